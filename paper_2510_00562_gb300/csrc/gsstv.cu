@@ -407,17 +407,15 @@ int gsstv_create(gsstv_handle** out, int n1, int n2, int n3, const gsstv_params*
     if (rc == GSSTV_OK) rc = dalloc(h, (void**)&h->v, (size_t)h->g.cube * sizeof(float));
     if (rc == GSSTV_OK) rc = dalloc(h, (void**)&h->sc, sizeof(Scal));
     if (rc == GSSTV_OK && (k1_configure(p->storage) != 0 || light_configure(p->storage) != 0 ||
-                           (p->storage == GSSTV_FP32 && k1_tma_configure(p->storage) != 0)))
+                           k1_tma_configure(p->storage) != 0))
         rc = GSSTV_ERR_CUDA;
     {
-        // The TMA-fed K1 serves float32 storage; 16-bit storage runs the
-        // cooperative-load K1.  GSSTV_K1=coop (a debugging aid) selects the
-        // cooperative kernel for float32 too.
+        // GSSTV_K1=coop (a debugging aid) selects the cooperative-load kernel
         const char* ev = std::getenv("GSSTV_K1");
-        h->k1_variant = (p->storage == GSSTV_FP32 && !(ev && std::strcmp(ev, "coop") == 0)) ? 1 : 0;
+        h->k1_variant = ev && std::strcmp(ev, "coop") == 0 ? 0 : 1;
     }
     h->k1_ctas = std::max(k1_grid_ctas(h->g), k1_tma_ctas(h->g));
-    h->k2_cap = k2_grid_ctas(h->g);
+    h->k2_cap = k2_grid_ctas(p->storage, h->g);
     if (rc == GSSTV_OK) rc = dalloc(h, (void**)&h->l1.cand[0], kCandCap * sizeof(float));
     if (rc == GSSTV_OK) rc = dalloc(h, (void**)&h->l1.cand[1], kCandCap * sizeof(float));
     if (rc == GSSTV_OK) rc = dalloc(h, (void**)&h->l1.hcnt, 2 * kHistBins * sizeof(unsigned long long));
@@ -433,9 +431,9 @@ int gsstv_create(gsstv_handle** out, int n1, int n2, int n3, const gsstv_params*
         for (auto& e : h->ev)
             if (rc == GSSTV_OK && cudaEventCreate(&e) != cudaSuccess) { e = nullptr; rc = GSSTV_ERR_CUDA; }
     }
-    for (int par = 0; par < 2 && rc == GSSTV_OK && h->k1_variant == 1; ++par) {
+    for (int par = 0; par < 2 && rc == GSSTV_OK && h->k1_variant == 1 && p->storage == GSSTV_FP32; ++par) {
         const IterBufs b = bufs(h, par);
-        if (k1_tma_maps(p->storage, h->g, b, &h->maps[par]) != 0) rc = GSSTV_ERR_CUDA;
+        if (k1_tma_maps(h->g, b, &h->maps[par]) != 0) rc = GSSTV_ERR_CUDA;
     }
     if (rc == GSSTV_OK) rc = upload_scalars(h, initial_scalars(h->p));
     if (rc != GSSTV_OK) {
@@ -657,7 +655,7 @@ int gsstv_autotune(gsstv_handle* h, int passes, int* chunk_out) {
     destroy_graphs(h);                                  // graphs hold the old launch shape
     TRY(rc);
     TRY(gsstv_reset_state(h));
-    if (chunk_out) *chunk_out = h->k1_chunk;
+    if (chunk_out) *chunk_out = std::max(h->k1_chunk, std::min(8, h->g.n3));
     return GSSTV_OK;
 }
 
@@ -1446,19 +1444,16 @@ int gsstv_slabs_create(gsstv_slabs** out, int n1, int n2, int n3, int nslabs, co
     if (rc == GSSTV_OK) {
         // each stage's launches, numbered across the slabs
         std::vector<int> gk1, gw, gr, gg, gk2;
-        int max_chunk = 0;
         for (int s = 0; s < nslabs; ++s) {
             const Geom& g = G->h[s]->g;
             const int c = k1_tma_part_chunk(g, G->k1p[s], 0);
             G->k1_chunk.push_back(c);
-            max_chunk = std::max(max_chunk, c);
             gk1.push_back(k1_tma_grid(g, G->k1p[s], c));
             gw.push_back(window_grid(g, G->winp[s], 1 << 30));
             gr.push_back(radix_grid(g, G->radp[s]));
             gg.push_back(gather_grid(g, G->gatp[s]));
             gk2.push_back(k2_grid(g, G->k2p[s], 1 << 30));
         }
-        for (auto& sp : G->k1p) sp.max_chunk = max_chunk;
         number_stage(G->k1p, gk1);
         number_stage(G->winp, gw);
         number_stage(G->radp, gr);

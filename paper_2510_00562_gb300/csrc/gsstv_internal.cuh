@@ -201,12 +201,18 @@ struct L1Work {
 // ---------------------------------------------------------------------------
 // small numerics helpers
 // ---------------------------------------------------------------------------
+// A compensated float sum, value s - c.  The exact rounding error of every
+// addition (Knuth's two-sum) is collected, so the sum of n values is good to
+// about n 2^-48: thresholds found from differently split sums then agree to
+// their float rounding (with Kahan's update, which rounds each corrected
+// addend, they differed by 1e-10, and one threshold in a few hundred passes by
+// a float ulp).
 struct Kahan {
     float s = 0.f, c = 0.f;
     __device__ __forceinline__ void add(float x) {
-        float y = x - c;
-        float t = s + y;
-        c = (t - s) - y;
+        const float t = __fadd_rn(s, x);
+        const float b = __fsub_rn(t, s);
+        c = __fsub_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)));
         s = t;
     }
     __device__ __forceinline__ double value() const { return (double)s - (double)c; }
@@ -384,7 +390,7 @@ struct IterParams {
 
 // Tensor maps over the current-parity buffers read by the TMA-fed K1.
 struct K1Maps {
-    CUtensorMap y1, y2, w1, w2, u, q, s, t, y3;
+    CUtensorMap y1v, y1h, y2v, y2h, w1, w2, u, q, s, t, y3;
 };
 
 // The bands one launch updates when a cube is stored as band slabs in
@@ -399,7 +405,6 @@ struct K1Maps {
 struct SlabPart {
     int band0 = 0, n3g = 0, o0 = 0, o1 = 0;
     int cta_base = 0, cta_total = 0;     // cta_total = 0: this launch alone
-    int max_chunk = 0;                   // K1: the longest band run of any launch of the stage
 };
 inline SlabPart whole_cube(const Geom& g) {
     SlabPart s;
@@ -411,12 +416,12 @@ inline SlabPart whole_cube(const Geom& g) {
 int k1_tma_ctas(const Geom& g);
 int k1_tma_chunk_candidates(const Geom& g, int* out, int cap);
 int k1_tma_configure(int storage);
-int k1_tma_maps(int storage, const Geom& g, const IterBufs& b, K1Maps* m);
-// CTAs of one K1 launch over the part's bands, and its bands per CTA (chunk
+int k1_tma_maps(const Geom& g, const IterBufs& b, K1Maps* m);
+// CTAs of one K1 launch over the part's bands, and its bands per item (chunk
 // as for launch_k1_tma)
 int k1_tma_grid(const Geom& g, const SlabPart& sp, int chunk);
 int k1_tma_part_chunk(const Geom& g, const SlabPart& sp, int chunk);
-// chunk: bands per CTA (0 or out of range: the wave/prologue model's choice)
+// chunk: bands per item (0 or out of range: the model's choice)
 int launch_k1_tma(int storage, const Geom& g, const K1Maps& m, const IterBufs& b, const IterParams& p,
                   Scal* sc, const L1Work& w, int chunk, const SlabPart& sp, cudaStream_t st);
 
@@ -451,7 +456,7 @@ int launch_search_gate(Scal* const* sc, int n, cudaGraphConditionalHandle cond, 
 int launch_search_finish(int mode, Scal* sc, const L1Work& w, int nvec, const unsigned long long* pn,
                          const double* ps, int parts, cudaStream_t st, int gated = 0,
                          cudaGraphConditionalHandle cond = 0);
-int k2_grid_ctas(const Geom& g);
+int k2_grid_ctas(int storage, const Geom& g);
 
 // ---------------------------------------------------------------------------
 // batches: every stage of a pass launched once for many independent cubes
@@ -476,6 +481,8 @@ struct BatchCube {
 };
 // Each launches one stage for cubes[0..n) on st (n <= kBatchMax).
 int launch_k1_batch(const BatchCube* cubes, int n, cudaStream_t st);
+// how launch_k1_batch splits the cubes: bands per item, band runs and CTAs of each
+void k1_batch_plan(const BatchCube* cubes, int n, int* chunk, int* gz, int* ctas);
 int launch_window_batch(const BatchCube* cubes, int n, cudaStream_t st);
 int launch_radix_batch(const BatchCube* cubes, int n, int level, cudaStream_t st);
 int launch_gather_batch(const BatchCube* cubes, int n, cudaStream_t st);

@@ -1,5 +1,5 @@
-// Tensor-memory-accelerator (TMA) helpers: host-side tensor-map encoding and
-// the device-side PTX for bulk tensor loads completed through mbarriers.
+// Tensor-memory-accelerator (TMA) helpers: the device-side PTX for bulk tensor
+// loads completed through mbarriers.
 //
 // Every wait on an mbarrier is bounded: after kMbarSpinLimit failed polls the
 // caller gets `false` and is expected to flag a timeout, drain its own loads
@@ -34,6 +34,10 @@ __device__ __forceinline__ void mbar_fence_init() {
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, unsigned bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                  : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, unsigned parity) {
@@ -78,14 +82,5 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
         "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
         : "memory");
 }
-
-// ---------------------------------------------------------------------------
-// host side
-// ---------------------------------------------------------------------------
-// Encodes a 3-D tiled map over `ncubes` stacked pitched cubes of `elem_bytes`
-// elements: dims (n2, n1, n3 * ncubes), row pitch p2 elements, box
-// (box_x, box_y, 1), zero fill outside.  Returns 0 on success.
-int tma_encode_cubes(CUtensorMap* map, const void* base, int elem_bytes, int n1, int n2, int n3,
-                     int p2, int ncubes, int box_x, int box_y);
 
 }  // namespace gsstv

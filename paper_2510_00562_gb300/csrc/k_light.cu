@@ -1057,7 +1057,7 @@ int launch_search_finish(int mode, Scal* sc, const L1Work& w, int nvec, const un
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
-int k2_grid_ctas(const Geom& g) { return k2_grid_part(g, whole_cube(g)); }
+int k2_grid_ctas(int, const Geom& g) { return k2_grid_part(g, whole_cube(g)); }
 
 int window_grid(const Geom& g, const SlabPart& sp, int part_cap) {
     return window_grid_n(part_voxels(g, sp), part_cap);
@@ -1171,8 +1171,11 @@ int launch_finish_batch(const BatchCube* cubes, int n, int mode, cudaStream_t st
                         cudaGraphConditionalHandle cond) {
     SearchBatchTab t{};
     if (search_table(cubes, n, t, [](const BatchCube&, const SlabPart&) { return 1; }) < 0) return -1;
-    if (mode == 2)                       // K1's partials: one set per CTA of the cube's K1 grid
-        for (int c = 0; c < n; ++c) t.c[c].parts = k1_tma_grid(cubes[c].g, whole_cube(cubes[c].g), cubes[c].k1_chunk);
+    if (mode == 2) {                     // K1's partials: one set per CTA of the cube's share of K1
+        int chunk[kBatchMax], gz[kBatchMax], ctas[kBatchMax];
+        k1_batch_plan(cubes, n, chunk, gz, ctas);
+        for (int c = 0; c < n; ++c) t.c[c].parts = ctas[c];
+    }
     k_finish_batch<<<2 * n, kFinishThreads, kFinishSmem, st>>>(t, mode, gated, cond);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }

@@ -1,27 +1,38 @@
-// K1, TMA-fed: the fused stencil pass of one P-PDS iteration (Algorithm 1),
-// float32 storage.
+// K1, the fused stencil pass of one P-PDS iteration (Algorithm 1).
 //
-// Same arithmetic as the cooperative-load kernel in k_stencil.cu (u step and
-// u' for band b+1; w1, w2 group soft-thresholds and w' on the tile plus a
-// one-pixel ring; y1, y2 ascent; window statistics of the l1 threshold
-// search), fed differently: each band's planes are brought into shared memory
-// by bulk tensor (TMA) copies that one thread issues two bands ahead,
-// completing on mbarriers.  One CTA of 512 threads per SM owns a 16 x 32 tile
-// and a run of bands.  Tiles whose halo stays off the image border take a
-// specialised path with no boundary masks.  Each CTA leaves its window
-// statistics and candidates (with their key histogram) for the finishing
-// launch that follows (k_search_finish, one CTA per vector), so that no CTA
-// of this launch runs the threshold search while the rest of the GPU idles.
+// For each band: the u step and u' of the next band; the w1, w2 group
+// soft-thresholds and w' on the tile plus a one-pixel ring; the y1, y2 ascent;
+// the window statistics of the l1 threshold search.  Tiles whose halo stays
+// off the image border take a specialised path with no boundary masks.
 //
-// Band march, one CTA barrier per band: while the w steps, u' of band b+1 and
-// the window statistics of band b run, the dual ascent of band b-1 (which
-// reads the w' and u' that the previous step completed) runs beside them.
-// Each thread keeps the four y values of its own voxel that the ascent needs
-// in registers for one band, so a y-group slot is free again as soon as its
-// band's w step is done: 3 y-group slots (y1, y2 with a 2-pixel halo, u and q
-// with a 1-pixel halo below/right, s, t, y3 with one row above) and 4 slots of
-// the 12 w planes (1-pixel halo, w' written in place) fit beside u' of three
-// bands and D^T y2 of the previous band: about 216 KB of shared memory.
+// One persistent CTA per SM works through (tile, band run) items, in the order
+// in which neighbouring tiles run at the same time over the same bands (their
+// halos then meet in L2).  Its warps have roles:
+//   16 tile warps   one voxel of the 16 x 32 tile per thread;
+//   2 ring warps    the one-pixel ring of w' and of u' (49 positions).  The
+//                   ascent reads on the ring only grid 0 above and right of the
+//                   tile, grid 1 below and left, grid 2 below and right, so 49
+//                   lanes with one position per grid cover it: the work of a
+//                   tile warp without its stores, and no tile warp does ring
+//                   work on top of its own before the band barrier;
+//   load warps      bring each band's planes into shared-memory rings, as far
+//                   ahead as slots are free and across item boundaries: one
+//                   warp of bulk tensor (TMA) copies for float32 storage, two
+//                   of 8-byte cp.async for 16-bit storage (the planes stay
+//                   16-bit in shared memory and are widened as they are read).
+// Full / empty mbarriers per slot couple the load warps to the others.  Every
+// wait is bounded; a wait that gives up raises a flag that ends the CTA.
+//
+// Band step, one barrier phase per band (an mbarrier with an arrival per
+// warp, so that arriving and waiting are apart): the dual ascent of the
+// previous band (it reads the w' and u' that the previous phase published);
+// the w steps and u' of the next band; arrive; the window statistics of the
+// next band, which nobody waits for, fill the time until the others arrive.
+// Each thread keeps the four y values of its own voxel that the ascent needs,
+// and D^T y2 of the previous band at its own u' position, in registers.
+//
+// What bounds it: instruction issue and the latency of 18 warps' dependency
+// chains (about 0.77 of the copy bandwidth on cubes that fill the GPU).
 #include <algorithm>
 #include <vector>
 #include <cmath>
@@ -54,14 +65,16 @@ EncodeFn encode_fn() {
 }
 }  // namespace
 
-int tma_encode_cubes(CUtensorMap* map, const void* base, int elem_bytes, int n1, int n2, int n3, int p2,
-                     int ncubes, int box_x, int box_y) {
+// A 3-D tiled map over `ncubes` stacked pitched float32 cubes of geometry g, of
+// which the first n1 rows and n2 columns of each band exist (zero fill outside),
+// box (box_x, box_y, 1).  Returns 0 on success.
+static int tma_encode_cubes(CUtensorMap* map, const void* base, const Geom& g, int n1, int n2, int ncubes, int box_x,
+                            int box_y) {
     EncodeFn fn = encode_fn();
     if (!fn) return -3;
-    const CUtensorMapDataType dt = elem_bytes == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-                                                   : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;  // 16-bit: bits only
-    cuuint64_t dims[3] = {(cuuint64_t)n2, (cuuint64_t)n1, (cuuint64_t)n3 * (cuuint64_t)ncubes};
-    cuuint64_t strides[2] = {(cuuint64_t)p2 * elem_bytes, (cuuint64_t)p2 * elem_bytes * n1};
+    const CUtensorMapDataType dt = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+    cuuint64_t dims[3] = {(cuuint64_t)n2, (cuuint64_t)n1, (cuuint64_t)g.n3 * (cuuint64_t)ncubes};
+    cuuint64_t strides[2] = {(cuuint64_t)g.p2 * 4u, (cuuint64_t)g.p2 * 4u * g.n1};
     cuuint32_t box[3] = {(cuuint32_t)box_x, (cuuint32_t)box_y, 1u};
     cuuint32_t estr[3] = {1u, 1u, 1u};
     const CUresult r = fn(map, dt, 3, const_cast<void*>(base), dims, strides, box, estr,
@@ -72,65 +85,66 @@ int tma_encode_cubes(CUtensorMap* map, const void* base, int elem_bytes, int n1,
 
 namespace {
 
+
 constexpr int pad128(int b) { return (b + 127) / 128 * 128; }
 
+constexpr int TY = 16, TX = 32;
+constexpr int OX = 4;                    // left halo columns: staged rows start 16-byte (16-bit: 8-byte) aligned
+constexpr int SW = TX + 2 * OX;          // width of the staged planes
+constexpr int YR = TY + 4, WR = TY + 2, UR = TY + 1, UC = TX + 1;
+constexpr int kTileWarps = 16, kRingWarps = 2, kConsWarps = kTileWarps + kRingWarps;
+constexpr int kCandBuf = 256;            // window candidates buffered per item and vector
+constexpr int kMaxRun = 4064;            // bands per item at most (16-bit histogram counters, see k1_plan)
+static_assert(TY * TX == 32 * kTileWarps, "one tile voxel per tile thread");
+
+template <typename T>
 struct Lay {
-    static constexpr int TY = 16, TX = 32, NT = 512;
-    static constexpr int OX = 4;                   // left halo columns: boxes start 16-byte aligned
-    static constexpr int SW = TX + 2 * OX;         // width of the staged planes
-    // the thread that issues the bulk copies: lane 0 of warp 8, a warp with no
-    // ring items (the ring warps are 0-7, 10 and 15), so the serial copy issue
-    // does not lengthen the slowest warp of a band step
-    static constexpr int PRODUCER = 256;
-    static constexpr int YR = TY + 4, WR = TY + 2, UR = TY + 1, UC = TX + 1;
-    static constexpr int Y_B = pad128(YR * SW * 4);
-    static constexpr int W_B = pad128(WR * SW * 4);
-    static constexpr int U_B = pad128(UR * SW * 4);
-    static constexpr int S_B = pad128(TY * TX * 4);
-    static constexpr int Y3_B = pad128((TY + 1) * TX * 4);
+    static constexpr bool F32 = std::is_same<T, float>::value;
+    static constexpr int LW = F32 ? 1 : 2;               // load warps
+    static constexpr int NT = 32 * (kConsWarps + LW);
+    static constexpr int ES = (int)sizeof(T);
+    static constexpr int Y_B = pad128(YR * SW * ES);
+    static constexpr int W_B = pad128(WR * SW * ES);
+    static constexpr int U_B = pad128(UR * SW * ES);
+    static constexpr int S_B = pad128(TY * TX * ES);
+    static constexpr int Y3_B = pad128((TY + 1) * TX * ES);
     static constexpr int YG_B = 4 * Y_B + 2 * U_B + 2 * S_B + Y3_B;
     static constexpr int WG_B = 12 * W_B;
-    static constexpr int NYS = 3, NWS = 4, NUS = 3;  // ring depths: y-group, w, u'
-    static constexpr int UP1 = UR * UC;              // floats of one u' plane
-    static constexpr int UP_B = pad128(NUS * UP1 * 4);
-    static constexpr int G_B = pad128(UR * UC * 4);
-    static constexpr int CB = 256;                   // window candidates buffered per CTA and vector
+    // ring depths: y-group, w, u'.  float32 w' overwrites w in place, so a w
+    // slot is held one band longer (until the ascent has read it); 16-bit
+    // storage keeps float32 w' in two slots of its own
+    static constexpr int NYS = 3, NWS = F32 ? 4 : 3, NUS = 3, NPS = F32 ? 0 : 2;
+    static constexpr int UP1 = UR * UC;                  // floats of one u' plane
+    static constexpr int WPL = pad128(WR * SW * 4) / 4;  // floats of one w' plane
     static constexpr int OFF_WG = NYS * YG_B;
-    static constexpr int OFF_UP = OFF_WG + NWS * WG_B;
-    static constexpr int OFF_G = OFF_UP + UP_B;
-    static constexpr int OFF_CB = OFF_G + G_B;
-    static constexpr int OFF_HIST = OFF_CB + 2 * CB * 4;      // K1 histogram: 2 x kK1Bins packed 16-bit counts
+    static constexpr int OFF_WP = OFF_WG + NWS * WG_B;
+    static constexpr int OFF_UP = OFF_WP + NPS * 12 * WPL * 4;
+    static constexpr int OFF_CB = OFF_UP + pad128(NUS * UP1 * 4);
+    static constexpr int OFF_HIST = OFF_CB + 4 * kCandBuf * 4;    // K1 histogram: 2 x kK1Bins packed 16-bit counts
     static constexpr int OFF_BAR = OFF_HIST + kK1Bins * 4;
-    static constexpr int SMEM = OFF_BAR + (NYS + NWS) * 8;
-    // float offsets inside a y-group slot, and between planes
-    static constexpr int YPL = Y_B / 4, WPL = W_B / 4;
-    static constexpr int O_U = 4 * YPL, O_Q = O_U + U_B / 4, O_S = O_Q + U_B / 4, O_T = O_S + S_B / 4,
-                         O_Y3 = O_T + S_B / 4;
-    // bytes each group's copies deliver
-    static constexpr unsigned YG_TX = 4u * YR * SW * 4 + 2u * UR * SW * 4 + 2u * TY * TX * 4 + (TY + 1u) * TX * 4;
-    static constexpr unsigned WG_TX = 12u * WR * SW * 4;
-    // one-pixel ring: w positions 2 (TX + 2) + 2 TY per set, u' positions (TX + 1) + TY
-    static constexpr int NWR = 2 * (TX + 2) + 2 * TY, NUR = (TX + 1) + TY;
-    static_assert(TY * TX == NT, "one tile voxel per thread");
-    // dynamic plus the kernel's static shared memory (the candidate counters:
-    // 128 bytes, see ptxas -v) within the 227 KB a CTA may use
-    static_assert(SMEM + 256 <= 227 * 1024, "shared memory");
-    // the ring work layout (see k1_tile): per set 4 warps of 4 + 4 column and
-    // 17 row items; the u' ring on 2 warps of 8 column items and at most 17
-    // row items
-    static_assert(NWR == 4 * (4 + 4 + 17) && TY == 16 && NUR == 2 * 8 + (TX + 1) && TX + 1 <= 2 * 17,
-                  "ring work layout");
+    static constexpr int SMEM = OFF_BAR + (2 * NYS + 2 * NWS + 1) * 8;
+    // element offsets inside a y-group slot, and between raw planes
+    static constexpr int YPL = Y_B / ES, WRAW = W_B / ES;
+    static constexpr int O_U = 4 * YPL, O_Q = O_U + U_B / ES, O_S = O_Q + U_B / ES, O_T = O_S + S_B / ES,
+                         O_Y3 = O_T + S_B / ES;
+    // bytes each group's bulk copies deliver
+    static constexpr unsigned YG_TX = ES * (4u * YR * SW + 2u * UR * SW + 2u * TY * TX + (TY + 1u) * TX);
+    static constexpr unsigned WG_TX = ES * 12u * WR * SW;
+    // dynamic plus the kernel's static shared memory within the 227 KB a CTA may use
+    static_assert(SMEM + 512 <= 227 * 1024, "shared memory");
+    static_assert(!F32 || WPL == WRAW, "w' in place");
 };
 
-struct K1TArgs {
+template <typename T>
+struct K1Args {
     Geom g;
-    float *u_n, *w1_n, *w2_n, *y1_n, *y2_n;
+    const T *u, *q, *s, *t, *y3, *y1, *y2, *w1, *w2;
+    T *u_n, *w1_n, *w2_n, *y1_n, *y2_n;
     IterParams p;
     Scal* sc;
     L1Work l1;
-    int chunk;
+    int chunk;          // bands per item
     SlabPart sp;
-    int hist_fits;      // every CTA of the stage counts at most 65535 voxels
 };
 
 // Window of the l1 threshold search for this launch (see gsstv_l1.cuh), and
@@ -140,25 +154,42 @@ struct K1Win {
     float lo_s, hi_s, lo_t, hi_t;
     bool hs, ht;
     unsigned hb_s, hb_t;
-    // the candidate lists' key histograms over the windows (null: not kept)
-    unsigned *nh_s, *nh_t;
-    NarrowGeom ng_s, ng_t;
 };
 
-// A thread's window statistics: count (a CTA covers at most a few thousand
-// voxels per thread slot, so 32 bits suffice) and compensated sum.
+// A thread's count and sum of sampled values above the histogram's range.
 struct K1Acc {
     unsigned n = 0;
-    Kahan s;
+    float s = 0.f;
 };
 
-// Per-CTA running state shared by the two tile paths.
-struct K1State {
-    K1Acc acc_s, acc_t;
-    float2 ks = make_float2(0.f, 0.f), kc = make_float2(0.f, 0.f);   // packed window sums (s, t)
-    K1Acc top_s, top_t;          // |x| above the histogram's range
-    unsigned n_y = 0, n_w = 0;   // groups issued so far (thread 0 only)
+// A thread's window statistics (a CTA covers at most a few thousand voxels per
+// thread slot, so 32-bit counts suffice), the compensated sums of s and t packed.
+struct K1Stat {
+    unsigned n_s = 0, n_t = 0;
+    float2 ks = make_float2(0.f, 0.f), kc = make_float2(0.f, 0.f);
+    K1Acc top_s, top_t;
 };
+
+// A position in a ring of N slots and the phase parity of its next use.
+template <int N>
+struct Ring {
+    int slot = 0;
+    unsigned ph = 0;
+    __device__ __forceinline__ void next() {
+        if (++slot == N) { slot = 0; ph ^= 1u; }
+    }
+};
+
+// Bounded wait that also gives up once another warp of the CTA has.
+__device__ __forceinline__ bool k1_wait(uint64_t* bar, unsigned parity, volatile int* abort) {
+    if (mbar_try_wait(bar, parity)) return true;
+    for (unsigned k = 0; k < kMbarSpinLimit; ++k) {
+        if (mbar_try_wait(bar, parity)) return true;
+        if ((k & 255u) == 255u && *abort) return false;
+    }
+    *abort = 1;
+    return false;
+}
 
 // Appends the lanes' window candidates to the CTA's shared buffer (one
 // shared-memory atomic per warp); values past its end go straight to the
@@ -175,11 +206,37 @@ __device__ __forceinline__ void append_shared(bool take, float x, float* buf, un
     if (lane == leader) base = atomicAdd(cnt, (unsigned)__popc(mask));
     base = __shfl_sync(0xffffffffu, base, leader);
     const unsigned k = base + __popc(mask & ((1u << lane) - 1u));
-    if (take && k < (unsigned)Lay::CB) buf[k] = x;
-    if (base + __popc(mask) > (unsigned)Lay::CB) {
-        const bool over = take && k >= (unsigned)Lay::CB;
+    if (take && k < (unsigned)kCandBuf) buf[k] = x;
+    if (base + __popc(mask) > (unsigned)kCandBuf) {
+        const bool over = take && k >= (unsigned)kCandBuf;
         append_candidate(over, x, cand, gcnt);
     }
+}
+
+// One warp: the buffered candidates of vector v join the global list (one
+// atomic) and its key histogram over the window, which the finish then narrows
+// without another pass over the candidates.
+__device__ __forceinline__ void flush_candidates(int v, float* buf, unsigned* cnt, Scal* sc, const L1Work& l1,
+                                              float lo, float hi) {
+    const int lane = threadIdx.x & 31;
+    const unsigned n = min(*cnt, (unsigned)kCandBuf);
+    if (n == 0) return;
+    unsigned base = 0;
+    if (lane == 0) base = atomicAdd(&sc->acc[v].m, n);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    const NarrowGeom ng = narrow_geom(__float_as_uint(lo), __float_as_uint(hi));
+    unsigned* h = l1.nh && ng.ok ? l1.nh + v * 3 * kNarrowBins : nullptr;
+    for (unsigned k = lane; k < n; k += 32u) {
+        const float x = buf[k];
+        if (base + k < kCandCap) l1.cand[v][base + k] = x;
+        if (h) narrow_add(h, ng, __float_as_uint(x));
+    }
+    __syncwarp();
+    if (lane == 0) {
+        if (h) atomicAdd(l1.nbinned + v, n);
+        *cnt = 0u;
+    }
+    __syncwarp();
 }
 
 // Counts x into the CTA's histogram (bins of the float key >> kHistShift from
@@ -193,13 +250,7 @@ __device__ __forceinline__ void hist_add(bool on, float x, unsigned hb, unsigned
     // above the range: an estimate from a sample, a plain sum suffices
     const bool up = on && !in && kb >= hb + (unsigned)kK1Bins;
     top.n += up ? 1u : 0u;
-    top.s.s += up ? x : 0.f;
-}
-
-// value of a set selector: an int, or a std::integral_constant
-template <typename X> __device__ __forceinline__ constexpr int set_of(X x) {
-    if constexpr (std::is_integral<X>::value) return x;
-    else return X::value;
+    top.s += up ? x : 0.f;
 }
 
 // Packed FP32 pairs (two lanes per instruction on sm_100 and later), used for
@@ -211,228 +262,225 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.f, -1.f), a); }
 
-using Set0 = std::integral_constant<int, 0>;
-using Set1 = std::integral_constant<int, 1>;
-using Store = std::true_type;
-using NoStore = std::false_type;
+// What a CTA's warps share: shared-memory regions and barriers.
+template <typename T>
+struct Sm {
+    unsigned char* sm;
+    uint64_t *yfull, *yempty, *wfull, *wempty, *evt;
+    unsigned* ccnt;
+    int* abort;
+    __device__ __forceinline__ Sm(unsigned char* p, unsigned* c, int* ab) : sm(p), ccnt(c), abort(ab) {
+        using L = Lay<T>;
+        yfull = reinterpret_cast<uint64_t*>(p + L::OFF_BAR);
+        yempty = yfull + L::NYS;
+        wfull = yempty + L::NYS;
+        wempty = wfull + L::NWS;
+        evt = wempty + L::NWS;
+    }
+    __device__ __forceinline__ T* yg(int slot) const { return reinterpret_cast<T*>(sm + slot * Lay<T>::YG_B); }
+    __device__ __forceinline__ T* wg(int slot) const {
+        return reinterpret_cast<T*>(sm + Lay<T>::OFF_WG + slot * Lay<T>::WG_B);
+    }
+    // w' of a band: in place of w (float32), or the band's slot of its own
+    __device__ __forceinline__ float* wp(int wslot, int pslot) const {
+        if constexpr (Lay<T>::F32) return reinterpret_cast<float*>(wg(wslot));
+        else return reinterpret_cast<float*>(sm + Lay<T>::OFF_WP) + pslot * (12 * Lay<T>::WPL);
+    }
+    __device__ __forceinline__ float* up(int slot) const {
+        return reinterpret_cast<float*>(sm + Lay<T>::OFF_UP) + slot * Lay<T>::UP1;
+    }
+    // candidates of vector v of an even or odd item: filled during the item,
+    // emptied while the next one fills the other
+    __device__ __forceinline__ float* cbuf(int v, int odd) const {
+        return reinterpret_cast<float*>(sm + Lay<T>::OFF_CB) + (2 * odd + v) * kCandBuf;
+    }
+    __device__ __forceinline__ unsigned* cnt(int v, int odd) const { return ccnt + 2 * odd + v; }
+    __device__ __forceinline__ unsigned* hist() const { return reinterpret_cast<unsigned*>(sm + Lay<T>::OFF_HIST); }
+};
 
-template <bool EDGE, bool HIST>
-__device__ __forceinline__ bool k1_tile(const K1Maps& M, const K1TArgs& a, unsigned char* sm, unsigned* ccnt,
-                                        int i0, int j0, int b0, int b1, K1State& S, const K1Win& W, float cs) {
-    using L = Lay;
-    constexpr int TY = L::TY, TX = L::TX, SW = L::SW, OX = L::OX, UC = L::UC;
-    constexpr int YPL = L::YPL, WPL = L::WPL;
+// One item: a tile's first row and column, and its bands [b0, b1).
+struct Item {
+    int i0, j0, b0, b1;
+};
+template <typename T>
+__device__ __forceinline__ Item item_of(const K1Args<T>& a, int it, int gx, int gy) {
+    const int bx = it % gx, r = it / gx;
+    const int by = r % gy, bz = r / gy;
+    Item m;
+    m.i0 = by * TY;
+    m.j0 = bx * TX;
+    m.b0 = a.sp.o0 + bz * a.chunk;
+    m.b1 = min(a.sp.o1, m.b0 + a.chunk);
+    return m;
+}
+__device__ __forceinline__ bool item_edge(const Item& m, const Geom& g) {
+    return !(m.i0 >= 2 && m.i0 + TY + 3 <= g.n1 && m.j0 >= 2 && m.j0 + TX + 3 <= g.n2);
+}
+
+// Ring positions and phases of a warp that consumes bands (kept across items).
+template <typename T>
+struct Cons {
+    Ring<Lay<T>::NYS> y;        // the next band's y-group
+    Ring<Lay<T>::NWS> w;        // the current band's w
+    int us = 0, ps = 0;         // u' slot of the next band, w' slot of the current one (16-bit)
+    unsigned ev = 0;            // parity of the next barrier phase
+    __device__ __forceinline__ void arrive(const Sm<T>& S) {
+        // float32: slots freed by this phase are reloaded by TMA: order this
+        // thread's generic accesses before those async-proxy writes
+        if constexpr (Lay<T>::F32) fence_proxy_async_smem();
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) mbar_arrive(S.evt);
+    }
+    __device__ __forceinline__ bool wait(const Sm<T>& S) {
+        const bool ok = k1_wait(S.evt, ev, S.abort);
+        ev ^= 1u;
+        return __all_sync(0xffffffffu, ok);
+    }
+};
+
+// D^T y2 of one band at row gi, column gj of the image, from global memory (y2
+// of the band at yv, yh): what D_s^T needs of the band before an item's first
+template <bool EDGE, typename T>
+__device__ __forceinline__ float dty_global(const T* yv, const T* yh, int gi, int gj, const Geom& g) {
+    const long long k = (long long)gi * g.p2 + gj;
+    if constexpr (EDGE) {
+        if (gi >= g.n1 || gj >= g.n2) return 0.f;
+        float d = 0.f;
+        if (gi >= 1) d += ldT(yv + k - g.p2);
+        if (gi <= g.n1 - 2) d -= ldT(yv + k);
+        if (gj >= 1) d += ldT(yh + k - 1);
+        if (gj <= g.n2 - 2) d -= ldT(yh + k);
+        return d;
+    } else {
+        return ((ldT(yv + k - g.p2) - ldT(yv + k)) + ldT(yh + k - 1)) - ldT(yh + k);
+    }
+}
+
+// u step (Eq. 21) and u' of one band at tile position (r, c) in [0, TY] x
+// [0, TX]: u' goes to upb, D^T y2 of the band replaces gprev (that of the
+// band before); returns u+.  gb: the band's place in the whole cube.
+template <bool EDGE, typename T>
+__device__ __forceinline__ float u_item(const K1Args<T>& a, const T* ys, float* upb, int gb, int r, int c, int gi,
+                                        int gj, float cs, float& gprev) {
+    using L = Lay<T>;
+    constexpr int YPL = L::YPL;
+    const Geom& g = a.g;
+    const IterParams& P = a.p;
+    const int kc = r * UC + c;
+    if constexpr (EDGE) {
+        if (gi >= g.n1 || gj >= g.n2) { upb[kc] = 0.f; gprev = 0.f; return 0.f; }
+    }
+    const int k = (r + 2) * SW + (c + OX);
+    float d1, gcur;                                 // D^T y1 and D^T y2 of the band
+    {
+        const T *v1 = ys + k, *h1 = ys + YPL + k, *v2 = ys + 2 * YPL + k, *h2 = ys + 3 * YPL + k;
+        const float2 d = sub2(add2(sub2(f2(ldT(v1 - SW), ldT(v2 - SW)), f2(ldT(v1), ldT(v2))),
+                                   f2(ldT(h1 - 1), ldT(h2 - 1))), f2(ldT(h1), ldT(h2)));
+        d1 = d.x;
+        gcur = d.y;
+    }
+    // D_s^T at the band's place in the whole cube (Neumann at its ends)
+    float dst_ = 0.f;
+    if (gb >= 1) dst_ += gprev;
+    if (gb <= a.sp.n3g - 2) dst_ -= gcur;
+    const int ku = r * SW + (c + OX);
+    const float y4 = cs * ldT(ys + L::O_Q + ku);
+    const float u = ldT(ys + L::O_U + ku);
+    const float un = fminf(fmaxf(u - P.gamma_u * (d1 + dst_ + y4), P.mu_lo), P.mu_hi);
+    upb[kc] = 2.f * un - u;
+    gprev = gcur;
+    return un;
+}
+
+// The eight dual entries that L reads at a grid position.
+struct YN {
+    float v00, vm0, v01, vm1, h00, h0m, h10, h1m;
+};
+template <typename T>
+__device__ __forceinline__ YN load_yn(const T* yv, const T* yh) {
+    YN y;
+    y.v00 = ldT(yv); y.vm0 = ldT(yv - SW); y.v01 = ldT(yv + 1); y.vm1 = ldT(yv - SW + 1);
+    y.h00 = ldT(yh); y.h0m = ldT(yh - 1); y.h10 = ldT(yh + SW); y.h1m = ldT(yh + SW - 1);
+    return y;
+}
+
+// (L_v, L_h) at the three grids of one position: the dual entries themselves,
+// the four-point means and the centred means.
+template <bool EDGE>
+__device__ __forceinline__ void l_pairs(const YN& y, bool mv, bool mh, float2 (&Lg)[3]) {
+    // (v, h) pairs: the centred means 0.5 (v00 + vm0), 0.5 (h00 + h0m), and
+    // the four-point means 0.25 (v00 + vm0 + v01 + vm1), 0.25 (h00 + h0m + h10 + h1m)
+    float2 sum = add2(f2(y.v00, y.h00), f2(y.vm0, y.h0m));
+    Lg[2] = mul2(sum, f2(0.5f, 0.5f));
+    sum = add2(add2(sum, f2(y.v01, y.h10)), f2(y.vm1, y.h1m));
+    const float2 four = mul2(sum, f2(0.25f, 0.25f));
+    Lg[0] = f2(!EDGE || mv ? y.v00 : 0.f, !EDGE || mv ? four.y : 0.f);
+    Lg[1] = f2(!EDGE || mh ? four.x : 0.f, !EDGE || mh ? y.h00 : 0.f);
+}
+
+// w step of one set (0 = w1, 1 = w2) from L y at each grid's position and the
+// six w values wk (k = 2 grid + component): w+ replaces wk, w' goes to the
+// set's planes 2 grid, 2 grid + 1 of wp at offset kw[grid] where L's output is
+// not structurally zero (on[grid]), zero elsewhere: L^T then reads w' unmasked.
+template <int SET, bool EDGE, typename T>
+__device__ __forceinline__ void w_step(const IterParams& P, const float2 (&Lg)[3], float (&wk)[6], float* wp,
+                                       const int (&kw)[3], const bool (&on)[3]) {
+    constexpr int WPL = Lay<T>::WPL;
+    const float gam = SET ? P.gamma_w2 : P.gamma_w1;
+    const float thr = SET ? P.thr_w2 : P.thr_w1;
+#pragma unroll
+    for (int gr = 0; gr < 3; ++gr) {
+        const float wv = wk[2 * gr], wh = wk[2 * gr + 1];
+        const float2 x = fma2(f2(gam, gam), Lg[gr], f2(wv, wh));
+        const float xv = x.x, xh = x.y;
+        // Eq. 24: max(1 - thr / ||x||, 0) x
+        float sc;
+        if constexpr (Lay<T>::F32) {
+            // 1 / ||x|| from rsqrt
+            const float n2 = xv * xv + xh * xh;
+            sc = n2 > thr * thr ? fmaxf(1.f - thr * rsqrtf(n2), 0.f) : 0.f;
+        } else {
+            const float n = sqrtf(xv * xv + xh * xh);
+            sc = n > thr ? 1.f - thr / n : 0.f;
+        }
+        const float2 nn = mul2(f2(sc, sc), x);
+        wk[2 * gr] = nn.x;
+        wk[2 * gr + 1] = nn.y;
+        const float nv = 2.f * nn.x - wv, nh = 2.f * nn.y - wh;
+        wp[(6 * SET + 2 * gr) * WPL + kw[gr]] = !EDGE || on[gr] ? nv : 0.f;
+        wp[(6 * SET + 2 * gr + 1) * WPL + kw[gr]] = !EDGE || on[gr] ? nh : 0.f;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// tile warps: one item
+// ---------------------------------------------------------------------------
+template <typename T, bool EDGE, bool HIST>
+__device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, const Item& m, Cons<T>& C, K1Stat& A,
+                                          const K1Win& W, float cs, int turn) {
+    using L = Lay<T>;
+    constexpr int YPL = L::YPL, WPL = L::WPL, WRAW = L::WRAW;
     const Geom& g = a.g;
     const IterParams& P = a.p;
     const int tid = threadIdx.x;
     const unsigned cube = (unsigned)g.cube;        // 6 cubes < 2^32 elements (checked at handle creation)
     const unsigned plane = (unsigned)g.n1 * (unsigned)g.p2;
-    uint64_t* ybar = reinterpret_cast<uint64_t*>(sm + L::OFF_BAR);
-    uint64_t* wbar = ybar + L::NYS;
-    float* up = reinterpret_cast<float*>(sm + L::OFF_UP);
-    float* gs = reinterpret_cast<float*>(sm + L::OFF_G);
-    float* cbuf = reinterpret_cast<float*>(sm + L::OFF_CB);
-    unsigned* hsm = reinterpret_cast<unsigned*>(sm + L::OFF_HIST);
-    const int bstart = max(b0 - 1, 0);
-    const int blast = min(b1, g.n3 - 1);
-
-    // ---- ring slots ----
-    auto ygb = [&](int band) { return sm + ((unsigned)(band - bstart) % L::NYS) * L::YG_B; };
-    auto wgb = [&](int band) { return sm + L::OFF_WG + ((unsigned)(band - b0) % L::NWS) * L::WG_B; };
-    auto yg = [&](int band) { return reinterpret_cast<const float*>(ygb(band)); };
-    auto wg = [&](int band) { return reinterpret_cast<float*>(wgb(band)); };
-    auto upl = [&](int band) { return up + ((unsigned)band % L::NUS) * L::UP1; };
-
-    auto issue_y = [&](int band) {
-        unsigned char* s = ygb(band);
-        uint64_t* bar = ybar + (band - bstart) % L::NYS;
-        mbar_arrive_expect_tx(bar, L::YG_TX);
-        tma_load_3d(s + 0 * L::Y_B, &M.y1, j0 - OX, i0 - 2, band, bar);
-        tma_load_3d(s + 1 * L::Y_B, &M.y1, j0 - OX, i0 - 2, g.n3 + band, bar);
-        tma_load_3d(s + 2 * L::Y_B, &M.y2, j0 - OX, i0 - 2, band, bar);
-        tma_load_3d(s + 3 * L::Y_B, &M.y2, j0 - OX, i0 - 2, g.n3 + band, bar);
-        tma_load_3d(s + 4 * L::O_U, &M.u, j0 - OX, i0, band, bar);
-        tma_load_3d(s + 4 * L::O_Q, &M.q, j0 - OX, i0, band, bar);
-        tma_load_3d(s + 4 * L::O_S, &M.s, j0, i0, band, bar);
-        tma_load_3d(s + 4 * L::O_T, &M.t, j0, i0, band, bar);
-        tma_load_3d(s + 4 * L::O_Y3, &M.y3, j0, i0 - 1, band, bar);
-        S.n_y++;
-    };
-    auto issue_w = [&](int band) {
-        unsigned char* s = wgb(band);
-        uint64_t* bar = wbar + (band - b0) % L::NWS;
-        mbar_arrive_expect_tx(bar, L::WG_TX);
-        for (int k = 0; k < 6; ++k) tma_load_3d(s + k * L::W_B, &M.w1, j0 - OX, i0 - 1, k * g.n3 + band, bar);
-        for (int k = 0; k < 6; ++k) tma_load_3d(s + (6 + k) * L::W_B, &M.w2, j0 - OX, i0 - 1, k * g.n3 + band, bar);
-        S.n_w++;
-    };
-    auto wait_y = [&](int band) {
-        return mbar_wait(ybar + (unsigned)(band - bstart) % L::NYS, ((unsigned)(band - bstart) / L::NYS) & 1);
-    };
-    auto wait_w = [&](int band) { return mbar_wait(wbar + (unsigned)(band - b0) % L::NWS, ((unsigned)(band - b0) / L::NWS) & 1); };
-
-    // D^T y = D_v^T y_v + D_h^T y_h at tile-relative (r, c); yv, yh: y planes
-    auto dty = [&](const float* yv, const float* yh, int r, int c) {
-        const int k = (r + 2) * SW + (c + OX);
-        if constexpr (EDGE) {
-            const int gi = i0 + r, gj = j0 + c;
-            float d = 0.f;
-            if (gi >= 1) d += yv[k - SW];
-            if (gi <= g.n1 - 2) d -= yv[k];
-            if (gj >= 1) d += yh[k - 1];
-            if (gj <= g.n2 - 2) d -= yh[k];
-            return d;
-        } else {
-            return ((yv[k - SW] - yv[k]) + yh[k - 1]) - yh[k];
-        }
-    };
-    // u step and u' of band bb at (r, c) in [0, TY] x [0, TX]; ys: y-group of
-    // bb; upb: u' plane of bb; with Store, u+ goes to *dst when `st`
-    auto u_item = [&](auto store_c, const float* ys, float* upb, int bb, int r, int c, float* dst, bool st) {
-        const int kc = r * UC + c;
-        if constexpr (EDGE) {
-            if (i0 + r >= g.n1 || j0 + c >= g.n2) { upb[kc] = 0.f; gs[kc] = 0.f; return; }
-        }
-        float d1, gcur;                                 // D^T y1 and D^T y2 of the band
-        if constexpr (EDGE) {
-            d1 = dty(ys, ys + YPL, r, c);
-            gcur = dty(ys + 2 * YPL, ys + 3 * YPL, r, c);
-        } else {
-            const int k = (r + 2) * SW + (c + OX);
-            const float *v1 = ys + k, *h1 = ys + YPL + k, *v2 = ys + 2 * YPL + k, *h2 = ys + 3 * YPL + k;
-            const float2 d = sub2(add2(sub2(f2(v1[-SW], v2[-SW]), f2(v1[0], v2[0])), f2(h1[-1], h2[-1])), f2(h1[0], h2[0]));
-            d1 = d.x;
-            gcur = d.y;
-        }
-        // D_s^T at the band's place in the whole cube (Neumann at its ends)
-        const float gprev = gs[kc];
-        const int gb = bb + a.sp.band0;
-        float dst_ = 0.f;
-        if (gb >= 1) dst_ += gprev;
-        if (gb <= a.sp.n3g - 2) dst_ -= gcur;
-        const int ku = r * SW + (c + OX);
-        const float y4 = cs * ys[L::O_Q + ku];
-        const float u = ys[L::O_U + ku];
-        const float un = fminf(fmaxf(u - P.gamma_u * (d1 + dst_ + y4), P.mu_lo), P.mu_hi);
-        upb[kc] = 2.f * un - u;
-        gs[kc] = gcur;
-        if constexpr (decltype(store_c)::value) {
-            if (st) *dst = un;
-        }
-    };
-    // w step of one set (0 = w1, 1 = w2; a compile-time constant or not) at
-    // (r, c) in [-1, TY] x [-1, TX]; w' overwrites w in place; with Store, w+
-    // goes to dst (the set's first plane) when `st`
-    auto w_item = [&](auto set_c, auto store_c, const float* ys, float* wst, int r, int c, float* dst, bool st) {
-        const int set = set_of(set_c);
-        const int kw = (r + 1) * SW + (c + OX);
-        const int gi = i0 + r, gj = j0 + c;
-        if constexpr (EDGE) {
-            if (gi < 0 || gi >= g.n1 || gj < 0 || gj >= g.n2) {
-#pragma unroll
-                for (int k = 0; k < 6; ++k) wst[(6 * set + k) * WPL + kw] = 0.f;
-                return;
-            }
-        }
-        const bool mv = !EDGE || gi < g.n1 - 1, mh = !EDGE || gj < g.n2 - 1;
-        const int ky = (r + 2) * SW + (c + OX);
-        const float* yv = ys + (2 * set) * YPL + ky;
-        const float* yh = yv + YPL;
-        auto V = [&](int dr, int dc) {
-            if constexpr (EDGE) return (gi + dr == g.n1 - 1) ? 0.f : yv[dr * SW + dc];
-            else return yv[dr * SW + dc];
-        };
-        auto H = [&](int dr, int dc) {
-            if constexpr (EDGE) return (gj + dc == g.n2 - 1) ? 0.f : yh[dr * SW + dc];
-            else return yh[dr * SW + dc];
-        };
-        const float v00 = V(0, 0), vm0 = V(-1, 0), v01 = V(0, 1), vm1 = V(-1, 1);
-        const float h00 = H(0, 0), h0m = H(0, -1), h10 = H(1, 0), h1m = H(1, -1);
-        // (v, h) pairs: the centred means 0.5 (v00 + vm0), 0.5 (h00 + h0m), and
-        // the four-point means 0.25 (v00 + vm0 + v01 + vm1), 0.25 (h00 + h0m + h10 + h1m)
-        float2 sum = add2(f2(v00, h00), f2(vm0, h0m));
-        const float2 cen = mul2(sum, f2(0.5f, 0.5f));
-        sum = add2(add2(sum, f2(v01, h10)), f2(vm1, h1m));
-        const float2 four = mul2(sum, f2(0.25f, 0.25f));
-        float2 Lg[3];                                   // (L_v, L_h) of the three grids
-        Lg[0] = f2(mv ? v00 : 0.f, mv ? four.y : 0.f);
-        Lg[1] = f2(mh ? four.x : 0.f, mh ? h00 : 0.f);
-        Lg[2] = cen;
-        const float gam = set ? P.gamma_w2 : P.gamma_w1;
-        const float thr = set ? P.thr_w2 : P.thr_w1;
-        const float thr2 = thr * thr;
-        float* wp = wst + (6 * set) * WPL + kw;
-#pragma unroll
-        for (int gr = 0; gr < 3; ++gr) {
-            const float wv = wp[(2 * gr) * WPL];
-            const float wh = wp[(2 * gr + 1) * WPL];
-            const float2 x = fma2(f2(gam, gam), Lg[gr], f2(wv, wh));
-            const float xv = x.x, xh = x.y;
-            // Eq. 24: max(1 - thr / ||x||, 0) x, with 1 / ||x|| from rsqrt
-            const float n2 = xv * xv + xh * xh;
-            const float sc = n2 > thr2 ? fmaxf(1.f - thr * rsqrtf(n2), 0.f) : 0.f;
-            const float2 nn = mul2(f2(sc, sc), x);
-            const float nv = nn.x, nh = nn.y;
-            wp[(2 * gr) * WPL] = 2.f * nv - wv;
-            wp[(2 * gr + 1) * WPL] = 2.f * nh - wh;
-            if constexpr (decltype(store_c)::value) {
-                if (st) {
-                    dst[(2 * gr) * cube] = nv;
-                    dst[(2 * gr + 1) * cube] = nh;
-                }
-            }
-        }
-    };
-
-    // ---- this thread's tile voxel and its share of the one-pixel ring ----
-    const int r_t = tid / TX, c_t = tid - (tid / TX) * TX;
-    const int gi_t = i0 + r_t, gj_t = j0 + c_t;
-    const bool valid_t = !EDGE || (gi_t < g.n1 && gj_t < g.n2);
-    const unsigned o_t = valid_t ? (unsigned)gi_t * (unsigned)g.p2 + (unsigned)gj_t : 0u;
-    const int ky_t = (r_t + 2) * SW + (c_t + OX);
-    // The one-pixel ring: w items on warps 0-7, u' items on warps 10 and 15
-    // (each scheduler, warp index mod 4, gets two or three ring warps besides
-    // its four tile warps).  A column of the ring walks rows 40 floats apart,
-    // so rows r and r + 4 fall in one shared-memory bank: a w warp takes four
-    // consecutive rows of each column, a u' warp eight (the mapping that gave
-    // a warp all 16 rows of a column made K1 0.6 % slower through bank
-    // conflicts).
-    int rw_r = 0, rw_c = 0, ru_r = 0, ru_c = 0;
-    const int wid = tid >> 5, lane = tid & 31;
-    // w ring: warps 0-7, warp w holds set w / 4 and quarter q = w % 4 of it:
-    // the left and right column items of rows 4q..4q+3 (distinct banks) and
-    // 17 of the 68 row items
-    const bool has_rw = wid < 8 && lane < 25;
-    const int rw_set = wid >= 4 ? 1 : 0;
-    if (has_rw) {
-        const int q = wid & 3;
-        if (lane < 4) { rw_r = 4 * q + lane; rw_c = -1; }
-        else if (lane < 8) { rw_r = 4 * q + lane - 4; rw_c = TX; }
-        else {
-            const int ri = 17 * q + lane - 8;           // 0..67
-            if (ri < TX + 2) { rw_r = -1; rw_c = ri - 1; } else { rw_r = TY; rw_c = ri - (TX + 2) - 1; }
-        }
-    }
-    // u' ring: warps 10 and 15, each 8 right-column items and half the row
-    const int uq = wid == 10 ? 0 : wid == 15 ? 1 : -1;
-    const bool has_ru = uq >= 0 && lane < (uq == 0 ? 25 : 24);
-    if (has_ru) {
-        if (lane < 8) { ru_r = 8 * uq + lane; ru_c = TX; }
-        else { ru_r = TY; ru_c = 17 * uq + lane - 8; }
-    }
+    const int r_t = tid / TX, c_t = tid % TX;
+    const int gi = m.i0 + r_t, gj = m.j0 + c_t;
+    const bool valid = !EDGE || (gi < g.n1 && gj < g.n2);
+    const unsigned o_t = valid ? (unsigned)gi * (unsigned)g.p2 + (unsigned)gj : 0u;
+    const int ky = (r_t + 2) * SW + (c_t + OX), kw = (r_t + 1) * SW + (c_t + OX);
+    const bool mv = !EDGE || gi < g.n1 - 1, mh = !EDGE || gj < g.n2 - 1;
+    const unsigned it32 = L::F32 ? 0u : (unsigned)a.sc->iter;      // seeds the 16-bit rounding streams
 
     // ---- dual ascent of y1, y2 at this thread's voxel of band tb ----
-    // Reads the band's completed w' and u' of the band and the next; yc: the
-    // voxel's y1 (v, h), y2 (v, h) of band tb.
-    auto t_item = [&](int tb, const float (&yc)[4]) {
-        if (!valid_t) return;
+    // Reads the band's completed w' (wp) and u' of the band (upb) and the next
+    // (upn); yc: the voxel's y1 (v, h), y2 (v, h) of band tb.
+    auto t_item = [&](int tb, const float* wp, const float* upb, const float* upn, const float (&yc)[4]) {
+        if (!valid) return;
         const bool nxt = tb + 1 < g.n3;
-        const float* upb = upl(tb);
-        const float* upn = upl(tb + 1);
-        const float* wp = wg(tb);
         const int kc = r_t * UC + c_t;
         const float u0 = upb[kc];
-        const bool mv = !EDGE || gi_t < g.n1 - 1, mh = !EDGE || gj_t < g.n2 - 1;
         // (vertical, horizontal) pairs: D u' and D D_s u' at the voxel
         const float2 ub = f2(upb[kc + UC], upb[kc + 1]);
         const float2 du_ = sub2(ub, f2(u0, u0));
@@ -440,23 +488,16 @@ __device__ __forceinline__ bool k1_tile(const K1Maps& M, const K1TArgs& a, unsig
         const float d0 = upn[kc] - u0;
         const float2 dd_ = sub2(sub2(f2(upn[kc + UC], upn[kc + 1]), ub), f2(d0, d0));
         const float2 dd = f2(nxt && mv ? dd_.x : 0.f, nxt && mh ? dd_.y : 0.f);
-        const float* wk = wp + (r_t + 1) * SW + (c_t + OX);
+        const float* wk = wp + kw;
         float2 lt[2];                                    // (L^T w')_v, (L^T w')_h of each set
 #pragma unroll
         for (int set = 0; set < 2; ++set) {
             auto Wk = [&](int k, int dr, int dc) { return wk[(6 * set + k) * WPL + dr * SW + dc]; };
-            auto A_ = [&](int dr, int dc) {
-                if constexpr (EDGE) return (gi_t + dr < g.n1 - 1) ? Wk(1, dr, dc) : 0.f;
-                else return Wk(1, dr, dc);
-            };
-            auto B_ = [&](int dr, int dc) {
-                if constexpr (EDGE) return (gj_t + dc < g.n2 - 1) ? Wk(2, dr, dc) : 0.f;
-                else return Wk(2, dr, dc);
-            };
-            // v: W0 + 0.25 (B(0,0) + B(1,0) + B(0,-1) + B(1,-1)) + 0.5 (W4(0,0) + W4(1,0))
-            // h: W3 + 0.25 (A(0,0) + A(0,1) + A(-1,0) + A(-1,1)) + 0.5 (W5(0,0) + W5(0,1))
-            const float2 s4 = add2(add2(add2(f2(B_(0, 0), A_(0, 0)), f2(B_(1, 0), A_(0, 1))), f2(B_(0, -1), A_(-1, 0))),
-                                   f2(B_(1, -1), A_(-1, 1)));
+            // v: W0 + 0.25 (W2(0,0) + W2(1,0) + W2(0,-1) + W2(1,-1)) + 0.5 (W4(0,0) + W4(1,0))
+            // h: W3 + 0.25 (W1(0,0) + W1(0,1) + W1(-1,0) + W1(-1,1)) + 0.5 (W5(0,0) + W5(0,1))
+            const float2 s4 = add2(add2(add2(f2(Wk(2, 0, 0), Wk(1, 0, 0)), f2(Wk(2, 1, 0), Wk(1, 0, 1))),
+                                        f2(Wk(2, 0, -1), Wk(1, -1, 0))),
+                                   f2(Wk(2, 1, -1), Wk(1, -1, 1)));
             const float2 s2 = add2(f2(Wk(4, 0, 0), Wk(5, 0, 0)), f2(Wk(4, 1, 0), Wk(5, 0, 1)));
             const float2 gg = fma2(f2(0.5f, 0.5f), s2, fma2(f2(0.25f, 0.25f), s4, f2(Wk(0, 0, 0), Wk(3, 0, 0))));
             lt[set] = f2(mv ? gg.x : 0.f, mh ? gg.y : 0.f);
@@ -464,225 +505,512 @@ __device__ __forceinline__ bool k1_tile(const K1Maps& M, const K1TArgs& a, unsig
         const unsigned ob = (unsigned)tb * plane + o_t;
         const float2 y1 = fma2(f2(P.gamma_y1, P.gamma_y1), sub2(du, lt[0]), f2(yc[0], yc[1]));
         const float2 y2 = fma2(f2(P.gamma_y2, P.gamma_y2), sub2(dd, lt[1]), f2(yc[2], yc[3]));
-        a.y1_n[ob] = y1.x;
-        a.y1_n[cube + ob] = y1.y;
-        a.y2_n[ob] = y2.x;
-        a.y2_n[cube + ob] = y2.y;
+        if constexpr (L::F32) {
+            a.y1_n[ob] = y1.x;
+            a.y1_n[cube + ob] = y1.y;
+            a.y2_n[ob] = y2.x;
+            a.y2_n[cube + ob] = y2.y;
+        } else {
+            SRStream sr(ob, it32, 3u);
+            stS(a.y1_n + ob, y1.x, sr);
+            stS(a.y1_n + (cube + ob), y1.y, sr);
+            stS(a.y2_n + ob, y2.x, sr);
+            stS(a.y2_n + (cube + ob), y2.y, sr);
+        }
     };
 
     // ---- l1 window statistics of s~, t~ at this thread's voxel ----
-    auto stats = [&](const float* ys, int b) {
+    auto stats = [&](const T* ys, int b) {
         float xs = 0.f, xt = 0.f;
-        if (valid_t) {
+        if (valid) {
             // s~ = s - g_s y4, t~ = t - g_t (D_v^T y3 + y4), each product and
             // difference rounded once as in s_t_tilde (the light pass computes
             // the same values), the (s, t) pair packed
-            const float qv = ys[L::O_Q + r_t * SW + (c_t + OX)];
-            const float y3v = ys[L::O_Y3 + (r_t + 1) * TX + c_t];
-            const float y3u = (!EDGE || gi_t >= 1) ? ys[L::O_Y3 + r_t * TX + c_t] : 0.f;
+            const float qv = ldT(ys + L::O_Q + r_t * SW + (c_t + OX));
+            const float y3v = ldT(ys + L::O_Y3 + (r_t + 1) * TX + c_t);
+            const float y3u = (!EDGE || gi >= 1) ? ldT(ys + L::O_Y3 + r_t * TX + c_t) : 0.f;
             const float y4 = __fmul_rn(cs, qv);
-            const float dvt = __fsub_rn(y3u, gi_t <= g.n1 - 2 ? y3v : 0.f);
-            const float2 m = mul2(f2(P.gamma_s, P.gamma_t), f2(y4, __fadd_rn(dvt, y4)));
-            const float2 x = sub2(f2(ys[L::O_S + r_t * TX + c_t], ys[L::O_T + r_t * TX + c_t]), m);
+            const float dvt = __fsub_rn(y3u, gi <= g.n1 - 2 ? y3v : 0.f);
+            const float2 mm = mul2(f2(P.gamma_s, P.gamma_t), f2(y4, __fadd_rn(dvt, y4)));
+            const float2 x = sub2(f2(ldT(ys + L::O_S + r_t * TX + c_t), ldT(ys + L::O_T + r_t * TX + c_t)), mm);
             xs = x.x;
             xt = x.y;
         }
         // an inactive window has lo = hi = +inf: nothing is counted or taken
         const float x_s = fabsf(xs), x_t = fabsf(xt);
-        const bool hs = valid_t && x_s > W.hi_s, ht = valid_t && x_t > W.hi_t;
+        const bool hs = valid && x_s > W.hi_s, ht = valid && x_t > W.hi_t;
         {
             // both vectors' compensated sums in packed pairs; a value not
             // taken adds zero, which leaves the represented sum unchanged
             const float2 x2 = f2(hs ? x_s : 0.f, ht ? x_t : 0.f);
-            const float2 y2 = sub2(x2, S.kc);
-            const float2 t2 = add2(S.ks, y2);
-            S.kc = sub2(sub2(t2, S.ks), y2);
-            S.ks = t2;
-            S.acc_s.n += hs ? 1u : 0u;
-            S.acc_t.n += ht ? 1u : 0u;
+            const float2 t2 = add2(A.ks, x2);
+            const float2 b2 = sub2(t2, A.ks);
+            A.kc = sub2(A.kc, add2(sub2(A.ks, sub2(t2, b2)), sub2(x2, b2)));
+            A.ks = t2;
+            A.n_s += hs ? 1u : 0u;
+            A.n_t += ht ? 1u : 0u;
         }
-        const bool cs_ = valid_t && !hs && x_s > W.lo_s, ct_ = valid_t && !ht && x_t > W.lo_t;
+        const bool cs_ = valid && !hs && x_s > W.lo_s, ct_ = valid && !ht && x_t > W.lo_t;
         if (__ballot_sync(0xffffffffu, cs_ || ct_)) {     // most warps have no candidate
-            append_shared(cs_, x_s, cbuf, ccnt, a.l1.cand[0], &a.sc->acc[0].m);
-            append_shared(ct_, x_t, cbuf + L::CB, ccnt + 1, a.l1.cand[1], &a.sc->acc[1].m);
+            append_shared(cs_, x_s, S.cbuf(0, turn & 1), S.cnt(0, turn & 1), a.l1.cand[0], &a.sc->acc[0].m);
+            append_shared(ct_, x_t, S.cbuf(1, turn & 1), S.cnt(1, turn & 1), a.l1.cand[1], &a.sc->acc[1].m);
         }
         if constexpr (HIST) {
             // a 1/32 sample: a warp (one row of the tile) counts its 32 voxels
             // at one band in 32, the band rotating with the row and the tile
             // so that every band is sampled; the branch is warp-uniform, so
             // the other 31 band steps cost one test
-            if ((((unsigned)b + 7u * (unsigned)r_t + 5u * (unsigned)(i0 >> 4) + 3u * (unsigned)(j0 >> 5)) & 31u) == 0u) {
-                hist_add(W.hs && valid_t, x_s, W.hb_s, hsm, S.top_s);
-                hist_add(W.ht && valid_t, x_t, W.hb_t, hsm + kK1Bins / 2, S.top_t);
+            if ((((unsigned)b + 7u * (unsigned)r_t + 5u * (unsigned)(m.i0 >> 4) + 3u * (unsigned)(m.j0 >> 5)) & 31u) == 0u) {
+                hist_add(W.hs && valid, x_s, W.hb_s, S.hist(), A.top_s);
+                hist_add(W.ht && valid, x_t, W.hb_t, S.hist() + kK1Bins / 2, A.top_t);
             }
         }
     };
-
-    // ---- prologue: D^T y2 of band b0-1 and u' of band b0 ----
-    if (tid == L::PRODUCER) {
-        for (int band = bstart; band <= min(bstart + L::NYS - 1, blast); ++band) issue_y(band);
-        issue_w(b0);
-        if (b0 + 1 < b1) issue_w(b0 + 1);
-    }
-    bool ok = true;
-    if (b0 >= 1) {
-        ok = wait_y(b0 - 1);
-        const float* yp = yg(b0 - 1);
-        for (int e = tid; e < L::UR * UC; e += L::NT) {
-            const int r = e / UC, c = e - r * UC;
-            if (EDGE && (i0 + r >= g.n1 || j0 + c >= g.n2)) { gs[e] = 0.f; continue; }
-            gs[e] = dty(yp + 2 * YPL, yp + 3 * YPL, r, c);
-        }
-    }
-    ok = wait_y(b0) && ok;
-    ok = __syncthreads_and(ok);
-    if (!ok) return false;
-    u_item(Store{}, yg(b0), upl(b0), b0, r_t, c_t, a.u_n + ((unsigned)b0 * plane + o_t), valid_t);
-    if (has_ru) u_item(NoStore{}, yg(b0), upl(b0), b0, ru_r, ru_c, nullptr, false);
-    __syncthreads();
-
-    // ---- band march, one barrier per band ----
-    // The ascent of the previous band needs nothing from this band's copies,
-    // so it runs before the waits on them; then the tile work of the band
-    // (the statistics, w steps, u' of the next band) is one straight run so
-    // that the compiler can interleave its independent chains, and the ring
-    // work follows.  u' of the band past the cube's last one is computed from
-    // a stale slot and not stored (its values are never used).
-    float yprev[4] = {0.f, 0.f, 0.f, 0.f};
-    auto step = [&](int b, auto do_t) -> bool {
-        const bool has_next = b + 1 < g.n3;
-        if (tid == L::PRODUCER) {
-            if (b + 2 <= blast && b + 2 - bstart >= L::NYS) issue_y(b + 2);
-            if (b + 2 < b1) issue_w(b + 2);
-        }
-        if constexpr (decltype(do_t)::value) t_item(b - 1, yprev);
-        bool okb = wait_w(b);
-        if (has_next) okb = wait_y(b + 1) && okb;
-        okb = __all_sync(0xffffffffu, okb);   // warp-uniform: the statistics use warp votes
-        if (okb) {
-            const float* ys = yg(b);
-            const float* ysn = yg(b + 1);
-            float* wst = wg(b);
-            float* upn = upl(b + 1);
-            const unsigned ob = (unsigned)b * plane + o_t;
-            float ycur[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) ycur[k] = ys[k * YPL + ky_t];
-            if (W.s || W.t) stats(ys, b);
-            w_item(Set0{}, Store{}, ys, wst, r_t, c_t, a.w1_n + ob, valid_t);
-            w_item(Set1{}, Store{}, ys, wst, r_t, c_t, a.w2_n + ob, valid_t);
-            u_item(Store{}, ysn, upn, b + 1, r_t, c_t, a.u_n + (ob + plane), valid_t && b + 1 < b1);
-            if (has_rw) w_item(rw_set, NoStore{}, ys, wst, rw_r, rw_c, nullptr, false);
-            if (has_ru && has_next) u_item(NoStore{}, ysn, upn, b + 1, ru_r, ru_c, nullptr, false);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) yprev[k] = ycur[k];
-        }
-        // the slots freed at this step are reloaded by TMA at the next one:
-        // order this thread's generic accesses before those async-proxy writes
-        fence_proxy_async_smem();
-        return !__syncthreads_or(!okb);
+    const bool win = W.s || W.t;
+    auto store_u = [&](unsigned ob, float un) {
+        if constexpr (L::F32) a.u_n[ob] = un;
+        else { SRStream sr(ob, it32, 2u); stS(a.u_n + ob, un, sr); }
     };
-    if (!step(b0, std::false_type{})) return false;
-    for (int b = b0 + 1; b < b1; ++b)
-        if (!step(b, std::true_type{})) return false;
-    t_item(b1 - 1, yprev);
+
+    // ---- band march, one barrier phase per band ----
+    // The step before the first band computes u' of the first band only; it
+    // shares the loop's code so that a launch fetches one copy of it (with
+    // separate code for the first steps and the last ascent, a launch of a few
+    // bands per CTA spent most of its time on instruction fetches).  u' of the
+    // band past the cube's last one is computed from a stale slot and not
+    // stored (its values are never used).
+    float gprev = 0.f;
+    if (m.b0 > 0) {
+        const T* yv = a.y2 + (unsigned)(m.b0 - 1) * plane;
+        gprev = dty_global<EDGE>(yv, yv + cube, gi, gj, g);
+    }
+    float yprev[4] = {0.f, 0.f, 0.f, 0.f};
+    const int w_last = C.w.slot == 0 ? L::NWS - 1 : C.w.slot - 1;    // the previous item's last w
+    int wslot_prev = w_last, ys_slot = 0, us_cur = 0, us_prev = 0;
+#pragma unroll 1
+    for (int b = m.b0 - 1;; ++b) {
+        const bool body = b >= m.b0, has_next = b + 1 < g.n3;
+        if (b > m.b0) t_item(b - 1, S.wp(wslot_prev, C.ps ^ 1), S.up(us_prev), S.up(us_cur), yprev);
+        if (b == m.b1) break;
+        bool ok = true;
+        if (body) ok = k1_wait(S.wfull + C.w.slot, C.w.ph, S.abort);
+        if (has_next) ok = k1_wait(S.yfull + C.y.slot, C.y.ph, S.abort) && ok;
+        if (!__all_sync(0xffffffffu, ok)) return false;    // warp-uniform: the statistics use warp votes
+        const unsigned ob = (unsigned)b * plane + o_t;
+        if (body) {
+            const T* ys = S.yg(ys_slot);
+            const T* wraw = S.wg(C.w.slot) + kw;
+            float* wp = S.wp(C.w.slot, C.ps) + kw;
+            if (EDGE && !valid) {
+#pragma unroll
+                for (int k = 0; k < 12; ++k) wp[k * WPL] = 0.f;
+            } else {
+                // every operand before the first store (the compiler cannot
+                // tell the shared-memory regions apart)
+                float w1[6], w2[6];
+#pragma unroll
+                for (int k = 0; k < 6; ++k) {
+                    w1[k] = ldT(wraw + k * WRAW);
+                    w2[k] = ldT(wraw + (6 + k) * WRAW);
+                }
+                const YN ya = load_yn(ys + ky, ys + YPL + ky);
+                const YN yb = load_yn(ys + 2 * YPL + ky, ys + 3 * YPL + ky);
+                yprev[0] = ya.v00; yprev[1] = ya.h00; yprev[2] = yb.v00; yprev[3] = yb.h00;
+                if constexpr (EDGE) {
+                    // staged as zero where D is structurally zero (see
+                    // k1_tma_maps): the ascent leaves the stored values there
+                    if (!mv) { yprev[0] = ldT(a.y1 + ob); yprev[2] = ldT(a.y2 + ob); }
+                    if (!mh) { yprev[1] = ldT(a.y1 + (cube + ob)); yprev[3] = ldT(a.y2 + (cube + ob)); }
+                }
+                float2 La[3], Lb[3];
+                l_pairs<EDGE>(ya, mv, mh, La);
+                l_pairs<EDGE>(yb, mv, mh, Lb);
+                const int k3[3] = {0, 0, 0};
+                const bool on[3] = {mv, mh, true};
+                w_step<0, EDGE, T>(P, La, w1, wp, k3, on);
+                w_step<1, EDGE, T>(P, Lb, w2, wp, k3, on);
+                if constexpr (L::F32) {
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) {
+                        a.w1_n[k * cube + ob] = w1[k];
+                        a.w2_n[k * cube + ob] = w2[k];
+                    }
+                } else {
+                    SRStream s1(ob, it32, 4u), s2(ob, it32, 5u);
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) {
+                        stS(a.w1_n + (k * cube + ob), w1[k], s1);
+                        stS(a.w2_n + (k * cube + ob), w2[k], s2);
+                    }
+                }
+            }
+        }
+        const T* yn = S.yg(C.y.slot);
+        const float un = u_item<EDGE>(a, yn, S.up(C.us), b + 1 + a.sp.band0, r_t, c_t, gi, gj, cs, gprev);
+        C.arrive(S);
+        const bool more = b + 1 < m.b1;
+        if (valid && more) store_u(ob + plane, un);
+        if (win && more) stats(yn, b + 1);
+        if (!C.wait(S)) return false;
+        if (tid == 0) {
+            // what every warp has finished with by now
+            if (body) mbar_arrive(S.yempty + ys_slot);
+            if (!more && has_next) mbar_arrive(S.yempty + C.y.slot);
+            if (!L::F32) {
+                if (body) mbar_arrive(S.wempty + C.w.slot);
+            } else if (body ? b > m.b0 : turn > 0) {
+                mbar_arrive(S.wempty + wslot_prev);
+            }
+        }
+        us_prev = us_cur;
+        us_cur = C.us;
+        C.us = C.us == L::NUS - 1 ? 0 : C.us + 1;
+        ys_slot = C.y.slot;
+        if (has_next) C.y.next();
+        if (body) {
+            wslot_prev = C.w.slot;
+            C.w.next();
+            C.ps ^= 1;
+        }
+    }
     return true;
 }
 
-// One CTA of K1: the tile (bx, by) and band run bz of a launch of gx x gy x gz
-// CTAs over one cube (a launch of its own, or the cube's share of a batch).
-__device__ __forceinline__ void k1_run(const K1Maps& maps, const K1TArgs& a, const int bx, const int by,
-                                       const int bz, const int gx, const int gy, const int gz) {
-    using L = Lay;
-    extern __shared__ __align__(128) unsigned char sm[];
-    __shared__ unsigned ccnt[2], cbase[2];
+// ---------------------------------------------------------------------------
+// ring warps: one item
+// ---------------------------------------------------------------------------
+template <typename T, bool EDGE>
+__device__ __forceinline__ bool ring_item(const K1Args<T>& a, const Sm<T>& S, const Item& m, Cons<T>& C, float cs) {
+    using L = Lay<T>;
+    constexpr int YPL = L::YPL, WRAW = L::WRAW;
     const Geom& g = a.g;
     const IterParams& P = a.p;
-    const int i0 = by * L::TY, j0 = bx * L::TX;
-    const int b0 = a.sp.o0 + bz * a.chunk;
-    const int b1 = min(a.sp.o1, b0 + a.chunk);
-    const int tid = threadIdx.x;
-    const float cs = (float)(1.0 - a.sc->c[P.parity]);
+    const int q = (threadIdx.x >> 5) - kTileWarps, lane = threadIdx.x & 31;
+    // w ring, a position per grid (row, column): grid 0 at (-1, c) and grids
+    // 1, 2 at (TY, c) for a column c of the tile; grids 0, 2 at (r, TX) and
+    // grid 1 at (r, -1) for a row r; the corners (-1, TX) of grid 0 and
+    // (TY, -1) of grid 1.  A column of the ring walks rows 40 floats apart, so
+    // rows r and r + 4 fall in one shared-memory bank: each warp takes half
+    // the rows and half the columns.
+    const bool has_w = lane < (q == 0 ? 25 : 24), has_u = has_w;
+    int pr[3], pc[3];
+    if (lane < 8) {
+        pr[0] = pr[1] = pr[2] = 8 * q + lane;
+        pc[0] = pc[2] = TX;
+        pc[1] = -1;
+    } else if (lane < 24) {
+        pr[0] = -1;
+        pr[1] = pr[2] = TY;
+        pc[0] = pc[1] = pc[2] = 16 * q + lane - 8;
+    } else {
+        pr[0] = -1;
+        pr[1] = pr[2] = TY;
+        pc[0] = TX;
+        pc[1] = pc[2] = -1;
+    }
+    // u' ring: the right column's rows and the row below
+    const int ur = lane < 8 ? 8 * q + lane : TY, uc = lane < 8 ? TX : lane < 24 ? 16 * q + lane - 8 : TX;
+    const int ui = m.i0 + ur, uj = m.j0 + uc;
+    int gi[3], gj[3], ky[3], kw[3];
+    bool in[3];                 // inside the image, and L's output not structurally zero
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        gi[k] = m.i0 + pr[k];
+        gj[k] = m.j0 + pc[k];
+        ky[k] = (pr[k] + 2) * SW + (pc[k] + OX);
+        kw[k] = (pr[k] + 1) * SW + (pc[k] + OX);
+        in[k] = !EDGE || (gi[k] >= 0 && gi[k] < g.n1 && gj[k] >= 0 && gj[k] < g.n2);
+    }
+    const bool mv = !EDGE || gi[0] < g.n1 - 1, mh = !EDGE || gj[1] < g.n2 - 1;
+    in[0] = in[0] && mv;
+    in[1] = in[1] && mh;
+    // L y of one set at the three positions (as l_pairs; the planes read
+    // outside a position's grid stay in the staged boxes)
+    auto ring_L = [&](const T* yv, const T* yh, float2 (&Lg)[3]) {
+        auto V = [&](int k, int dr, int dc) { return ldT(yv + ky[k] + dr * SW + dc); };
+        auto H = [&](int k, int dr, int dc) { return ldT(yh + ky[k] + dr * SW + dc); };
+        const float h4 = 0.25f * (((H(0, 0, 0) + H(0, 0, -1)) + H(0, 1, 0)) + H(0, 1, -1));
+        const float v4 = 0.25f * (((V(1, 0, 0) + V(1, -1, 0)) + V(1, 0, 1)) + V(1, -1, 1));
+        Lg[0] = f2(mv ? V(0, 0, 0) : 0.f, mv ? h4 : 0.f);
+        Lg[1] = f2(mh ? v4 : 0.f, mh ? H(1, 0, 0) : 0.f);
+        Lg[2] = f2(0.5f * (V(2, 0, 0) + V(2, -1, 0)), 0.5f * (H(2, 0, 0) + H(2, 0, -1)));
+    };
+
+    float gprev = 0.f;
+    if (has_u && m.b0 > 0) {
+        const T* yv = a.y2 + (long long)(m.b0 - 1) * g.n1 * g.p2;
+        gprev = dty_global<EDGE>(yv, yv + g.cube, ui, uj, g);
+    }
+    int ys_slot = 0;
+#pragma unroll 1
+    for (int b = m.b0 - 1; b < m.b1; ++b) {
+        const bool body = b >= m.b0, has_next = b + 1 < g.n3;
+        bool ok = true;
+        if (body) ok = k1_wait(S.wfull + C.w.slot, C.w.ph, S.abort);
+        if (has_next) ok = k1_wait(S.yfull + C.y.slot, C.y.ph, S.abort) && ok;
+        if (!__all_sync(0xffffffffu, ok)) return false;
+        if (body && has_w) {
+            const T* ys = S.yg(ys_slot);
+            const T* wraw = S.wg(C.w.slot);
+            float* wp = S.wp(C.w.slot, C.ps);
+            float w1[6], w2[6];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                w1[k] = ldT(wraw + k * WRAW + kw[k / 2]);
+                w2[k] = ldT(wraw + (6 + k) * WRAW + kw[k / 2]);
+            }
+            float2 La[3], Lb[3];
+            ring_L(ys, ys + YPL, La);
+            ring_L(ys + 2 * YPL, ys + 3 * YPL, Lb);
+            w_step<0, EDGE, T>(P, La, w1, wp, kw, in);
+            w_step<1, EDGE, T>(P, Lb, w2, wp, kw, in);
+        }
+        if (has_u && has_next)
+            u_item<EDGE>(a, S.yg(C.y.slot), S.up(C.us), b + 1 + a.sp.band0, ur, uc, ui, uj, cs, gprev);
+        C.arrive(S);
+        if (!C.wait(S)) return false;
+        C.us = C.us == L::NUS - 1 ? 0 : C.us + 1;
+        ys_slot = C.y.slot;
+        if (has_next) C.y.next();
+        if (body) {
+            C.w.next();
+            C.ps ^= 1;
+        }
+    }
+    return true;
+}
+
+// ---------------------------------------------------------------------------
+// load warps
+// ---------------------------------------------------------------------------
+// The groups of an item in the order they are asked for: each band's y-group
+// and w, and the y-group of the band after the last (for its u').  issue_y
+// (band, slot), issue_w(band, slot) fill a slot; wait_empty(bar, parity) waits
+// for it to be free.  Returns false when a wait gave up.
+template <typename T, typename FY, typename FW, typename FE>
+__device__ __forceinline__ bool load_item(const Item& m, const Geom& g, Ring<Lay<T>::NYS>& y, Ring<Lay<T>::NWS>& w,
+                                          const Sm<T>& S, FY&& issue_y, FW&& issue_w, FE&& wait_empty) {
+    const int blast = min(m.b1, g.n3 - 1);
+#pragma unroll 1
+    for (int b = m.b0; b <= blast; ++b) {
+        if (!wait_empty(S.yempty + y.slot, y.ph ^ 1u)) return false;
+        issue_y(b, y.slot);
+        y.next();
+        if (b == m.b1) break;
+        if (!wait_empty(S.wempty + w.slot, w.ph ^ 1u)) return false;
+        issue_w(b, w.slot);
+        w.next();
+    }
+    return true;
+}
+
+// float32: one thread issues bulk tensor copies
+// (ny, nw: groups issued)
+__device__ __forceinline__ void load_tma(const K1Maps& M, const K1Args<float>& a, const Sm<float>& S, int bid, int nblk,
+                                         int items, int gx, int gy, unsigned& ny, unsigned& nw) {
+    using L = Lay<float>;
+    Ring<L::NYS> y;
+    Ring<L::NWS> w;
+    const Geom& g = a.g;
+    bool ok = true;
+    for (int it = bid; it < items && ok; it += nblk) {
+        const Item m = item_of(a, it, gx, gy);
+        ok = load_item<float>(
+            m, g, y, w, S,
+            [&](int band, int slot) {
+                unsigned char* s = reinterpret_cast<unsigned char*>(S.yg(slot));
+                uint64_t* bar = S.yfull + slot;
+                mbar_arrive_expect_tx(bar, L::YG_TX);
+                // (a cube of one row / column has no vertical / horizontal
+                // differences: start past its map's one row / aligned column)
+                const int iv = g.n1 > 1 ? m.i0 - 2 : 16, jh = g.n2 > 1 ? m.j0 - OX : 64;
+                tma_load_3d(s + 0 * L::Y_B, &M.y1v, m.j0 - OX, iv, band, bar);
+                tma_load_3d(s + 1 * L::Y_B, &M.y1h, jh, m.i0 - 2, band, bar);
+                tma_load_3d(s + 2 * L::Y_B, &M.y2v, m.j0 - OX, iv, band, bar);
+                tma_load_3d(s + 3 * L::Y_B, &M.y2h, jh, m.i0 - 2, band, bar);
+                tma_load_3d(s + 4 * L::O_U, &M.u, m.j0 - OX, m.i0, band, bar);
+                tma_load_3d(s + 4 * L::O_Q, &M.q, m.j0 - OX, m.i0, band, bar);
+                tma_load_3d(s + 4 * L::O_S, &M.s, m.j0, m.i0, band, bar);
+                tma_load_3d(s + 4 * L::O_T, &M.t, m.j0, m.i0, band, bar);
+                tma_load_3d(s + 4 * L::O_Y3, &M.y3, m.j0, m.i0 - 1, band, bar);
+                ny++;
+            },
+            [&](int band, int slot) {
+                unsigned char* s = reinterpret_cast<unsigned char*>(S.wg(slot));
+                uint64_t* bar = S.wfull + slot;
+                mbar_arrive_expect_tx(bar, L::WG_TX);
+                for (int k = 0; k < 6; ++k)
+                    tma_load_3d(s + k * L::W_B, &M.w1, m.j0 - OX, m.i0 - 1, k * g.n3 + band, bar);
+                for (int k = 0; k < 6; ++k)
+                    tma_load_3d(s + (6 + k) * L::W_B, &M.w2, m.j0 - OX, m.i0 - 1, k * g.n3 + band, bar);
+                nw++;
+            },
+            [&](uint64_t* bar, unsigned parity) { return k1_wait(bar, parity, S.abort); });
+    }
+}
+
+// Waits (bounded) for the copies in flight to land, before the CTA gives its
+// shared memory back after a wait gave up.
+__device__ __forceinline__ void drain_tma(const Sm<float>& S, unsigned ny, unsigned nw) {
+    using L = Lay<float>;
+    for (unsigned k = 0; k < (unsigned)L::NYS && k < ny; ++k)
+        (void)mbar_wait(S.yfull + (ny - 1u - k) % L::NYS, ((ny - 1u - k) / L::NYS) & 1u);
+    for (unsigned k = 0; k < (unsigned)L::NWS && k < nw; ++k)
+        (void)mbar_wait(S.wfull + (nw - 1u - k) % L::NWS, ((nw - 1u - k) / L::NWS) & 1u);
+}
+
+// 16-bit: the load warps copy 8 bytes (four columns) per lane and instruction, the
+// first n of them from src and zero after (outside the image); a slot's full barrier counts every load thread.
+__device__ __forceinline__ void cp8(void* dst, const void* src, int n) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(n) : "memory");
+}
+template <typename T>
+__device__ __forceinline__ void load_async(const K1Args<T>& a, const Sm<T>& S, int bid, int nblk, int items, int gx,
+                                           int gy) {
+    using L = Lay<T>;
+    constexpr int NL = 32 * L::LW;
+    Ring<L::NYS> y;
+    Ring<L::NWS> w;
+    const Geom& g = a.g;
+    const int lt = threadIdx.x - 32 * kConsWarps;
+    const long long plane = (long long)g.n1 * g.p2;
+    auto done = [&](uint64_t* bar) {
+        asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+    };
+    for (int it = bid; it < items; it += nblk) {
+        const Item m = item_of(a, it, gx, gy);
+        // `n` planes of `rows` rows from (row0, col0), `quads` quads a row:
+        // plane k from base(k), into dst + k * stride; nr, nc: the image's rows
+        // and columns, the rest is zero
+        auto planes = [&](int n, int rows, int quads, int row0, int col0, T* dst, int stride, int nr, int nc,
+                          auto&& base) {
+            for (int e = lt; e < rows * quads; e += NL) {
+                const int r = e / quads, c = 4 * (e - r * quads);
+                const int gi = row0 + r, gj = col0 + c;
+                const bool in = gi >= 0 && gi < nr && gj >= 0 && gj < nc;
+                const int bytes = in ? min(nc - gj, 4) * L::ES : 0;
+                const long long o = in ? (long long)gi * g.p2 + gj : 0;
+                T* d = dst + r * 4 * quads + c;
+                for (int k = 0; k < n; ++k) cp8(d + k * stride, base(k) + o, bytes);
+            }
+        };
+        const bool ok = load_item<T>(
+            m, g, y, w, S,
+            [&](int band, int slot) {
+                T* s = S.yg(slot);
+                const long long bo = band * plane;
+                // (y_v without the last row, y_h without the last column, as in k1_tma_maps)
+                planes(2, YR, SW / 4, m.i0 - 2, m.j0 - OX, s, 2 * L::YPL, g.n1 - 1, g.n2,
+                       [&](int k) { return (k ? a.y2 : a.y1) + bo; });
+                planes(2, YR, SW / 4, m.i0 - 2, m.j0 - OX, s + L::YPL, 2 * L::YPL, g.n1, g.n2 - 1,
+                       [&](int k) { return (k ? a.y2 : a.y1) + g.cube + bo; });
+                planes(2, UR, SW / 4, m.i0, m.j0 - OX, s + L::O_U, L::O_Q - L::O_U, g.n1, g.n2,
+                       [&](int k) { return (k ? a.q : a.u) + bo; });
+                planes(2, TY, TX / 4, m.i0, m.j0, s + L::O_S, L::O_T - L::O_S, g.n1, g.n2,
+                       [&](int k) { return (k ? a.t : a.s) + bo; });
+                planes(1, TY + 1, TX / 4, m.i0 - 1, m.j0, s + L::O_Y3, 0, g.n1, g.n2, [&](int) { return a.y3 + bo; });
+                done(S.yfull + slot);
+            },
+            [&](int band, int slot) {
+                const long long bo = band * plane;
+                planes(12, WR, SW / 4, m.i0 - 1, m.j0 - OX, S.wg(slot), L::WRAW, g.n1, g.n2,
+                       [&](int k) { return (k < 6 ? a.w1 + k * g.cube : a.w2 + (k - 6) * g.cube) + bo; });
+                done(S.wfull + slot);
+            },
+            [&](uint64_t* bar, unsigned parity) { return __all_sync(0xffffffffu, k1_wait(bar, parity, S.abort)); });
+        if (!ok) break;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// One CTA of K1: items bid, bid + nblk, ... of the gx x gy x gz items (tiles
+// by band runs) of one cube.
+template <typename T>
+__device__ __forceinline__ void k1_run(const K1Maps* maps, const K1Args<T>& a, const int bid, const int nblk,
+                                       const int gx, const int gy, const int gz) {
+    using L = Lay<T>;
+    extern __shared__ __align__(128) unsigned char sm[];
+    __shared__ unsigned ccnt[4];
+    __shared__ int abort_flag;
+    __shared__ float wred[kTileWarps * 12];
+    const IterParams& P = a.p;
+    const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
+    const int items = gx * gy * gz;
+    const Sm<T> S(sm, ccnt, &abort_flag);
+    if (tid == 0) {
+        const unsigned full = L::F32 ? 1u : 32u * L::LW;
+        for (int k = 0; k < L::NYS; ++k) { mbar_init(S.yfull + k, full); mbar_init(S.yempty + k, 1); }
+        for (int k = 0; k < L::NWS; ++k) { mbar_init(S.wfull + k, full); mbar_init(S.wempty + k, 1); }
+        mbar_init(S.evt, kConsWarps);
+        mbar_fence_init();
+        for (int k = 0; k < 4; ++k) ccnt[k] = 0u;
+        abort_flag = 0;
+    }
+    for (int k = tid; k < kK1Bins; k += L::NT) S.hist()[k] = 0u;
+    __syncthreads();
+
     K1Win W;
     W.s = !P.tau_exact && a.sc->radius[0] > 0.0 && a.sc->ctl[0].window_ok;
     W.t = !P.tau_exact && a.sc->radius[1] > 0.0 && a.sc->ctl[1].window_ok;
     W.lo_s = W.s ? a.sc->ctl[0].theta_lo : INFINITY; W.hi_s = W.s ? a.sc->ctl[0].theta_hi : INFINITY;
     W.lo_t = W.t ? a.sc->ctl[1].theta_lo : INFINITY; W.hi_t = W.t ? a.sc->ctl[1].theta_hi : INFINITY;
-    // the histograms: on after a recent miss, while a CTA's voxels fit the
-    // 16-bit counters
-    const bool hist_fits = a.hist_fits != 0;
+    // the histograms: on after a recent miss
     W.hb_s = a.sc->ctl[0].hbase;
     W.hb_t = a.sc->ctl[1].hbase;
-    W.hs = W.s && hist_fits && a.sc->ctl[0].hist_left > 0 && hist_base_ok(W.hb_s);
-    W.ht = W.t && hist_fits && a.sc->ctl[1].hist_left > 0 && hist_base_ok(W.hb_t);
-    W.ng_s = narrow_geom(__float_as_uint(W.lo_s), __float_as_uint(W.hi_s));
-    W.ng_t = narrow_geom(__float_as_uint(W.lo_t), __float_as_uint(W.hi_t));
-    W.nh_s = W.s && a.l1.nh && W.ng_s.ok ? a.l1.nh : nullptr;
-    W.nh_t = W.t && a.l1.nh && W.ng_t.ok ? a.l1.nh + 3 * kNarrowBins : nullptr;
-
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::OFF_BAR);
-    if (tid == 0) {
-        for (int k = 0; k < L::NYS + L::NWS; ++k) mbar_init(bars + k, 1);
-        mbar_fence_init();
-        ccnt[0] = ccnt[1] = 0;
-    }
-    if (W.hs || W.ht) {
-        unsigned* hsm = reinterpret_cast<unsigned*>(sm + L::OFF_HIST);
-        for (int k = tid; k < kK1Bins; k += L::NT) hsm[k] = 0u;
+    W.hs = W.s && a.sc->ctl[0].hist_left > 0 && hist_base_ok(W.hb_s);
+    W.ht = W.t && a.sc->ctl[1].hist_left > 0 && hist_base_ok(W.hb_t);
+    const bool hist = W.hs || W.ht;
+    K1Stat A;
+    unsigned ny = 0, nw = 0;
+    if (wid < kTileWarps) {
+        const float cs = (float)(1.0 - a.sc->c[P.parity]);      // y4 = (1 - c) q
+        Cons<T> C;
+        int turn = 0;
+        for (int it = bid; it < items; it += nblk, ++turn) {
+            const Item m = item_of(a, it, gx, gy);
+            const bool ok = item_edge(m, a.g)
+                                ? (hist ? tile_item<T, true, true>(a, S, m, C, A, W, cs, turn)
+                                        : tile_item<T, true, false>(a, S, m, C, A, W, cs, turn))
+                                : (hist ? tile_item<T, false, true>(a, S, m, C, A, W, cs, turn)
+                                        : tile_item<T, false, false>(a, S, m, C, A, W, cs, turn));
+            if (!ok) break;
+        }
+    } else if (wid < kConsWarps) {
+        const float cs = (float)(1.0 - a.sc->c[P.parity]);
+        const int v = wid - kTileWarps;                         // warps 0, 1: vector v's candidates
+        const bool mine = v == 0 ? W.s : v == 1 && W.t;
+        Cons<T> C;
+        int turn = 0;
+        for (int it = bid; it < items; it += nblk, ++turn) {
+            const Item m = item_of(a, it, gx, gy);
+            const bool ok = item_edge(m, a.g) ? ring_item<T, true>(a, S, m, C, cs) : ring_item<T, false>(a, S, m, C, cs);
+            if (!ok) break;
+            if (mine)
+                flush_candidates(v, S.cbuf(v, turn & 1), S.cnt(v, turn & 1), a.sc, a.l1, v ? W.lo_t : W.lo_s,
+                                 v ? W.hi_t : W.hi_s);
+        }
+    } else {
+        if constexpr (L::F32) {
+            if (lane == 0) load_tma(*maps, a, S, bid, nblk, items, gx, gy, ny, nw);
+            __syncwarp();
+        } else {
+            load_async<T>(a, S, bid, nblk, items, gx, gy);
+        }
     }
     __syncthreads();
-
-    K1State S;
-    const bool edge = !(i0 >= 2 && i0 + L::TY + 3 <= g.n1 && j0 >= 2 && j0 + L::TX + 3 <= g.n2);
-    const bool hist = W.hs || W.ht;
-    const bool ok = edge ? (hist ? k1_tile<true, true>(maps, a, sm, ccnt, i0, j0, b0, b1, S, W, cs)
-                                 : k1_tile<true, false>(maps, a, sm, ccnt, i0, j0, b0, b1, S, W, cs))
-                         : (hist ? k1_tile<false, true>(maps, a, sm, ccnt, i0, j0, b0, b1, S, W, cs)
-                                 : k1_tile<false, false>(maps, a, sm, ccnt, i0, j0, b0, b1, S, W, cs));
-    if (!ok) {
-        // a load never arrived: record it, let this CTA's copies land (bounded)
-        // before its shared memory is released, and skip the statistics (the
-        // producer holds the counts of the copies it issued)
-        if (tid == L::PRODUCER) {
-            atomicOr(&a.sc->error, 4);
-            for (int k = 0; k < L::NYS; ++k)
-                if (S.n_y > (unsigned)k) (void)mbar_wait(bars + k, ((S.n_y - 1 - k) / L::NYS) & 1);
-            for (int k = 0; k < L::NWS; ++k)
-                if (S.n_w > (unsigned)k)
-                    (void)mbar_wait(bars + L::NYS + k, ((S.n_w - 1 - k) / L::NWS) & 1);
-        }
-        __syncthreads();
+    if (abort_flag) {                                           // a load never arrived
+        if (tid == 0) atomicOr(&a.sc->error, 4);
+        if constexpr (L::F32)
+            if (tid == 32 * kConsWarps) drain_tma(S, ny, nw);
     }
 
     // this CTA among every CTA of the pass stage (all slabs of a split cube)
-    const int cta = a.sp.cta_base + bx + gx * (by + gy * bz);
+    const int cta = a.sp.cta_base + bid;
     if (W.s || W.t) {
-        // the buffered window candidates join the global list (one atomic per vector)
-        __syncthreads();
-        if (tid < 2) {
-            const unsigned n = min(ccnt[tid], (unsigned)L::CB);
-            cbase[tid] = n ? atomicAdd(&a.sc->acc[tid].m, n) : 0u;
-        }
-        __syncthreads();
-        const float* cbuf = reinterpret_cast<const float*>(sm + L::OFF_CB);
-        for (int v = 0; v < 2; ++v) {
-            const unsigned n = min(ccnt[v], (unsigned)L::CB);
-            for (unsigned k = tid; k < n; k += L::NT)
-                if (cbase[v] + k < kCandCap) a.l1.cand[v][cbase[v] + k] = cbuf[v * L::CB + k];
-            // and into the list's key histogram over the window, which the
-            // finish then narrows without another pass over the candidates
-            unsigned* h = v == 0 ? W.nh_s : W.nh_t;
-            if (h) {
-                const NarrowGeom& ng = v == 0 ? W.ng_s : W.ng_t;
-                for (unsigned k = tid; k < n; k += L::NT) narrow_add(h, ng, __float_as_uint(cbuf[v * L::CB + k]));
-                if (tid == 0 && n) atomicAdd(a.l1.nbinned + v, n);
-            }
-        }
-        if (W.hs || W.ht) {
+        if (hist) {
             // the histogram joins the global one (unpacked, nonzero bins only)
-            const unsigned* hsm = reinterpret_cast<const unsigned*>(sm + L::OFF_HIST);
             for (int k = tid; k < kK1Bins; k += L::NT) {
-                const unsigned w = hsm[k];
+                const unsigned w = S.hist()[k];
                 const int v = k / (kK1Bins / 2), b = 2 * (k - v * (kK1Bins / 2));
                 unsigned* gh = a.l1.khist + v * kK1Bins + b;
                 if (w & 0xffffu) atomicAdd(gh, w & 0xffffu);
@@ -691,42 +1019,48 @@ __device__ __forceinline__ void k1_run(const K1Maps& maps, const K1TArgs& a, con
         }
         // the CTA's window statistics (counts and sums above the windows) and
         // the histograms' above-range statistics, reduced together: 32-bit
-        // counts and float-pair sums through the warps, one barrier, thread 0
-        // finishes (no FP64 outside thread 0)
-        unsigned n4[4] = {S.acc_s.n, S.acc_t.n, S.top_s.n, S.top_t.n};
-        float hi4[4] = {S.ks.x, S.ks.y, S.top_s.s.s, S.top_t.s.s};
-        float lo4[4] = {-S.kc.x, -S.kc.y, -S.top_s.s.c, -S.top_t.s.c};
+        // counts and float-pair sums through the tile warps, then through
+        // warp 0 (no FP64 outside one thread)
+        unsigned n4[4] = {A.n_s, A.n_t, A.top_s.n, A.top_t.n};
+        float hi4[4] = {A.ks.x, A.ks.y, A.top_s.s, A.top_t.s};
+        float lo4[4] = {-A.kc.x, -A.kc.y, 0.f, 0.f};
+        auto reduce = [&](int from) {
+            for (int o = from; o > 0; o >>= 1) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                n4[q] += __shfl_xor_sync(0xffffffffu, n4[q], o);
-                const float bh = __shfl_xor_sync(0xffffffffu, hi4[q], o), bl = __shfl_xor_sync(0xffffffffu, lo4[q], o);
-                pair_add(hi4[q], lo4[q], bh, bl);
+                for (int q = 0; q < 4; ++q) {
+                    n4[q] += __shfl_xor_sync(0xffffffffu, n4[q], o);
+                    const float bh = __shfl_xor_sync(0xffffffffu, hi4[q], o);
+                    const float bl = __shfl_xor_sync(0xffffffffu, lo4[q], o);
+                    pair_add(hi4[q], lo4[q], bh, bl);
+                }
             }
-        }
-        float* wbuf = reinterpret_cast<float*>(sm + L::OFF_G);          // idle now: 16 warps x 12 values
-        if ((tid & 31) == 0) {
+        };
+        if (wid < kTileWarps) {
+            reduce(16);
+            if (lane == 0) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                wbuf[(tid >> 5) * 12 + q] = __uint_as_float(n4[q]);
-                wbuf[(tid >> 5) * 12 + 4 + q] = hi4[q];
-                wbuf[(tid >> 5) * 12 + 8 + q] = lo4[q];
+                for (int q = 0; q < 4; ++q) {
+                    wred[wid * 12 + q] = __uint_as_float(n4[q]);
+                    wred[wid * 12 + 4 + q] = hi4[q];
+                    wred[wid * 12 + 8 + q] = lo4[q];
+                }
             }
         }
         __syncthreads();
-        if (tid == 0) {
+        if (wid == 0) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                unsigned long long n = 0;
-                float h = wbuf[4 + q], l = wbuf[8 + q];
-                n += __float_as_uint(wbuf[q]);
-                for (int w = 1; w < L::NT / 32; ++w) {
-                    n += __float_as_uint(wbuf[w * 12 + q]);
-                    pair_add(h, l, wbuf[w * 12 + 4 + q], wbuf[w * 12 + 8 + q]);
+                n4[q] = lane < kTileWarps ? __float_as_uint(wred[lane * 12 + q]) : 0u;
+                hi4[q] = lane < kTileWarps ? wred[lane * 12 + 4 + q] : 0.f;
+                lo4[q] = lane < kTileWarps ? wred[lane * 12 + 8 + q] : 0.f;
+            }
+            reduce(kTileWarps / 2);
+            if (lane == 0) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    a.l1.k1_n[4 * cta + q] = n4[q];
+                    a.l1.k1_s[4 * cta + q] = (double)hi4[q] + (double)lo4[q];
                 }
-                a.l1.k1_n[4 * cta + q] = n;
-                a.l1.k1_s[4 * cta + q] = (double)h + (double)l;
             }
         }
     }
@@ -738,8 +1072,14 @@ __device__ __forceinline__ void k1_run(const K1Maps& maps, const K1TArgs& a, con
     }
 }
 
-__global__ void __launch_bounds__(512, 1) k1_tma(const __grid_constant__ K1Maps maps, const K1TArgs a) {
-    k1_run(maps, a, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x, gridDim.y, gridDim.z);
+__global__ void __launch_bounds__(Lay<float>::NT, 1) k1_tma(const __grid_constant__ K1Maps maps,
+                                                            const __grid_constant__ K1Args<float> a, int gx, int gy,
+                                                            int gz) {
+    k1_run<float>(&maps, a, blockIdx.x, gridDim.x, gx, gy, gz);
+}
+template <typename T>
+__global__ void __launch_bounds__(Lay<T>::NT, 1) k1_half(const __grid_constant__ K1Args<T> a, int gx, int gy, int gz) {
+    k1_run<T>(nullptr, a, blockIdx.x, gridDim.x, gx, gy, gz);
 }
 
 // K1 over many cubes in one launch: the cube of a CTA from a table of first
@@ -747,9 +1087,9 @@ __global__ void __launch_bounds__(512, 1) k1_tma(const __grid_constant__ K1Maps 
 struct K1BatchTab {
     int n;
     int start[kBatchMax + 1];
-    short gx[kBatchMax], gy[kBatchMax], gz[kBatchMax];
+    int gx[kBatchMax], gy[kBatchMax], gz[kBatchMax];
     const K1Maps* maps[kBatchMax];
-    K1TArgs args[kBatchMax];
+    K1Args<float> args[kBatchMax];
 };
 
 __device__ __forceinline__ int batch_cube_of(const int* start, int n, int blk) {
@@ -761,77 +1101,91 @@ __device__ __forceinline__ int batch_cube_of(const int* start, int n, int blk) {
     return lo;
 }
 
-__global__ void __launch_bounds__(512, 1) k1_tma_batch(const __grid_constant__ K1BatchTab t) {
+__global__ void __launch_bounds__(Lay<float>::NT, 1) k1_tma_batch(const __grid_constant__ K1BatchTab t) {
     const int c = batch_cube_of(t.start, t.n, blockIdx.x);
     // the cube's arguments by value: the table is indexed by a run-time
     // cube, so each field is loaded once instead of at each use
-    const K1TArgs a = t.args[c];
+    const K1Args<float> a = t.args[c];
     if (__ldcg(&a.sc->done)) return;        // this cube has stopped
-    const int gx = t.gx[c], gy = t.gy[c], gz = t.gz[c];
-    const int l = blockIdx.x - t.start[c];
-    const int bx = l % gx, by = (l / gx) % gy, bz = l / (gx * gy);
     const K1Maps* maps = t.maps[c];
-    if (threadIdx.x == Lay::PRODUCER) {
+    if (threadIdx.x == 32 * kConsWarps) {
         // the cube's tensor maps sit in global memory (the copies' descriptors)
-        tma_prefetch_map(&maps->y1); tma_prefetch_map(&maps->y2); tma_prefetch_map(&maps->w1);
-        tma_prefetch_map(&maps->w2); tma_prefetch_map(&maps->u); tma_prefetch_map(&maps->q);
+        tma_prefetch_map(&maps->y1v); tma_prefetch_map(&maps->y1h); tma_prefetch_map(&maps->y2v);
+        tma_prefetch_map(&maps->y2h); tma_prefetch_map(&maps->w1); tma_prefetch_map(&maps->w2); tma_prefetch_map(&maps->u); tma_prefetch_map(&maps->q);
         tma_prefetch_map(&maps->s); tma_prefetch_map(&maps->t); tma_prefetch_map(&maps->y3);
     }
-    k1_run(*maps, a, bx, by, bz, gx, gy, gz);
+    k1_run<float>(maps, a, blockIdx.x - t.start[c], t.start[c + 1] - t.start[c], t.gx[c], t.gy[c], t.gz[c]);
 }
 
-// Bands per CTA.  One CTA runs per SM, so a launch of U CTAs on S SMs takes
-// ceil(U / S) waves and the last wave leaves SMs idle; every CTA also pays a
-// prologue of about 1.5 band steps (its first copies, D^T y2 of the band
-// before, u' of its first band).  Picks the split of the bands (runs of at
-// least 8) that minimises idle fraction + prologue fraction.
-int tma_chunk(int nb, int tiles) {
-    const double kSms = (double)device_sms();
-    constexpr double kPrologue = 1.5;
-    const int max_chunks = std::max(1, nb / 8);
-    int best_len = nb;
+// ---------------------------------------------------------------------------
+// host: how a cube is split
+// ---------------------------------------------------------------------------
+// Band steps that an item costs beyond its bands: u' of its first band, the
+// copies of the bands before and after it, and the wait for its first planes.
+constexpr double kItemCost = 1.5;
+
+int tiles_of(const Geom& g) { return ((g.n2 + TX - 1) / TX) * ((g.n1 + TY - 1) / TY); }
+
+// Band steps of the slowest of `ctas` CTAs when `tiles` tiles of nb bands run
+// as items of len bands.
+double run_cost(int nb, int tiles, int len, int ctas) {
+    const long long items = (long long)tiles * ((nb + len - 1) / len);
+    return (double)((items + ctas - 1) / ctas) * (len + kItemCost);
+}
+
+// Bands per item for `ctas` persistent CTAs: the split of the bands whose
+// slowest CTA does the fewest band steps.
+int best_run(int nb, int tiles, int ctas) {
+    int best_len = std::min(nb, kMaxRun);
     double best = 1e30;
-    for (int chunks = 1; chunks <= max_chunks; ++chunks) {
-        const int len = (nb + chunks - 1) / chunks;
-        const int used = (nb + len - 1) / len;                 // chunks actually launched
-        const double units = (double)tiles * used;
-        const double waves = std::ceil(units / kSms);
-        const double waste = (waves - units / kSms) / waves + kPrologue / len;
-        if (waste < best - 1e-12) { best = waste; best_len = len; }
+    int prev = 0;
+    for (int runs = 1; runs <= nb; ++runs) {
+        const int len = (nb + runs - 1) / runs;
+        if (len == prev || len > kMaxRun) continue;
+        prev = len;
+        const double c = run_cost(nb, tiles, len, ctas);
+        if (c < best * (1.0 - 1e-12)) { best = c; best_len = len; }
     }
     return best_len;
 }
 
-}  // namespace
-
-// CTAs of the largest launch any allowed band run gives (runs of at least 8
-// bands, or all of them when there are fewer): the per-CTA statistics arrays
-// are sized for it.
-int k1_tma_ctas(const Geom& g) {
-    const int tx = (g.n2 + Lay::TX - 1) / Lay::TX, ty = (g.n1 + Lay::TY - 1) / Lay::TY;
-    const int shortest = std::min(8, g.n3);
-    return tx * ty * ((g.n3 + shortest - 1) / shortest);
+// One launch's split: bands per item and CTAs.  One CTA per SM, and more only
+// for cubes so large that a CTA's sampled histogram could pass its 16-bit
+// counters (an item counts at most 512 voxels for every 32 of its bands).
+struct Plan {
+    int chunk, gz, ctas;
+};
+Plan k1_plan(const Geom& g, int nb, int chunk, int ctas) {
+    Plan p;
+    const int tiles = tiles_of(g);
+    p.chunk = chunk >= 1 && chunk <= std::min(nb, kMaxRun) ? chunk : best_run(nb, tiles, ctas);
+    p.gz = (nb + p.chunk - 1) / p.chunk;
+    const long long items = (long long)tiles * p.gz;
+    const long long per = std::max(1, 127 / ((p.chunk + 31) / 32));       // items a CTA may count
+    p.ctas = (int)std::min(items, std::max((long long)ctas, (items + per - 1) / per));
+    return p;
 }
 
-// Run lengths worth timing: the model's choice and the next best by its
-// estimate, at most `cap` distinct lengths, the model's choice first.
+}  // namespace
+
+// CTAs of the largest launch any run length gives: the per-CTA statistics
+// arrays are sized for it.
+int k1_tma_ctas(const Geom& g) {
+    return std::max(device_sms(), tiles_of(g) * ((g.n3 + std::min(8, g.n3) - 1) / std::min(8, g.n3)));
+}
+
+// Run lengths worth timing: the model's choice first, then the next best of
+// at least 8 bands by its estimate, at most `cap` distinct lengths.
 int k1_tma_chunk_candidates(const Geom& g, int* out, int cap) {
-    const double kSms = (double)device_sms();
-    constexpr double kPrologue = 1.5;
-    const int tx = (g.n2 + Lay::TX - 1) / Lay::TX, ty = (g.n1 + Lay::TY - 1) / Lay::TY;
-    const int tiles = tx * ty;
-    const int max_chunks = std::max(1, g.n3 / 8);
+    const int tiles = tiles_of(g), sms = device_sms();
     std::vector<std::pair<double, int>> c;
-    for (int chunks = 1; chunks <= max_chunks; ++chunks) {
-        const int len = (g.n3 + chunks - 1) / chunks;
-        if (!c.empty() && c.back().second == len) continue;
-        const int used = (g.n3 + len - 1) / len;
-        const double units = (double)tiles * used;
-        const double waves = std::ceil(units / kSms);
-        c.push_back({(waves - units / kSms) / waves + kPrologue / len, len});
+    for (int runs = 1; runs <= std::max(1, g.n3 / 8); ++runs) {
+        const int len = (g.n3 + runs - 1) / runs;
+        if (len > kMaxRun || (!c.empty() && c.back().second == len)) continue;
+        c.push_back({run_cost(g.n3, tiles, len, sms), len});
     }
     std::stable_sort(c.begin(), c.end(), [](const auto& x, const auto& y) { return x.first < y.first; });
-    const int first = tma_chunk(g.n3, tiles);
+    const int first = best_run(g.n3, tiles, sms);
     int n = 0;
     if (cap > 0) out[n++] = first;
     for (const auto& e : c)
@@ -839,49 +1193,106 @@ int k1_tma_chunk_candidates(const Geom& g, int* out, int cap) {
     return n;
 }
 
-// The TMA-fed kernel is built for float32 storage only (16-bit storage runs
-// the cooperative-load kernel of k_stencil.cu).
 int k1_tma_configure(int storage) {
-    if (storage != 0) return -1;
-    const cudaError_t e = cudaFuncSetAttribute(k1_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay::SMEM);
+    cudaError_t e = cudaErrorInvalidValue;
+    switch (storage) {
+        case 0: e = cudaFuncSetAttribute(k1_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<float>::SMEM); break;
+        case 1: e = cudaFuncSetAttribute(k1_half<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<__nv_bfloat16>::SMEM); break;
+        case 2: e = cudaFuncSetAttribute(k1_half<__half>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<__half>::SMEM); break;
+    }
     return e == cudaSuccess ? 0 : -3;
 }
 
-// tensor maps over the current-parity buffers of one iteration
-int k1_tma_maps(int storage, const Geom& g, const IterBufs& b, K1Maps* m) {
-    if (storage != 0) return -1;
-    constexpr int sw = Lay::SW, ty = Lay::TY;
+// tensor maps over the current-parity buffers of one iteration (float32)
+int k1_tma_maps(const Geom& g, const IterBufs& b, K1Maps* m) {
     int rc = 0;
-    rc |= tma_encode_cubes(&m->y1, b.y1, 4, g.n1, g.n2, g.n3, g.p2, 2, sw, ty + 4);
-    rc |= tma_encode_cubes(&m->y2, b.y2, 4, g.n1, g.n2, g.n3, g.p2, 2, sw, ty + 4);
-    rc |= tma_encode_cubes(&m->w1, b.w1, 4, g.n1, g.n2, g.n3, g.p2, 6, sw, ty + 2);
-    rc |= tma_encode_cubes(&m->w2, b.w2, 4, g.n1, g.n2, g.n3, g.p2, 6, sw, ty + 2);
-    rc |= tma_encode_cubes(&m->u, b.u, 4, g.n1, g.n2, g.n3, g.p2, 1, sw, ty + 1);
-    rc |= tma_encode_cubes(&m->q, b.q, 4, g.n1, g.n2, g.n3, g.p2, 1, sw, ty + 1);
-    rc |= tma_encode_cubes(&m->s, b.s, 4, g.n1, g.n2, g.n3, g.p2, 1, Lay::TX, ty);
-    rc |= tma_encode_cubes(&m->t, b.t, 4, g.n1, g.n2, g.n3, g.p2, 1, Lay::TX, ty);
-    rc |= tma_encode_cubes(&m->y3, b.y3, 4, g.n1, g.n2, g.n3, g.p2, 1, Lay::TX, ty + 1);
+    // y_v without its last row and y_h without its last column (where D is
+    // structurally zero and L and D^T read them as zero): the copies' zero fill
+    // then masks them, and no load in the kernel needs a test
+    const float *y1 = (const float*)b.y1, *y2 = (const float*)b.y2;
+    const int rv = std::max(g.n1 - 1, 1), ch = std::max(g.n2 - 1, 1);
+    rc |= tma_encode_cubes(&m->y1v, y1, g, rv, g.n2, 1, SW, YR);
+    rc |= tma_encode_cubes(&m->y1h, y1 + g.cube, g, g.n1, ch, 1, SW, YR);
+    rc |= tma_encode_cubes(&m->y2v, y2, g, rv, g.n2, 1, SW, YR);
+    rc |= tma_encode_cubes(&m->y2h, y2 + g.cube, g, g.n1, ch, 1, SW, YR);
+    rc |= tma_encode_cubes(&m->w1, b.w1, g, g.n1, g.n2, 6, SW, WR);
+    rc |= tma_encode_cubes(&m->w2, b.w2, g, g.n1, g.n2, 6, SW, WR);
+    rc |= tma_encode_cubes(&m->u, b.u, g, g.n1, g.n2, 1, SW, UR);
+    rc |= tma_encode_cubes(&m->q, b.q, g, g.n1, g.n2, 1, SW, UR);
+    rc |= tma_encode_cubes(&m->s, b.s, g, g.n1, g.n2, 1, TX, TY);
+    rc |= tma_encode_cubes(&m->t, b.t, g, g.n1, g.n2, 1, TX, TY);
+    rc |= tma_encode_cubes(&m->y3, b.y3, g, g.n1, g.n2, 1, TX, TY + 1);
     return rc ? -3 : 0;
 }
 
-namespace {
-// bands per CTA for the part's nb updated bands
-int part_chunk(const Geom& g, int nb, int chunk) {
-    const int tx = (g.n2 + Lay::TX - 1) / Lay::TX, ty = (g.n1 + Lay::TY - 1) / Lay::TY;
-    return chunk >= std::min(8, nb) && chunk <= nb ? chunk : tma_chunk(nb, tx * ty);
-}
-}  // namespace
-
 int k1_tma_part_chunk(const Geom& g, const SlabPart& sp, int chunk) {
-    return sp.o1 > sp.o0 ? part_chunk(g, sp.o1 - sp.o0, chunk) : 0;
+    return sp.o1 > sp.o0 ? k1_plan(g, sp.o1 - sp.o0, chunk, device_sms()).chunk : 0;
 }
 
 int k1_tma_grid(const Geom& g, const SlabPart& sp, int chunk) {
-    const int nb = sp.o1 - sp.o0;
-    if (nb <= 0) return 0;
-    const int tx = (g.n2 + Lay::TX - 1) / Lay::TX, ty = (g.n1 + Lay::TY - 1) / Lay::TY;
-    const int c = part_chunk(g, nb, chunk);
-    return tx * ty * ((nb + c - 1) / c);
+    return sp.o1 > sp.o0 ? k1_plan(g, sp.o1 - sp.o0, chunk, device_sms()).ctas : 0;
+}
+
+namespace {
+template <typename T>
+K1Args<T> k1_args(const Geom& g, const IterBufs& b, const IterParams& p, Scal* sc, const L1Work& w, int chunk,
+                  const SlabPart& sp) {
+    K1Args<T> a;
+    a.g = g;
+    a.u = (const T*)b.u; a.q = (const T*)b.q; a.s = (const T*)b.s; a.t = (const T*)b.t; a.y3 = (const T*)b.y3;
+    a.y1 = (const T*)b.y1; a.y2 = (const T*)b.y2; a.w1 = (const T*)b.w1; a.w2 = (const T*)b.w2;
+    a.u_n = (T*)b.u_n; a.w1_n = (T*)b.w1_n; a.w2_n = (T*)b.w2_n; a.y1_n = (T*)b.y1_n; a.y2_n = (T*)b.y2_n;
+    a.p = p;
+    a.sc = sc;
+    a.l1 = w;
+    a.chunk = chunk;
+    a.sp = sp;
+    return a;
+}
+}  // namespace
+
+// The CTAs that each cube of a batch gets: persistent like a single cube's,
+// the SMs shared out so that the cube whose CTAs do the most band steps does
+// as few as possible (bisection on that count; every cube at least one CTA).
+void k1_batch_plan(const BatchCube* cubes, int n, int* chunk, int* gz, int* ctas) {
+    const int sms = device_sms();
+    // the fewest CTAs with which cube q stays within `steps` band steps
+    auto fewest = [&](const BatchCube& q, double steps, int* len_out) -> int {
+        const int nb = q.g.n3, tiles = tiles_of(q.g);
+        int best = 1 << 30, prev = 0;
+        for (int runs = 1; runs <= nb; ++runs) {
+            int len = (nb + runs - 1) / runs;
+            if (q.k1_chunk >= 1 && q.k1_chunk <= nb) len = q.k1_chunk;      // the cube's own (autotuned) run
+            if (len == prev) continue;
+            prev = len;
+            const long long per = (long long)(steps / (len + kItemCost));
+            if (len <= kMaxRun && per >= 1) {
+                const long long items = (long long)tiles * ((nb + len - 1) / len);
+                const long long c = (items + per - 1) / per;
+                if (c < best) { best = (int)c; *len_out = len; }
+            }
+            if (len == q.k1_chunk) break;
+        }
+        return best;
+    };
+    double lo = 0.0, hi = 1.0;
+    for (int c = 0; c < n; ++c) hi += (double)tiles_of(cubes[c].g) * (cubes[c].g.n3 + kItemCost) * 2.0;
+    const int budget = std::max(sms, n);
+    int len = 0;
+    for (int k = 0; k < 40 && hi - lo > 1e-3 * hi; ++k) {
+        const double mid = 0.5 * (lo + hi);
+        long long sum = 0;
+        for (int c = 0; c < n; ++c) sum += fewest(cubes[c], mid, &len);
+        if (sum <= budget) hi = mid; else lo = mid;
+    }
+    for (int c = 0; c < n; ++c) {
+        len = std::min(cubes[c].g.n3, kMaxRun);
+        const int want = std::min(std::max(1, fewest(cubes[c], hi, &len)), budget);
+        const Plan p = k1_plan(cubes[c].g, cubes[c].g.n3, len, want);
+        chunk[c] = p.chunk;
+        gz[c] = p.gz;
+        ctas[c] = p.ctas;
+    }
 }
 
 int launch_k1_batch(const BatchCube* cubes, int n, cudaStream_t st) {
@@ -889,59 +1300,46 @@ int launch_k1_batch(const BatchCube* cubes, int n, cudaStream_t st) {
     static_assert(sizeof(K1BatchTab) <= 32000, "kernel parameter space");
     K1BatchTab t{};
     t.n = n;
+    int chunk[kBatchMax], gz[kBatchMax], ctas[kBatchMax];
+    k1_batch_plan(cubes, n, chunk, gz, ctas);
     int total = 0;
     for (int c = 0; c < n; ++c) {
         const BatchCube& q = cubes[c];
-        const SlabPart whole = whole_cube(q.g);
-        K1TArgs& a = t.args[c];
-        a.g = q.g;
-        a.u_n = (float*)q.b.u_n; a.w1_n = (float*)q.b.w1_n; a.w2_n = (float*)q.b.w2_n;
-        a.y1_n = (float*)q.b.y1_n; a.y2_n = (float*)q.b.y2_n;
-        a.p = q.p;
-        a.sc = q.sc;
-        a.l1 = q.l1;
-        a.sp = whole;
-        a.chunk = part_chunk(q.g, q.g.n3, q.k1_chunk);
-        a.hist_fits = a.chunk * Lay::NT <= 65535;
-        const int tx = (q.g.n2 + Lay::TX - 1) / Lay::TX, ty = (q.g.n1 + Lay::TY - 1) / Lay::TY;
-        const int tz = (q.g.n3 + a.chunk - 1) / a.chunk;
-        if (tx > 32767 || ty > 32767 || tz > 32767) return -1;
-        t.gx[c] = (short)tx; t.gy[c] = (short)ty; t.gz[c] = (short)tz;
+        t.args[c] = k1_args<float>(q.g, q.b, q.p, q.sc, q.l1, chunk[c], whole_cube(q.g));
+        const int tx = (q.g.n2 + TX - 1) / TX, ty = (q.g.n1 + TY - 1) / TY;
+        t.gx[c] = tx; t.gy[c] = ty; t.gz[c] = gz[c];
         t.maps[c] = q.maps;
         t.start[c] = total;
-        total += tx * ty * tz;
+        total += ctas[c];
     }
     t.start[n] = total;
-    k1_tma_batch<<<total, Lay::NT, Lay::SMEM, st>>>(t);
+    k1_tma_batch<<<total, Lay<float>::NT, Lay<float>::SMEM, st>>>(t);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
 int k1_batch_configure() {
-    const cudaError_t e = cudaFuncSetAttribute(k1_tma_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay::SMEM);
+    const cudaError_t e = cudaFuncSetAttribute(k1_tma_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<float>::SMEM);
     return e == cudaSuccess ? 0 : -3;
 }
 
 int launch_k1_tma(int storage, const Geom& g, const K1Maps& m, const IterBufs& b, const IterParams& p,
                   Scal* sc, const L1Work& w, int chunk, const SlabPart& sp, cudaStream_t st) {
-    if (storage != 0) return -1;
     const int nb = sp.o1 - sp.o0;
     if (nb <= 0 || sp.o0 < 0 || sp.o1 > g.n3) return -1;
-    K1TArgs a;
-    a.g = g;
-    a.u_n = (float*)b.u_n; a.w1_n = (float*)b.w1_n; a.w2_n = (float*)b.w2_n;
-    a.y1_n = (float*)b.y1_n; a.y2_n = (float*)b.y2_n;
-    a.p = p;
-    a.sc = sc;
-    a.l1 = w;
-    a.sp = sp;
-    const int tx = (g.n2 + Lay::TX - 1) / Lay::TX, ty = (g.n1 + Lay::TY - 1) / Lay::TY;
-    a.chunk = part_chunk(g, nb, chunk);
-    // the histogram's packed 16-bit counters hold a CTA's voxels; a split cube
-    // passes the longest run of all its launches in sp.max_chunk, so that
-    // every launch of the stage agrees
-    a.hist_fits = std::max(a.chunk, sp.max_chunk) * Lay::NT <= 65535;
-    dim3 grid(tx, ty, (nb + a.chunk - 1) / a.chunk);
-    k1_tma<<<grid, Lay::NT, Lay::SMEM, st>>>(m, a);
+    const Plan pl = k1_plan(g, nb, chunk, device_sms());
+    const int gx = (g.n2 + TX - 1) / TX, gy = (g.n1 + TY - 1) / TY;
+    auto half = [&](auto zero) {
+        using T = decltype(zero);
+        k1_half<T><<<pl.ctas, Lay<T>::NT, Lay<T>::SMEM, st>>>(k1_args<T>(g, b, p, sc, w, pl.chunk, sp), gx, gy, pl.gz);
+    };
+    switch (storage) {
+        case 0:
+            k1_tma<<<pl.ctas, Lay<float>::NT, Lay<float>::SMEM, st>>>(m, k1_args<float>(g, b, p, sc, w, pl.chunk, sp), gx, gy, pl.gz);
+            break;
+        case 1: half(__nv_bfloat16()); break;
+        case 2: half(__half()); break;
+        default: return -1;
+    }
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
