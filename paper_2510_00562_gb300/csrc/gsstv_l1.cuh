@@ -116,10 +116,11 @@ __device__ __forceinline__ unsigned long long narrow_res(unsigned long long w) {
 // The key histogram of vector v's candidate list when every one of its m
 // candidates was counted into it (built by the passes that appended them,
 // over the same window), else null.
-__device__ __forceinline__ const unsigned* narrow_pre(const L1Work& w, int v, unsigned m) {
+__device__ __forceinline__ unsigned* narrow_pre(const L1Work& w, int v, unsigned m) {
     return (w.nh && m > 0u && __ldcg(w.nbinned + v) == m) ? w.nh + v * 3 * kNarrowBins : nullptr;
 }
-// Clears vector v's list histogram after its finish has read it (whole block).
+// Clears vector v's list histogram unless its finish has (l1_narrow clears it
+// as it reads it); whole block.
 __device__ __forceinline__ void narrow_clear(const L1Work& w, int v) {
     if (!w.nh) return;
     const unsigned used = __ldcg(w.nbinned + v);
@@ -133,7 +134,7 @@ __device__ __forceinline__ void narrow_clear(const L1Work& w, int v) {
 // scr: 3 kNarrowBins unsigned of shared memory; sh_d: 4 doubles of shared
 // memory; pre (optional): the candidates' key
 // histogram over (klo, khi], already built (the first round reads it instead
-// of binning the candidates).  On
+// of binning the candidates, and clears it and its counter nbinned).  On
 // return 0: (klo, khi] narrowed, n_hi / s_hi now count everything above khi,
 // and the *m_st values in the new window are staged as floats in scr.
 // Returns 1 when phi at the window's lower end is negative (the root lies
@@ -142,7 +143,7 @@ __device__ __forceinline__ void narrow_clear(const L1Work& w, int v) {
 // narrow in a few rounds.
 static __device__ int l1_narrow(const float* cand, bool cand_shared, unsigned m, double& n_hi, double& s_hi,
                                 unsigned& klo, unsigned& khi, double r, unsigned* scr, unsigned* m_st, int* sh_i,
-                                double* sh_d, const unsigned* pre = nullptr) {
+                                double* sh_d, unsigned* pre = nullptr, unsigned* nbinned = nullptr) {
     // every candidate, from global memory (batched loads) or from shared memory
     auto each = [&](auto&& f) {
         if (cand_shared) {
@@ -163,21 +164,18 @@ static __device__ int l1_narrow(const float* cand, bool cand_shared, unsigned m,
         if (round == 0 && pre) {
             // 16-byte loads, all of a thread's issued before its stores (one
             // CTA copying from L2 is bound by the loads' latency)
-            const uint4* p4 = reinterpret_cast<const uint4*>(pre);
+            uint4* p4 = reinterpret_cast<uint4*>(pre);
             uint4* s4 = reinterpret_cast<uint4*>(scr);
             constexpr int kW4 = 2 * kNarrowBins / 4;
-            uint4 q[2];
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const int k = (int)threadIdx.x + j * (int)blockDim.x;
-                if (k < kW4) q[j] = __ldcg(p4 + k);
+            const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+            for (int k0 = (int)threadIdx.x; k0 < kW4; k0 += 2 * (int)blockDim.x) {
+                const int k1 = k0 + (int)blockDim.x;
+                const uint4 q0 = __ldcg(p4 + k0), q1 = k1 < kW4 ? __ldcg(p4 + k1) : zero;
+                s4[k0] = q0;
+                p4[k0] = zero;
+                if (k1 < kW4) { s4[k1] = q1; p4[k1] = zero; }
             }
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const int k = (int)threadIdx.x + j * (int)blockDim.x;
-                if (k < kW4) s4[k] = q[j];
-            }
-            for (int k = (int)threadIdx.x + 2 * (int)blockDim.x; k < kW4; k += blockDim.x) s4[k] = __ldcg(p4 + k);
+            if (threadIdx.x == 0) *nbinned = 0u;
         } else {
             for (int k = threadIdx.x; k < 2 * kNarrowBins; k += blockDim.x) scr[k] = 0u;
             __syncthreads();
@@ -216,42 +214,34 @@ static __device__ int l1_narrow(const float* cand, bool cand_shared, unsigned m,
             return phi_at((double)__uint_as_float(lk), V(lk), Nsuf, Ssuf);
         };
         // The bin whose lower edge is the highest with phi >= 0 (phi does not
-        // increase with the edge, so those edges come first).  Warp 0 alone:
-        // FP64 runs at a small fraction of the FP32 rate on this part, and one
-        // warp's FP64 instruction costs what the whole block's would divided
-        // by its warps.  Each lane sums a chunk of at most 64 bins; the
-        // highest lane whose chunk's lowest edge has phi >= 0 holds the bin,
-        // which the lanes then find two bins each.
-        if (threadIdx.x < 32) {
-            const int lane = (int)threadIdx.x;
-            // phi at an edge e inside the window (b > 0) is A + u0 X with
-            // A = s_hi - r and the exact integer X = Ssuf - (Nsuf + n_hi) e/u0,
-            // so phi >= 0 exactly when X >= T = ceil(-A / u0) (u0 a power of
-            // two: the quotient is exact): the lanes test in integers, lane 0
-            // alone computes T in FP64.  Windows so narrow against the sums
-            // that T leaves 62 bits take the FP64 test.
-            long long T = 0, NH = 0;
-            int int_ok = 0;
-            if (lane == 0) {
+        // increase with the edge, so those edges come first).  The block's
+        // threads take a few bins each (two with 1024 threads), in integers:
+        // phi at an edge e inside the window (b > 0) is A + u0 X with A =
+        // s_hi - r and the exact integer X = Ssuf - (Nsuf + n_hi) e/u0, so
+        // phi >= 0 exactly when X >= T = ceil(-A / u0) (u0 a power of two: the
+        // quotient is exact); thread 0 alone computes T in FP64, which runs at
+        // a small fraction of the FP32 rate on this part.  Windows so narrow
+        // against the sums that T leaves 62 bits take the FP64 test.  (One
+        // warp with 64 bins a lane took 8 us of this step's 12, measured on
+        // 512x512x224.)
+        __shared__ unsigned long long nr_N[32], nr_S[32];
+        __shared__ long long nr_T, nr_H;
+        __shared__ int nr_int, nr_best;
+        {
+            const int tid = (int)threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = ((int)blockDim.x + 31) >> 5;
+            if (tid == 0) {
                 const double q = ceil(-(s_hi - r) / u0);
-                int_ok = fabs(q) < 4.6e18 && n_hi >= 0.0 && n_hi < 9.0e15;
-                T = int_ok ? (long long)q : 0;
-                NH = int_ok ? (long long)n_hi : 0;
+                const bool ok = fabs(q) < 4.6e18 && n_hi >= 0.0 && n_hi < 9.0e15;
+                nr_int = ok ? 1 : 0;
+                nr_T = ok ? (long long)q : 0;
+                nr_H = ok ? (long long)n_hi : 0;
+                nr_best = -1;
             }
-            int_ok = __shfl_sync(0xffffffffu, int_ok, 0);
-            T = __shfl_sync(0xffffffffu, T, 0);
-            NH = __shfl_sync(0xffffffffu, NH, 0);
-            auto edge_ok = [&](int b, unsigned long long Nsuf, unsigned long long Ssuf) -> bool {
-                if (b == 0 || !int_ok) return edge_phi(b, Nsuf, Ssuf) >= 0.0;
-                const unsigned lk = (base + (unsigned)b) << shift;
-                const __int128 X = (__int128)Ssuf - (__int128)(Nsuf + (unsigned long long)NH) * (__int128)V(lk);
-                return X >= (__int128)T;
-            };
-            const int per = (nb + 31) / 32;
-            const int c0 = lane * per, c1 = min(nb, c0 + per);
+            const int per = (nb + (int)blockDim.x - 1) / (int)blockDim.x;
+            const int c0 = tid * per, c1 = min(nb, c0 + per);
             unsigned long long Nc = 0, Sc = 0;
             for (int b = c0; b < c1; ++b) { Nc += narrow_count(hw[b]); Sc += bin_int(b); }
-            // inclusive suffix over the lanes: the bins from c0 up
+            // inclusive suffix over the warp's lanes, then the warps above
             unsigned long long Ni = Nc, Si = Sc;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -259,43 +249,38 @@ static __device__ int l1_narrow(const float* cand, bool cand_shared, unsigned m,
                 const unsigned long long y = __shfl_down_sync(0xffffffffu, Si, o);
                 if (lane + o < 32) { Ni += x; Si += y; }
             }
-            const bool ok = c0 < c1 && edge_ok(c0, Ni, Si);
-            const unsigned okm = __ballot_sync(0xffffffffu, ok);
-            if (okm == 0u) {
-                if (lane == 0) {
-                    sh_i[0] = -1;
-                    // phi at the window's lower end, and the count above it
-                    sh_d[2] = edge_phi(0, Ni, Si);
-                    sh_d[3] = n_hi + (double)Ni;
-                }
-            } else {
-                const int L = 31 - __clz(okm);
-                const int l0 = L * per, l1 = min(nb, l0 + per);
-                // the bins above lane L's chunk
-                const unsigned long long Nup = __shfl_sync(0xffffffffu, Ni - Nc, L);
-                const unsigned long long Sup = __shfl_sync(0xffffffffu, Si - Sc, L);
-                const int bA = l0 + 2 * lane, bB = bA + 1;
-                const unsigned long long nA = bA < l1 ? narrow_count(hw[bA]) : 0ull, sA = bA < l1 ? bin_int(bA) : 0ull;
-                const unsigned long long nB = bB < l1 ? narrow_count(hw[bB]) : 0ull, sB = bB < l1 ? bin_int(bB) : 0ull;
-                unsigned long long Nj = nA + nB, Sj = sA + sB;      // inclusive suffix from bA
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const unsigned long long x = __shfl_down_sync(0xffffffffu, Nj, o);
-                    const unsigned long long y = __shfl_down_sync(0xffffffffu, Sj, o);
-                    if (lane + o < 32) { Nj += x; Sj += y; }
-                }
-                const bool okA = bA < l1 && edge_ok(bA, Nup + Nj, Sup + Sj);
-                const bool okB = bB < l1 && edge_ok(bB, Nup + Nj - nA, Sup + Sj - sA);
-                const int mine = okB ? bB : okA ? bA : -1;
-                const int best = __reduce_max_sync(0xffffffffu, mine);
-                if (mine == best) {
-                    // the bins above the chosen one
-                    const unsigned long long an = best == bB ? Nup + Nj - nA - nB : Nup + Nj - nA;
-                    const unsigned long long as = best == bB ? Sup + Sj - sA - sB : Sup + Sj - sA;
-                    sh_i[0] = best;
-                    sh_d[0] = n_hi + (double)an;
-                    sh_d[1] = s_hi + (double)as * u0;
-                }
+            if (lane == 0) { nr_N[wid] = Ni; nr_S[wid] = Si; }
+            __syncthreads();
+            const bool above = lane > wid && lane < nw;
+            const unsigned long long Nw = warp_sum(above ? nr_N[lane] : 0ull), Sw = warp_sum(above ? nr_S[lane] : 0ull);
+            unsigned long long Nr = Nw + (Ni - Nc), Sr = Sw + (Si - Sc);    // the bins above this thread's
+            const bool int_ok = nr_int != 0;
+            const long long T = nr_T, NH = nr_H;
+            auto edge_ok = [&](int b, unsigned long long Nsuf, unsigned long long Ssuf) -> bool {
+                if (b == 0 || !int_ok) return edge_phi(b, Nsuf, Ssuf) >= 0.0;
+                const unsigned lk = (base + (unsigned)b) << shift;
+                const __int128 X = (__int128)Ssuf - (__int128)(Nsuf + (unsigned long long)NH) * (__int128)V(lk);
+                return X >= (__int128)T;
+            };
+            int mine = -1;
+            for (int b = c1 - 1; b >= c0 && mine < 0; --b) {
+                const unsigned long long n = narrow_count(hw[b]), sb = bin_int(b);
+                if (edge_ok(b, Nr + n, Sr + sb)) mine = b;
+                else { Nr += n; Sr += sb; }
+            }
+            const int best_w = __reduce_max_sync(0xffffffffu, mine);
+            if (lane == 0 && best_w >= 0) atomicMax(&nr_best, best_w);
+            __syncthreads();
+            const int best = nr_best;
+            if (mine == best && best >= 0) {               // the bins above the chosen one
+                sh_i[0] = best;
+                sh_d[0] = n_hi + (double)Nr;
+                sh_d[1] = s_hi + (double)Sr * u0;
+            } else if (best < 0 && tid == 0) {
+                sh_i[0] = -1;
+                // phi at the window's lower end, and the count above it
+                sh_d[2] = edge_phi(0, Nr, Sr);
+                sh_d[3] = n_hi + (double)Nr;
             }
         }
         __syncthreads();
@@ -347,7 +332,8 @@ static __device__ int l1_window_finish(double n_hi, double s_hi, const float* ca
                                        double* tau_out, double* red_d,
                                        unsigned long long* red_u, WinInfo* info = nullptr,
                                        float* stage = nullptr, unsigned stage_cap = 0,
-                                       unsigned* scr = nullptr, const unsigned* pre = nullptr) {
+                                       unsigned* scr = nullptr, unsigned* pre = nullptr,
+                                       unsigned* nbinned = nullptr) {
     // The scalar tests in FP64 on thread 0 (FP64 is scarce on this part),
     // shared with the block.
     __shared__ int wp_rc, wp_narrow, wp_pre;
@@ -356,7 +342,6 @@ static __device__ int l1_window_finish(double n_hi, double s_hi, const float* ca
         const double phi_hi = s_hi - n_hi * theta_hi - r;
         if (info) info->phi_hi = phi_hi;
         wp_rc = m_raw > kCandCap ? 1 : phi_hi > 0.0 ? 2 : -1;     // 2: root above the window
-        wp_narrow = wp_rc < 0 && scr && m_raw > kNarrowMin && theta_lo >= 0.0;
         // the window's ends as float keys: (klo, khi] holds every candidate
         unsigned klo = __float_as_uint((float)theta_lo), khi = __float_as_uint((float)theta_hi);
         if ((double)__uint_as_float(klo) > theta_lo) klo -= 1u;        // rounding of the ends
@@ -365,6 +350,10 @@ static __device__ int l1_window_finish(double n_hi, double s_hi, const float* ca
         wp_khi = khi;
         // a key histogram built over the float window fits only that window
         wp_pre = pre && (double)(float)theta_lo == theta_lo && (double)(float)theta_hi == theta_hi;
+        // a list that comes with its histogram is narrowed whenever one warp
+        // could not take it in one step (reading the bins costs about 2 us,
+        // Michelot's steps on a few hundred values 5 us)
+        wp_narrow = wp_rc < 0 && scr && theta_lo >= 0.0 && m_raw > (wp_pre ? 32u : kNarrowMin);
     }
     __syncthreads();
     if (wp_rc >= 0) {
@@ -390,7 +379,7 @@ static __device__ int l1_window_finish(double n_hi, double s_hi, const float* ca
             src_shared = true;
         }
         // (red_d serves as the narrowing's scalars)
-        const int rc = l1_narrow(src, src_shared, m, nh, sh, klo, khi, r, scr, &m_st, nr_i, red_d, pre);
+        const int rc = l1_narrow(src, src_shared, m, nh, sh, klo, khi, r, scr, &m_st, nr_i, red_d, pre, nbinned);
         if (rc == 1) {
             // phi(theta_lo) < 0: as below, inside the ball or a miss below
             if (info) { info->phi_lo = red_d[2]; info->n_lo = red_d[3]; }
@@ -446,7 +435,25 @@ static __device__ int l1_window_finish(double n_hi, double s_hi, const float* ca
             state = __shfl_sync(0xffffffffu, state, 0);
             tf = __shfl_sync(0xffffffffu, tf, 0);
             int rc = state == 2 ? 0 : state == 3 ? 1 : 0;
-            if (state == 0) {
+            if (state == 0 && m <= 32u) {
+                // one value per lane: those with phi(x) < 0 lie above the root
+                // and are the active set (the fixed point of Michelot's steps,
+                // found at once)
+                const float x = lane < m ? stage[lane] : 0.f;
+                Kahan ge;
+                unsigned n_ge = 0;
+                for (unsigned k = 0; k < m; ++k) {
+                    const float xk = __shfl_sync(0xffffffffu, x, k);
+                    if (xk >= x) { ge.add(xk); ++n_ge; }
+                }
+                const double phi = s_hi + ge.value() - (n_hi + (double)n_ge) * (double)x - r;
+                const bool active = lane < m && phi < 0.0;
+                Kahan ka;
+                if (active) ka.add(x);
+                warp_sum_pair(ka, h, l);
+                const unsigned c = (unsigned)__popc(__ballot_sync(0xffffffffu, active));
+                if (lane == 0) tau = (s_hi + ((double)h + (double)l) - r) / (n_hi + (double)c);
+            } else if (state == 0) {
                 unsigned prev = m;
                 for (int it = 0; it < 200; ++it) {
                     Kahan ka;

@@ -11,6 +11,7 @@
 // which the next iteration applies when it reads q.  It also reduces the two
 // norms of the stopping rule (Eq. 28).
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <mutex>
 #include <type_traits>
@@ -91,12 +92,33 @@ struct K2Args {
     SlabPart sp;        // the bands updated, and this launch's CTAs among the stage's
 };
 
-// The CTA `bid` of `nblk` that share one cube's K2 (a launch of its own, or
-// the cube's share of a batch launch).
+// A thread's part of the three norms |q|^2, |u+ - u|^2, |u|^2.
+struct K2Norms {
+    Kahan q, du, u;
+};
+
+// Kahan's update of a compensated sum, and its sums in the order of the block:
+// the norms of 16-bit storage.  Its iterates round by random bits, so a last
+// place of the l2-ball scale moves a fraction of them by a whole 16-bit place;
+// the order of this sum is therefore part of what a run reproduces.
+struct KahanSum {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        float y = x - c;
+        float t = s + y;
+        c = (t - s) - y;
+        s = t;
+    }
+    __device__ __forceinline__ double value() const { return (double)s - (double)c; }
+};
+struct K2NormsStrip {
+    KahanSum q, du, u;
+};
+
+// The rows of one strip per thread and item, top to bottom, t' of the row below
+// carried over: 16-bit storage, whose rounding streams follow the strips.
 template <typename T>
-__device__ __forceinline__ void k2_body(const K2Args<T>& a, const int bid, const int nblk) {
-    __shared__ double red_d[64];
-    __shared__ int is_last;
+__device__ __forceinline__ void k2_strips(const K2Args<T>& a, const int bid, const int nblk, K2NormsStrip& N) {
     const Geom g = a.g;
     const IterParams& P = a.p;
     const float cs = (float)(1.0 - a.sc->c[P.parity]);
@@ -106,7 +128,6 @@ __device__ __forceinline__ void k2_body(const K2Args<T>& a, const int bid, const
     const int quads = g.p2 / 4;
     const int strips = (g.n1 + K2_ROWS - 1) / K2_ROWS;
     const long long items = (long long)(a.sp.o1 - a.sp.o0) * strips * quads;
-    Kahan aq, adu, au;
     for (long long it = bid * (long long)NT + threadIdx.x; it < items; it += (long long)nblk * NT) {
         const int qd = (int)(it % quads);
         const long long rest = it / quads;
@@ -151,10 +172,10 @@ __device__ __forceinline__ void k2_body(const K2Args<T>& a, const int bid, const
                     const float qn = y4p - P.gamma_y4 * comp(v4, k);
                     set_comp(qn4, k, qn);
                     if (j + k < g.n2) {
-                        aq.add(qn * qn);
+                        N.q.add(qn * qn);
                         const float du = un - uo;
-                        adu.add(du * du);
-                        au.add(uo * uo);
+                        N.du.add(du * du);
+                        N.u.add(uo * uo);
                     }
                 }
             }
@@ -175,31 +196,161 @@ __device__ __forceinline__ void k2_body(const K2Args<T>& a, const int bid, const
             st4S(a.y3_n + g.at(b, g.n1 - 1, j), y3prev, sr);
         }
     }
-    const double q2 = block_sum(aq.value(), red_d);
-    const double du2 = block_sum(adu.value(), red_d);
-    const double u2 = block_sum(au.value(), red_d);
+}
+
+// float32: one row of four columns per thread and item, every load of the item
+// issued at once (t' of the row below is computed again from its t, y3, q,
+// which the neighbouring rows' threads read too: cache hits).  A persistent
+// grid walks the cube in memory order, so that no wave of CTAs is left half
+// empty.  (The strips above, one thread marching down 8 rows, were bound by
+// the latency of 9 dependent row loads on small cubes, 20 us whatever the
+// size up to 128 x 128 x 64, and left their third wave a quarter full at
+// 256 x 256 x 128, 80 us.)
+// big: the block's shared sums that take a thread's partials before they could
+// overflow float.
+__device__ __forceinline__ void k2_rows(const K2Args<float>& a, const int bid, const int nblk, K2Norms& N, double* big) {
+    const Geom g = a.g;
+    const IterParams& P = a.p;
+    const unsigned quads = (unsigned)g.p2 / 4u, n1 = (unsigned)g.n1;
+    const unsigned total = (unsigned)(a.sp.o1 - a.sp.o0) * n1 * quads;     // < 2^30 for any cube that fits
+    const unsigned row0 = (unsigned)a.sp.o0 * n1;
+    const float cs = (float)(1.0 - a.sc->c[P.parity]);
+    const float tau_s = (float)a.sc->ctl[0].tau;
+    const float tau_t = (float)a.sc->ctl[1].tau;
+    for (unsigned e = (unsigned)bid * NT + threadIdx.x; e < total; e += (unsigned)nblk * NT) {
+        const unsigned r = e / quads;
+        const int j = (int)(e - r * quads) * 4;
+        const unsigned row = row0 + r;                                      // b * n1 + i
+        const int i = (int)(row % n1);
+        const long long o = (long long)row * g.p2 + j;
+        const bool dn = i < g.n1 - 1;
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 s4 = Vec4<float>::ld(a.s + o), t4 = Vec4<float>::ld(a.t + o);
+        const float4 y34 = Vec4<float>::ld(a.y3 + o), q4 = Vec4<float>::ld(a.q + o);
+        const float4 u0 = Vec4<float>::ld(a.u + o), u1 = Vec4<float>::ld(a.u_n + o);
+        const float4 v4 = Vec4<float>::ld(a.v + o);
+        const float4 yu4 = i >= 1 ? Vec4<float>::ld(a.y3 + o - g.p2) : zero;
+        const float4 td4 = dn ? Vec4<float>::ld(a.t + o + g.p2) : zero;
+        const float4 yd4 = dn ? Vec4<float>::ld(a.y3 + o + g.p2) : zero;
+        const float4 qd4 = dn ? Vec4<float>::ld(a.q + o + g.p2) : zero;
+        float4 sp4, tp4, qn4, y3n4;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float y4 = __fmul_rn(cs, comp(q4, k));
+            float xs, xt, xsd, xtd;
+            s_t_tilde(comp(s4, k), comp(t4, k), comp(y34, k), comp(yu4, k), comp(q4, k), cs, i, g.n1, P.gamma_s,
+                      P.gamma_t, xs, xt);
+            const float sp = soft(xs, tau_s), tp = soft(xt, tau_t);
+            const float sb = 2.f * sp - comp(s4, k), tb = 2.f * tp - comp(t4, k);
+            set_comp(sp4, k, sp);
+            set_comp(tp4, k, tp);
+            // t' of the row below (the last row has D_v t' = 0: y3 is unchanged there)
+            s_t_tilde(0.f, comp(td4, k), comp(yd4, k), comp(y34, k), comp(qd4, k), cs, i + 1, g.n1, P.gamma_s,
+                      P.gamma_t, xsd, xtd);
+            const float tbd = 2.f * soft(xtd, tau_t) - comp(td4, k);
+            set_comp(y3n4, k, dn ? comp(y34, k) + P.gamma_y3 * (tbd - tb) : comp(y34, k));
+            const float uo = comp(u0, k), un = comp(u1, k);
+            const float ub = 2.f * un - uo;
+            const float y4p = y4 + P.gamma_y4 * (ub + sb + tb);
+            const float qn = y4p - P.gamma_y4 * comp(v4, k);
+            set_comp(qn4, k, qn);
+            if (j + k < g.n2) {
+                N.q.add(qn * qn);
+                const float du = un - uo;
+                N.du.add(du * du);
+                N.u.add(uo * uo);
+            }
+        }
+        if (fmaxf(fmaxf(N.q.s, N.du.s), N.u.s) > 1e36f) {
+            atomicAdd(big, N.q.value());
+            atomicAdd(big + 1, N.du.value());
+            atomicAdd(big + 2, N.u.value());
+            N = K2Norms();
+        }
+        Vec4<float>::st(a.y3_n + o, y3n4);
+        Vec4<float>::st(a.s_n + o, sp4);
+        Vec4<float>::st(a.t_n + o, tp4);
+        Vec4<float>::st(a.q_n + o, qn4);
+    }
+}
+
+// The CTA `bid` of `nblk` that share one cube's K2 (a launch of its own, or
+// the cube's share of a batch launch).
+template <typename T>
+__device__ __forceinline__ void k2_body(const K2Args<T>& a, const int bid, const int nblk) {
+    constexpr int NW = NT / 32;
+    __shared__ double red_d[64];
+    __shared__ int is_last;
+    const IterParams& P = a.p;
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cta = a.sp.cta_base + bid;
     const int ncta = a.sp.cta_total > 0 ? a.sp.cta_total : nblk;
-    if (threadIdx.x == 0) {
-        a.part[3 * cta] = q2;
-        a.part[3 * cta + 1] = du2;
-        a.part[3 * cta + 2] = u2;
+    if constexpr (std::is_same<T, float>::value) {
+        __shared__ double big[3];
+        if (threadIdx.x < 3) big[threadIdx.x] = 0.0;
+        __syncthreads();
+        K2Norms N;
+        k2_rows(a, bid, nblk, N, big);
+        // the CTA's norms: float pairs through each warp (no lane's sum is
+        // above 1e36), the warps' in FP64 by three lanes
+        const Kahan* k3[3] = {&N.q, &N.du, &N.u};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            float h, l;
+            warp_sum_pair(*k3[k], h, l);
+            if (lane == 0) red_d[k * NW + wid] = (double)h + (double)l;
+        }
+        __syncthreads();
+        if (threadIdx.x < 3) {
+            double r = big[threadIdx.x];
+            for (int k = 0; k < NW; ++k) r += red_d[threadIdx.x * NW + k];
+            a.part[3 * cta + threadIdx.x] = r;
+            __threadfence();
+        }
+    } else {
+        K2NormsStrip N;
+        k2_strips(a, bid, nblk, N);
+        const double q2 = block_sum(N.q.value(), red_d);
+        const double du2 = block_sum(N.du.value(), red_d);
+        const double u2 = block_sum(N.u.value(), red_d);
+        if (threadIdx.x == 0) {
+            a.part[3 * cta] = q2;
+            a.part[3 * cta + 1] = du2;
+            a.part[3 * cta + 2] = u2;
+        }
     }
-    __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) is_last = (atomicAdd(&a.sc->k2_ticket, 1u) == (unsigned)(ncta - 1));
+    if (threadIdx.x == 0) {
+        __threadfence();
+        is_last = (atomicAdd(&a.sc->k2_ticket, 1u) == (unsigned)(ncta - 1));
+    }
     __syncthreads();
     if (!is_last) return;
     __threadfence();
     double s0 = 0, s1 = 0, s2 = 0;
-    for (int k = threadIdx.x; k < ncta; k += NT) {
-        s0 += __ldcg(a.part + 3 * k);
-        s1 += __ldcg(a.part + 3 * k + 1);
-        s2 += __ldcg(a.part + 3 * k + 2);
+    if constexpr (std::is_same<T, float>::value) {
+        // one warp per norm sums the CTAs' partials
+        if (wid < 3) {
+            double r = 0.0;
+#pragma unroll 4
+            for (int k = lane; k < ncta; k += 32) r += __ldcg(a.part + 3 * k + wid);
+            r = warp_sum(r);
+            if (lane == 0) red_d[wid] = r;
+        }
+        __syncthreads();
+        s0 = red_d[0];
+        s1 = red_d[1];
+        s2 = red_d[2];
+    } else {
+        for (int k = threadIdx.x; k < ncta; k += NT) {
+            s0 += __ldcg(a.part + 3 * k);
+            s1 += __ldcg(a.part + 3 * k + 1);
+            s2 += __ldcg(a.part + 3 * k + 2);
+        }
+        s0 = block_sum(s0, red_d);
+        s1 = block_sum(s1, red_d);
+        s2 = block_sum(s2, red_d);
     }
-    s0 = block_sum(s0, red_d);
-    s1 = block_sum(s1, red_d);
-    s2 = block_sum(s2, red_d);
     if (threadIdx.x == 0) {
         Scal* sc = a.sc;
         double c = 1.0;
@@ -573,27 +724,41 @@ __device__ __noinline__ void k1_window_finish(const SearchArgs& a, const unsigne
         return;
     }
     const bool hist_v = __ldcg(&a.sc->k1_hist[v]) != 0;
-    unsigned long long n = 0, hn = 0;
-    double s = 0.0, hs = 0.0;
-    for (int k = threadIdx.x; k < parts; k += blockDim.x) {
-        n += __ldcg(pn + 4 * k + v);
-        s += __ldcg(ps + 4 * k + v);
-        hn += __ldcg(pn + 4 * k + 2 + v);
-        hs += __ldcg(ps + 4 * k + 2 + v);
+    // the CTAs' partials (one per SM): one warp, so that the FP64 additions
+    // (scarce on this part) are not issued by every warp of the block
+    if (threadIdx.x < 32) {
+        unsigned long long n = 0;
+        double s = 0.0;
+#pragma unroll 4
+        for (int k = threadIdx.x; k < parts; k += 32) {
+            n += __ldcg(pn + 4 * k + v);
+            s += __ldcg(ps + 4 * k + v);
+        }
+        n = warp_sum(n);
+        s = warp_sum(s);
+        if (threadIdx.x == 0) { red_u[0] = n; red_d[0] = s; }
     }
-    n = block_sum(n, red_u);
-    s = block_sum(s, red_d);
+    __syncthreads();
+    const unsigned long long n = red_u[0];
+    const double s = red_d[0];
+    __syncthreads();
     const unsigned m = __ldcg(&a.sc->acc[v].m);
     const double tlo = C.theta_lo, thi = C.theta_hi;
     double tau = 0.0;
     WinInfo wi;
     const int miss = l1_window_finish((double)n, s, a.w.cand[v], m, tlo, thi, r, &tau, red_d, red_u, &wi, fstage,
-                                      kFinishStage, scr, narrow_pre(a.w, v, m));
+                                      kFinishStage, scr, narrow_pre(a.w, v, m), a.w.nbinned + v);
     narrow_clear(a.w, v);
     int hist_hit = 0;
     float h_lo = 0.f, h_hi = 0.f;
     double h_m = 0.0;
     if (miss && hist_v) {
+        unsigned long long hn = 0;
+        double hs = 0.0;
+        for (int k = threadIdx.x; k < parts; k += blockDim.x) {
+            hn += __ldcg(pn + 4 * k + 2 + v);
+            hs += __ldcg(ps + 4 * k + 2 + v);
+        }
         hn = block_sum(hn, red_u);
         hs = block_sum(hs, red_d);
         hist_hit = l1_hist_bracket(a.w.khist + v * kK1Bins, C.hbase, (double)hn, hs, r, (double)kHistSample,
@@ -657,7 +822,7 @@ __device__ __forceinline__ void finish_body(const SearchArgs& a, int mode, const
         }
         double tau = 0.0;
         const int rc = l1_window_finish(n, sm, a.w.cand[v], m, lo, hi, r, &tau, red_d, red_u, nullptr, fstage,
-                                        kFinishStage, scr, narrow_pre(a.w, v, m));
+                                        kFinishStage, scr, narrow_pre(a.w, v, m), a.w.nbinned + v);
         narrow_clear(a.w, v);
         if (threadIdx.x == 0) {
             if (mode == 0) {
@@ -808,9 +973,14 @@ long long part_voxels(const Geom& g, const SlabPart& sp) {
     return (long long)(sp.o1 - sp.o0) * g.n1 * g.n2;
 }
 
-int k2_grid_part(const Geom& g, const SlabPart& sp) {
-    const long long items = (long long)(sp.o1 - sp.o0) * ((g.n1 + K2_ROWS - 1) / K2_ROWS) * (g.p2 / 4);
-    return grid_for(items);
+// CTAs of K2 that fit the GPU at once (its launch bounds)
+int k2_resident() { return 3 * device_sms(); }
+
+int k2_grid_part(int storage, const Geom& g, const SlabPart& sp) {
+    const long long nb = sp.o1 - sp.o0;
+    if (storage != 0) return grid_for(nb * ((g.n1 + K2_ROWS - 1) / K2_ROWS) * (g.p2 / 4));
+    const long long ctas = (nb * g.n1 * (g.p2 / 4) + NT - 1) / NT;
+    return (int)std::max(1ll, std::min<long long>(ctas, k2_resident()));
 }
 
 int radix_grid_n(long long n) {
@@ -833,7 +1003,7 @@ int launch_k2_t(const Geom& g, const IterBufs& b, const IterParams& p, Scal* sc,
     a.sc = sc;
     a.part = part;
     a.sp = sp;
-    const int ctas = std::min(k2_grid_part(g, sp), part_cap);
+    const int ctas = std::min(k2_grid_part(std::is_same<T, float>::value ? 0 : 1, g, sp), part_cap);
     k2_light<T><<<ctas, NT, 0, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
@@ -1057,14 +1227,14 @@ int launch_search_finish(int mode, Scal* sc, const L1Work& w, int nvec, const un
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
-int k2_grid_ctas(int, const Geom& g) { return k2_grid_part(g, whole_cube(g)); }
+int k2_grid_ctas(int storage, const Geom& g) { return k2_grid_part(storage, g, whole_cube(g)); }
 
 int window_grid(const Geom& g, const SlabPart& sp, int part_cap) {
     return window_grid_n(part_voxels(g, sp), part_cap);
 }
 int radix_grid(const Geom& g, const SlabPart& sp) { return radix_grid_n(part_voxels(g, sp)); }
 int gather_grid(const Geom& g, const SlabPart& sp) { return gather_grid_n(part_voxels(g, sp)); }
-int k2_grid(const Geom& g, const SlabPart& sp, int part_cap) { return std::min(k2_grid_part(g, sp), part_cap); }
+int k2_grid(const Geom& g, const SlabPart& sp, int part_cap) { return std::min(k2_grid_part(0, g, sp), part_cap); }
 
 int launch_k2(int storage, const Geom& g, const IterBufs& b, const IterParams& p, Scal* sc,
               double* part, int part_cap, const SlabPart& sp, cudaStream_t st) {
@@ -1186,6 +1356,9 @@ int launch_k2_batch(const BatchCube* cubes, int n, cudaStream_t st) {
     K2BatchTab t{};
     t.n = n;
     int total = 0;
+    // the CTAs that fit the GPU, shared out by size (each cube at least one)
+    double all = 0.0;
+    for (int c = 0; c < n; ++c) all += (double)cubes[c].g.cube;
     for (int c = 0; c < n; ++c) {
         const BatchCube& q = cubes[c];
         K2Args<float>& a = t.c[c];
@@ -1198,7 +1371,8 @@ int launch_k2_batch(const BatchCube* cubes, int n, cudaStream_t st) {
         a.part = q.k2_part;
         a.sp = whole_cube(q.g);
         t.start[c] = total;
-        total += std::min(k2_grid_part(q.g, a.sp), q.k2_cap);
+        const int share = (int)std::ceil(k2_resident() * ((double)q.g.cube / all));
+        total += std::max(1, std::min({share, k2_grid_part(0, q.g, a.sp), q.k2_cap}));
     }
     t.start[n] = total;
     k2_batch<<<total, NT, 0, st>>>(t);
