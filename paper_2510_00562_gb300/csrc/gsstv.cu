@@ -224,13 +224,16 @@ int enqueue_iteration(gsstv_handle* h, int par, bool timed, cudaStream_t st, boo
     auto k1_finish = [&](int gated, cudaGraphConditionalHandle cond) -> int {
         if (h->k1_variant == 1)
             return map_launch(launch_search_finish(2, h->sc, h->l1, 2, h->l1.k1_n, h->l1.k1_s,
-                                                   k1_tma_grid(h->g, whole, h->k1_chunk), st, gated, cond));
+                                                   k1_tma_grid(sto, h->g, whole, h->k1_chunk), st, gated, cond));
         return gated ? map_launch(launch_search_gate(&h->sc, 1, cond, st)) : GSSTV_OK;
     };
     auto search = [&](cudaStream_t s) -> int {
-        TRY(map_launch(launch_window(sto, h->g, b, ip, h->sc, h->l1, h->k1_ctas, whole, s)));
+        // (16-bit storage: the CTAs that the cooperative K1's partials allow, whose
+        // sums a run reproduces)
+        const int cap = sto == GSSTV_FP32 ? h->k1_ctas : k1_grid_ctas(h->g);
+        TRY(map_launch(launch_window(sto, h->g, b, ip, h->sc, h->l1, cap, whole, s)));
         TRY(map_launch(launch_search_finish(0, h->sc, h->l1, 2, h->l1.k1_n, h->l1.k1_s,
-                                            window_grid(h->g, whole, h->k1_ctas), s)));
+                                            window_grid(h->g, whole, cap), s)));
         for (int level = 0; level < 3; ++level)
             TRY(map_launch(launch_fallback(sto, level, h->g, b, ip, h->sc, h->l1, whole, s)));
         TRY(map_launch(launch_gather(sto, h->g, b, ip, h->sc, h->l1, whole, s)));
@@ -622,7 +625,9 @@ int gsstv_set_state(gsstv_handle* h, const gsstv_state_view* v) {
 int gsstv_autotune(gsstv_handle* h, int passes, int* chunk_out) {
     if (chunk_out) *chunk_out = 0;
     if (!h || passes < 1) return GSSTV_ERR_ARG;
-    if (h->k1_variant != 1) return GSSTV_OK;          // the cooperative kernel has no run length to tune
+    // the cooperative kernel has no run length to tune; 16-bit storage keeps the
+    // run its sums are split by
+    if (h->k1_variant != 1 || h->p.storage != GSSTV_FP32) return GSSTV_OK;
     int cand[6];
     const int nc = k1_tma_chunk_candidates(h->g, cand, 6);
     const gsstv_stats saved_stats = h->stats;
@@ -1448,7 +1453,7 @@ int gsstv_slabs_create(gsstv_slabs** out, int n1, int n2, int n3, int nslabs, co
             const Geom& g = G->h[s]->g;
             const int c = k1_tma_part_chunk(g, G->k1p[s], 0);
             G->k1_chunk.push_back(c);
-            gk1.push_back(k1_tma_grid(g, G->k1p[s], c));
+            gk1.push_back(k1_tma_grid(GSSTV_FP32, g, G->k1p[s], c));
             gw.push_back(window_grid(g, G->winp[s], 1 << 30));
             gr.push_back(radix_grid(g, G->radp[s]));
             gg.push_back(gather_grid(g, G->gatp[s]));

@@ -277,9 +277,26 @@ __device__ __forceinline__ void pair_add(float& hi, float& lo, float bhi, float 
     hi = __fadd_rn(s, e);
     lo = __fsub_rn(e, __fsub_rn(hi, s));
 }
+// Kahan's update of a compensated sum: the sums of 16-bit storage.  Its
+// iterates round by random bits, so a last place of a threshold or of the
+// l2-ball scale moves a fraction of them by a whole 16-bit place; the update
+// and the order of these sums are therefore part of what a run reproduces.
+struct KahanSum {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        float y = x - c;
+        float t = s + y;
+        c = (t - s) - y;
+        s = t;
+    }
+    __device__ __forceinline__ double value() const { return (double)s - (double)c; }
+};
+template <typename T>
+using KahanOf = std::conditional_t<std::is_same<T, float>::value, Kahan, KahanSum>;
 // The CTA's sum of the threads' compensated sums; the result (a double) is
 // valid on thread 0 only.  buf: >= 32 float2 of shared memory.
-__device__ __forceinline__ double block_sum_pair(const Kahan& k, float2* buf) {
+template <typename K>
+__device__ __forceinline__ double block_sum_pair(const K& k, float2* buf) {
     float hi = k.s, lo = -k.c;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -339,9 +356,10 @@ __device__ __forceinline__ void s_t_tilde(float s, float t, float y3, float y3_u
 // ---------------------------------------------------------------------------
 // window accounting for one |x| value, used by K1 and by the gather pass
 // ---------------------------------------------------------------------------
+template <typename T>
 struct WinAcc {
     unsigned long long n = 0;
-    Kahan s;
+    KahanOf<T> s;
 };
 
 // Appends the lanes' candidates with one atomic per warp.
@@ -419,7 +437,7 @@ int k1_tma_configure(int storage);
 int k1_tma_maps(const Geom& g, const IterBufs& b, K1Maps* m);
 // CTAs of one K1 launch over the part's bands, and its bands per item (chunk
 // as for launch_k1_tma)
-int k1_tma_grid(const Geom& g, const SlabPart& sp, int chunk);
+int k1_tma_grid(int storage, const Geom& g, const SlabPart& sp, int chunk);
 int k1_tma_part_chunk(const Geom& g, const SlabPart& sp, int chunk);
 // chunk: bands per item (0 or out of range: the model's choice)
 int launch_k1_tma(int storage, const Geom& g, const K1Maps& m, const IterBufs& b, const IterParams& p,
@@ -428,6 +446,8 @@ int launch_k1_tma(int storage, const Geom& g, const K1Maps& m, const IterBufs& b
 int launch_k1(int storage, const Geom& g, const IterBufs& b, const IterParams& p, Scal* sc,
               const L1Work& w, int n_cta_slots, cudaStream_t st);
 int k1_grid_ctas(const Geom& g);
+// bands per CTA of the cooperative K1
+int k1_coop_chunk(const Geom& g);
 int k1_configure(int storage);
 int light_configure(int storage);
 // CTAs of one launch of the threshold passes and of K2 over the part's bands

@@ -97,20 +97,7 @@ struct K2Norms {
     Kahan q, du, u;
 };
 
-// Kahan's update of a compensated sum, and its sums in the order of the block:
-// the norms of 16-bit storage.  Its iterates round by random bits, so a last
-// place of the l2-ball scale moves a fraction of them by a whole 16-bit place;
-// the order of this sum is therefore part of what a run reproduces.
-struct KahanSum {
-    float s = 0.f, c = 0.f;
-    __device__ __forceinline__ void add(float x) {
-        float y = x - c;
-        float t = s + y;
-        c = (t - s) - y;
-        s = t;
-    }
-    __device__ __forceinline__ double value() const { return (double)s - (double)c; }
-};
+// The norms of 16-bit storage, in the order of the block.
 struct K2NormsStrip {
     KahanSum q, du, u;
 };
@@ -389,6 +376,7 @@ __global__ void __launch_bounds__(NT, 3) k2_light(const K2Args<T> a) {
 // ---------------------------------------------------------------------------
 template <typename T>
 struct CubeSrc {
+    using Storage = T;
     Geom g;
     const T *s, *t, *y3, *q;
     const Scal* sc;
@@ -439,6 +427,7 @@ struct CubeSrc {
 };
 
 struct FlatSrc {
+    using Storage = float;
     const float* x;
     long long n;
     template <typename F>
@@ -648,7 +637,7 @@ __device__ __forceinline__ void window_body(const Src& src, const SearchArgs& a,
     if (!need[0] && !need[1]) return;
     const float lo0 = a.sc->ctl[0].g_lo, hi0 = a.sc->ctl[0].g_hi;
     const float lo1 = a.sc->ctl[1].g_lo, hi1 = a.sc->ctl[1].g_hi;
-    WinAcc w0, w1;
+    WinAcc<typename Src::Storage> w0, w1;
     GSSTV_BLOCK_CAND(bc);
     if (need[0]) bc.keep_hist(a.w, 0, lo0, hi0);
     if (need[1]) bc.keep_hist(a.w, 1, lo1, hi1);
@@ -772,7 +761,8 @@ __device__ __noinline__ void k1_window_finish(const SearchArgs& a, const unsigne
         if (!miss) {
             l1_record_tau(C, tau, (double)min(m, kCandCap), thi - tlo, true);
             C.hits++;
-            if (C.hist_left > 0) C.hist_left--;
+            // (counted down where K1 keeps the histogram: float32 storage)
+            if (C.hist_left > 0 && __ldcg(&a.sc->k1_win[v]) == 1) C.hist_left--;
         } else if (hist_hit) {
             C.prefix = 0; C.n_above = 0; C.s_above = 0.0;
             C.need = NEED_WINDOW;

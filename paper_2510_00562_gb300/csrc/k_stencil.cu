@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(NT, 2) k1_stencil(const K1Args<T> a) {
     const bool win_t = !P.tau_exact && a.sc->radius[1] > 0.0 && a.sc->ctl[1].window_ok;
     const float lo_s = a.sc->ctl[0].theta_lo, hi_s = a.sc->ctl[0].theta_hi;
     const float lo_t = a.sc->ctl[1].theta_lo, hi_t = a.sc->ctl[1].theta_hi;
-    WinAcc acc_s, acc_t;
+    WinAcc<T> acc_s, acc_t;
 
     auto Yp = [&](int slot, int pl) { return ys + (slot * 4 + pl) * Y_PL; };
 
@@ -430,12 +430,8 @@ int launch_k1_t(const Geom& g, const IterBufs& b, const IterParams& p, Scal* sc,
     a.p = p;
     a.sc = sc;
     a.l1 = w;
-    const int tiles = ((g.n2 + TX - 1) / TX) * ((g.n1 + TY - 1) / TY);
-    const int target = device_sms() * 16;                  // about 16 CTAs per SM
-    int chunks = (target + tiles - 1) / tiles;
-    chunks = max(1, min(chunks, (g.n3 + 7) / 8));          // at least 8 bands per CTA
-    a.chunk = (g.n3 + chunks - 1) / chunks;
-    chunks = (g.n3 + a.chunk - 1) / a.chunk;
+    a.chunk = k1_coop_chunk(g);
+    const int chunks = (g.n3 + a.chunk - 1) / a.chunk;
     dim3 grid((g.n2 + TX - 1) / TX, (g.n1 + TY - 1) / TY, chunks);
     k1_stencil<T><<<grid, NT, smem, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
@@ -454,14 +450,18 @@ int k1_configure(int storage) {
     return e == cudaSuccess ? 0 : -3;
 }
 
+int k1_coop_chunk(const Geom& g) {
+    const int tiles = ((g.n2 + TX - 1) / TX) * ((g.n1 + TY - 1) / TY);
+    const int target = device_sms() * 16;                  // about 16 CTAs per SM
+    int chunks = (target + tiles - 1) / tiles;
+    chunks = std::max(1, std::min(chunks, (g.n3 + 7) / 8));     // at least 8 bands per CTA
+    return (g.n3 + chunks - 1) / chunks;
+}
+
 int k1_grid_ctas(const Geom& g) {
     const int tiles = ((g.n2 + TX - 1) / TX) * ((g.n1 + TY - 1) / TY);
-    const int target = device_sms() * 16;
-    int chunks = (target + tiles - 1) / tiles;
-    chunks = std::max(1, std::min(chunks, (g.n3 + 7) / 8));
-    const int chunk = (g.n3 + chunks - 1) / chunks;
-    chunks = (g.n3 + chunk - 1) / chunk;
-    return tiles * chunks;
+    const int chunk = k1_coop_chunk(g);
+    return tiles * ((g.n3 + chunk - 1) / chunk);
 }
 
 int launch_k1(int storage, const Geom& g, const IterBufs& b, const IterParams& p, Scal* sc,

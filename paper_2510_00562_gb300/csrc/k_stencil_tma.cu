@@ -122,7 +122,9 @@ struct Lay {
     static constexpr int OFF_CB = OFF_UP + pad128(NUS * UP1 * 4);
     static constexpr int OFF_HIST = OFF_CB + 4 * kCandBuf * 4;    // K1 histogram: 2 x kK1Bins packed 16-bit counts
     static constexpr int OFF_BAR = OFF_HIST + kK1Bins * 4;
-    static constexpr int SMEM = OFF_BAR + (2 * NYS + 2 * NWS + 1) * 8;
+    // 16-bit: the window's values of three bands (see Ordered)
+    static constexpr int OFF_X = pad128(OFF_BAR + (2 * NYS + 2 * NWS + 1) * 8);
+    static constexpr int SMEM = F32 ? OFF_BAR + (2 * NYS + 2 * NWS + 1) * 8 : OFF_X + NUS * TY * TX * 8;
     // element offsets inside a y-group slot, and between raw planes
     static constexpr int YPL = Y_B / ES, WRAW = W_B / ES;
     static constexpr int O_U = 4 * YPL, O_Q = O_U + U_B / ES, O_S = O_Q + U_B / ES, O_T = O_S + S_B / ES,
@@ -144,6 +146,7 @@ struct K1Args {
     Scal* sc;
     L1Work l1;
     int chunk;          // bands per item
+    int unit;           // 16-bit: bands per piece of the window's sums (chunk is a multiple of it)
     SlabPart sp;
 };
 
@@ -168,6 +171,30 @@ struct K1Stat {
     unsigned n_s = 0, n_t = 0;
     float2 ks = make_float2(0.f, 0.f), kc = make_float2(0.f, 0.f);
     K1Acc top_s, top_t;
+};
+
+// 16-bit storage: the sums above the windows in the order and the pieces of the
+// cooperative kernel (a thread's sum over `unit` bands of the tile's rows r and
+// r + 8, row r before row r + 8 at each band), so that both kernels find the
+// same thresholds: a threshold one float ulp off flips random roundings of a
+// 16-bit iterate.  The warps of rows 0-7 add up what all 16 rows' warps leave
+// in shared memory, one band late; finished pieces join a float pair.  (Sums
+// split otherwise, with a histogram and exact additions, moved one threshold in
+// 32 passes of a 256x256x200 float16 solve by an ulp and the result by up to a
+// float16 place; a pass took 0.91 ms either way, 1.47 ms in the cooperative
+// kernel's launches, and at 512x512x224 bfloat16 3.55 ms, 3.25 and 6.05 ms.)
+struct Ordered {
+    KahanSum s, t;
+    float hs = 0.f, ls = 0.f, ht = 0.f, lt = 0.f;
+    __device__ __forceinline__ void add(float2 x) {            // a component below zero: not above its window
+        if (x.x >= 0.f) s.add(x.x);
+        if (x.y >= 0.f) t.add(x.y);
+    }
+    __device__ __forceinline__ void close() {
+        pair_add(hs, ls, s.s, -s.c);
+        pair_add(ht, lt, t.s, -t.c);
+        s = t = KahanSum();
+    }
 };
 
 // A position in a ring of N slots and the phase parity of its next use.
@@ -295,6 +322,10 @@ struct Sm {
         return reinterpret_cast<float*>(sm + Lay<T>::OFF_CB) + (2 * odd + v) * kCandBuf;
     }
     __device__ __forceinline__ unsigned* cnt(int v, int odd) const { return ccnt + 2 * odd + v; }
+    // 16-bit: |s~|, |t~| of one band where they are above their windows, else -1
+    __device__ __forceinline__ float2* above(int slot) const {
+        return reinterpret_cast<float2*>(sm + Lay<T>::OFF_X) + slot * (TY * TX);
+    }
     __device__ __forceinline__ unsigned* hist() const { return reinterpret_cast<unsigned*>(sm + Lay<T>::OFF_HIST); }
 };
 
@@ -457,7 +488,7 @@ __device__ __forceinline__ void w_step(const IterParams& P, const float2 (&Lg)[3
 // ---------------------------------------------------------------------------
 template <typename T, bool EDGE, bool HIST>
 __device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, const Item& m, Cons<T>& C, K1Stat& A,
-                                          const K1Win& W, float cs, int turn) {
+                                          Ordered& O, const K1Win& W, float cs, int turn) {
     using L = Lay<T>;
     constexpr int YPL = L::YPL, WPL = L::WPL, WRAW = L::WRAW;
     const Geom& g = a.g;
@@ -539,7 +570,11 @@ __device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, co
         // an inactive window has lo = hi = +inf: nothing is counted or taken
         const float x_s = fabsf(xs), x_t = fabsf(xt);
         const bool hs = valid && x_s > W.hi_s, ht = valid && x_t > W.hi_t;
-        {
+        A.n_s += hs ? 1u : 0u;
+        A.n_t += ht ? 1u : 0u;
+        if constexpr (!L::F32) {
+            S.above(C.us)[tid] = f2(hs ? x_s : -1.f, ht ? x_t : -1.f);
+        } else {
             // both vectors' compensated sums in packed pairs; a value not
             // taken adds zero, which leaves the represented sum unchanged
             const float2 x2 = f2(hs ? x_s : 0.f, ht ? x_t : 0.f);
@@ -547,8 +582,6 @@ __device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, co
             const float2 b2 = sub2(t2, A.ks);
             A.kc = sub2(A.kc, add2(sub2(A.ks, sub2(t2, b2)), sub2(x2, b2)));
             A.ks = t2;
-            A.n_s += hs ? 1u : 0u;
-            A.n_t += ht ? 1u : 0u;
         }
         const bool cs_ = valid && !hs && x_s > W.lo_s, ct_ = valid && !ht && x_t > W.lo_t;
         if (__ballot_sync(0xffffffffu, cs_ || ct_)) {     // most warps have no candidate
@@ -587,6 +620,7 @@ __device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, co
     float yprev[4] = {0.f, 0.f, 0.f, 0.f};
     const int w_last = C.w.slot == 0 ? L::NWS - 1 : C.w.slot - 1;    // the previous item's last w
     int wslot_prev = w_last, ys_slot = 0, us_cur = 0, us_prev = 0;
+    int piece = 0;
 #pragma unroll 1
     for (int b = m.b0 - 1;; ++b) {
         const bool body = b >= m.b0, has_next = b + 1 < g.n3;
@@ -652,6 +686,16 @@ __device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, co
         if (valid && more) store_u(ob + plane, un);
         if (win && more) stats(yn, b + 1);
         if (!C.wait(S)) return false;
+        if constexpr (!L::F32) {
+            // band b, whose values every warp left before this phase (the slot
+            // is written again two phases on)
+            if (win && body && tid < TY * TX / 2) {
+                const float2* x = S.above(us_cur) + tid;
+                O.add(x[0]);
+                O.add(x[TY * TX / 2]);
+                if (++piece == a.unit || !more) { O.close(); piece = 0; }
+            }
+        }
         if (tid == 0) {
             // what every warp has finished with by now
             if (body) mbar_arrive(S.yempty + ys_slot);
@@ -957,10 +1001,12 @@ __device__ __forceinline__ void k1_run(const K1Maps* maps, const K1Args<T>& a, c
     // the histograms: on after a recent miss
     W.hb_s = a.sc->ctl[0].hbase;
     W.hb_t = a.sc->ctl[1].hbase;
-    W.hs = W.s && a.sc->ctl[0].hist_left > 0 && hist_base_ok(W.hb_s);
-    W.ht = W.t && a.sc->ctl[1].hist_left > 0 && hist_base_ok(W.hb_t);
+    // (float32 storage only: 16-bit storage searches as the cooperative kernel does)
+    W.hs = L::F32 && W.s && a.sc->ctl[0].hist_left > 0 && hist_base_ok(W.hb_s);
+    W.ht = L::F32 && W.t && a.sc->ctl[1].hist_left > 0 && hist_base_ok(W.hb_t);
     const bool hist = W.hs || W.ht;
     K1Stat A;
+    Ordered O;
     unsigned ny = 0, nw = 0;
     if (wid < kTileWarps) {
         const float cs = (float)(1.0 - a.sc->c[P.parity]);      // y4 = (1 - c) q
@@ -969,10 +1015,10 @@ __device__ __forceinline__ void k1_run(const K1Maps* maps, const K1Args<T>& a, c
         for (int it = bid; it < items; it += nblk, ++turn) {
             const Item m = item_of(a, it, gx, gy);
             const bool ok = item_edge(m, a.g)
-                                ? (hist ? tile_item<T, true, true>(a, S, m, C, A, W, cs, turn)
-                                        : tile_item<T, true, false>(a, S, m, C, A, W, cs, turn))
-                                : (hist ? tile_item<T, false, true>(a, S, m, C, A, W, cs, turn)
-                                        : tile_item<T, false, false>(a, S, m, C, A, W, cs, turn));
+                                ? (hist ? tile_item<T, true, L::F32>(a, S, m, C, A, O, W, cs, turn)
+                                        : tile_item<T, true, false>(a, S, m, C, A, O, W, cs, turn))
+                                : (hist ? tile_item<T, false, L::F32>(a, S, m, C, A, O, W, cs, turn)
+                                        : tile_item<T, false, false>(a, S, m, C, A, O, W, cs, turn));
             if (!ok) break;
         }
     } else if (wid < kConsWarps) {
@@ -1021,6 +1067,10 @@ __device__ __forceinline__ void k1_run(const K1Maps* maps, const K1Args<T>& a, c
         // the histograms' above-range statistics, reduced together: 32-bit
         // counts and float-pair sums through the tile warps, then through
         // warp 0 (no FP64 outside one thread)
+        if constexpr (!L::F32) {
+            A.ks = f2(O.hs, O.ht);
+            A.kc = f2(-O.ls, -O.lt);
+        }
         unsigned n4[4] = {A.n_s, A.n_t, A.top_s.n, A.top_t.n};
         float hi4[4] = {A.ks.x, A.ks.y, A.top_s.s, A.top_t.s};
         float lo4[4] = {-A.kc.x, -A.kc.y, 0.f, 0.f};
@@ -1067,7 +1117,8 @@ __device__ __forceinline__ void k1_run(const K1Maps* maps, const K1Args<T>& a, c
     // what this pass counted, for the finishing launch that follows (every
     // CTA agrees; the first writes it)
     if (cta == 0 && tid == 0) {
-        a.sc->k1_win[0] = W.s; a.sc->k1_win[1] = W.t;
+        constexpr int on = L::F32 ? 1 : 2;                      // 2: no histogram is ever kept
+        a.sc->k1_win[0] = W.s ? on : 0; a.sc->k1_win[1] = W.t ? on : 0;
         a.sc->k1_hist[0] = W.hs; a.sc->k1_hist[1] = W.ht;
     }
 }
@@ -1133,15 +1184,16 @@ double run_cost(int nb, int tiles, int len, int ctas) {
     return (double)((items + ctas - 1) / ctas) * (len + kItemCost);
 }
 
-// Bands per item for `ctas` persistent CTAs: the split of the bands whose
-// slowest CTA does the fewest band steps.
-int best_run(int nb, int tiles, int ctas) {
+// Bands per item for `ctas` persistent CTAs: the split of the bands (in multiples
+// of unit) whose slowest CTA does the fewest band steps.
+int best_run(int nb, int tiles, int ctas, int unit = 1) {
     int best_len = std::min(nb, kMaxRun);
     double best = 1e30;
     int prev = 0;
     for (int runs = 1; runs <= nb; ++runs) {
-        const int len = (nb + runs - 1) / runs;
-        if (len == prev || len > kMaxRun) continue;
+        int len = (nb + runs - 1) / runs;
+        len = (len + unit - 1) / unit * unit;
+        if (len == prev || (len > kMaxRun && unit == 1)) continue;
         prev = len;
         const double c = run_cost(nb, tiles, len, ctas);
         if (c < best * (1.0 - 1e-12)) { best = c; best_len = len; }
@@ -1163,6 +1215,17 @@ Plan k1_plan(const Geom& g, int nb, int chunk, int ctas) {
     const long long items = (long long)tiles * p.gz;
     const long long per = std::max(1, 127 / ((p.chunk + 31) / 32));       // items a CTA may count
     p.ctas = (int)std::min(items, std::max((long long)ctas, (items + per - 1) / per));
+    return p;
+}
+
+// 16-bit storage: items of whole pieces of the window's sums (no histogram, so
+// no limit on the run or the items a CTA takes).
+Plan k1_plan_half(const Geom& g, int nb) {
+    Plan p;
+    const int tiles = tiles_of(g);
+    p.chunk = best_run(nb, tiles, device_sms(), k1_coop_chunk(g));
+    p.gz = (nb + p.chunk - 1) / p.chunk;
+    p.ctas = (int)std::min<long long>((long long)tiles * p.gz, device_sms());
     return p;
 }
 
@@ -1229,8 +1292,9 @@ int k1_tma_part_chunk(const Geom& g, const SlabPart& sp, int chunk) {
     return sp.o1 > sp.o0 ? k1_plan(g, sp.o1 - sp.o0, chunk, device_sms()).chunk : 0;
 }
 
-int k1_tma_grid(const Geom& g, const SlabPart& sp, int chunk) {
-    return sp.o1 > sp.o0 ? k1_plan(g, sp.o1 - sp.o0, chunk, device_sms()).ctas : 0;
+int k1_tma_grid(int storage, const Geom& g, const SlabPart& sp, int chunk) {
+    if (sp.o1 <= sp.o0) return 0;
+    return (storage == 0 ? k1_plan(g, sp.o1 - sp.o0, chunk, device_sms()) : k1_plan_half(g, sp.o1 - sp.o0)).ctas;
 }
 
 namespace {
@@ -1246,6 +1310,7 @@ K1Args<T> k1_args(const Geom& g, const IterBufs& b, const IterParams& p, Scal* s
     a.sc = sc;
     a.l1 = w;
     a.chunk = chunk;
+    a.unit = 0;
     a.sp = sp;
     return a;
 }
@@ -1326,11 +1391,13 @@ int launch_k1_tma(int storage, const Geom& g, const K1Maps& m, const IterBufs& b
                   Scal* sc, const L1Work& w, int chunk, const SlabPart& sp, cudaStream_t st) {
     const int nb = sp.o1 - sp.o0;
     if (nb <= 0 || sp.o0 < 0 || sp.o1 > g.n3) return -1;
-    const Plan pl = k1_plan(g, nb, chunk, device_sms());
+    const Plan pl = storage == 0 ? k1_plan(g, nb, chunk, device_sms()) : k1_plan_half(g, nb);
     const int gx = (g.n2 + TX - 1) / TX, gy = (g.n1 + TY - 1) / TY;
     auto half = [&](auto zero) {
         using T = decltype(zero);
-        k1_half<T><<<pl.ctas, Lay<T>::NT, Lay<T>::SMEM, st>>>(k1_args<T>(g, b, p, sc, w, pl.chunk, sp), gx, gy, pl.gz);
+        K1Args<T> args = k1_args<T>(g, b, p, sc, w, pl.chunk, sp);
+        args.unit = k1_coop_chunk(g);
+        k1_half<T><<<pl.ctas, Lay<T>::NT, Lay<T>::SMEM, st>>>(args, gx, gy, pl.gz);
     };
     switch (storage) {
         case 0:
