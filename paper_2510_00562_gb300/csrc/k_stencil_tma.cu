@@ -1154,9 +1154,11 @@ __device__ __forceinline__ int batch_cube_of(const int* start, int n, int blk) {
 
 __global__ void __launch_bounds__(Lay<float>::NT, 1) k1_tma_batch(const __grid_constant__ K1BatchTab t) {
     const int c = batch_cube_of(t.start, t.n, blockIdx.x);
-    // the cube's arguments by value: the table is indexed by a run-time
-    // cube, so each field is loaded once instead of at each use
-    const K1Args<float> a = t.args[c];
+    // the cube's arguments where they lie, in the constant bank: a copy of them
+    // went to local memory (96 registers are all in use), and its loads lengthened
+    // every band step (464 against 306 us a launch for eight cubes of 0.05 to
+    // 4.2 million voxels)
+    const K1Args<float>& a = t.args[c];
     if (__ldcg(&a.sc->done)) return;        // this cube has stopped
     const K1Maps* maps = t.maps[c];
     if (threadIdx.x == 32 * kConsWarps) {
