@@ -360,14 +360,15 @@ def run_reference(args):
 GRAPH_PASSES = 16            # passes per CUDA graph (graph_iters), the solver's default
 
 
-def gpu_launches(steps, search_passes, graph_passes=GRAPH_PASSES):
-    """Kernels launched in `steps` timed passes: whole graphs of graph_passes
-    passes launch K1, its window finish (which opens the search launches'
-    conditional node when needed) and K2, plus the seven search launches in
-    the passes whose node opened (search_passes); the remaining passes run
-    eagerly, all ten launches each."""
+def gpu_launches(steps, variant="tma", search_passes=0, graph_passes=GRAPH_PASSES):
+    """Kernels launched in `steps` timed passes: K1, the threshold search and
+    K2.  (The cooperative K1: K1, a gate and K2 in whole graphs of graph_passes
+    passes, seven search launches more in those that searched, and nine
+    launches in each pass that runs eagerly.)"""
+    if variant != "coop":
+        return 3 * steps
     in_graphs = (steps // graph_passes) * graph_passes if graph_passes > 0 else 0
-    return 3 * in_graphs + 7 * search_passes + 10 * (steps - in_graphs)
+    return 3 * in_graphs + 7 * search_passes + 9 * (steps - in_graphs)
 
 
 def run_gpu(args):
@@ -483,7 +484,7 @@ def run_gpu(args):
                 "note": "one gsstv_solve_host call of `steps` iterations after an untimed one (the "
                         "solver's graphs built): pinned H2D of v, state reset, iterations, D2H of u, s, t",
                 "clocks": clk_e2e.summary()},
-        "gpu_launches": gpu_launches(args.steps, st["search_passes"], args.graph_passes),
+        "gpu_launches": gpu_launches(args.steps, variant, st["search_passes"], args.graph_passes),
         "quality": quality,
     }
     if pf:

@@ -218,33 +218,32 @@ int enqueue_iteration(gsstv_handle* h, int par, bool timed, cudaStream_t st, boo
                              : cudaEventRecord(h->ev[h->ev_used + 1], st)));
         h->ev_used += 2;
     }
-    // the TMA-fed K1 leaves its window's finish to a launch of its own (the
-    // cooperative K1 finishes it in its last CTA); in a graph that launch, or
-    // a gate kernel, decides whether the search launches run
-    auto k1_finish = [&](int gated, cudaGraphConditionalHandle cond) -> int {
-        if (h->k1_variant == 1)
-            return map_launch(launch_search_finish(2, h->sc, h->l1, 2, h->l1.k1_n, h->l1.k1_s,
-                                                   k1_tma_grid(sto, h->g, whole, h->k1_chunk), st, gated, cond));
-        return gated ? map_launch(launch_search_gate(&h->sc, 1, cond, st)) : GSSTV_OK;
-    };
-    auto search = [&](cudaStream_t s) -> int {
+    if (h->k1_variant == 1) {
         // (16-bit storage: the CTAs that the cooperative K1's partials allow, whose
         // sums a run reproduces)
         const int cap = sto == GSSTV_FP32 ? h->k1_ctas : k1_grid_ctas(h->g);
-        TRY(map_launch(launch_window(sto, h->g, b, ip, h->sc, h->l1, cap, whole, s)));
-        TRY(map_launch(launch_search_finish(0, h->sc, h->l1, 2, h->l1.k1_n, h->l1.k1_s,
-                                            window_grid(h->g, whole, cap), s)));
-        for (int level = 0; level < 3; ++level)
-            TRY(map_launch(launch_fallback(sto, level, h->g, b, ip, h->sc, h->l1, whole, s)));
-        TRY(map_launch(launch_gather(sto, h->g, b, ip, h->sc, h->l1, whole, s)));
-        TRY(map_launch(launch_search_finish(1, h->sc, h->l1, 2, nullptr, nullptr, 0, s)));
-        return GSSTV_OK;
-    };
-    if (in_graph) {
-        TRY(capture_if_search(st, h->cap2, [&](cudaGraphConditionalHandle c) { return k1_finish(1, c); }, search));
+        TRY(map_launch(launch_search(sto, h->g, b, ip, h->sc, h->l1, cap, k1_tma_grid(sto, h->g, whole, h->k1_chunk),
+                                     in_graph ? 1 : 0, st)));
     } else {
-        TRY(k1_finish(0, 0));
-        TRY(search(st));
+        // the cooperative K1 finishes its window in its last CTA; the search
+        // launches return at once unless a vector needs them
+        auto search = [&](cudaStream_t s) -> int {
+            TRY(map_launch(launch_window(sto, h->g, b, ip, h->sc, h->l1, h->k1_ctas, whole, s)));
+            TRY(map_launch(launch_search_finish(0, h->sc, h->l1, 2, h->l1.k1_n, h->l1.k1_s,
+                                                window_grid(h->g, whole, h->k1_ctas), s)));
+            for (int level = 0; level < 3; ++level)
+                TRY(map_launch(launch_fallback(sto, level, h->g, b, ip, h->sc, h->l1, whole, s)));
+            TRY(map_launch(launch_gather(sto, h->g, b, ip, h->sc, h->l1, whole, s)));
+            TRY(map_launch(launch_search_finish(1, h->sc, h->l1, 2, nullptr, nullptr, 0, s)));
+            return GSSTV_OK;
+        };
+        if (in_graph) {
+            TRY(capture_if_search(st, h->cap2, [&](cudaGraphConditionalHandle c) {
+                return map_launch(launch_search_gate(&h->sc, 1, c, st));
+            }, search));
+        } else {
+            TRY(search(st));
+        }
     }
     TRY(map_launch(launch_k2(sto, h->g, b, ip, h->sc, h->k2_part, h->k2_cap, whole, st)));
     return GSSTV_OK;
@@ -892,7 +891,6 @@ struct gsstv_batch {
     int* live = nullptr;           // device: cubes still iterating
     int* live_host = nullptr;      // page-locked copy
     cudaStream_t cap = nullptr;    // private capture stream
-    cudaStream_t cap2 = nullptr;   // and one for the bodies of conditional graph nodes
     cudaGraphExec_t gexec = nullptr;
     int graph_len = 0;
     std::vector<int> graph_chunks;  // the cubes' K1 band runs the graph was built with
@@ -904,7 +902,6 @@ int gsstv_batch_destroy(gsstv_batch* b) {
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
     if (b->caller) cudaStreamSynchronize(b->caller);
     if (b->cap) cudaStreamDestroy(b->cap);
-    if (b->cap2) cudaStreamDestroy(b->cap2);
     if (b->dmaps) cudaFree(b->dmaps);
     if (b->live) cudaFree(b->live);
     if (b->live_host) cudaFreeHost(b->live_host);
@@ -971,10 +968,6 @@ int gsstv_batch_create(gsstv_batch** out, int ncubes, const int* n1, const int* 
             b->cap = nullptr;
             rc = GSSTV_ERR_CUDA;
         }
-        if (rc == GSSTV_OK && cudaStreamCreateWithFlags(&b->cap2, cudaStreamNonBlocking) != cudaSuccess) {
-            b->cap2 = nullptr;
-            rc = GSSTV_ERR_CUDA;
-        }
         for (int c = 0; c < ncubes && rc == GSSTV_OK; ++c)
             rc = cuda_rc(cudaMemcpy(b->dmaps + 2 * c, b->h[c]->maps, 2 * sizeof(K1Maps), cudaMemcpyHostToDevice));
     }
@@ -1014,17 +1007,7 @@ int batch_enqueue(gsstv_batch* b, const std::vector<int>& set, int par, cudaStre
     TRY(map_launch(launch_k1_batch(cubes, nc, st)));
     // K1's window finish, then the search launches behind a conditional node
     // that it opens (the fused solve is always captured)
-    auto k1_finish = [&](cudaGraphConditionalHandle c) -> int {
-        return map_launch(launch_finish_batch(cubes, nc, 2, st, 1, c));
-    };
-    TRY(capture_if_search(st, b->cap2, k1_finish, [&](cudaStream_t q) -> int {
-        TRY(map_launch(launch_window_batch(cubes, nc, q)));
-        TRY(map_launch(launch_finish_batch(cubes, nc, 0, q)));
-        for (int level = 0; level < 3; ++level) TRY(map_launch(launch_radix_batch(cubes, nc, level, q)));
-        TRY(map_launch(launch_gather_batch(cubes, nc, q)));
-        TRY(map_launch(launch_finish_batch(cubes, nc, 1, q)));
-        return GSSTV_OK;
-    }));
+    TRY(map_launch(launch_search_batch(cubes, nc, st)));
     TRY(map_launch(launch_k2_batch(cubes, nc, st)));
     return GSSTV_OK;
 }

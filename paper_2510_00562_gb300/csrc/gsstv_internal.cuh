@@ -146,6 +146,16 @@ struct L1Acc {
     unsigned int pad;
 };
 
+// Stages of a pass's search launch (k_search): the current one, and of each
+// stage the items drawn and done.  Zero between passes.
+constexpr int kSearchStages = 8;
+constexpr unsigned kSearchSpinLimit = 1u << 23;   // polls (0.1 us and more each) before a wait gives up
+struct SearchSync {
+    unsigned stage = 0;
+    unsigned next[kSearchStages] = {}, done[kSearchStages] = {};
+    unsigned pad = 0;
+};
+
 struct Scal {
     double c[2];               // y4 = (1 - c[p]) q at iteration parity p
     L1Ctl ctl[2];
@@ -164,6 +174,7 @@ struct Scal {
     long long gate_opens;      // passes whose threshold search launches ran (graphs)
     unsigned int fin_ticket;   // CTAs of K1's window finish done (the last sets the search gate)
     unsigned int pad2;
+    SearchSync search;
 };
 
 constexpr int kHistBins = 2048;        // radix histogram bins per vector
@@ -473,6 +484,10 @@ int launch_search_gate(Scal* const* sc, int n, cudaGraphConditionalHandle cond, 
 // for every vector that needs it: one launch after the pass(es) it finishes.
 // gated (mode 2 in a graph): its last CTA also sets `cond` to whether a
 // threshold search is still needed.
+// K1's window finish and, where a vector needs it, the rest of the search, in
+// one launch.  parts: K1's CTAs; count: count the pass in gate_opens if it searched
+int launch_search(int storage, const Geom& g, const IterBufs& b, const IterParams& p, Scal* sc, const L1Work& w,
+                  int part_cap, int parts, int count, cudaStream_t st);
 int launch_search_finish(int mode, Scal* sc, const L1Work& w, int nvec, const unsigned long long* pn,
                          const double* ps, int parts, cudaStream_t st, int gated = 0,
                          cudaGraphConditionalHandle cond = 0);
@@ -503,11 +518,7 @@ struct BatchCube {
 int launch_k1_batch(const BatchCube* cubes, int n, cudaStream_t st);
 // how launch_k1_batch splits the cubes: bands per item, band runs and CTAs of each
 void k1_batch_plan(const BatchCube* cubes, int n, int* chunk, int* gz, int* ctas);
-int launch_window_batch(const BatchCube* cubes, int n, cudaStream_t st);
-int launch_radix_batch(const BatchCube* cubes, int n, int level, cudaStream_t st);
-int launch_gather_batch(const BatchCube* cubes, int n, cudaStream_t st);
-int launch_finish_batch(const BatchCube* cubes, int n, int mode, cudaStream_t st, int gated = 0,
-                        cudaGraphConditionalHandle cond = 0);
+int launch_search_batch(const BatchCube* cubes, int n, cudaStream_t st);
 int launch_k2_batch(const BatchCube* cubes, int n, cudaStream_t st);
 int batch_configure();
 

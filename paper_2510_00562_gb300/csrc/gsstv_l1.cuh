@@ -792,9 +792,11 @@ static __device__ void l1_radix_select(L1Ctl& c, RadixLevel lv, const unsigned l
                                        const unsigned long long* hres, double r, double* sh_d,
                                        unsigned long long* sh_u, int* sh_i) {
     const int nb = lv.nbins();
-    const int nt = blockDim.x;
+    // (chunks for 256 threads at most: thread 0 walks the chunks' sums in FP64)
+    const int nt = min((int)blockDim.x, 256);
     const int per = (nb + nt - 1) / nt;
-    const int k0 = threadIdx.x * per;
+    const bool has = (int)threadIdx.x < nt;
+    const int k0 = has ? threadIdx.x * per : nb;
     const int k1 = min(nb, k0 + per);
     // 1. chunk totals
     unsigned long long cnt = 0;
@@ -808,8 +810,10 @@ static __device__ void l1_radix_select(L1Ctl& c, RadixLevel lv, const unsigned l
         }
     }
     // sh_d[0..nt) chunk sums, sh_u[0..nt) chunk counts; suffixes by thread 0
-    sh_d[threadIdx.x] = sum;
-    sh_u[threadIdx.x] = cnt;
+    if (has) {
+        sh_d[threadIdx.x] = sum;
+        sh_u[threadIdx.x] = cnt;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         double s = c.s_above;
@@ -825,8 +829,8 @@ static __device__ void l1_radix_select(L1Ctl& c, RadixLevel lv, const unsigned l
     }
     __syncthreads();
     // 2. inside the chunk, from the top bin down: phi(lo_k) >= 0 ?
-    double s_run = sh_d[threadIdx.x];
-    unsigned long long n_run = sh_u[threadIdx.x];
+    double s_run = has ? sh_d[threadIdx.x] : 0.0;
+    unsigned long long n_run = has ? sh_u[threadIdx.x] : 0ull;
     int best = -1;
     double best_phi = 0.0, best_s_above = 0.0;
     unsigned long long best_n_above = 0, best_cnt = 0;

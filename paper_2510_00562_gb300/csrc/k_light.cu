@@ -352,6 +352,7 @@ __device__ __forceinline__ void k2_body(const K2Args<T>& a, const int bid, const
         sc->u2 = s2;
         sc->iter++;
         sc->k2_ticket = 0;
+        sc->search = SearchSync();
         // the stopping rule of a batch cube (Eq. 28, or the pass cap): on the
         // device, so that a batch runs as one graph without host polling
         if (P.max_iter > 0) {
@@ -389,16 +390,20 @@ struct CubeSrc {
     // want_t: whether the pass needs |s~| / |t~| (uniform over the launch); the
     // inputs of a vector not wanted are not read, and its value passed to f is
     // meaningless.
+    // The thread takes items first + its index, then every stride (both in
+    // threads, the stride a multiple of 32; threads at or past it take none).
     template <typename F>
-    __device__ void visit(const int bid, const int nblk, F&& f, const bool want_s, const bool want_t) const {
+    __device__ void visit(const unsigned first, const unsigned stride, F&& f, const bool want_s,
+                          const bool want_t) const {
         const float cs = (float)(1.0 - sc->c[parity]);
         const unsigned quads = (unsigned)g.p2 / 4u;
         const unsigned n1 = (unsigned)g.n1;
         const unsigned total = (unsigned)nb * n1 * quads;       // < 2^31 for any cube that fits
         const unsigned row0 = (unsigned)o0 * n1;
-        for (unsigned base = bid * blockDim.x; base < total; base += nblk * blockDim.x) {
+        const bool mine = first + threadIdx.x < stride;
+        for (unsigned base = first; base < total; base += stride) {
             const unsigned item = base + threadIdx.x;
-            const bool live = item < total;
+            const bool live = mine && item < total;
             const unsigned row = row0 + (live ? item / quads : 0u);   // b * n1 + i
             const int j = (int)(item - (row - row0) * quads) * 4;
             const int i = (int)(row % n1);
@@ -431,8 +436,8 @@ struct FlatSrc {
     const float* x;
     long long n;
     template <typename F>
-    __device__ void visit(const int bid, const int nblk, F&& f, bool, bool) const {
-        for (long long base = bid * (long long)blockDim.x; base < n; base += (long long)nblk * blockDim.x) {
+    __device__ void visit(const unsigned first, const unsigned stride, F&& f, bool, bool) const {
+        for (long long base = first; base < n; base += stride) {
             const long long l = base + threadIdx.x;
             const bool valid = l < n;
             f(valid, valid ? fabsf(x[l]) : 0.f, 0.f);
@@ -448,16 +453,11 @@ struct SearchArgs {
     __device__ int total(int nblk) const { return cta_total > 0 ? cta_total : nblk; }
 };
 
-// Radix histogram pass of one level for every vector that needs it; the last
-// CTA selects the bracket.
+// Radix histogram pass of one level for every vector that needs it.
 template <typename Src>
-__device__ __forceinline__ void radix_body(const Src& src, const SearchArgs& a, const int level, const int bid,
-                                           const int nblk) {
+__device__ __forceinline__ void radix_count(const Src& src, const SearchArgs& a, const int level, const int bid,
+                                            const int nblk) {
     extern __shared__ __align__(16) unsigned hsm[];   // [2][2048] counts, low and high residue halves
-    __shared__ double sh_d[NT];
-    __shared__ unsigned long long sh_u[NT];
-    __shared__ int sh_i[1];
-    __shared__ int is_last;
     const int want = NEED_RADIX0 + level;
     bool need[2];
     need[0] = a.sc->ctl[0].need == want;
@@ -472,7 +472,7 @@ __device__ __forceinline__ void radix_body(const Src& src, const SearchArgs& a, 
     unsigned* hc = hsm;
     unsigned* hrl = hsm + 2 * kHistBins;
     unsigned* hrh = hsm + 4 * kHistBins;
-    for (int k = threadIdx.x; k < 6 * kHistBins; k += NT) hsm[k] = 0;
+    for (int k = threadIdx.x; k < 6 * kHistBins; k += blockDim.x) hsm[k] = 0;
     __syncthreads();
     const unsigned pre0 = a.sc->ctl[0].prefix, pre1 = a.sc->ctl[1].prefix;
     auto insert = [&](int v, bool take, unsigned key) {
@@ -486,7 +486,7 @@ __device__ __forceinline__ void radix_body(const Src& src, const SearchArgs& a, 
             }
         }
     };
-    src.visit(bid, nblk, [&](bool valid, float x0, float x1) {
+    src.visit(bid * blockDim.x, nblk * blockDim.x, [&](bool valid, float x0, float x1) {
         if (need[0]) {
             const unsigned key = __float_as_uint(x0);
             insert(0, valid && lv.inside(key, pre0), key);
@@ -497,24 +497,47 @@ __device__ __forceinline__ void radix_body(const Src& src, const SearchArgs& a, 
         }
     }, need[0], need[1]);
     __syncthreads();
-    for (int k = threadIdx.x; k < 2 * kHistBins; k += NT) {
+    for (int k = threadIdx.x; k < 2 * kHistBins; k += blockDim.x) {
         if ((k % kHistBins) >= nb) continue;
         if (hc[k]) atomicAdd(a.w.hcnt + k, (unsigned long long)hc[k]);
         const unsigned long long res = ((unsigned long long)hrh[k] << 10) + hrl[k];
         if (res) atomicAdd(a.w.hres + k, res);
     }
+}
+
+// Selects the bracket of one level once every CTA has counted; one whole block.
+__device__ __forceinline__ void radix_finish(const SearchArgs& a, const int level) {
+    __shared__ double sh_d[NT];
+    __shared__ unsigned long long sh_u[NT];
+    __shared__ int sh_i[1];
+    const int want = NEED_RADIX0 + level;
+    const RadixLevel lv{level};
+    bool need[2];
+    need[0] = a.sc->ctl[0].need == want;
+    need[1] = a.nvec > 1 && a.sc->ctl[1].need == want;
+    for (int v = 0; v < 2; ++v) {
+        if (!need[v]) continue;
+        l1_radix_select(a.sc->ctl[v], lv, a.w.hcnt + v * kHistBins, a.w.hres + v * kHistBins,
+                        a.sc->radius[v], sh_d, sh_u, sh_i);
+    }
+    for (int k = threadIdx.x; k < 2 * kHistBins; k += blockDim.x) { a.w.hcnt[k] = 0; a.w.hres[k] = 0; }
+}
+
+// A level in a launch of its own; the last CTA selects the bracket.
+template <typename Src>
+__device__ __forceinline__ void radix_body(const Src& src, const SearchArgs& a, const int level, const int bid,
+                                           const int nblk) {
+    __shared__ int is_last;
+    const int want = NEED_RADIX0 + level;
+    if (a.sc->ctl[0].need != want && !(a.nvec > 1 && a.sc->ctl[1].need == want)) return;
+    radix_count(src, a, level, bid, nblk);
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) is_last = (atomicAdd(&a.sc->fb_ticket, 1u) == (unsigned)(a.total(nblk) - 1));
     __syncthreads();
     if (!is_last) return;
     __threadfence();
-    for (int v = 0; v < 2; ++v) {
-        if (!need[v]) continue;
-        l1_radix_select(a.sc->ctl[v], lv, a.w.hcnt + v * kHistBins, a.w.hres + v * kHistBins,
-                        a.sc->radius[v], sh_d, sh_u, sh_i);
-    }
-    for (int k = threadIdx.x; k < 2 * kHistBins; k += NT) { a.w.hcnt[k] = 0; a.w.hres[k] = 0; }
+    radix_finish(a, level);
     if (threadIdx.x == 0) a.sc->fb_ticket = 0;
 }
 
@@ -608,7 +631,7 @@ __device__ __forceinline__ void gather_body(const Src& src, const SearchArgs& a,
     GSSTV_BLOCK_CAND(bc);
     if (need[0]) bc.keep_hist(a.w, 0, lo0, hi0);
     if (need[1]) bc.keep_hist(a.w, 1, lo1, hi1);
-    src.visit(bid, nblk, [&](bool valid, float x0, float x1) {
+    src.visit(bid * blockDim.x, nblk * blockDim.x, [&](bool valid, float x0, float x1) {
         if (need[0]) bc.append(0, valid && x0 > lo0 && x0 <= hi0, x0, a.w.cand[0], &a.sc->acc[0].m);
         if (need[1]) bc.append(1, valid && x1 > lo1 && x1 <= hi1, x1, a.w.cand[1], &a.sc->acc[1].m);
     }, need[0], need[1]);
@@ -628,7 +651,7 @@ __global__ void __launch_bounds__(NT) k_gather(const Src src, const SearchArgs a
 // partial sums go to pn / ps (the stencil pass's partial arrays, free by now).
 template <typename Src>
 __device__ __forceinline__ void window_body(const Src& src, const SearchArgs& a, unsigned long long* pn, double* ps,
-                                            const int bid, const int nblk) {
+                                            const int bid, const unsigned stride) {
     __shared__ double red_d[64];
     __shared__ unsigned long long red_u[64];
     bool need[2];
@@ -641,7 +664,7 @@ __device__ __forceinline__ void window_body(const Src& src, const SearchArgs& a,
     GSSTV_BLOCK_CAND(bc);
     if (need[0]) bc.keep_hist(a.w, 0, lo0, hi0);
     if (need[1]) bc.keep_hist(a.w, 1, lo1, hi1);
-    src.visit(bid, nblk, [&](bool valid, float x0, float x1) {
+    src.visit(bid * blockDim.x, stride, [&](bool valid, float x0, float x1) {
         if (need[0]) {
             const bool hi = valid && x0 > hi0;
             if (hi) { w0.n++; w0.s.add(x0); }
@@ -669,7 +692,7 @@ __device__ __forceinline__ void window_body(const Src& src, const SearchArgs& a,
 template <typename Src>
 __global__ void __launch_bounds__(NT) k_window(const Src src, const SearchArgs a, unsigned long long* pn,
                                                double* ps) {
-    window_body(src, a, pn, ps, blockIdx.x, gridDim.x);
+    window_body(src, a, pn, ps, blockIdx.x, gridDim.x * blockDim.x);
 }
 
 // The finish of K1's window (mode 2), of the retry window (mode 0) or of the
@@ -875,6 +898,121 @@ __global__ void __launch_bounds__(kFinishThreads) k_search_finish(const SearchAr
     if (gated) finish_gate(a.sc, gridDim.x, cond, [&] { return scal_needs_search(a.sc); });
 }
 
+// ---------------------------------------------------------------------------
+// the threshold search of a pass in one launch
+// ---------------------------------------------------------------------------
+// Between K1 and K2: the finish of K1's window (two CTAs, one per vector) and,
+// when a vector's window missed, the retry, radix and gather passes on all CTAs.
+// The stages follow one another inside the launch.  (With the search launches in
+// a conditional graph node, every pass paid 8.5 us between the finish and K2 for
+// the node alone, opened or not; passes launched one by one paid for seven
+// launches that returned at once.)
+//
+// A stage is a number of items that CTAs draw from a counter; the CTA that
+// completes a stage's last item decides the next stage and publishes it.  A CTA
+// only ever waits for items that running CTAs hold, so the launch needs no
+// co-residency and may share the GPU with others of its kind.  K2 clears the
+// counters for the next pass.  Waits are bounded.
+enum { ST_FINISH = 0, ST_WINDOW, ST_WINDOW_END, ST_RADIX0, ST_RADIX1, ST_RADIX2, ST_GATHER, ST_GATHER_END, ST_EXIT };
+static_assert(ST_GATHER_END < kSearchStages, "counters per stage");
+
+struct SearchShape {
+    int parts;              // K1's partials
+    unsigned win_threads;   // threads that share the retry pass (a multiple of 256)
+    int win_items, pass_items;
+    int count;              // count the passes that searched (graph launches)
+};
+
+__device__ __forceinline__ unsigned search_stage(const SearchSync* y) {
+    unsigned w;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(w) : "l"(&y->stage) : "memory");
+    return w;
+}
+
+// The stage after `st` from the vectors' needs (thread 0).
+__device__ __forceinline__ int search_next(const SearchArgs& a, int st) {
+    if (st == ST_WINDOW) return ST_WINDOW_END;
+    if (st == ST_GATHER) return ST_GATHER_END;
+    int next = ST_EXIT;
+    for (int v = 0; v < a.nvec; ++v) {
+        const int need = __ldcg(&a.sc->ctl[v].need);
+        const int s = need == NEED_WINDOW ? ST_WINDOW : need == NEED_RADIX0 ? ST_RADIX0 : need == NEED_RADIX1 ? ST_RADIX1
+                    : need == NEED_RADIX2 ? ST_RADIX2 : need == NEED_GATHER ? ST_GATHER : ST_EXIT;
+        if (s > st) next = min(next, s);
+    }
+    return next;
+}
+
+template <typename Src>
+__device__ __forceinline__ void search_body(const Src& src, const SearchArgs& a, unsigned long long* pn, double* ps,
+                                            const SearchShape& h, const int bid) {
+    __shared__ int sh_stage, sh_item, sh_last;
+    SearchSync* y = &a.sc->search;
+    // whole block: an item of stage st is done; the last of n publishes the next stage
+    auto complete = [&](int st, int n) {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            sh_last = atomicAdd(&y->done[st], 1u) == (unsigned)(n - 1);
+        }
+        __syncthreads();
+        if (!sh_last) return;
+        __threadfence();
+        if (st >= ST_RADIX0 && st <= ST_RADIX2) {
+            radix_finish(a, st - ST_RADIX0);
+            __threadfence();
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) {
+            const unsigned next = (unsigned)search_next(a, st);
+            if (st == ST_FINISH && next != ST_EXIT && h.count) a.sc->gate_opens++;
+            __threadfence();
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&y->stage), "r"(next) : "memory");
+        }
+    };
+    if (bid < a.nvec) {
+        finish_body(a, 2, pn, ps, h.parts, bid);
+        complete(ST_FINISH, a.nvec);
+    }
+    for (int st = ST_FINISH;;) {
+        if (threadIdx.x == 0) {
+            unsigned w = search_stage(y);
+            for (unsigned k = 0; w <= (unsigned)st && k < kSearchSpinLimit; ++k) {
+                __nanosleep(100);
+                w = search_stage(y);
+            }
+            if (w <= (unsigned)st) {
+                atomicOr(&a.sc->error, 4);
+                w = ST_EXIT;
+            }
+            sh_stage = (int)w;
+        }
+        __syncthreads();
+        st = sh_stage;
+        if (st >= ST_EXIT) return;
+        const int n = st == ST_WINDOW ? h.win_items : st == ST_WINDOW_END || st == ST_GATHER_END ? a.nvec : h.pass_items;
+        for (;;) {
+            if (threadIdx.x == 0) sh_item = (int)atomicAdd(&y->next[st], 1u);
+            __syncthreads();
+            const int item = sh_item;
+            if (item >= n) break;
+            if (st == ST_WINDOW) window_body(src, a, pn, ps, item, h.win_threads);
+            else if (st == ST_WINDOW_END) finish_body(a, 0, pn, ps, h.win_items, item);
+            else if (st == ST_GATHER) gather_body(src, a, item, n);
+            else if (st == ST_GATHER_END) finish_body(a, 1, pn, ps, 0, item);
+            else radix_count(src, a, st - ST_RADIX0, item, n);
+            complete(st, n);
+        }
+        __syncthreads();
+    }
+}
+
+template <typename Src>
+__global__ void __launch_bounds__(kFinishThreads) k_search(const Src src, const SearchArgs a, unsigned long long* pn,
+                                                           double* ps, const SearchShape h) {
+    search_body(src, a, pn, ps, h, blockIdx.x);
+}
+
 // out = soft(x, tau) for the standalone projection
 __global__ void k_apply_flat(const float* x, float* out, long long n, const Scal* sc) {
     const double tau = sc->ctl[0].tau;
@@ -1055,6 +1193,31 @@ int launch_window_t(const Geom& g, const IterBufs& b, const IterParams& p, Scal*
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
+// the shape of a cube's search launch.  win_ctas: 256-thread CTAs that the retry
+// pass is split by; a radix item sees at most 2^21 values (its shared bins are
+// 32-bit).
+SearchShape search_shape(long long voxels, int win_ctas, int parts, int count, int ctas) {
+    SearchShape h;
+    h.parts = parts;
+    h.win_threads = 256u * (unsigned)win_ctas;
+    h.win_items = (win_ctas * 256 + kFinishThreads - 1) / kFinishThreads;
+    h.pass_items = (int)std::max<long long>(ctas, (voxels + (1ll << 21) - 1) >> 21);
+    h.count = count;
+    return h;
+}
+
+template <typename T>
+int launch_search_t(const Geom& g, const IterBufs& b, const IterParams& p, Scal* sc, const L1Work& w, int part_cap,
+                    int parts, int count, cudaStream_t st) {
+    const SlabPart whole = whole_cube(g);
+    const CubeSrc<T> src = make_cube_src<T>(g, b, p, sc, whole);
+    const int win = window_grid_n(part_voxels(g, whole), part_cap);
+    const int ctas = std::max(2, (win * 256 + kFinishThreads - 1) / kFinishThreads);
+    const SearchShape h = search_shape(part_voxels(g, whole), win, parts, count, ctas);
+    k_search<CubeSrc<T>><<<ctas, kFinishThreads, kFinishSmem, st>>>(src, cube_args(sc, w, whole), w.k1_n, w.k1_s, h);
+    return cudaGetLastError() == cudaSuccess ? 0 : -3;
+}
+
 template <typename S, typename D>
 int launch_convert(const S* src, long long sp, long long sc_, D* dst, long long dp, long long dc,
                    const Geom& g, int ncubes, const double* scale, cudaStream_t st) {
@@ -1095,7 +1258,7 @@ struct SearchCube {
     SearchArgs a;
     unsigned long long* pn;
     double* ps;
-    int parts;
+    SearchShape h;
 };
 struct SearchBatchTab {
     int n;
@@ -1108,37 +1271,14 @@ struct K2BatchTab {
     K2Args<float> c[kBatchMax];
 };
 
-__global__ void __launch_bounds__(NT) k_window_batch(const __grid_constant__ SearchBatchTab t) {
-    const int c = batch_cube_of(t.start, t.n, blockIdx.x);
+// The search of every cube of a batch.  The first CTAs are two per cube, its
+// window's finishes; the rest help the cubes that start[] gives them to.
+__global__ void __launch_bounds__(kFinishThreads) k_search_batch(const __grid_constant__ SearchBatchTab t) {
+    const int k = (int)blockIdx.x - 2 * t.n;
+    const int c = k < 0 ? (int)blockIdx.x >> 1 : batch_cube_of(t.start, t.n, k);
     const SearchCube& q = t.c[c];
     if (__ldcg(&q.a.sc->done)) return;
-    window_body(q.src, q.a, q.pn, q.ps, blockIdx.x - t.start[c], t.start[c + 1] - t.start[c]);
-}
-__global__ void __launch_bounds__(NT) k_radix_batch(const __grid_constant__ SearchBatchTab t, const int level) {
-    const int c = batch_cube_of(t.start, t.n, blockIdx.x);
-    const SearchCube& q = t.c[c];
-    if (__ldcg(&q.a.sc->done)) return;
-    radix_body(q.src, q.a, level, blockIdx.x - t.start[c], t.start[c + 1] - t.start[c]);
-}
-__global__ void __launch_bounds__(NT) k_gather_batch(const __grid_constant__ SearchBatchTab t) {
-    const int c = batch_cube_of(t.start, t.n, blockIdx.x);
-    const SearchCube& q = t.c[c];
-    if (__ldcg(&q.a.sc->done)) return;
-    gather_body(q.src, q.a, blockIdx.x - t.start[c], t.start[c + 1] - t.start[c]);
-}
-// one CTA per cube and vector
-__global__ void __launch_bounds__(kFinishThreads) k_finish_batch(const __grid_constant__ SearchBatchTab t,
-                                                                  const int mode, int gated,
-                                                                  cudaGraphConditionalHandle cond) {
-    const SearchCube& q = t.c[blockIdx.x >> 1];
-    if (!__ldcg(&q.a.sc->done)) finish_body(q.a, mode, q.pn, q.ps, q.parts, blockIdx.x & 1);
-    // every CTA counts, a stopped cube's too (the first cube's scalars hold the count)
-    if (gated)
-        finish_gate(t.c[0].a.sc, gridDim.x, cond, [&] {
-            bool any = false;
-            for (int c = 0; c < t.n; ++c) any = any || scal_needs_search(t.c[c].a.sc);
-            return any;
-        });
+    search_body(q.src, q.a, q.pn, q.ps, q.h, k < 0 ? (int)blockIdx.x & 1 : 2);
 }
 __global__ void __launch_bounds__(NT, 3) k2_batch(const __grid_constant__ K2BatchTab t) {
     const int c = batch_cube_of(t.start, t.n, blockIdx.x);
@@ -1147,28 +1287,6 @@ __global__ void __launch_bounds__(NT, 3) k2_batch(const __grid_constant__ K2Batc
     const K2Args<float> a = t.c[c];
     if (__ldcg(&a.sc->done)) return;
     k2_body(a, blockIdx.x - t.start[c], t.start[c + 1] - t.start[c]);
-}
-
-// the search table of a stage; grid(q): CTAs of cube q's share
-template <typename G>
-int search_table(const BatchCube* cubes, int n, SearchBatchTab& t, G&& grid) {
-    if (n < 1 || n > kBatchMax) return -1;
-    static_assert(sizeof(SearchBatchTab) <= 32000, "kernel parameter space");
-    t.n = n;
-    int total = 0;
-    for (int c = 0; c < n; ++c) {
-        const BatchCube& q = cubes[c];
-        const SlabPart whole = whole_cube(q.g);
-        t.c[c].src = make_cube_src<float>(q.g, q.b, q.p, q.sc, whole);
-        t.c[c].a = cube_args(q.sc, q.l1, whole);
-        t.c[c].pn = q.l1.k1_n;
-        t.c[c].ps = q.l1.k1_s;
-        t.c[c].parts = window_grid_n(part_voxels(q.g, whole), q.k1_ctas);
-        t.start[c] = total;
-        total += grid(q, whole);
-    }
-    t.start[n] = total;
-    return total;
 }
 
 }  // namespace
@@ -1205,8 +1323,24 @@ int light_configure(int storage) {
     if (e != cudaSuccess) return -3;
     e = cudaFuncSetAttribute(k_radix<FlatSrc>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return -3;
+    switch (storage) {
+        case 0: e = cudaFuncSetAttribute(k_search<CubeSrc<float>>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFinishSmem); break;
+        case 1: e = cudaFuncSetAttribute(k_search<CubeSrc<__nv_bfloat16>>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFinishSmem); break;
+        case 2: e = cudaFuncSetAttribute(k_search<CubeSrc<__half>>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFinishSmem); break;
+    }
+    if (e != cudaSuccess) return -3;
     e = cudaFuncSetAttribute(k_search_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, kFinishSmem);
     return e == cudaSuccess ? 0 : -3;
+}
+
+int launch_search(int storage, const Geom& g, const IterBufs& b, const IterParams& p, Scal* sc, const L1Work& w,
+                  int part_cap, int parts, int count, cudaStream_t st) {
+    switch (storage) {
+        case 0: return launch_search_t<float>(g, b, p, sc, w, part_cap, parts, count, st);
+        case 1: return launch_search_t<__nv_bfloat16>(g, b, p, sc, w, part_cap, parts, count, st);
+        case 2: return launch_search_t<__half>(g, b, p, sc, w, part_cap, parts, count, st);
+    }
+    return -1;
 }
 
 int launch_search_finish(int mode, Scal* sc, const L1Work& w, int nvec, const unsigned long long* pn,
@@ -1267,36 +1401,6 @@ int launch_window(int storage, const Geom& g, const IterBufs& b, const IterParam
     return -1;
 }
 
-int launch_window_batch(const BatchCube* cubes, int n, cudaStream_t st) {
-    SearchBatchTab t{};
-    const int total = search_table(cubes, n, t, [](const BatchCube& q, const SlabPart& w) {
-        return window_grid_n(part_voxels(q.g, w), q.k1_ctas);
-    });
-    if (total < 0) return -1;
-    k_window_batch<<<total, NT, 0, st>>>(t);
-    return cudaGetLastError() == cudaSuccess ? 0 : -3;
-}
-
-int launch_radix_batch(const BatchCube* cubes, int n, int level, cudaStream_t st) {
-    SearchBatchTab t{};
-    const int total = search_table(cubes, n, t, [](const BatchCube& q, const SlabPart& w) {
-        return radix_grid_n(part_voxels(q.g, w));
-    });
-    if (total < 0) return -1;
-    k_radix_batch<<<total, NT, 6 * kHistBins * sizeof(unsigned), st>>>(t, level);
-    return cudaGetLastError() == cudaSuccess ? 0 : -3;
-}
-
-int launch_gather_batch(const BatchCube* cubes, int n, cudaStream_t st) {
-    SearchBatchTab t{};
-    const int total = search_table(cubes, n, t, [](const BatchCube& q, const SlabPart& w) {
-        return gather_grid_n(part_voxels(q.g, w));
-    });
-    if (total < 0) return -1;
-    k_gather_batch<<<total, NT, 0, st>>>(t);
-    return cudaGetLastError() == cudaSuccess ? 0 : -3;
-}
-
 // Whether any cube still needs a threshold search after K1's finish: sets the
 // condition of the graph node that holds the search launches (one thread, so
 // that no two calls race).
@@ -1327,16 +1431,33 @@ int launch_search_gate(Scal* const* sc, int n, cudaGraphConditionalHandle cond, 
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
-int launch_finish_batch(const BatchCube* cubes, int n, int mode, cudaStream_t st, int gated,
-                        cudaGraphConditionalHandle cond) {
+int launch_search_batch(const BatchCube* cubes, int n, cudaStream_t st) {
+    if (n < 1 || n > kBatchMax) return -1;
+    static_assert(sizeof(SearchBatchTab) <= 32000, "kernel parameter space");
     SearchBatchTab t{};
-    if (search_table(cubes, n, t, [](const BatchCube&, const SlabPart&) { return 1; }) < 0) return -1;
-    if (mode == 2) {                     // K1's partials: one set per CTA of the cube's share of K1
-        int chunk[kBatchMax], gz[kBatchMax], ctas[kBatchMax];
-        k1_batch_plan(cubes, n, chunk, gz, ctas);
-        for (int c = 0; c < n; ++c) t.c[c].parts = ctas[c];
+    t.n = n;
+    int chunk[kBatchMax], gz[kBatchMax], ctas[kBatchMax];
+    k1_batch_plan(cubes, n, chunk, gz, ctas);            // K1's partials: one set per CTA of the cube
+    double all = 0.0;
+    for (int c = 0; c < n; ++c) all += (double)cubes[c].g.cube;
+    const int helpers = std::max(0, device_sms() - 2 * n);
+    int total = 0;
+    for (int c = 0; c < n; ++c) {
+        const BatchCube& q = cubes[c];
+        const SlabPart whole = whole_cube(q.g);
+        const long long vox = part_voxels(q.g, whole);
+        SearchCube& e = t.c[c];
+        e.src = make_cube_src<float>(q.g, q.b, q.p, q.sc, whole);
+        e.a = cube_args(q.sc, q.l1, whole);
+        e.pn = q.l1.k1_n;
+        e.ps = q.l1.k1_s;
+        t.start[c] = total;
+        const int share = (int)(helpers * ((double)q.g.cube / all));
+        e.h = search_shape(vox, window_grid_n(vox, q.k1_ctas), ctas[c], 1, 2 + share);
+        total += share;
     }
-    k_finish_batch<<<2 * n, kFinishThreads, kFinishSmem, st>>>(t, mode, gated, cond);
+    t.start[n] = total;
+    k_search_batch<<<2 * n + total, kFinishThreads, kFinishSmem, st>>>(t);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -1373,10 +1494,7 @@ int k1_batch_configure();
 
 int batch_configure() {
     if (k1_batch_configure() != 0) return -3;
-    cudaError_t e = cudaFuncSetAttribute(k_radix_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(6 * kHistBins * sizeof(unsigned)));
-    if (e != cudaSuccess) return -3;
-    e = cudaFuncSetAttribute(k_finish_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFinishSmem);
+    const cudaError_t e = cudaFuncSetAttribute(k_search_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFinishSmem);
     return e == cudaSuccess ? 0 : -3;
 }
 
