@@ -342,7 +342,8 @@ int error_of(const Scal& s) {
     return GSSTV_OK;
 }
 
-Scal initial_scalars(const gsstv_params& p) {
+// defer: K2 places the search's next windows (a whole cube's launches)
+Scal initial_scalars(const gsstv_params& p, int defer) {
     Scal s;
     std::memset(&s, 0, sizeof(s));
     s.radius[0] = p.alpha;
@@ -350,6 +351,7 @@ Scal initial_scalars(const gsstv_params& p) {
     for (int v = 0; v < 2; ++v) {
         s.ctl[v].window_ok = 1;       // first window (0, 0]: is the vector inside the ball?
         s.ctl[v].need = NEED_NONE;
+        s.ctl[v].defer = defer;
     }
     return s;
 }
@@ -437,7 +439,7 @@ int gsstv_create(gsstv_handle** out, int n1, int n2, int n3, const gsstv_params*
         const IterBufs b = bufs(h, par);
         if (k1_tma_maps(h->g, b, &h->maps[par]) != 0) rc = GSSTV_ERR_CUDA;
     }
-    if (rc == GSSTV_OK) rc = upload_scalars(h, initial_scalars(h->p));
+    if (rc == GSSTV_OK) rc = upload_scalars(h, initial_scalars(h->p, h->k1_variant == 1));
     if (rc != GSSTV_OK) {
         free_all(h);
         delete h;
@@ -490,7 +492,7 @@ int gsstv_reset_state(gsstv_handle* h) {
     }
     TRY(map_launch(launch_pitched_to_storage(h->p.storage, h->v, h->u[0], h->g, h->st)));
     h->parity = 0;
-    return upload_scalars(h, initial_scalars(h->p));
+    return upload_scalars(h, initial_scalars(h->p, h->k1_variant == 1));
 }
 
 int gsstv_iterate(gsstv_handle* h, int n, int* iters_done) {
@@ -618,7 +620,7 @@ int gsstv_set_state(gsstv_handle* h, const gsstv_state_view* v) {
     TRY(map_launch(launch_pack(sto, v->y3, h->y3[par], h->g, 1, h->st)));
     TRY(map_launch(launch_pack(sto, v->y4, h->q[par], h->g, 1, h->st)));
     // y4 is now stored unscaled (c = 0); the threshold search starts afresh
-    return upload_scalars(h, initial_scalars(h->p));
+    return upload_scalars(h, initial_scalars(h->p, h->k1_variant == 1));
 }
 
 int gsstv_autotune(gsstv_handle* h, int passes, int* chunk_out) {
@@ -1365,7 +1367,7 @@ int slabs_read_scalars(gsstv_slabs* G, Scal* out) {
 }
 
 int slabs_upload_scalars(gsstv_slabs* G) {
-    Scal s = initial_scalars(G->p);
+    Scal s = initial_scalars(G->p, 0);
     TRY(cuda_rc(cudaMemcpyAsync(G->sc, &s, sizeof(Scal), cudaMemcpyHostToDevice, G->st)));
     return cuda_rc(cudaStreamSynchronize(G->st));
 }

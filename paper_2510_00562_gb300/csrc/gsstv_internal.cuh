@@ -137,6 +137,11 @@ struct L1Ctl {
     unsigned hbase;
     int hist_left;
     long long hits, exact_runs, retry_hits;
+    // deferred placement of the next window (l1_record_tau): what it was
+    // recorded with, and the threshold of the last placement
+    int defer, pend, rec_hit, rec_hist;
+    double rec_m, rec_w, tau_last;
+    int have_last, pad;
 };
 
 struct L1Acc {
@@ -271,6 +276,11 @@ __device__ __forceinline__ double key_value(unsigned key) { return (double)__uin
 __device__ __forceinline__ double key_ulp(unsigned key) {
     const unsigned e = (key >> 23) & 0xffu;
     return __longlong_as_double((long long)((e == 0u ? 1u : e) + 873u) << 52);
+}
+// and its reciprocal (exact)
+__device__ __forceinline__ double key_ulp_inv(unsigned key) {
+    const unsigned e = (key >> 23) & 0xffu;
+    return __longlong_as_double((long long)(1173u - (e == 0u ? 1u : e)) << 52);
 }
 
 // Sums over the CTA carried as unevaluated float pairs (hi + lo, Knuth's

@@ -230,7 +230,7 @@ static __device__ int l1_narrow(const float* cand, bool cand_shared, unsigned m,
         {
             const int tid = (int)threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = ((int)blockDim.x + 31) >> 5;
             if (tid == 0) {
-                const double q = ceil(-(s_hi - r) / u0);
+                const double q = ceil(-(s_hi - r) * key_ulp_inv(k0));    // (u0 a power of two)
                 const bool ok = fabs(q) < 4.6e18 && n_hi >= 0.0 && n_hi < 9.0e15;
                 nr_int = ok ? 1 : 0;
                 nr_T = ok ? (long long)q : 0;
@@ -711,14 +711,14 @@ static __device__ int l1_hist_bracket(const unsigned* hist_g, unsigned hbase, do
 // (kCandTargetWide while the histogram is on) candidates are expected (density
 // measured at the last window).  `hit`: tau came from K1's window.  Thread 0
 // only.
-static __device__ void l1_record_tau(L1Ctl& c, double tau_new, double m_used, double width_used, bool hit) {
+static __device__ void l1_place_window(L1Ctl& c, double tau_new, double m_used, double width_used, bool hit,
+                                       bool hist_on) {
     c.tau_prev2 = c.tau_prev;
     c.have_prev2 = c.have_prev;
-    c.tau_prev = c.tau;
-    c.have_prev = c.have_tau;
-    c.tau = tau_new;
-    c.have_tau = 1;
-    c.need = NEED_NONE;
+    c.tau_prev = c.tau_last;
+    c.have_prev = c.have_last;
+    c.tau_last = tau_new;
+    c.have_last = 1;
     if (width_used > 0.0 && m_used > 0.0) c.dens = m_used / width_used;
     if (!(tau_new > 0.0)) {            // ball inactive: window (0, 0]
         c.theta_lo = 0.f;
@@ -732,7 +732,7 @@ static __device__ void l1_record_tau(L1Ctl& c, double tau_new, double m_used, do
     double hw;
     if (!trend) {
         hw = 1e-3 * tau_new;
-    } else if (c.hist_left > 0 && c.have_prev2 && c.tau_prev2 > 0.0) {
+    } else if (hist_on && c.have_prev2 && c.tau_prev2 > 0.0) {
         // the passes after a miss, while the thresholds move fast: the window
         // spans the linear and the quadratic extrapolations (tau + d1 and
         // tau + 2 d1 - d0) with a margin of half their distance and a tenth
@@ -749,7 +749,7 @@ static __device__ void l1_record_tau(L1Ctl& c, double tau_new, double m_used, do
     // a wide window while the thresholds move fast (the passes after a miss,
     // with K1's histogram on), where a hit saves a retry pass; else a narrow
     // one, which K1 and the finish handle faster
-    if (c.dens > 0.0) hw = fmin(hw, 0.5 * (c.hist_left > 0 ? kCandTargetWide : kCandTarget) / c.dens);
+    if (c.dens > 0.0) hw = fmin(hw, 0.5 * (hist_on ? kCandTargetWide : kCandTarget) / c.dens);
     // the histogram of the next pass: four octaves from a quarter of the
     // predicted threshold
     c.hbase = center > 0.0 ? (__float_as_uint(__double2float_rd(0.25 * center)) >> kHistShift) : 0u;
@@ -758,6 +758,24 @@ static __device__ void l1_record_tau(L1Ctl& c, double tau_new, double m_used, do
     c.theta_lo = __double2float_rd(lo);
     c.theta_hi = __double2float_ru(hi);
     c.window_ok = 1;
+}
+
+// A threshold found: K2 may run.  Where K2 places the next window (defer), the
+// placement waits for it; else it is done here.  Thread 0 only.
+static __device__ void l1_record_tau(L1Ctl& c, double tau_new, double m_used, double width_used, bool hit) {
+    const int hist_on = c.hist_left > 0;
+    c.tau = tau_new;
+    c.have_tau = 1;
+    c.need = NEED_NONE;
+    if (c.defer) {
+        c.rec_m = m_used;
+        c.rec_w = width_used;
+        c.rec_hit = hit;
+        c.rec_hist = hist_on;
+        c.pend = 1;
+    } else {
+        l1_place_window(c, tau_new, m_used, width_used, hit, hist_on);
+    }
 }
 
 // Radix level geometry: bin of a key and its residue (the bits below the bin).

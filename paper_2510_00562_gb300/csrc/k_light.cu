@@ -90,6 +90,7 @@ struct K2Args {
     Scal* sc;
     double* part;       // 3 doubles per CTA
     SlabPart sp;        // the bands updated, and this launch's CTAs among the stage's
+    int windows;        // 1: the first CTA places the next windows
 };
 
 // A thread's part of the three norms |q|^2, |u+ - u|^2, |u|^2.
@@ -263,9 +264,25 @@ __device__ __forceinline__ void k2_rows(const K2Args<float>& a, const int bid, c
 
 // The CTA `bid` of `nblk` that share one cube's K2 (a launch of its own, or
 // the cube's share of a batch launch).
+// The next windows of the threshold search, placed beside K2 by a CTA of its own
+// (one warp per vector): K1 needs them, K2 does not, and in the search launch
+// they stood 5 us in K2's way (code that runs once, in FP64).
+__device__ __forceinline__ void k2_windows(Scal* sc) {
+    if ((threadIdx.x & 31) || threadIdx.x >= 64) return;
+    L1Ctl& c = sc->ctl[threadIdx.x >> 5];
+    if (!c.pend) return;
+    c.pend = 0;
+    l1_place_window(c, c.tau, c.rec_m, c.rec_w, c.rec_hit != 0, c.rec_hist != 0);
+}
+
+// (CTA -1, where the launch has one, places the next windows)
 template <typename T>
 __device__ __forceinline__ void k2_body(const K2Args<T>& a, const int bid, const int nblk) {
     constexpr int NW = NT / 32;
+    if (bid < 0) {
+        k2_windows(a.sc);
+        return;
+    }
     __shared__ double red_d[64];
     __shared__ int is_last;
     const IterParams& P = a.p;
@@ -369,7 +386,7 @@ __device__ __forceinline__ void k2_body(const K2Args<T>& a, const int bid, const
 
 template <typename T>
 __global__ void __launch_bounds__(NT, 3) k2_light(const K2Args<T> a) {
-    k2_body(a, blockIdx.x, gridDim.x);
+    k2_body(a, (int)blockIdx.x - a.windows, (int)gridDim.x - a.windows);
 }
 
 // ---------------------------------------------------------------------------
@@ -709,57 +726,143 @@ __global__ void __launch_bounds__(NT) k_window(const Src src, const SearchArgs a
 constexpr int kFinishThreads = 1024;
 constexpr unsigned kFinishStage = 32768;
 
+// tau inside the window (lo, hi] of m values by one warp: 0 found, 1 below, 2
+// above (as l1_window_finish).  Newton's steps on phi from the window's middle,
+// where the window was predicted around: from the right of the root a step lands
+// left of it, from there they do not pass it, and a repeated count means the
+// active set is the root's.
+__device__ __forceinline__ int warp_window(const float* x, unsigned m, double n_hi, double s_hi, float lo, float hi,
+                                           double r, double* tau_out) {
+    const unsigned lane = threadIdx.x & 31u;
+    if (s_hi - n_hi * (double)hi - r > 0.0) return 2;
+    float tf = -INFINITY;                                 // first the sum of all values: phi at lo
+    unsigned prev = 0xffffffffu;
+    double tau = 0.0;
+#pragma unroll 1
+    for (int it = 0; it < 200; ++it) {
+        Kahan k;
+        unsigned c = 0;
+#pragma unroll 1
+        for (unsigned e = lane; e < m; e += 32u) {
+            const float y = x[e];
+            const bool in = y > tf;
+            k.add(in ? y : 0.f);
+            c += in ? 1u : 0u;
+        }
+        c = __reduce_add_sync(0xffffffffu, c);
+        float h = k.s, l = -k.c;
+#pragma unroll 1
+        for (int o = 16; o > 0; o >>= 1) {
+            const float oh = __shfl_xor_sync(0xffffffffu, h, o), ol = __shfl_xor_sync(0xffffffffu, l, o);
+            pair_add(h, l, oh, ol);
+        }
+        const double num = s_hi + ((double)h + (double)l) - r, den = n_hi + (double)c;
+        if (it == 0) {
+            if (num - den * (double)lo < 0.0) {           // phi(lo) < 0: inside the ball, or a miss below
+                *tau_out = 0.0;
+                return lo <= 0.f ? 0 : 1;
+            }
+            tf = 0.5f * (lo + hi);
+        } else {
+            tau = num / den;
+            tf = __double2float_rd(tau);
+            if (c == prev) break;
+            prev = c;
+        }
+    }
+    *tau_out = tau;
+    return 0;
+}
+
 // K1's window of vector v, after the fused pass: the CTAs' counts and sums
 // above the window summed, tau found on the candidates (l1_window_finish); on
 // a miss, K1's sampled histogram (when it was on) brackets tau for one retry
 // pass, else the next window is placed from the bounds the miss gives or the
 // radix passes run.  The whole block; K1's partials: pn / ps, four per CTA.
-__device__ __noinline__ void k1_window_finish(const SearchArgs& a, const unsigned long long* pn, const double* ps,
+__device__ __noinline__ int k1_window_finish(const SearchArgs& a, const unsigned long long* pn, const double* ps,
                                               int parts, const int v, float* fstage, unsigned* scr, double* red_d,
                                               unsigned long long* red_u) {
     __shared__ int sh_flag;
+    __shared__ int sh_rc;
     L1Ctl& C = a.sc->ctl[v];
-    const double r = a.sc->radius[v];
-    if (!(r > 0.0)) {
+    // everything the finish starts from in one round of loads: the scalars, the
+    // first candidates, and in warp 0 K1's partials (one per SM; one warp, so
+    // that the FP64 additions, scarce on this part, are not issued by every warp)
+    const double r = __ldcg(&a.sc->radius[v]);
+    const int win = __ldcg(&a.sc->k1_win[v]), hist_w = __ldcg(&a.sc->k1_hist[v]), hist_left = __ldcg(&C.hist_left);
+    const unsigned m = __ldcg(&a.sc->acc[v].m), nbin = a.w.nh ? __ldcg(a.w.nbinned + v) : 0u;
+    const float tlo_f = __ldcg(&C.theta_lo), thi_f = __ldcg(&C.theta_hi);
+    const float x0 = __ldcg(a.w.cand[v] + threadIdx.x);          // (the list holds kCandCap floats)
+    unsigned n = 0;                                              // (fewer than 2^32 voxels)
+    double s = 0.0;
+    if (threadIdx.x < 32) {
+#pragma unroll 5
+        for (int k = threadIdx.x; k < parts; k += 32) {
+            n += (unsigned)__ldcg(pn + 4 * k + v);
+            s += __ldcg(ps + 4 * k + v);
+        }
+    }
+    fstage[threadIdx.x] = x0;
+    if (!(__double_as_longlong(r) > 0)) {
         if (threadIdx.x == 0) {
             C.tau = __int_as_float(0x7f800000);
             C.have_tau = 1;
             C.need = NEED_NONE;
             C.window_ok = 0;
         }
-        return;
+        return NEED_NONE;
     }
-    if (!__ldcg(&a.sc->k1_win[v])) {
+    if (!win) {
         if (threadIdx.x == 0) {
             C.need = NEED_RADIX0; C.prefix = 0; C.n_above = 0; C.s_above = 0.0; C.exact_runs++;
         }
-        return;
+        return NEED_RADIX0;
     }
-    const bool hist_v = __ldcg(&a.sc->k1_hist[v]) != 0;
-    // the CTAs' partials (one per SM): one warp, so that the FP64 additions
-    // (scarce on this part) are not issued by every warp of the block
+    const bool hist_v = hist_w != 0;
+    __syncthreads();
     if (threadIdx.x < 32) {
-        unsigned long long n = 0;
-        double s = 0.0;
-#pragma unroll 4
-        for (int k = threadIdx.x; k < parts; k += 32) {
-            n += __ldcg(pn + 4 * k + v);
-            s += __ldcg(ps + 4 * k + v);
+        n = __reduce_add_sync(0xffffffffu, n);
+#pragma unroll 1
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        // A window of few values (the steady state): warp 0 finds tau alone.
+        // This launch runs its code once, so the instruction fetches are what
+        // it waits for (the same steps took 21 us after passes that stay in L2
+        // and 34 us after larger ones): short loops over all the values beat the
+        // narrowing by the list's histogram up to here.
+        double tau = 0.0;
+        const int rc = m > (unsigned)kFinishThreads ? -1 : warp_window(fstage, m, (double)n, s, tlo_f, thi_f, r, &tau);
+        if (threadIdx.x == 0) {
+            sh_rc = rc;
+            red_d[0] = s;
+            red_u[0] = n;
+            if (rc == 0) {
+                l1_record_tau(C, tau, (double)m, (double)thi_f - (double)tlo_f, true);
+                atomicAdd(reinterpret_cast<unsigned long long*>(&C.hits), 1ull);
+                // (counted down where K1 keeps the histogram: float32 storage)
+                if (hist_left > 0 && win == 1) C.hist_left = hist_left - 1;
+                a.sc->acc[v].m = 0;
+            }
         }
-        n = warp_sum(n);
-        s = warp_sum(s);
-        if (threadIdx.x == 0) { red_u[0] = n; red_d[0] = s; }
     }
     __syncthreads();
-    const unsigned long long n = red_u[0];
-    const double s = red_d[0];
+    if (sh_rc == 0) {
+        if (nbin) {
+            uint4* h4 = reinterpret_cast<uint4*>(a.w.nh + v * 3 * kNarrowBins);
+            for (int k = threadIdx.x; k < 2 * kNarrowBins / 4; k += kFinishThreads) h4[k] = make_uint4(0u, 0u, 0u, 0u);
+            if (threadIdx.x == 0) a.w.nbinned[v] = 0u;
+        }
+        if (hist_v) a.w.khist[v * kK1Bins + threadIdx.x] = 0u;
+        return NEED_NONE;
+    }
+    n = (unsigned)red_u[0];
+    s = red_d[0];
     __syncthreads();
-    const unsigned m = __ldcg(&a.sc->acc[v].m);
-    const double tlo = C.theta_lo, thi = C.theta_hi;
+    const double tlo = tlo_f, thi = thi_f;
     double tau = 0.0;
     WinInfo wi;
     const int miss = l1_window_finish((double)n, s, a.w.cand[v], m, tlo, thi, r, &tau, red_d, red_u, &wi, fstage,
-                                      kFinishStage, scr, narrow_pre(a.w, v, m), a.w.nbinned + v);
+                                      kFinishStage, scr, m > 0u && nbin == m ? a.w.nh + v * 3 * kNarrowBins : nullptr,
+                                      a.w.nbinned + v);
     narrow_clear(a.w, v);
     int hist_hit = 0;
     float h_lo = 0.f, h_hi = 0.f;
@@ -784,8 +887,7 @@ __device__ __noinline__ void k1_window_finish(const SearchArgs& a, const unsigne
         if (!miss) {
             l1_record_tau(C, tau, (double)min(m, kCandCap), thi - tlo, true);
             C.hits++;
-            // (counted down where K1 keeps the histogram: float32 storage)
-            if (C.hist_left > 0 && __ldcg(&a.sc->k1_win[v]) == 1) C.hist_left--;
+            if (hist_left > 0 && win == 1) C.hist_left = hist_left - 1;
         } else if (hist_hit) {
             C.prefix = 0; C.n_above = 0; C.s_above = 0.0;
             C.need = NEED_WINDOW;
@@ -798,24 +900,22 @@ __device__ __noinline__ void k1_window_finish(const SearchArgs& a, const unsigne
         a.sc->acc[v].m = 0;
     }
     __syncthreads();
+    return -1;
 }
 
 constexpr size_t kFinishSmem = kFinishStage * sizeof(float) + 3 * kNarrowBins * sizeof(unsigned);
-__device__ __forceinline__ void finish_body(const SearchArgs& a, int mode, const unsigned long long* pn,
+__device__ __forceinline__ int finish_body(const SearchArgs& a, int mode, const unsigned long long* pn,
                                             const double* ps, int parts, const int v) {
     extern __shared__ __align__(16) float fstage[];         // kFinishStage floats + the narrowing scratch
     __shared__ double red_d[64];
     __shared__ unsigned long long red_u[64];
     const int want = mode == 0 ? NEED_WINDOW : NEED_GATHER;
     unsigned* scr = reinterpret_cast<unsigned*>(fstage + kFinishStage);
-    if (v >= a.nvec) return;
-    if (mode == 2) {
-        k1_window_finish(a, pn, ps, parts, v, fstage, scr, red_d, red_u);
-        return;
-    }
+    if (v >= a.nvec) return -1;
+    if (mode == 2) return k1_window_finish(a, pn, ps, parts, v, fstage, scr, red_d, red_u);
     {
         L1Ctl& C = a.sc->ctl[v];
-        if (C.need != want) return;                         // uniform over the CTA
+        if (C.need != want) return -1;                      // uniform over the CTA
         const double r = a.sc->radius[v];
         const unsigned m = __ldcg(&a.sc->acc[v].m);
         const double lo = C.g_lo, hi = C.g_hi;
@@ -860,9 +960,9 @@ __device__ __forceinline__ void finish_body(const SearchArgs& a, int mode, const
         }
         __syncthreads();
     }
+    return -1;
 }
 
-// one CTA per vector
 // After K1's window finish (mode 2) in a graph: the last of the launch's
 // CTAs opens the conditional node of the search launches when a cube still
 // needs a search (one thread, so that no two calls race).  need_any() reads the
@@ -948,31 +1048,43 @@ __device__ __forceinline__ void search_body(const Src& src, const SearchArgs& a,
                                             const SearchShape& h, const int bid) {
     __shared__ int sh_stage, sh_item, sh_last;
     SearchSync* y = &a.sc->search;
+    auto publish = [&](int next) {                       // (thread 0)
+        __threadfence();
+        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&y->stage), "r"((unsigned)next) : "memory");
+    };
     // whole block: an item of stage st is done; the last of n publishes the next stage
     auto complete = [&](int st, int n) {
         __syncthreads();
         if (threadIdx.x == 0) {
             __threadfence();
             sh_last = atomicAdd(&y->done[st], 1u) == (unsigned)(n - 1);
+            __threadfence();
         }
         __syncthreads();
         if (!sh_last) return;
-        __threadfence();
         if (st >= ST_RADIX0 && st <= ST_RADIX2) {
+            __threadfence();
             radix_finish(a, st - ST_RADIX0);
             __threadfence();
             __syncthreads();
         }
-        if (threadIdx.x == 0) {
-            const unsigned next = (unsigned)search_next(a, st);
-            if (st == ST_FINISH && next != ST_EXIT && h.count) a.sc->gate_opens++;
-            __threadfence();
-            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&y->stage), "r"(next) : "memory");
-        }
+        if (threadIdx.x == 0) publish(search_next(a, st));
     };
     if (bid < a.nvec) {
-        finish_body(a, 2, pn, ps, h.parts, bid);
-        complete(ST_FINISH, a.nvec);
+        // the finishes' count carries in its upper half whether a vector still
+        // needs a search, so that the usual pass reads nothing back
+        const bool need = finish_body(a, 2, pn, ps, h.parts, bid) != NEED_NONE;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            const unsigned was = atomicAdd(&y->done[ST_FINISH], need ? 0x10001u : 1u);
+            if ((was & 0xffffu) == (unsigned)(a.nvec - 1)) {
+                __threadfence();
+                const int next = need || (was >> 16) ? search_next(a, ST_FINISH) : (int)ST_EXIT;
+                if (next != ST_EXIT && h.count) a.sc->gate_opens++;
+                publish(next);
+            }
+        }
     }
     for (int st = ST_FINISH;;) {
         if (threadIdx.x == 0) {
@@ -1101,8 +1213,9 @@ long long part_voxels(const Geom& g, const SlabPart& sp) {
     return (long long)(sp.o1 - sp.o0) * g.n1 * g.n2;
 }
 
-// CTAs of K2 that fit the GPU at once (its launch bounds)
-int k2_resident() { return 3 * device_sms(); }
+// CTAs of K2 that fit the GPU at once (its launch bounds), beside the one that
+// places the windows
+int k2_resident() { return 3 * device_sms() - 1; }
 
 int k2_grid_part(int storage, const Geom& g, const SlabPart& sp) {
     const long long nb = sp.o1 - sp.o0;
@@ -1131,8 +1244,9 @@ int launch_k2_t(const Geom& g, const IterBufs& b, const IterParams& p, Scal* sc,
     a.sc = sc;
     a.part = part;
     a.sp = sp;
+    a.windows = sp.cta_total == 0 ? 1 : 0;                 // (a slab's windows are placed by the finish)
     const int ctas = std::min(k2_grid_part(std::is_same<T, float>::value ? 0 : 1, g, sp), part_cap);
-    k2_light<T><<<ctas, NT, 0, st>>>(a);
+    k2_light<T><<<ctas + a.windows, NT, 0, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -1286,7 +1400,7 @@ __global__ void __launch_bounds__(NT, 3) k2_batch(const __grid_constant__ K2Batc
     // loaded once instead of at each use
     const K2Args<float> a = t.c[c];
     if (__ldcg(&a.sc->done)) return;
-    k2_body(a, blockIdx.x - t.start[c], t.start[c + 1] - t.start[c]);
+    k2_body(a, (int)blockIdx.x - t.start[c] - 1, t.start[c + 1] - t.start[c] - 1);
 }
 
 }  // namespace
@@ -1483,7 +1597,8 @@ int launch_k2_batch(const BatchCube* cubes, int n, cudaStream_t st) {
         a.sp = whole_cube(q.g);
         t.start[c] = total;
         const int share = (int)std::ceil(k2_resident() * ((double)q.g.cube / all));
-        total += std::max(1, std::min({share, k2_grid_part(0, q.g, a.sp), q.k2_cap}));
+        a.windows = 1;
+        total += std::max(1, std::min({share, k2_grid_part(0, q.g, a.sp), q.k2_cap})) + 1;
     }
     t.start[n] = total;
     k2_batch<<<total, NT, 0, st>>>(t);
