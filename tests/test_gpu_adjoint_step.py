@@ -1,0 +1,46 @@
+"""The single transposed pass (gsstv_vjp_step) against the FP64 reverse mode at
+the edges of its tiles (32 x 16, runs of bands), in place and not.  Tolerance as
+for one pass elsewhere: float32 arithmetic on float32 inputs, a few roundings of
+6e-8 per term amplified by the stencil sums: 1e-5 relative."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import adjoint as A
+from oracle import ppds as o
+from paper_2510_00562_gb300 import synth
+from paper_2510_00562_gb300.solver import GRAD_PARAMS, STATE_KEYS, GeoSSTVSolver, make_params
+
+pytestmark = pytest.mark.gpu
+
+
+def rel(a, b):
+    return np.linalg.norm(a - b) / np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("shape", [(16, 32, 2), (17, 33, 5), (15, 31, 3), (48, 65, 4), (33, 1, 2)])
+def test_one_pass_at_tile_edges(shape, in_place):
+    n1, n2, n3 = shape
+    rs = synth.random_state(n1, n2, n3, seed=n2, scale=0.1)
+    rng = np.random.default_rng(5)
+    v = rng.uniform(0, 1, (n3, n1, n2)).astype(np.float32)
+    kw = dict(eps=0.02 * v.size ** 0.5, alpha=0.4 * np.abs(rs["s"]).sum(dtype=np.float64),
+              beta=0.4 * np.abs(rs["t"]).sum(dtype=np.float64), omega=0.05)
+    bn = {k: rng.standard_normal(rs[k].shape).astype(np.float32) for k in STATE_KEYS}
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(x, dtype=np.float32)).cuda()  # noqa: E731
+    with GeoSSTVSolver(n1, n2, n3, make_params(graph_iters=0, **kw)) as sol:
+        sol.load(dev(v))
+        x = {k: dev(rs[k]) for k in STATE_KEYS}
+        sol.set_state(x)
+        sol.iterate(1)
+        bar, vbar, pbar = sol.vjp_step(x, sol.get_state(), {k: dev(bn[k]) for k in STATE_KEYS}, in_place=in_place)
+        got = {k: t.cpu().numpy().astype(np.float64) for k, t in bar.items()}
+        vbar = vbar.cpu().numpy().astype(np.float64)
+    ref, vref, pref = A.step_vjp(o.State(**{k: rs[k].astype(np.float64) for k in STATE_KEYS}), v.astype(np.float64),
+                                 o.Params(**kw), o.State(**{k: bn[k].astype(np.float64) for k in STATE_KEYS}))
+    for k in STATE_KEYS:
+        assert rel(got[k], getattr(ref, k)) < 1e-5, k
+    assert rel(vbar, vref) < 1e-5
+    for k in GRAD_PARAMS:
+        assert pbar[k] == pytest.approx(pref[k], rel=1e-5, abs=1e-9 * np.linalg.norm(vref)), k
