@@ -341,7 +341,7 @@ static __device__ int l1_window_finish(double n_hi, double s_hi, const float* ca
     if (threadIdx.x == 0) {
         const double phi_hi = s_hi - n_hi * theta_hi - r;
         if (info) info->phi_hi = phi_hi;
-        wp_rc = m_raw > kCandCap ? 1 : phi_hi > 0.0 ? 2 : -1;     // 2: root above the window
+        wp_rc = m_raw > kCandCap ? 1 : !(phi_hi <= 0.0) ? 2 : -1;     // 2: root above the window (or no number)
         // the window's ends as float keys: (klo, khi] holds every candidate
         unsigned klo = __float_as_uint((float)theta_lo), khi = __float_as_uint((float)theta_hi);
         if ((double)__uint_as_float(klo) > theta_lo) klo -= 1u;        // rounding of the ends

@@ -454,10 +454,46 @@ struct FlatSrc {
     long long n;
     template <typename F>
     __device__ void visit(const unsigned first, const unsigned stride, F&& f, bool, bool) const {
-        for (long long base = first; base < n; base += stride) {
+        long long done = 0;
+        if (!(reinterpret_cast<unsigned long long>(x) & 15ull)) {
+            // four values per thread and two loads in flight
+            const float4* x4 = reinterpret_cast<const float4*>(x);
+            const long long quads = n >> 2;
+            done = quads << 2;
+            const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+            const bool mine = first + threadIdx.x < stride;
+            for (long long base = first; base < quads; base += 2ll * stride) {
+                const long long l0 = base + threadIdx.x, l1 = l0 + stride;
+                const bool v0 = mine && l0 < quads, v1 = mine && l1 < quads;
+                const float4 q0 = v0 ? __ldg(x4 + l0) : zero, q1 = v1 ? __ldg(x4 + l1) : zero;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) f(v0, fabsf(comp(q0, k)), 0.f);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) f(v1, fabsf(comp(q1, k)), 0.f);
+            }
+        }
+        for (long long base = done + first; base < n; base += stride) {
             const long long l = base + threadIdx.x;
-            const bool valid = l < n;
+            const bool valid = first + threadIdx.x < stride && l < n;
             f(valid, valid ? fabsf(x[l]) : 0.f, 0.f);
+        }
+    }
+};
+
+// One value in 32 of a flat vector: of every whole block of 1024 a run of 32,
+// its place hashed (a fixed stride could fall in step with the data).
+struct SampleSrc {
+    using Storage = float;
+    const float* x;
+    long long n;            // sampled values, a multiple of 32
+    template <typename F>
+    __device__ void visit(const unsigned first, const unsigned stride, F&& f, bool, bool) const {
+        for (long long base = first; base < n; base += stride) {
+            const long long e = base + threadIdx.x;
+            const bool valid = first + threadIdx.x < stride && e < n;
+            const unsigned run = ((unsigned)(e >> 5) * 2654435761u) >> 27;
+            const long long l = ((e >> 5) << 10) + 32u * run + (e & 31);
+            f(valid, valid ? fabsf(__ldg(x + l)) : 0.f, 0.f);
         }
     }
 };
@@ -683,7 +719,9 @@ __device__ __forceinline__ void window_body(const Src& src, const SearchArgs& a,
     if (need[1]) bc.keep_hist(a.w, 1, lo1, hi1);
     src.visit(bid * blockDim.x, stride, [&](bool valid, float x0, float x1) {
         if (need[0]) {
-            const bool hi = valid && x0 > hi0;
+            // (a flat vector's NaN counts as above, so that the window misses and
+            // the radix passes decide)
+            const bool hi = valid && (std::is_same<Src, FlatSrc>::value ? !(x0 <= hi0) : x0 > hi0);
             if (hi) { w0.n++; w0.s.add(x0); }
             bc.append(0, valid && !hi && x0 > lo0, x0, a.w.cand[0], &a.sc->acc[0].m);
         }
@@ -774,6 +812,80 @@ __device__ __forceinline__ int warp_window(const float* x, unsigned m, double n_
     return 0;
 }
 
+// The same by the whole block for at most kBlockWindow values of the list, held in
+// registers (157x203x61: a pass 139 -> 131 us; the narrowing took about 34 us a
+// finish).
+constexpr int kBlockPer = 8;
+constexpr unsigned kBlockWindow = 1024 * kBlockPer;
+__device__ __forceinline__ int block_window(const float* cand, unsigned m, double n_hi, double s_hi, float lo, float hi,
+                                            double r, double* tau_out) {
+    __shared__ float2 part[32];
+    __shared__ unsigned cnt[32];
+    __shared__ float sh_tf;
+    __shared__ int sh_state;                              // 0 go on, 1 found, 2 inside the ball, 3 below, 4 above
+    __shared__ double sh_tau;
+    const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    float x[kBlockPer];
+#pragma unroll
+    for (int k = 0; k < kBlockPer; ++k) {
+        const unsigned e = threadIdx.x + (unsigned)k * blockDim.x;
+        x[k] = e < m ? __ldcg(cand + e) : -INFINITY;      // (never above a threshold)
+    }
+    float tf = -INFINITY;
+    unsigned prev = 0xffffffffu;
+#pragma unroll 1
+    for (int it = 0; it < 200; ++it) {
+        Kahan k;
+        unsigned c = 0;
+#pragma unroll
+        for (int e = 0; e < kBlockPer; ++e) {
+            const bool in = x[e] > tf;
+            k.add(in ? x[e] : 0.f);
+            c += in ? 1u : 0u;
+        }
+        c = __reduce_add_sync(0xffffffffu, c);
+        float h = k.s, l = -k.c;
+#pragma unroll 1
+        for (int o = 16; o > 0; o >>= 1) {
+            const float oh = __shfl_xor_sync(0xffffffffu, h, o), ol = __shfl_xor_sync(0xffffffffu, l, o);
+            pair_add(h, l, oh, ol);
+        }
+        if (lane == 0) { part[wid] = make_float2(h, l); cnt[wid] = c; }
+        __syncthreads();
+        if (wid == 0) {
+            h = lane < nw ? part[lane].x : 0.f;
+            l = lane < nw ? part[lane].y : 0.f;
+            c = __reduce_add_sync(0xffffffffu, lane < nw ? cnt[lane] : 0u);
+#pragma unroll 1
+            for (int o = 16; o > 0; o >>= 1) {
+                const float oh = __shfl_xor_sync(0xffffffffu, h, o), ol = __shfl_xor_sync(0xffffffffu, l, o);
+                pair_add(h, l, oh, ol);
+            }
+            const double num = s_hi + ((double)h + (double)l) - r, den = n_hi + (double)c;
+            int state = 0;
+            double tau = 0.0;
+            if (it == 0) {
+                tf = 0.5f * (lo + hi);
+                if (s_hi - n_hi * (double)hi - r > 0.0) state = 4;
+                else if (num - den * (double)lo < 0.0) state = lo <= 0.f ? 2 : 3;
+            } else {
+                tau = num / den;
+                tf = __double2float_rd(tau);
+                if (c == prev) state = 1;
+                prev = c;
+            }
+            if (lane == 0) { sh_tf = tf; sh_state = state; sh_tau = tau; }
+        }
+        __syncthreads();
+        tf = sh_tf;
+        if (sh_state) break;
+        __syncthreads();
+    }
+    const int state = sh_state;
+    *tau_out = state == 2 ? 0.0 : sh_tau;
+    return state == 3 ? 1 : state == 4 ? 2 : 0;
+}
+
 // K1's window of vector v, after the fused pass: the CTAs' counts and sums
 // above the window summed, tau found on the candidates (l1_window_finish); on
 // a miss, K1's sampled histogram (when it was on) brackets tau for one retry
@@ -835,17 +947,25 @@ __device__ __noinline__ int k1_window_finish(const SearchArgs& a, const unsigned
             sh_rc = rc;
             red_d[0] = s;
             red_u[0] = n;
-            if (rc == 0) {
-                l1_record_tau(C, tau, (double)m, (double)thi_f - (double)tlo_f, true);
-                atomicAdd(reinterpret_cast<unsigned long long*>(&C.hits), 1ull);
-                // (counted down where K1 keeps the histogram: float32 storage)
-                if (hist_left > 0 && win == 1) C.hist_left = hist_left - 1;
-                a.sc->acc[v].m = 0;
-            }
+            red_d[1] = tau;
+            red_d[2] = (double)n;
         }
     }
     __syncthreads();
+    if (m > (unsigned)kFinishThreads && m <= kBlockWindow) {
+        double tau = 0.0;
+        const int rc = block_window(a.w.cand[v], m, red_d[2], red_d[0], tlo_f, thi_f, r, &tau);
+        if (threadIdx.x == 0) { sh_rc = rc; red_d[1] = tau; }
+        __syncthreads();
+    }
     if (sh_rc == 0) {
+        if (threadIdx.x == 0) {
+            l1_record_tau(C, red_d[1], (double)m, (double)thi_f - (double)tlo_f, true);
+            atomicAdd(reinterpret_cast<unsigned long long*>(&C.hits), 1ull);
+            // (counted down where K1 keeps the histogram: float32 storage)
+            if (hist_left > 0 && win == 1) C.hist_left = hist_left - 1;
+            a.sc->acc[v].m = 0;
+        }
         if (nbin) {
             uint4* h4 = reinterpret_cast<uint4*>(a.w.nh + v * 3 * kNarrowBins);
             for (int k = threadIdx.x; k < 2 * kNarrowBins / 4; k += kFinishThreads) h4[k] = make_uint4(0u, 0u, 0u, 0u);
@@ -1017,7 +1137,7 @@ enum { ST_FINISH = 0, ST_WINDOW, ST_WINDOW_END, ST_RADIX0, ST_RADIX1, ST_RADIX2,
 static_assert(ST_GATHER_END < kSearchStages, "counters per stage");
 
 struct SearchShape {
-    int parts;              // K1's partials
+    int parts;              // K1's partials (-1: no K1, the first stage is set already)
     unsigned win_threads;   // threads that share the retry pass (a multiple of 256)
     int win_items, pass_items;
     int count;              // count the passes that searched (graph launches)
@@ -1070,7 +1190,7 @@ __device__ __forceinline__ void search_body(const Src& src, const SearchArgs& a,
         }
         if (threadIdx.x == 0) publish(search_next(a, st));
     };
-    if (bid < a.nvec) {
+    if (h.parts >= 0 && bid < a.nvec) {
         // the finishes' count carries in its upper half whether a vector still
         // needs a search, so that the usual pass reads nothing back
         const bool need = finish_body(a, 2, pn, ps, h.parts, bid) != NEED_NONE;
@@ -1125,12 +1245,50 @@ __global__ void __launch_bounds__(kFinishThreads) k_search(const Src src, const 
     search_body(src, a, pn, ps, h, blockIdx.x);
 }
 
+// The standalone projection between its two searches: tau of the sample (1 / scale
+// of the values) places the window of one pass over all of them.  0.5 % about
+// tau is several standard deviations of the sample's for vectors this long; a
+// miss costs the radix passes.  A sample inside its ball says nothing about a
+// root near zero: the radix passes run at once.
+__global__ void k_flat_window(Scal* sc, double radius, double scale) {
+    if (threadIdx.x != 0) return;
+    L1Ctl& c = sc->ctl[0];
+    sc->radius[0] = radius;
+    sc->search = SearchSync();
+    sc->acc[0].m = 0u;
+    c.prefix = 0; c.n_above = 0; c.s_above = 0.0;
+    if (c.tau > 0.0 && isfinite(c.tau)) {
+        double hw = 0.005 * c.tau;
+        if (c.dens > 0.0) hw = fmin(hw, 0.25 * (double)kCandCap / (c.dens * scale));
+        c.g_lo = __double2float_rd(c.tau - hw);
+        c.g_hi = __double2float_ru(c.tau + hw);
+        c.need = NEED_WINDOW;
+        sc->search.stage = ST_WINDOW;
+    } else {
+        c.need = NEED_RADIX0;
+        sc->search.stage = ST_RADIX0;
+    }
+}
+
 // out = soft(x, tau) for the standalone projection
-__global__ void k_apply_flat(const float* x, float* out, long long n, const Scal* sc) {
+__global__ void __launch_bounds__(NT) k_apply_flat(const float* x, float* out, long long n, const Scal* sc) {
     const double tau = sc->ctl[0].tau;
     const float tf = (float)tau;
-    for (long long l = blockIdx.x * (long long)NT + threadIdx.x; l < n; l += (long long)gridDim.x * NT)
-        out[l] = tau > 0.0 ? soft(x[l], tf) : x[l];
+    const bool on = tau > 0.0;
+    long long done = 0;
+    if (!((reinterpret_cast<unsigned long long>(x) | reinterpret_cast<unsigned long long>(out)) & 15ull)) {
+        const float4* x4 = reinterpret_cast<const float4*>(x);
+        float4* o4 = reinterpret_cast<float4*>(out);
+        const long long quads = n >> 2;
+        done = quads << 2;
+        for (long long l = blockIdx.x * (long long)NT + threadIdx.x; l < quads; l += (long long)gridDim.x * NT) {
+            float4 q = x4[l];
+            if (on) q = make_float4(soft(q.x, tf), soft(q.y, tf), soft(q.z, tf), soft(q.w, tf));
+            o4[l] = q;
+        }
+    }
+    for (long long l = done + blockIdx.x * (long long)NT + threadIdx.x; l < n; l += (long long)gridDim.x * NT)
+        out[l] = on ? soft(x[l], tf) : x[l];
 }
 
 // ---------------------------------------------------------------------------
@@ -1699,50 +1857,79 @@ int launch_scale_unpack(int storage, const void* q, const double* c, float* dst,
 // ---------------------------------------------------------------------------
 // standalone projection of a flat device vector onto an l1 ball
 // ---------------------------------------------------------------------------
+// Vectors from this length on are searched by a sample and one pass.
+constexpr long long kSampleFrom = 1ll << 21;
+
+// One allocation holds the scratch.  A short vector is searched by the radix
+// stages of one launch; a long one by those stages on a sample of 1/32, which
+// place the window of one pass over all values (58.7 M values: a call with three
+// radix passes and a gather over all of them took 1290 us, now 544: sample 89,
+// pass 168, output 66 us; 4096 values in seven launches and four allocations 357
+// us, now 260).
 int l1_project_standalone(const float* x, long long n, double radius, float* out, double* tau,
                           cudaStream_t st) {
-    if (light_configure(0) != 0) return -3;
-    Scal* sc = nullptr;
+    const bool sampled = n >= kSampleFrom && radius > 0.0;
+    if (cudaFuncSetAttribute(k_search<FlatSrc>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFinishSmem) != cudaSuccess ||
+        cudaFuncSetAttribute(k_search<SampleSrc>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFinishSmem) != cudaSuccess)
+        return -3;
+    const size_t parts = 4 * (size_t)device_sms(), b_hist = 2 * kHistBins * sizeof(unsigned long long);
+    // (a gathered bracket holds at most kGatherMax values, a window kCandCap)
+    const size_t b_cand = (sampled ? (size_t)kCandCap : (size_t)kGatherMax) * sizeof(float);
+    const size_t b_nh = 6 * kNarrowBins * sizeof(unsigned);
+    size_t off = 0;
+    auto take = [&](size_t b) { const size_t o = off; off += (b + 255) / 256 * 256; return o; };
+    const size_t o_sc = take(sizeof(Scal)), o_cnt = take(b_hist), o_res = take(b_hist), o_nh = take(b_nh),
+                 o_nb = take(2 * sizeof(unsigned)), o_zero = off, o_pn = take(parts * 8), o_ps = take(parts * 8),
+                 o_cand = take(b_cand);
+    char* mem = nullptr;
+    if (cudaMalloc(&mem, off) != cudaSuccess) {
+        cudaGetLastError();
+        return -2;
+    }
+    Scal* sc = reinterpret_cast<Scal*>(mem + o_sc);
     L1Work w{};
-    size_t bytes_hist = 2 * kHistBins * sizeof(unsigned long long);
+    w.hcnt = reinterpret_cast<unsigned long long*>(mem + o_cnt);
+    w.hres = reinterpret_cast<unsigned long long*>(mem + o_res);
+    w.nh = reinterpret_cast<unsigned*>(mem + o_nh);
+    w.nbinned = reinterpret_cast<unsigned*>(mem + o_nb);
+    w.cand[0] = w.cand[1] = reinterpret_cast<float*>(mem + o_cand);
+    unsigned long long* pn = reinterpret_cast<unsigned long long*>(mem + o_pn);
+    double* ps = reinterpret_cast<double*>(mem + o_ps);
+    const SearchArgs a{sc, w, 1};
+    auto search = [&](const auto& src, long long cnt) {
+        const int win = window_grid_n(cnt, 4 * device_sms());
+        const int ctas = (win * 256 + kFinishThreads - 1) / kFinishThreads;
+        k_search<<<ctas, kFinishThreads, kFinishSmem, st>>>(src, a, pn, ps, search_shape(cnt, win, -1, 0, ctas));
+    };
     int rc = 0;
-    if (cudaMalloc(&sc, sizeof(Scal)) != cudaSuccess) return -2;
-    if (cudaMalloc(&w.hcnt, bytes_hist) != cudaSuccess || cudaMalloc(&w.hres, bytes_hist) != cudaSuccess ||
-        cudaMalloc(&w.cand[0], kCandCap * sizeof(float)) != cudaSuccess) {
-        rc = -2;
+    Scal h{};
+    const long long ns = (n >> 10) << 5;
+    const double scale = sampled ? (double)n / (double)ns : 1.0;
+    h.radius[0] = radius / scale;
+    h.ctl[0].need = radius > 0.0 ? NEED_RADIX0 : NEED_NONE;
+    h.ctl[0].tau = radius > 0.0 ? 0.0 : (double)INFINITY;
+    h.search.stage = ST_RADIX0;
+    if (cudaMemsetAsync(mem, 0, o_zero, st) != cudaSuccess ||
+        cudaMemcpyAsync(sc, &h, sizeof(Scal), cudaMemcpyHostToDevice, st) != cudaSuccess)
+        rc = -3;
+    if (rc == 0) {
+        if (sampled) {
+            search(SampleSrc{x, ns}, ns);
+            k_flat_window<<<1, 32, 0, st>>>(sc, radius, scale);
+        }
+        if (radius > 0.0) search(FlatSrc{x, n}, n);
+        k_apply_flat<<<grid_for(n), NT, 0, st>>>(x, out, n, sc);
+        if (cudaGetLastError() != cudaSuccess) rc = -3;
     }
     if (rc == 0) {
-        w.cand[1] = w.cand[0];
-        Scal h{};
-        h.radius[0] = radius;
-        h.ctl[0].need = radius > 0.0 ? NEED_RADIX0 : NEED_NONE;
-        h.ctl[0].tau = radius > 0.0 ? 0.0 : (double)INFINITY;
-        if (cudaMemcpyAsync(sc, &h, sizeof(Scal), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-            cudaMemsetAsync(w.hcnt, 0, bytes_hist, st) != cudaSuccess ||
-            cudaMemsetAsync(w.hres, 0, bytes_hist, st) != cudaSuccess)
+        if (cudaMemcpyAsync(&h, sc, sizeof(Scal), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaStreamSynchronize(st) != cudaSuccess)
             rc = -3;
-        const FlatSrc src{x, n};
-        const SearchArgs a{sc, w, 1};
-        for (int level = 0; level < 3 && rc == 0; ++level) rc = launch_radix_src(src, n, a, level, st);
-        if (rc == 0) {
-            k_gather<FlatSrc><<<gather_grid_n(n), NT, 0, st>>>(src, a);
-            k_search_finish<<<1, kFinishThreads, kFinishSmem, st>>>(a, 1, nullptr, nullptr, 0, 0, 0);
-            k_apply_flat<<<grid_for(n), NT, 0, st>>>(x, out, n, sc);
-            if (cudaGetLastError() != cudaSuccess) rc = -3;
-        }
-        if (rc == 0) {
-            if (cudaMemcpyAsync(&h, sc, sizeof(Scal), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-                cudaStreamSynchronize(st) != cudaSuccess)
-                rc = -3;
-            else if (h.error) rc = -6;
-            else if (tau) *tau = h.ctl[0].tau;
-        }
+        else if (h.error) rc = -6;
+        else if (tau) *tau = h.ctl[0].tau;
     }
     cudaStreamSynchronize(st);
-    cudaFree(sc);
-    cudaFree(w.hcnt);
-    cudaFree(w.hres);
-    cudaFree(w.cand[0]);
+    cudaFree(mem);
     return rc;
 }
 
