@@ -603,9 +603,10 @@ __global__ void __launch_bounds__(NT) k_radix(const Src src, const SearchArgs a,
 // lists with one atomic per vector at the end of the pass (a warp-level global
 // atomic per candidate serialises on the counter once windows are wide).
 // What overflows the shared buffer goes straight to the global list.
-constexpr int kBlkCand = 1024;
+constexpr int kBlkCand = 1024;           // per vector in a 256-thread CTA's static shared memory
 struct BlockCand {
-    float (*buf)[kBlkCand];
+    float* buf[2];
+    unsigned cap;
     unsigned* cnt;     // [2]
     unsigned* base;    // [2]
     // the lists' key histograms over the windows (null: not kept)
@@ -632,9 +633,9 @@ struct BlockCand {
         if (lane == leader) b = atomicAdd(cnt + v, (unsigned)__popc(mask));
         b = __shfl_sync(0xffffffffu, b, leader);
         const unsigned k = b + __popc(mask & ((1u << lane) - 1u));
-        if (take && k < (unsigned)kBlkCand) buf[v][k] = x;
-        if (b + __popc(mask) > (unsigned)kBlkCand) {
-            const bool over = take && k >= (unsigned)kBlkCand;
+        if (take && k < cap) buf[v][k] = x;
+        if (b + __popc(mask) > cap) {
+            const bool over = take && k >= cap;
             append_candidate(over, x, gcand, gcnt);
             if (over && nh[v]) {
                 narrow_add(nh[v], ng[v], __float_as_uint(x));
@@ -646,12 +647,12 @@ struct BlockCand {
     __device__ void flush(float* const* gcand, Scal* sc) {
         __syncthreads();
         if (threadIdx.x < 2) {
-            const unsigned n = min(cnt[threadIdx.x], (unsigned)kBlkCand);
+            const unsigned n = min(cnt[threadIdx.x], cap);
             base[threadIdx.x] = n ? atomicAdd(&sc->acc[threadIdx.x].m, n) : 0u;
         }
         __syncthreads();
         for (int v = 0; v < 2; ++v) {
-            const unsigned n = min(cnt[v], (unsigned)kBlkCand);
+            const unsigned n = min(cnt[v], cap);
             for (unsigned k = threadIdx.x; k < n; k += blockDim.x)
                 if (base[v] + k < kCandCap) gcand[v][base[v] + k] = buf[v][k];
         }
@@ -660,28 +661,35 @@ struct BlockCand {
     // key histogram (kept by keep_hist)
     __device__ void bin(int v) {
         if (!nh[v]) return;
-        const unsigned n = min(cnt[v], (unsigned)kBlkCand);
+        const unsigned n = min(cnt[v], cap);
         for (unsigned k = threadIdx.x; k < n; k += blockDim.x) narrow_add(nh[v], ng[v], __float_as_uint(buf[v][k]));
         if (threadIdx.x == 0 && n) atomicAdd(nbinned + v, n);
     }
 };
-#define GSSTV_BLOCK_CAND(name)                                   \
-    __shared__ float name##_buf[2][kBlkCand];                    \
-    __shared__ unsigned name##_cnt[2], name##_base[2];           \
-    BlockCand name{name##_buf, name##_cnt, name##_base};         \
+// The buffers: the static ones, or `store` (cap floats per vector).
+struct CandStore {
+    float* p = nullptr;
+    unsigned cap = 0;
+};
+#define GSSTV_BLOCK_CAND(name, store)                                                                  \
+    __shared__ float name##_buf[2][kBlkCand];                                                          \
+    __shared__ unsigned name##_cnt[2], name##_base[2];                                                 \
+    BlockCand name{{store.p ? store.p : name##_buf[0], store.p ? store.p + store.cap : name##_buf[1]}, \
+                   store.p ? store.cap : (unsigned)kBlkCand, name##_cnt, name##_base};                 \
     name.init()
 
 // Gathers the bracket bin of every vector that needs it (k_search_finish
 // finishes tau).
 template <typename Src>
-__device__ __forceinline__ void gather_body(const Src& src, const SearchArgs& a, const int bid, const int nblk) {
+__device__ __forceinline__ void gather_body(const Src& src, const SearchArgs& a, const int bid, const int nblk,
+                                            const CandStore store = CandStore()) {
     bool need[2];
     need[0] = a.sc->ctl[0].need == NEED_GATHER;
     need[1] = a.nvec > 1 && a.sc->ctl[1].need == NEED_GATHER;
     if (!need[0] && !need[1]) return;
     const float lo0 = a.sc->ctl[0].g_lo, hi0 = a.sc->ctl[0].g_hi;
     const float lo1 = a.sc->ctl[1].g_lo, hi1 = a.sc->ctl[1].g_hi;
-    GSSTV_BLOCK_CAND(bc);
+    GSSTV_BLOCK_CAND(bc, store);
     if (need[0]) bc.keep_hist(a.w, 0, lo0, hi0);
     if (need[1]) bc.keep_hist(a.w, 1, lo1, hi1);
     src.visit(bid * blockDim.x, nblk * blockDim.x, [&](bool valid, float x0, float x1) {
@@ -704,7 +712,8 @@ __global__ void __launch_bounds__(NT) k_gather(const Src src, const SearchArgs a
 // partial sums go to pn / ps (the stencil pass's partial arrays, free by now).
 template <typename Src>
 __device__ __forceinline__ void window_body(const Src& src, const SearchArgs& a, unsigned long long* pn, double* ps,
-                                            const int bid, const unsigned stride) {
+                                            const int bid, const unsigned stride,
+                                            const CandStore store = CandStore()) {
     __shared__ double red_d[64];
     __shared__ unsigned long long red_u[64];
     bool need[2];
@@ -714,7 +723,7 @@ __device__ __forceinline__ void window_body(const Src& src, const SearchArgs& a,
     const float lo0 = a.sc->ctl[0].g_lo, hi0 = a.sc->ctl[0].g_hi;
     const float lo1 = a.sc->ctl[1].g_lo, hi1 = a.sc->ctl[1].g_hi;
     WinAcc<typename Src::Storage> w0, w1;
-    GSSTV_BLOCK_CAND(bc);
+    GSSTV_BLOCK_CAND(bc, store);
     if (need[0]) bc.keep_hist(a.w, 0, lo0, hi0);
     if (need[1]) bc.keep_hist(a.w, 1, lo1, hi1);
     src.visit(bid * blockDim.x, stride, [&](bool valid, float x0, float x1) {
@@ -1166,7 +1175,12 @@ __device__ __forceinline__ int search_next(const SearchArgs& a, int st) {
 template <typename Src>
 __device__ __forceinline__ void search_body(const Src& src, const SearchArgs& a, unsigned long long* pn, double* ps,
                                             const SearchShape& h, const int bid) {
+    extern __shared__ __align__(16) float fstage[];
     __shared__ int sh_stage, sh_item, sh_last;
+    // an item's candidates wait in the finish's stage, free in these stages: 152
+    // CTAs with 1024 places a vector overflowed into single atomics on the global
+    // list (a retry pass of 512x512x224 appends 180-360 thousand)
+    const CandStore store{fstage, kFinishStage / 2};
     SearchSync* y = &a.sc->search;
     auto publish = [&](int next) {                       // (thread 0)
         __threadfence();
@@ -1228,9 +1242,9 @@ __device__ __forceinline__ void search_body(const Src& src, const SearchArgs& a,
             __syncthreads();
             const int item = sh_item;
             if (item >= n) break;
-            if (st == ST_WINDOW) window_body(src, a, pn, ps, item, h.win_threads);
+            if (st == ST_WINDOW) window_body(src, a, pn, ps, item, h.win_threads, store);
             else if (st == ST_WINDOW_END) finish_body(a, 0, pn, ps, h.win_items, item);
-            else if (st == ST_GATHER) gather_body(src, a, item, n);
+            else if (st == ST_GATHER) gather_body(src, a, item, n, store);
             else if (st == ST_GATHER_END) finish_body(a, 1, pn, ps, 0, item);
             else radix_count(src, a, st - ST_RADIX0, item, n);
             complete(st, n);
