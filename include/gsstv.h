@@ -299,8 +299,10 @@ int gsstv_unrolled_vjp(gsstv_handle* h, int iters, int ckpt_every, const float* 
  * of the indicator of B_{1,alpha}): d_out = sign(x) max(|x| - tau, 0), with
  * tau >= 0 the root of sum max(|x_i| - tau, 0) = radius, or d_out = d_x when
  * ||x||_1 <= radius; radius = 0 gives d_out = 0.  d_x, d_out: device, n
- * floats (may alias); tau_out: host double (may be NULL).  Allocates its
- * scratch with cudaMalloc and synchronises the stream before returning. */
+ * floats (may alias); tau_out: host double (may be NULL).  Takes its scratch
+ * (at most 5 MB) from a memory pool of the library's own on the device, which
+ * keeps at most 8 MB between calls (from cudaMalloc where the device has no
+ * pools), and synchronises the stream before returning. */
 int gsstv_project_l1ball(const float* d_x, int64_t n, double radius,
                          float* d_out, double* tau_out, void* stream);
 

@@ -826,7 +826,8 @@ __device__ __forceinline__ int warp_window(const float* x, unsigned m, double n_
 // finish).
 constexpr int kBlockPer = 8;
 constexpr unsigned kBlockWindow = 1024 * kBlockPer;
-__device__ __forceinline__ int block_window(const float* cand, unsigned m, double n_hi, double s_hi, float lo, float hi,
+template <typename Load>
+__device__ __forceinline__ int block_window(Load&& load, unsigned m, double n_hi, double s_hi, float lo, float hi,
                                             double r, double* tau_out) {
     __shared__ float2 part[32];
     __shared__ unsigned cnt[32];
@@ -838,7 +839,7 @@ __device__ __forceinline__ int block_window(const float* cand, unsigned m, doubl
 #pragma unroll
     for (int k = 0; k < kBlockPer; ++k) {
         const unsigned e = threadIdx.x + (unsigned)k * blockDim.x;
-        x[k] = e < m ? __ldcg(cand + e) : -INFINITY;      // (never above a threshold)
+        x[k] = e < m ? load(e) : -INFINITY;               // (never above a threshold)
     }
     float tf = -INFINITY;
     unsigned prev = 0xffffffffu;
@@ -963,7 +964,8 @@ __device__ __noinline__ int k1_window_finish(const SearchArgs& a, const unsigned
     __syncthreads();
     if (m > (unsigned)kFinishThreads && m <= kBlockWindow) {
         double tau = 0.0;
-        const int rc = block_window(a.w.cand[v], m, red_d[2], red_d[0], tlo_f, thi_f, r, &tau);
+        const float* cand = a.w.cand[v];
+        const int rc = block_window([cand](unsigned e) { return __ldcg(cand + e); }, m, red_d[2], red_d[0], tlo_f, thi_f, r, &tau);
         if (threadIdx.x == 0) { sh_rc = rc; red_d[1] = tau; }
         __syncthreads();
     }
@@ -1281,6 +1283,39 @@ __global__ void k_flat_window(Scal* sc, double radius, double scale) {
     } else {
         c.need = NEED_RADIX0;
         sc->search.stage = ST_RADIX0;
+    }
+}
+
+// The standalone projection of at most kBlockWindow values by one CTA, the values
+// in its registers: with everything a candidate the finish's steps are the whole
+// search.  (4096 values took 59 us in the radix stages, whose code runs once.)  As
+// there, a NaN leaves the vector as it is and an infinity makes tau infinite.
+__global__ void __launch_bounds__(1024) k_project_small(const float* x, float* out, unsigned n, double radius,
+                                                        double* tau_out) {
+    __shared__ double sh_tau;
+    bool nan = false, inf = false;
+    for (unsigned e = threadIdx.x; e < n; e += blockDim.x) {
+        const float y = x[e];
+        nan = nan || y != y;
+        inf = inf || fabsf(y) == INFINITY;
+    }
+    nan = __syncthreads_or(nan);
+    inf = __syncthreads_or(inf);
+    double tau = nan ? 0.0 : (double)INFINITY;
+    if (radius > 0.0 && !nan && !inf)
+        (void)block_window([x](unsigned e) { return fabsf(x[e]); }, n, 0.0, 0.0, 0.f, 0.f, radius, &tau);
+    if (radius == 0.0) tau = (double)INFINITY;
+    if (threadIdx.x == 0) {
+        sh_tau = tau;
+        *tau_out = tau;
+    }
+    __syncthreads();
+    tau = sh_tau;
+    const float tf = (float)tau;
+    const bool on = tau > 0.0;
+    for (unsigned e = threadIdx.x; e < n; e += blockDim.x) {
+        const float y = x[e];
+        out[e] = on ? soft(y, tf) : y;
     }
 }
 
@@ -1871,17 +1906,82 @@ int launch_scale_unpack(int storage, const void* q, const double* c, float* dst,
 // ---------------------------------------------------------------------------
 // standalone projection of a flat device vector onto an l1 ball
 // ---------------------------------------------------------------------------
+// Scratch of the standalone projection: stream-ordered, from a memory pool of the
+// library's own on each device that keeps at most 8 MB between calls (a pair of
+// cudaMalloc and cudaFree took 0.15 ms of every call).  Without a pool, cudaMalloc.
+struct PoolScratch {
+    void* p = nullptr;
+    cudaStream_t st;
+    bool pooled = false;
+    explicit PoolScratch(cudaStream_t s) : st(s) {}
+    static cudaMemPool_t pool() {
+        constexpr int kMaxDev = 64;
+        static std::once_flag once[kMaxDev];
+        static cudaMemPool_t pools[kMaxDev];
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) return nullptr;
+        std::call_once(once[dev], [dev] {
+            cudaMemPoolProps props{};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            cudaMemPool_t q = nullptr;
+            unsigned long long keep = 8ull << 20;
+            if (cudaMemPoolCreate(&q, &props) != cudaSuccess ||
+                cudaMemPoolSetAttribute(q, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+                if (q) cudaMemPoolDestroy(q);
+                q = nullptr;
+                cudaGetLastError();
+            }
+            pools[dev] = q;
+        });
+        return pools[dev];
+    }
+    bool get(size_t bytes) {
+        const cudaMemPool_t q = pool();
+        if (q) {
+            if (cudaMallocFromPoolAsync(&p, bytes, q, st) == cudaSuccess) {
+                pooled = true;
+                return true;
+            }
+            cudaGetLastError();
+        }
+        if (cudaMalloc(&p, bytes) == cudaSuccess) return true;
+        cudaGetLastError();
+        p = nullptr;
+        return false;
+    }
+    ~PoolScratch() {
+        if (!p) return;
+        if (pooled) cudaFreeAsync(p, st);
+        else cudaFree(p);
+    }
+};
+
 // Vectors from this length on are searched by a sample and one pass.
 constexpr long long kSampleFrom = 1ll << 21;
 
-// One allocation holds the scratch.  A short vector is searched by the radix
+// One allocation holds the scratch.  A vector of at most kBlockWindow values is
+// one CTA's; a short one is searched by the radix
 // stages of one launch; a long one by those stages on a sample of 1/32, which
 // place the window of one pass over all values (58.7 M values: a call with three
 // radix passes and a gather over all of them took 1290 us, now 544: sample 89,
-// pass 168, output 66 us; 4096 values in seven launches and four allocations 357
-// us, now 260).
+// pass 168, output 66 us, and 484 with pooled scratch; 4096 values in seven
+// launches and four allocations 357
+// us, now 52).
 int l1_project_standalone(const float* x, long long n, double radius, float* out, double* tau,
                           cudaStream_t st) {
+    PoolScratch scr(st);
+    if (n <= (long long)kBlockWindow) {
+        double t = 0.0;
+        if (!scr.get(sizeof(double))) return -2;
+        k_project_small<<<1, 1024, 0, st>>>(x, out, (unsigned)n, radius, (double*)scr.p);
+        const bool ok = cudaGetLastError() == cudaSuccess &&
+                        cudaMemcpyAsync(&t, scr.p, sizeof(t), cudaMemcpyDeviceToHost, st) == cudaSuccess;
+        if (cudaStreamSynchronize(st) != cudaSuccess || !ok) return -3;
+        if (tau) *tau = t;
+        return 0;
+    }
     const bool sampled = n >= kSampleFrom && radius > 0.0;
     if (cudaFuncSetAttribute(k_search<FlatSrc>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFinishSmem) != cudaSuccess ||
         cudaFuncSetAttribute(k_search<SampleSrc>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFinishSmem) != cudaSuccess)
@@ -1895,11 +1995,8 @@ int l1_project_standalone(const float* x, long long n, double radius, float* out
     const size_t o_sc = take(sizeof(Scal)), o_cnt = take(b_hist), o_res = take(b_hist), o_nh = take(b_nh),
                  o_nb = take(2 * sizeof(unsigned)), o_zero = off, o_pn = take(parts * 8), o_ps = take(parts * 8),
                  o_cand = take(b_cand);
-    char* mem = nullptr;
-    if (cudaMalloc(&mem, off) != cudaSuccess) {
-        cudaGetLastError();
-        return -2;
-    }
+    if (!scr.get(off)) return -2;
+    char* mem = (char*)scr.p;
     Scal* sc = reinterpret_cast<Scal*>(mem + o_sc);
     L1Work w{};
     w.hcnt = reinterpret_cast<unsigned long long*>(mem + o_cnt);
@@ -1943,7 +2040,6 @@ int l1_project_standalone(const float* x, long long n, double radius, float* out
         else if (tau) *tau = h.ctl[0].tau;
     }
     cudaStreamSynchronize(st);
-    cudaFree(mem);
     return rc;
 }
 

@@ -1,5 +1,5 @@
-"""The l1-ball projection of vectors long enough for the sampled search, against
-torch in float64: lengths at the edges of its blocks, unaligned vectors, values
+"""The l1-ball projection of vectors long enough for the sampled search, and of
+those short enough for one CTA, against torch in float64: lengths at the edges of its blocks, unaligned vectors, values
 whose sample says little (a period, a few large outliers, ties, all in the
 ball), and NaN.  Tolerances: those of the projection's other tests for tau (1e-6
 relative); an output is one float32 subtraction of tau rounded to float32, 2^-23
@@ -50,8 +50,24 @@ def test_long_vectors(kind, n, frac):
         assert float((out.double() - want).abs().max()) <= 2.0 ** -23 * float(y.abs().max())
 
 
-def test_nan_leaves_the_vector():
-    x = vector("normal", N)
-    x[12345] = float("nan")
+@pytest.mark.parametrize("n", [1, 31, 1024, 8191, 8192, 8193])
+@pytest.mark.parametrize("frac", [0.0, 0.02, 0.6, 0.9999, 2.0])
+def test_short_vectors(n, frac):
+    for x in (vector("normal", n), vector("ties", n)):
+        r = frac * float(x.abs().sum(dtype=torch.float64))
+        out, tau = project_l1ball(x, r)
+        if r == 0.0:
+            assert torch.equal(out, torch.zeros_like(x))
+            continue
+        ref = exact(x, r)
+        assert tau == pytest.approx(ref, rel=1e-6, abs=1e-12)
+        want = x.double().sign() * (x.double().abs() - ref).clamp(min=0.0)
+        assert float((out.double() - want).abs().max()) <= 2.0 ** -23 * float(x.abs().max())
+
+
+@pytest.mark.parametrize("n", [100, 10000, N])
+def test_nan_leaves_the_vector(n):
+    x = vector("normal", n)
+    x[77] = float("nan")
     out, tau = project_l1ball(x, 10.0)
     assert tau == 0.0 and torch.equal(out.nan_to_num(7.0), x.nan_to_num(7.0))
