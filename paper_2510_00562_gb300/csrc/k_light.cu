@@ -821,13 +821,9 @@ __device__ __forceinline__ int warp_window(const float* x, unsigned m, double n_
     return 0;
 }
 
-// The same by the whole block for at most kBlockWindow values of the list, held in
-// registers (157x203x61: a pass 139 -> 131 us; the narrowing took about 34 us a
-// finish).
-constexpr int kBlockPer = 8;
-constexpr unsigned kBlockWindow = 1024 * kBlockPer;
-template <typename Load>
-__device__ __forceinline__ int block_window(Load&& load, unsigned m, double n_hi, double s_hi, float lo, float hi,
+// The same by the whole block on m values in shared memory (a finish through the
+// narrowing took 34 us and more; 157x203x61: a pass 139 -> 131 us).
+__device__ __forceinline__ int block_window(const float* x, unsigned m, double n_hi, double s_hi, float lo, float hi,
                                             double r, double* tau_out) {
     __shared__ float2 part[32];
     __shared__ unsigned cnt[32];
@@ -835,22 +831,17 @@ __device__ __forceinline__ int block_window(Load&& load, unsigned m, double n_hi
     __shared__ int sh_state;                              // 0 go on, 1 found, 2 inside the ball, 3 below, 4 above
     __shared__ double sh_tau;
     const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    float x[kBlockPer];
-#pragma unroll
-    for (int k = 0; k < kBlockPer; ++k) {
-        const unsigned e = threadIdx.x + (unsigned)k * blockDim.x;
-        x[k] = e < m ? load(e) : -INFINITY;               // (never above a threshold)
-    }
     float tf = -INFINITY;
     unsigned prev = 0xffffffffu;
 #pragma unroll 1
     for (int it = 0; it < 200; ++it) {
         Kahan k;
         unsigned c = 0;
-#pragma unroll
-        for (int e = 0; e < kBlockPer; ++e) {
-            const bool in = x[e] > tf;
-            k.add(in ? x[e] : 0.f);
+#pragma unroll 4
+        for (unsigned e = threadIdx.x; e < m; e += blockDim.x) {
+            const float y = x[e];
+            const bool in = y > tf;
+            k.add(in ? y : 0.f);
             c += in ? 1u : 0u;
         }
         c = __reduce_add_sync(0xffffffffu, c);
@@ -962,10 +953,13 @@ __device__ __noinline__ int k1_window_finish(const SearchArgs& a, const unsigned
         }
     }
     __syncthreads();
-    if (m > (unsigned)kFinishThreads && m <= kBlockWindow) {
+    if (m > (unsigned)kFinishThreads && m <= kFinishStage) {
         double tau = 0.0;
         const float* cand = a.w.cand[v];
-        const int rc = block_window([cand](unsigned e) { return __ldcg(cand + e); }, m, red_d[2], red_d[0], tlo_f, thi_f, r, &tau);
+#pragma unroll 8
+        for (unsigned e = threadIdx.x + kFinishThreads; e < m; e += kFinishThreads) fstage[e] = __ldcg(cand + e);
+        __syncthreads();
+        const int rc = block_window(fstage, m, red_d[2], red_d[0], tlo_f, thi_f, r, &tau);
         if (threadIdx.x == 0) { sh_rc = rc; red_d[1] = tau; }
         __syncthreads();
     }
@@ -1286,16 +1280,18 @@ __global__ void k_flat_window(Scal* sc, double radius, double scale) {
     }
 }
 
-// The standalone projection of at most kBlockWindow values by one CTA, the values
-// in its registers: with everything a candidate the finish's steps are the whole
+// The standalone projection of at most kSmallProject values by one CTA: with everything a candidate the finish's steps are the whole
 // search.  (4096 values took 59 us in the radix stages, whose code runs once.)  As
 // there, a NaN leaves the vector as it is and an infinity makes tau infinite.
+constexpr unsigned kSmallProject = 8192;
 __global__ void __launch_bounds__(1024) k_project_small(const float* x, float* out, unsigned n, double radius,
                                                         double* tau_out) {
+    __shared__ float xs[kSmallProject];
     __shared__ double sh_tau;
     bool nan = false, inf = false;
     for (unsigned e = threadIdx.x; e < n; e += blockDim.x) {
         const float y = x[e];
+        xs[e] = fabsf(y);
         nan = nan || y != y;
         inf = inf || fabsf(y) == INFINITY;
     }
@@ -1303,7 +1299,7 @@ __global__ void __launch_bounds__(1024) k_project_small(const float* x, float* o
     inf = __syncthreads_or(inf);
     double tau = nan ? 0.0 : (double)INFINITY;
     if (radius > 0.0 && !nan && !inf)
-        (void)block_window([x](unsigned e) { return fabsf(x[e]); }, n, 0.0, 0.0, 0.f, 0.f, radius, &tau);
+        (void)block_window(xs, n, 0.0, 0.0, 0.f, 0.f, radius, &tau);
     if (radius == 0.0) tau = (double)INFINITY;
     if (threadIdx.x == 0) {
         sh_tau = tau;
@@ -1961,7 +1957,7 @@ struct PoolScratch {
 // Vectors from this length on are searched by a sample and one pass.
 constexpr long long kSampleFrom = 1ll << 21;
 
-// One allocation holds the scratch.  A vector of at most kBlockWindow values is
+// One allocation holds the scratch.  A vector of at most kSmallProject values is
 // one CTA's; a short one is searched by the radix
 // stages of one launch; a long one by those stages on a sample of 1/32, which
 // place the window of one pass over all values (58.7 M values: a call with three
@@ -1972,7 +1968,7 @@ constexpr long long kSampleFrom = 1ll << 21;
 int l1_project_standalone(const float* x, long long n, double radius, float* out, double* tau,
                           cudaStream_t st) {
     PoolScratch scr(st);
-    if (n <= (long long)kBlockWindow) {
+    if (n <= (long long)kSmallProject) {
         double t = 0.0;
         if (!scr.get(sizeof(double))) return -2;
         k_project_small<<<1, 1024, 0, st>>>(x, out, (unsigned)n, radius, (double*)scr.p);
