@@ -94,8 +94,8 @@ typedef struct gsstv_stats {
     int64_t tau_retry_hits;    /* l1 thresholds found by one retry pass over a
                                   window placed after a miss                  */
     int64_t search_passes;     /* graph-launched passes whose threshold search
-                                  launches ran (the rest skip them: K1's
-                                  window found both thresholds)               */
+                                  went past K1's window (which found both
+                                  thresholds in the rest)                     */
 } gsstv_stats;
 
 /* Device views of the full state (float32, each a (N3,N1,N2) cube or a stack

@@ -678,7 +678,7 @@ struct CandStore {
                    store.p ? store.cap : (unsigned)kBlkCand, name##_cnt, name##_base};                 \
     name.init()
 
-// Gathers the bracket bin of every vector that needs it (k_search_finish
+// Gathers the bracket bin of every vector that needs it (finish_body
 // finishes tau).
 template <typename Src>
 __device__ __forceinline__ void gather_body(const Src& src, const SearchArgs& a, const int bid, const int nblk,
@@ -707,7 +707,7 @@ __global__ void __launch_bounds__(NT) k_gather(const Src src, const SearchArgs a
 }
 
 // One windowed pass after K1's window missed: count and sum of |x| above the
-// retry window and its values as candidates (k_search_finish runs Michelot's
+// retry window and its values as candidates (finish_body runs Michelot's
 // finish; a second miss leaves the threshold to the radix passes).  Per-CTA
 // partial sums go to pn / ps (the stencil pass's partial arrays, free by now).
 template <typename Src>
