@@ -55,5 +55,5 @@ def unrolled_geosstv(v: torch.Tensor, eps, alpha, beta, omega, iters: int,
     if solver is None:
         n3, n1, n2 = v.shape
         solver = GeoSSTVSolver(n1, n2, n3, storage="fp32", graph_iters=16, **params)
-    u = _Unrolled.apply(v, eps, alpha, beta, omega, solver, iters, ckpt_every)
-    return u
+    with solver.fixed_sums():       # as the backward re-runs the passes
+        return _Unrolled.apply(v, eps, alpha, beta, omega, solver, iters, ckpt_every)

@@ -61,6 +61,7 @@ _SIGS = {
     "gsstv_create": (c_int, [ctypes.POINTER(c_void_p), c_int, c_int, c_int,
                              ctypes.POINTER(GsstvParams), c_void_p]),
     "gsstv_set_params": (c_int, [c_void_p, ctypes.POINTER(GsstvParams)]),
+    "gsstv_set_fixed_sums": (c_int, [c_void_p, c_int]),
     "gsstv_destroy": (c_int, [c_void_p]),
     "gsstv_load_observation": (c_int, [c_void_p, c_void_p]),
     "gsstv_reset_state": (c_int, [c_void_p]),
@@ -159,6 +160,10 @@ def gsstv_create(n1: int, n2: int, n3: int, params: GsstvParams, stream: int | N
 
 def gsstv_set_params(h, params: GsstvParams):
     _check(load().gsstv_set_params(h, ctypes.byref(params)), "gsstv_set_params")
+
+
+def gsstv_set_fixed_sums(h, on: bool):
+    _check(load().gsstv_set_fixed_sums(h, 1 if on else 0), "gsstv_set_fixed_sums")
 
 
 def gsstv_destroy(h):

@@ -46,7 +46,8 @@ struct gsstv_handle {
     int k1_variant = 1;           // 1: TMA-fed K1, 0: cooperative-load K1 (GSSTV_K1=coop)
     int k1_chunk = 0;             // bands per K1 CTA (0: the wave/prologue model's choice)
     K1Maps maps[2];               // tensor maps of the buffers read at parity 0 / 1
-    cudaGraphExec_t gexec[2]{};
+    int fixed = 0;                // sums in their fixed order (gsstv_set_fixed_sums)
+    cudaGraphExec_t gexec[2][2]{};  // [fixed][parity]
     int graph_len = 0;
     int timing = 0;
     std::vector<cudaEvent_t> ev;
@@ -101,8 +102,9 @@ int dalloc(gsstv_handle* h, void** out, size_t bytes) {
 }
 
 void free_all(gsstv_handle* h) {
-    for (int k = 0; k < 2; ++k)
-        if (h->gexec[k]) { cudaGraphExecDestroy(h->gexec[k]); h->gexec[k] = nullptr; }
+    for (auto& row : h->gexec)
+        for (cudaGraphExec_t& x : row)
+            if (x) { cudaGraphExecDestroy(x); x = nullptr; }
     cudaStreamSynchronize(h->st);
     for (auto& row : h->timed_exec)
         for (cudaGraphExec_t& x : row)
@@ -116,8 +118,9 @@ void free_all(gsstv_handle* h) {
 }
 
 void destroy_graphs(gsstv_handle* h) {
-    for (int k = 0; k < 2; ++k)
-        if (h->gexec[k]) { cudaGraphExecDestroy(h->gexec[k]); h->gexec[k] = nullptr; }
+    for (auto& row : h->gexec)
+        for (cudaGraphExec_t& x : row)
+            if (x) { cudaGraphExecDestroy(x); x = nullptr; }
     h->graph_len = 0;
     if (h->timed_len) cudaStreamSynchronize(h->st);
     for (auto& row : h->timed_exec)
@@ -150,6 +153,7 @@ IterParams iparams(const gsstv_handle* h, int par) {
     ip.eps = p.eps;
     ip.parity = par;
     ip.tau_exact = p.tau_mode == GSSTV_TAU_EXACT;
+    ip.fixed_sums = h->fixed && p.storage == GSSTV_FP32;
     ip.max_iter = 0;                   // the stopping rule runs on the host for a single handle
     ip.check_every = 0;
     ip.tol = 0.0;
@@ -219,11 +223,11 @@ int enqueue_iteration(gsstv_handle* h, int par, bool timed, cudaStream_t st, boo
         h->ev_used += 2;
     }
     if (h->k1_variant == 1) {
-        // (16-bit storage: the CTAs that the cooperative K1's partials allow, whose
-        // sums a run reproduces)
-        const int cap = sto == GSSTV_FP32 ? h->k1_ctas : k1_grid_ctas(h->g);
-        TRY(map_launch(launch_search(sto, h->g, b, ip, h->sc, h->l1, cap, k1_tma_grid(sto, h->g, whole, h->k1_chunk),
-                                     in_graph ? 1 : 0, st)));
+        // (where a run reproduces its sums: the CTAs that the cooperative K1's
+        // partials allow)
+        const int cap = sto == GSSTV_FP32 && !ip.fixed_sums ? h->k1_ctas : k1_grid_ctas(h->g);
+        const int parts = k1_tma_grid(sto, h->g, whole, h->k1_chunk, ip.fixed_sums);
+        TRY(map_launch(launch_search(sto, h->g, b, ip, h->sc, h->l1, cap, parts, in_graph ? 1 : 0, st)));
     } else {
         // the cooperative K1 finishes its window in its last CTA; the search
         // launches return at once unless a vector needs them
@@ -270,7 +274,9 @@ int build_graph_exec(gsstv_handle* h, int par, int len, bool timed, cudaGraphExe
     cudaGraphDestroy(graph);
     return cuda_rc(e);
 }
-int build_graph(gsstv_handle* h, int par, int len) { return build_graph_exec(h, par, len, false, &h->gexec[par]); }
+int build_graph(gsstv_handle* h, int par, int len) {
+    return build_graph_exec(h, par, len, false, &h->gexec[h->fixed][par]);
+}
 
 int flush_timing(gsstv_handle* h) {
     if (h->ev_used == 0) return GSSTV_OK;
@@ -291,12 +297,12 @@ int run_block(gsstv_handle* h, int n) {
     while (n > 0) {
         if (!h->timing && G > 0 && n >= G) {
             if (h->graph_len != G) destroy_graphs(h);
-            if (!h->gexec[h->parity]) TRY(build_graph(h, h->parity, G));
+            if (!h->gexec[h->fixed][h->parity]) TRY(build_graph(h, h->parity, G));
             h->graph_len = G;
-            TRY(cuda_rc(cudaGraphLaunch(h->gexec[h->parity], h->st)));
+            TRY(cuda_rc(cudaGraphLaunch(h->gexec[h->fixed][h->parity], h->st)));
             n -= G;
             h->stats.iterations += G;
-        } else if (h->timing && G > 0 && n >= G && 2 * G * gsstv_handle::kTimedSlots <= (int)h->ev.size()) {
+        } else if (h->timing && !h->fixed && G > 0 && n >= G && 2 * G * gsstv_handle::kTimedSlots <= (int)h->ev.size()) {
             // the same graphs with K1 between timing events: the graph of
             // slot k records events [2 G k, 2 G (k + 1)) of the pool, which
             // are read (flush_timing) before the slot is launched again
@@ -458,6 +464,12 @@ int gsstv_set_params(gsstv_handle* h, const gsstv_params* p) {
     double r[2] = {p->alpha, p->beta};
     TRY(cuda_rc(cudaMemcpyAsync(&h->sc->radius[0], r, sizeof(r), cudaMemcpyHostToDevice, h->st)));
     return cuda_rc(cudaStreamSynchronize(h->st));
+}
+
+int gsstv_set_fixed_sums(gsstv_handle* h, int on) {
+    if (!h) return GSSTV_ERR_ARG;
+    h->fixed = on ? 1 : 0;
+    return GSSTV_OK;
 }
 
 int gsstv_destroy(gsstv_handle* h) {
@@ -632,9 +644,10 @@ int gsstv_autotune(gsstv_handle* h, int passes, int* chunk_out) {
     int cand[6];
     const int nc = k1_tma_chunk_candidates(h->g, cand, 6);
     const gsstv_stats saved_stats = h->stats;
-    const int saved_timing = h->timing;
+    const int saved_timing = h->timing, saved_fixed = h->fixed;
     double best = INFINITY;
     int best_chunk = 0;
+    h->fixed = 0;                                       // (fixed sums have one split)
     int rc = flush_timing(h);
     for (int k = 0; k < nc && rc == GSSTV_OK; ++k) {
         h->k1_chunk = cand[k];
@@ -656,6 +669,7 @@ int gsstv_autotune(gsstv_handle* h, int passes, int* chunk_out) {
         }
     }
     h->timing = saved_timing;
+    h->fixed = saved_fixed;
     h->stats = saved_stats;
     h->k1_chunk = rc == GSSTV_OK ? best_chunk : 0;
     destroy_graphs(h);                                  // graphs hold the old launch shape
@@ -696,7 +710,7 @@ int gsstv_set_timing(gsstv_handle* h, int on) {
     // build the timed graphs of the current parity now, so that timed passes
     // do not wait for them
     const int G = h->p.graph_iters > 0 ? ((h->p.graph_iters + 1) / 2) * 2 : 0;
-    if (on && G > 0 && 2 * G * gsstv_handle::kTimedSlots <= (int)h->ev.size()) {
+    if (on && !h->fixed && G > 0 && 2 * G * gsstv_handle::kTimedSlots <= (int)h->ev.size()) {
         if (h->timed_len != G) destroy_graphs(h);
         h->timed_len = G;
         for (int k = 0; k < gsstv_handle::kTimedSlots; ++k) {
@@ -762,6 +776,15 @@ int vjp_launch(gsstv_handle* h, const gsstv_state_view* x, const gsstv_state_vie
                                           work, prm, h->st));
 }
 
+// The passes of a differentiated run take their sums in the fixed order, whatever
+// the handle is set to.
+struct FixedSums {
+    gsstv_handle* h;
+    int was;
+    explicit FixedSums(gsstv_handle* hh) : h(hh), was(hh->fixed) { h->fixed = 1; }
+    ~FixedSums() { h->fixed = was; }
+};
+
 // device scratch of one gsstv_unrolled_vjp call, released on every return
 struct Scratch {
     void* p = nullptr;
@@ -826,6 +849,7 @@ int gsstv_unrolled_vjp(gsstv_handle* h, int iters, int ckpt_every, const float* 
     // (otherwise unused) first segment slot, and the sweep re-runs nothing;
     // otherwise the last segment needs no run here.
     const bool keep_all = C == 1;
+    const FixedSums fixed(h);
     TRY(gsstv_reset_state(h));
     for (int c = 0; c < nck; ++c) {
         const gsstv_state_view v = slot(c);

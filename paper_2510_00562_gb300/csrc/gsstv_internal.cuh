@@ -298,10 +298,12 @@ __device__ __forceinline__ void pair_add(float& hi, float& lo, float bhi, float 
     hi = __fadd_rn(s, e);
     lo = __fsub_rn(e, __fsub_rn(hi, s));
 }
-// Kahan's update of a compensated sum: the sums of 16-bit storage.  Its
-// iterates round by random bits, so a last place of a threshold or of the
-// l2-ball scale moves a fraction of them by a whole 16-bit place; the update
-// and the order of these sums are therefore part of what a run reproduces.
+// Kahan's update of a compensated sum, for the sums whose rounding is part of
+// what a run reproduces: those of 16-bit storage (its iterates round by random
+// bits, so a last place of a threshold or of the l2-ball scale moves a fraction
+// of them by a whole 16-bit place) and those of a differentiated float32 run
+// (gsstv_set_fixed_sums: a threshold one float ulp off moves its FP64 adjoints
+// by 1e-8 to 1e-5).
 struct KahanSum {
     float s = 0.f, c = 0.f;
     __device__ __forceinline__ void add(float x) {
@@ -312,8 +314,6 @@ struct KahanSum {
     }
     __device__ __forceinline__ double value() const { return (double)s - (double)c; }
 };
-template <typename T>
-using KahanOf = std::conditional_t<std::is_same<T, float>::value, Kahan, KahanSum>;
 // The CTA's sum of the threads' compensated sums; the result (a double) is
 // valid on thread 0 only.  buf: >= 32 float2 of shared memory.
 template <typename K>
@@ -377,10 +377,10 @@ __device__ __forceinline__ void s_t_tilde(float s, float t, float y3, float y3_u
 // ---------------------------------------------------------------------------
 // window accounting for one |x| value, used by K1 and by the gather pass
 // ---------------------------------------------------------------------------
-template <typename T>
+template <typename K>
 struct WinAcc {
     unsigned long long n = 0;
-    KahanOf<T> s;
+    K s;
 };
 
 // Appends the lanes' candidates with one atomic per warp.
@@ -420,6 +420,7 @@ struct IterParams {
     double eps;
     int parity;                  // iteration parity (selects c[])
     int tau_exact;               // 1: skip the window statistics
+    int fixed_sums;              // 1: sums in their fixed order (gsstv_set_fixed_sums; float32 storage)
     // the stopping rule applied on the device (batch cubes; max_iter = 0: off)
     int max_iter;
     int check_every;
@@ -456,11 +457,12 @@ int k1_tma_ctas(const Geom& g);
 int k1_tma_chunk_candidates(const Geom& g, int* out, int cap);
 int k1_tma_configure(int storage);
 int k1_tma_maps(const Geom& g, const IterBufs& b, K1Maps* m);
-// CTAs of one K1 launch over the part's bands, and its bands per item (chunk
-// as for launch_k1_tma)
-int k1_tma_grid(int storage, const Geom& g, const SlabPart& sp, int chunk);
+// CTAs of one K1 launch over the part's bands, and its bands per item (chunk,
+// fixed_sums as for launch_k1_tma)
+int k1_tma_grid(int storage, const Geom& g, const SlabPart& sp, int chunk, int fixed_sums = 0);
 int k1_tma_part_chunk(const Geom& g, const SlabPart& sp, int chunk);
-// chunk: bands per item (0 or out of range: the model's choice)
+// chunk: bands per item (0 or out of range, and always where the sums are in
+// their fixed order: the model's choice)
 int launch_k1_tma(int storage, const Geom& g, const K1Maps& m, const IterBufs& b, const IterParams& p,
                   Scal* sc, const L1Work& w, int chunk, const SlabPart& sp, cudaStream_t st);
 

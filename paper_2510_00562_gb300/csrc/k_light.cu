@@ -98,13 +98,15 @@ struct K2Norms {
     Kahan q, du, u;
 };
 
-// The norms of 16-bit storage, in the order of the block.
+// The norms of the strips, in the order of the block.
 struct K2NormsStrip {
     KahanSum q, du, u;
 };
 
 // The rows of one strip per thread and item, top to bottom, t' of the row below
-// carried over: 16-bit storage, whose rounding streams follow the strips.
+// carried over: 16-bit storage, whose rounding streams follow the strips, and
+// float32 with its sums in their fixed order (a thread's Kahan sums over a strip
+// of four columns: the last place of the l2-ball scale).
 template <typename T>
 __device__ __forceinline__ void k2_strips(const K2Args<T>& a, const int bid, const int nblk, K2NormsStrip& N) {
     const Geom g = a.g;
@@ -276,7 +278,7 @@ __device__ __forceinline__ void k2_windows(Scal* sc) {
 }
 
 // (CTA -1, where the launch has one, places the next windows)
-template <typename T>
+template <typename T, bool STRIPS = !std::is_same<T, float>::value>
 __device__ __forceinline__ void k2_body(const K2Args<T>& a, const int bid, const int nblk) {
     constexpr int NW = NT / 32;
     if (bid < 0) {
@@ -289,7 +291,7 @@ __device__ __forceinline__ void k2_body(const K2Args<T>& a, const int bid, const
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cta = a.sp.cta_base + bid;
     const int ncta = a.sp.cta_total > 0 ? a.sp.cta_total : nblk;
-    if constexpr (std::is_same<T, float>::value) {
+    if constexpr (!STRIPS) {
         __shared__ double big[3];
         if (threadIdx.x < 3) big[threadIdx.x] = 0.0;
         __syncthreads();
@@ -332,7 +334,7 @@ __device__ __forceinline__ void k2_body(const K2Args<T>& a, const int bid, const
     if (!is_last) return;
     __threadfence();
     double s0 = 0, s1 = 0, s2 = 0;
-    if constexpr (std::is_same<T, float>::value) {
+    if constexpr (!STRIPS) {
         // one warp per norm sums the CTAs' partials
         if (wid < 3) {
             double r = 0.0;
@@ -384,9 +386,9 @@ __device__ __forceinline__ void k2_body(const K2Args<T>& a, const int bid, const
     }
 }
 
-template <typename T>
+template <typename T, bool STRIPS>
 __global__ void __launch_bounds__(NT, 3) k2_light(const K2Args<T> a) {
-    k2_body(a, (int)blockIdx.x - a.windows, (int)gridDim.x - a.windows);
+    k2_body<T, STRIPS>(a, (int)blockIdx.x - a.windows, (int)gridDim.x - a.windows);
 }
 
 // ---------------------------------------------------------------------------
@@ -394,7 +396,7 @@ __global__ void __launch_bounds__(NT, 3) k2_light(const K2Args<T> a) {
 // ---------------------------------------------------------------------------
 template <typename T>
 struct CubeSrc {
-    using Storage = T;
+    using Sum = KahanSum;       // of a retry pass above its window (reproduced, as K1's)
     Geom g;
     const T *s, *t, *y3, *q;
     const Scal* sc;
@@ -449,7 +451,7 @@ struct CubeSrc {
 };
 
 struct FlatSrc {
-    using Storage = float;
+    using Sum = Kahan;          // tau is a result in FP64
     const float* x;
     long long n;
     template <typename F>
@@ -483,7 +485,7 @@ struct FlatSrc {
 // One value in 32 of a flat vector: of every whole block of 1024 a run of 32,
 // its place hashed (a fixed stride could fall in step with the data).
 struct SampleSrc {
-    using Storage = float;
+    using Sum = Kahan;
     const float* x;
     long long n;            // sampled values, a multiple of 32
     template <typename F>
@@ -722,7 +724,7 @@ __device__ __forceinline__ void window_body(const Src& src, const SearchArgs& a,
     if (!need[0] && !need[1]) return;
     const float lo0 = a.sc->ctl[0].g_lo, hi0 = a.sc->ctl[0].g_hi;
     const float lo1 = a.sc->ctl[1].g_lo, hi1 = a.sc->ctl[1].g_hi;
-    WinAcc<typename Src::Storage> w0, w1;
+    WinAcc<typename Src::Sum> w0, w1;
     GSSTV_BLOCK_CAND(bc, store);
     if (need[0]) bc.keep_hist(a.w, 0, lo0, hi0);
     if (need[1]) bc.keep_hist(a.w, 1, lo1, hi1);
@@ -1420,9 +1422,9 @@ long long part_voxels(const Geom& g, const SlabPart& sp) {
 // places the windows
 int k2_resident() { return 3 * device_sms() - 1; }
 
-int k2_grid_part(int storage, const Geom& g, const SlabPart& sp) {
+int k2_grid_part(bool strips, const Geom& g, const SlabPart& sp) {
     const long long nb = sp.o1 - sp.o0;
-    if (storage != 0) return grid_for(nb * ((g.n1 + K2_ROWS - 1) / K2_ROWS) * (g.p2 / 4));
+    if (strips) return grid_for(nb * ((g.n1 + K2_ROWS - 1) / K2_ROWS) * (g.p2 / 4));
     const long long ctas = (nb * g.n1 * (g.p2 / 4) + NT - 1) / NT;
     return (int)std::max(1ll, std::min<long long>(ctas, k2_resident()));
 }
@@ -1448,8 +1450,11 @@ int launch_k2_t(const Geom& g, const IterBufs& b, const IterParams& p, Scal* sc,
     a.part = part;
     a.sp = sp;
     a.windows = sp.cta_total == 0 ? 1 : 0;                 // (a slab's windows are placed by the finish)
-    const int ctas = std::min(k2_grid_part(std::is_same<T, float>::value ? 0 : 1, g, sp), part_cap);
-    k2_light<T><<<ctas + a.windows, NT, 0, st>>>(a);
+    constexpr bool f32 = std::is_same<T, float>::value;
+    const bool strips = !f32 || p.fixed_sums;
+    const int ctas = std::min(k2_grid_part(strips, g, sp), part_cap) + a.windows;
+    if (strips) k2_light<T, true><<<ctas, NT, 0, st>>>(a);
+    else if constexpr (f32) k2_light<T, false><<<ctas, NT, 0, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -1668,14 +1673,18 @@ int launch_search_finish(int mode, Scal* sc, const L1Work& w, int nvec, const un
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
-int k2_grid_ctas(int storage, const Geom& g) { return k2_grid_part(storage, g, whole_cube(g)); }
+// (the partials of a float32 cube serve both of its grids)
+int k2_grid_ctas(int storage, const Geom& g) {
+    const int strips = k2_grid_part(true, g, whole_cube(g));
+    return storage != 0 ? strips : std::max(strips, k2_grid_part(false, g, whole_cube(g)));
+}
 
 int window_grid(const Geom& g, const SlabPart& sp, int part_cap) {
     return window_grid_n(part_voxels(g, sp), part_cap);
 }
 int radix_grid(const Geom& g, const SlabPart& sp) { return radix_grid_n(part_voxels(g, sp)); }
 int gather_grid(const Geom& g, const SlabPart& sp) { return gather_grid_n(part_voxels(g, sp)); }
-int k2_grid(const Geom& g, const SlabPart& sp, int part_cap) { return std::min(k2_grid_part(0, g, sp), part_cap); }
+int k2_grid(const Geom& g, const SlabPart& sp, int part_cap) { return std::min(k2_grid_part(false, g, sp), part_cap); }
 
 int launch_k2(int storage, const Geom& g, const IterBufs& b, const IterParams& p, Scal* sc,
               double* part, int part_cap, const SlabPart& sp, cudaStream_t st) {
@@ -1801,7 +1810,7 @@ int launch_k2_batch(const BatchCube* cubes, int n, cudaStream_t st) {
         t.start[c] = total;
         const int share = (int)std::ceil(k2_resident() * ((double)q.g.cube / all));
         a.windows = 1;
-        total += std::max(1, std::min({share, k2_grid_part(0, q.g, a.sp), q.k2_cap})) + 1;
+        total += std::max(1, std::min({share, k2_grid_part(false, q.g, a.sp), q.k2_cap})) + 1;
     }
     t.start[n] = total;
     k2_batch<<<total, NT, 0, st>>>(t);

@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(NT, 2) k1_stencil(const K1Args<T> a) {
     const bool win_t = !P.tau_exact && a.sc->radius[1] > 0.0 && a.sc->ctl[1].window_ok;
     const float lo_s = a.sc->ctl[0].theta_lo, hi_s = a.sc->ctl[0].theta_hi;
     const float lo_t = a.sc->ctl[1].theta_lo, hi_t = a.sc->ctl[1].theta_hi;
-    WinAcc<T> acc_s, acc_t;
+    WinAcc<KahanSum> acc_s, acc_t;
 
     auto Yp = [&](int slot, int pl) { return ys + (slot * 4 + pl) * Y_PL; };
 

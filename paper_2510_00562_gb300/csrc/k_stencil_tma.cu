@@ -147,7 +147,7 @@ struct K1Args {
     Scal* sc;
     L1Work l1;
     int chunk;          // bands per item
-    int unit;           // 16-bit: bands per piece of the window's sums (chunk is a multiple of it)
+    int unit;           // sums in a fixed order: bands per piece (chunk is a multiple of it)
     SlabPart sp;
 };
 
@@ -184,6 +184,13 @@ struct K1Stat {
 // 32 passes of a 256x256x200 float16 solve by an ulp and the result by up to a
 // float16 place; a pass took 0.91 ms either way, 1.47 ms in the cooperative
 // kernel's launches, and at 512x512x224 bfloat16 3.55 ms, 3.25 and 6.05 ms.)
+//
+// float32 storage with the sums in their fixed order (FIX, gsstv_set_fixed_sums):
+// a thread's Kahan sum over `unit` bands of its own voxel, in one launch shape for
+// every run.  A solve sums more exactly and splits as the SMs are filled best; the
+// thresholds of the two differ by 1e-10, which rounds to another float once in some
+// hundred passes, and the FP64 adjoints of a run of 9 to 40 passes then moved by
+// 1e-8 to 9e-6 (5 of 40 runs).
 struct Ordered {
     KahanSum s, t;
     float hs = 0.f, ls = 0.f, ht = 0.f, lt = 0.f;
@@ -195,6 +202,12 @@ struct Ordered {
         pair_add(hs, ls, s.s, -s.c);
         pair_add(ht, lt, t.s, -t.c);
         s = t = KahanSum();
+    }
+    // a piece's packed sums of the two vectors
+    __device__ __forceinline__ void close(float2& ks, float2& kc) {
+        pair_add(hs, ls, ks.x, -kc.x);
+        pair_add(ht, lt, ks.y, -kc.y);
+        ks = kc = make_float2(0.f, 0.f);
     }
 };
 
@@ -487,7 +500,7 @@ __device__ __forceinline__ void w_step(const IterParams& P, const float2 (&Lg)[3
 // ---------------------------------------------------------------------------
 // tile warps: one item
 // ---------------------------------------------------------------------------
-template <typename T, bool EDGE, bool HIST>
+template <typename T, bool FIX, bool EDGE, bool HIST>
 __device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, const Item& m, Cons<T>& C, K1Stat& A,
                                           Ordered& O, const K1Win& W, float cs, int turn) {
     using L = Lay<T>;
@@ -579,10 +592,17 @@ __device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, co
             // both vectors' compensated sums in packed pairs; a value not
             // taken adds zero, which leaves the represented sum unchanged
             const float2 x2 = f2(hs ? x_s : 0.f, ht ? x_t : 0.f);
-            const float2 t2 = add2(A.ks, x2);
-            const float2 b2 = sub2(t2, A.ks);
-            A.kc = sub2(A.kc, add2(sub2(A.ks, sub2(t2, b2)), sub2(x2, b2)));
-            A.ks = t2;
+            if constexpr (FIX) {
+                const float2 y2 = sub2(x2, A.kc);
+                const float2 t2 = add2(A.ks, y2);
+                A.kc = sub2(sub2(t2, A.ks), y2);
+                A.ks = t2;
+            } else {
+                const float2 t2 = add2(A.ks, x2);
+                const float2 b2 = sub2(t2, A.ks);
+                A.kc = sub2(A.kc, add2(sub2(A.ks, sub2(t2, b2)), sub2(x2, b2)));
+                A.ks = t2;
+            }
         }
         const bool cs_ = valid && !hs && x_s > W.lo_s, ct_ = valid && !ht && x_t > W.lo_t;
         if (__ballot_sync(0xffffffffu, cs_ || ct_)) {     // most warps have no candidate
@@ -685,7 +705,12 @@ __device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, co
         C.arrive(S);
         const bool more = b + 1 < m.b1;
         if (valid && more) store_u(ob + plane, un);
-        if (win && more) stats(yn, b + 1);
+        if (win && more) {
+            stats(yn, b + 1);
+            if constexpr (FIX) {
+                if (++piece == a.unit || b + 2 == m.b1) { O.close(A.ks, A.kc); piece = 0; }
+            }
+        }
         if (!C.wait(S)) return false;
         if constexpr (!L::F32) {
             // band b, whose values every warp left before this phase (the slot
@@ -970,7 +995,7 @@ __device__ __forceinline__ void load_async(const K1Args<T>& a, const Sm<T>& S, i
 
 // One CTA of K1: items bid, bid + nblk, ... of the gx x gy x gz items (tiles
 // by band runs) of one cube.
-template <typename T>
+template <typename T, bool FIX = false>
 __device__ __forceinline__ void k1_run(const K1Maps* maps, const K1Args<T>& a, const int bid, const int nblk,
                                        const int gx, const int gy, const int gz) {
     using L = Lay<T>;
@@ -1002,9 +1027,11 @@ __device__ __forceinline__ void k1_run(const K1Maps* maps, const K1Args<T>& a, c
     // the histograms: on after a recent miss
     W.hb_s = a.sc->ctl[0].hbase;
     W.hb_t = a.sc->ctl[1].hbase;
-    // (float32 storage only: 16-bit storage searches as the cooperative kernel does)
-    W.hs = L::F32 && W.s && a.sc->ctl[0].hist_left > 0 && hist_base_ok(W.hb_s);
-    W.ht = L::F32 && W.t && a.sc->ctl[1].hist_left > 0 && hist_base_ok(W.hb_t);
+    // (float32 storage only: 16-bit storage searches as the cooperative kernel does;
+    // sums in a fixed order: only where a piece fits the counters)
+    const bool keep = L::F32 && (!FIX || a.unit * (TY * TX) <= 65535);
+    W.hs = keep && W.s && a.sc->ctl[0].hist_left > 0 && hist_base_ok(W.hb_s);
+    W.ht = keep && W.t && a.sc->ctl[1].hist_left > 0 && hist_base_ok(W.hb_t);
     const bool hist = W.hs || W.ht;
     K1Stat A;
     Ordered O;
@@ -1016,10 +1043,10 @@ __device__ __forceinline__ void k1_run(const K1Maps* maps, const K1Args<T>& a, c
         for (int it = bid; it < items; it += nblk, ++turn) {
             const Item m = item_of(a, it, gx, gy);
             const bool ok = item_edge(m, a.g)
-                                ? (hist ? tile_item<T, true, L::F32>(a, S, m, C, A, O, W, cs, turn)
-                                        : tile_item<T, true, false>(a, S, m, C, A, O, W, cs, turn))
-                                : (hist ? tile_item<T, false, L::F32>(a, S, m, C, A, O, W, cs, turn)
-                                        : tile_item<T, false, false>(a, S, m, C, A, O, W, cs, turn));
+                                ? (hist ? tile_item<T, FIX, true, L::F32>(a, S, m, C, A, O, W, cs, turn)
+                                        : tile_item<T, FIX, true, false>(a, S, m, C, A, O, W, cs, turn))
+                                : (hist ? tile_item<T, FIX, false, L::F32>(a, S, m, C, A, O, W, cs, turn)
+                                        : tile_item<T, FIX, false, false>(a, S, m, C, A, O, W, cs, turn));
             if (!ok) break;
         }
     } else if (wid < kConsWarps) {
@@ -1068,7 +1095,7 @@ __device__ __forceinline__ void k1_run(const K1Maps* maps, const K1Args<T>& a, c
         // the histograms' above-range statistics, reduced together: 32-bit
         // counts and float-pair sums through the tile warps, then through
         // warp 0 (no FP64 outside one thread)
-        if constexpr (!L::F32) {
+        if constexpr (!L::F32 || FIX) {
             A.ks = f2(O.hs, O.ht);
             A.kc = f2(-O.ls, -O.lt);
         }
@@ -1128,6 +1155,11 @@ __global__ void __launch_bounds__(Lay<float>::NT, 1) k1_tma(const __grid_constan
                                                             const __grid_constant__ K1Args<float> a, int gx, int gy,
                                                             int gz) {
     k1_run<float>(&maps, a, blockIdx.x, gridDim.x, gx, gy, gz);
+}
+__global__ void __launch_bounds__(Lay<float>::NT, 1) k1_tma_fixed(const __grid_constant__ K1Maps maps,
+                                                                  const __grid_constant__ K1Args<float> a, int gx,
+                                                                  int gy, int gz) {
+    k1_run<float, true>(&maps, a, blockIdx.x, gridDim.x, gx, gy, gz);
 }
 template <typename T>
 __global__ void __launch_bounds__(Lay<T>::NT, 1) k1_half(const __grid_constant__ K1Args<T> a, int gx, int gy, int gz) {
@@ -1232,6 +1264,39 @@ Plan k1_plan_half(const Geom& g, int nb) {
     return p;
 }
 
+// float32 sums in their fixed order: the bands of a piece.  Runs of at least 8
+// bands, or all of fewer, chosen as if each piece were a CTA of its own: the split
+// whose last wave leaves the least of the SMs idle, a CTA's start counted as 1.5
+// bands.  Part of what the sums are, so it follows no measurement.
+int fixed_piece(int nb, int tiles) {
+    const double sms = (double)device_sms();
+    int len_best = nb;
+    double best = 1e30;
+    for (int runs = 1; runs <= std::max(1, nb / 8); ++runs) {
+        const int len = (nb + runs - 1) / runs;
+        const double units = (double)tiles * ((nb + len - 1) / len);
+        const double waves = std::ceil(units / sms);
+        const double waste = (waves - units / sms) / waves + 1.5 / len;
+        if (waste < best - 1e-12) { best = waste; len_best = len; }
+    }
+    return len_best;
+}
+// Items of whole pieces; with a histogram (see k1_run) within its counters as in k1_plan.
+Plan k1_plan_fixed(const Geom& g, int nb) {
+    Plan p;
+    const int tiles = tiles_of(g), unit = fixed_piece(nb, tiles);
+    p.chunk = best_run(nb, tiles, device_sms(), unit);
+    if (unit * (TY * TX) <= 65535) p.chunk = std::min(p.chunk, kMaxRun / unit * unit);
+    p.gz = (nb + p.chunk - 1) / p.chunk;
+    const long long items = (long long)tiles * p.gz;
+    const long long per = std::max(1, 127 / ((p.chunk + 31) / 32));
+    p.ctas = (int)std::min(items, std::max((long long)device_sms(), (items + per - 1) / per));
+    return p;
+}
+Plan k1_plan_of(int storage, const Geom& g, int nb, int chunk, int fixed_sums) {
+    return storage != 0 ? k1_plan_half(g, nb) : fixed_sums ? k1_plan_fixed(g, nb) : k1_plan(g, nb, chunk, device_sms());
+}
+
 }  // namespace
 
 // CTAs of the largest launch any run length gives: the per-CTA statistics
@@ -1262,7 +1327,11 @@ int k1_tma_chunk_candidates(const Geom& g, int* out, int cap) {
 int k1_tma_configure(int storage) {
     cudaError_t e = cudaErrorInvalidValue;
     switch (storage) {
-        case 0: e = cudaFuncSetAttribute(k1_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<float>::SMEM); break;
+        case 0:
+            e = cudaFuncSetAttribute(k1_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<float>::SMEM);
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(k1_tma_fixed, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<float>::SMEM);
+            break;
         case 1: e = cudaFuncSetAttribute(k1_half<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<__nv_bfloat16>::SMEM); break;
         case 2: e = cudaFuncSetAttribute(k1_half<__half>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<__half>::SMEM); break;
     }
@@ -1295,9 +1364,8 @@ int k1_tma_part_chunk(const Geom& g, const SlabPart& sp, int chunk) {
     return sp.o1 > sp.o0 ? k1_plan(g, sp.o1 - sp.o0, chunk, device_sms()).chunk : 0;
 }
 
-int k1_tma_grid(int storage, const Geom& g, const SlabPart& sp, int chunk) {
-    if (sp.o1 <= sp.o0) return 0;
-    return (storage == 0 ? k1_plan(g, sp.o1 - sp.o0, chunk, device_sms()) : k1_plan_half(g, sp.o1 - sp.o0)).ctas;
+int k1_tma_grid(int storage, const Geom& g, const SlabPart& sp, int chunk, int fixed_sums) {
+    return sp.o1 > sp.o0 ? k1_plan_of(storage, g, sp.o1 - sp.o0, chunk, fixed_sums).ctas : 0;
 }
 
 namespace {
@@ -1394,7 +1462,7 @@ int launch_k1_tma(int storage, const Geom& g, const K1Maps& m, const IterBufs& b
                   Scal* sc, const L1Work& w, int chunk, const SlabPart& sp, cudaStream_t st) {
     const int nb = sp.o1 - sp.o0;
     if (nb <= 0 || sp.o0 < 0 || sp.o1 > g.n3) return -1;
-    const Plan pl = storage == 0 ? k1_plan(g, nb, chunk, device_sms()) : k1_plan_half(g, nb);
+    const Plan pl = k1_plan_of(storage, g, nb, chunk, p.fixed_sums);
     const int gx = (g.n2 + TX - 1) / TX, gy = (g.n1 + TY - 1) / TY;
     auto half = [&](auto zero) {
         using T = decltype(zero);
@@ -1403,9 +1471,13 @@ int launch_k1_tma(int storage, const Geom& g, const K1Maps& m, const IterBufs& b
         k1_half<T><<<pl.ctas, Lay<T>::NT, Lay<T>::SMEM, st>>>(args, gx, gy, pl.gz);
     };
     switch (storage) {
-        case 0:
-            k1_tma<<<pl.ctas, Lay<float>::NT, Lay<float>::SMEM, st>>>(m, k1_args<float>(g, b, p, sc, w, pl.chunk, sp), gx, gy, pl.gz);
+        case 0: {
+            K1Args<float> args = k1_args<float>(g, b, p, sc, w, pl.chunk, sp);
+            args.unit = p.fixed_sums ? fixed_piece(nb, gx * gy) : 0;
+            if (p.fixed_sums) k1_tma_fixed<<<pl.ctas, Lay<float>::NT, Lay<float>::SMEM, st>>>(m, args, gx, gy, pl.gz);
+            else k1_tma<<<pl.ctas, Lay<float>::NT, Lay<float>::SMEM, st>>>(m, args, gx, gy, pl.gz);
             break;
+        }
         case 1: half(__nv_bfloat16()); break;
         case 2: half(__half()); break;
         default: return -1;

@@ -6,6 +6,8 @@ column (horizontal) -- contiguous, the layout of include/gsstv.h.
 """
 from __future__ import annotations
 
+import contextlib
+
 import torch
 
 from . import binding as B
@@ -45,6 +47,7 @@ class GeoSSTVSolver:
         self.params = params if params is not None else make_params(**kw)
         self.stream = stream or torch.cuda.current_stream()
         self.h = B.gsstv_create(n1, n2, n3, self.params, self.stream.cuda_stream)
+        self._fixed = False
 
     # -- lifetime ------------------------------------------------------------
     def close(self):
@@ -84,6 +87,19 @@ class GeoSSTVSolver:
                 setattr(params, k, STORAGE.get(v, v) if k == "storage" else v)
         B.gsstv_set_params(self.h, params)
         self.params = params
+
+    @contextlib.contextmanager
+    def fixed_sums(self):
+        """Within it, passes take their global sums in the order in which
+        unrolled_vjp takes them (gsstv_set_fixed_sums): for a forward run whose
+        result seeds unrolled_vjp."""
+        was, self._fixed = self._fixed, True
+        B.gsstv_set_fixed_sums(self.h, True)
+        try:
+            yield self
+        finally:
+            self._fixed = was
+            B.gsstv_set_fixed_sums(self.h, was)
 
     def solve(self, v: torch.Tensor):
         """Runs max_iter passes from the standard start; returns (u, s, t, iters)."""
