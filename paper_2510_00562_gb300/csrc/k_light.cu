@@ -1285,23 +1285,38 @@ __global__ void k_flat_window(Scal* sc, double radius, double scale) {
 // The standalone projection of at most kSmallProject values by one CTA: with everything a candidate the finish's steps are the whole
 // search.  (4096 values took 59 us in the radix stages, whose code runs once.)  As
 // there, a NaN leaves the vector as it is and an infinity makes tau infinite.
+// The block's sums are float pairs, so values whose sum could pass the largest
+// float (2^13 of them at 2^112 and more) are scaled by 2^-32 first: exact, but for
+// bits below 2^-200 of the largest value.
 constexpr unsigned kSmallProject = 8192;
+constexpr float kProjectHuge = 0x1p112f, kProjectDown = 0x1p-32f;
+static_assert(kSmallProject <= 1u << 13, "a sum of values below kProjectHuge stays a float");
 __global__ void __launch_bounds__(1024) k_project_small(const float* x, float* out, unsigned n, double radius,
                                                         double* tau_out) {
     __shared__ float xs[kSmallProject];
     __shared__ double sh_tau;
-    bool nan = false, inf = false;
+    bool nan = false, inf = false, huge = false;
     for (unsigned e = threadIdx.x; e < n; e += blockDim.x) {
         const float y = x[e];
         xs[e] = fabsf(y);
         nan = nan || y != y;
         inf = inf || fabsf(y) == INFINITY;
+        huge = huge || fabsf(y) >= kProjectHuge;
     }
     nan = __syncthreads_or(nan);
     inf = __syncthreads_or(inf);
+    huge = __syncthreads_or(huge);
     double tau = nan ? 0.0 : (double)INFINITY;
-    if (radius > 0.0 && !nan && !inf)
-        (void)block_window(xs, n, 0.0, 0.0, 0.f, 0.f, radius, &tau);
+    if (radius > 0.0 && !nan && !inf) {
+        double down = 1.0;
+        if (huge) {
+            down = (double)kProjectDown;
+            for (unsigned e = threadIdx.x; e < n; e += blockDim.x) xs[e] *= kProjectDown;
+            __syncthreads();
+        }
+        (void)block_window(xs, n, 0.0, 0.0, 0.f, 0.f, radius * down, &tau);
+        tau /= down;
+    }
     if (radius == 0.0) tau = (double)INFINITY;
     if (threadIdx.x == 0) {
         sh_tau = tau;

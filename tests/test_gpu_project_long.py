@@ -71,3 +71,18 @@ def test_nan_leaves_the_vector(n):
     x[77] = float("nan")
     out, tau = project_l1ball(x, 10.0)
     assert tau == 0.0 and torch.equal(out.nan_to_num(7.0), x.nan_to_num(7.0))
+
+
+@pytest.mark.parametrize("n", [64, 4096, 8192, 8193, N + 5])
+@pytest.mark.parametrize("top", [2e37, 1e36, 3e38])
+@pytest.mark.parametrize("frac", [0.02, 0.6, 2.0])
+def test_a_norm_above_the_largest_float(n, top, frac):
+    """Finite values whose sum of absolute values float32 cannot hold."""
+    g = torch.Generator(device="cuda").manual_seed(n)
+    x = top * (2.0 * torch.rand(n, device="cuda", generator=g) - 1.0)
+    r = frac * float(x.abs().sum(dtype=torch.float64))
+    out, tau = project_l1ball(x, r)
+    ref = exact(x, r)
+    assert tau == pytest.approx(ref, rel=1e-6)
+    want = x.double().sign() * (x.double().abs() - ref).clamp(min=0.0)
+    assert float((out.double() - want).abs().max()) <= 2.0 ** -23 * float(x.double().abs().max())
