@@ -776,17 +776,21 @@ constexpr int kFinishThreads = 1024;
 constexpr unsigned kFinishStage = 32768;
 
 // tau inside the window (lo, hi] of m values by one warp: 0 found, 1 below, 2
-// above (as l1_window_finish).  Newton's steps on phi from the window's middle,
-// where the window was predicted around: from the right of the root a step lands
-// left of it, from there they do not pass it, and a repeated count means the
-// active set is the root's.
+// above or no number (as l1_window_finish), -1 not settled.  Newton's steps on phi
+// from the window's middle, where the window was predicted around: from the right
+// of the root a step lands left of it, from there they do not pass it, so that the
+// counts fall, and a repeated count means the active set is the root's.  (A count
+// that rises again has met a value equal to tau but for its rounding.)  Sums that
+// overflow give a tau that is no number.
+__device__ __forceinline__ bool window_settled(int it, unsigned c, unsigned prev) {
+    return c == prev || (it > 2 && c > prev);
+}
 __device__ __forceinline__ int warp_window(const float* x, unsigned m, double n_hi, double s_hi, float lo, float hi,
                                            double r, double* tau_out) {
     const unsigned lane = threadIdx.x & 31u;
-    if (s_hi - n_hi * (double)hi - r > 0.0) return 2;
+    if (!(s_hi - n_hi * (double)hi - r <= 0.0)) return 2;
     float tf = -INFINITY;                                 // first the sum of all values: phi at lo
     unsigned prev = 0xffffffffu;
-    double tau = 0.0;
 #pragma unroll 1
     for (int it = 0; it < 200; ++it) {
         Kahan k;
@@ -813,14 +817,16 @@ __device__ __forceinline__ int warp_window(const float* x, unsigned m, double n_
             }
             tf = 0.5f * (lo + hi);
         } else {
-            tau = num / den;
+            const double tau = num / den;
             tf = __double2float_rd(tau);
-            if (c == prev) break;
+            if (window_settled(it, c, prev)) {
+                *tau_out = tau;
+                return isfinite(tau) ? 0 : -1;
+            }
             prev = c;
         }
     }
-    *tau_out = tau;
-    return 0;
+    return -1;
 }
 
 // The same by the whole block on m values in shared memory (a finish through the
@@ -830,7 +836,7 @@ __device__ __forceinline__ int block_window(const float* x, unsigned m, double n
     __shared__ float2 part[32];
     __shared__ unsigned cnt[32];
     __shared__ float sh_tf;
-    __shared__ int sh_state;                              // 0 go on, 1 found, 2 inside the ball, 3 below, 4 above
+    __shared__ int sh_state;                              // 0 go on, 1 found, 2 inside the ball, 3 below, 4 above, 5 no number
     __shared__ double sh_tau;
     const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     float tf = -INFINITY;
@@ -869,12 +875,12 @@ __device__ __forceinline__ int block_window(const float* x, unsigned m, double n
             double tau = 0.0;
             if (it == 0) {
                 tf = 0.5f * (lo + hi);
-                if (s_hi - n_hi * (double)hi - r > 0.0) state = 4;
+                if (!(s_hi - n_hi * (double)hi - r <= 0.0)) state = 4;
                 else if (num - den * (double)lo < 0.0) state = lo <= 0.f ? 2 : 3;
             } else {
                 tau = num / den;
                 tf = __double2float_rd(tau);
-                if (c == prev) state = 1;
+                if (window_settled(it, c, prev)) state = isfinite(tau) ? 1 : 5;
                 prev = c;
             }
             if (lane == 0) { sh_tf = tf; sh_state = state; sh_tau = tau; }
@@ -886,7 +892,7 @@ __device__ __forceinline__ int block_window(const float* x, unsigned m, double n
     }
     const int state = sh_state;
     *tau_out = state == 2 ? 0.0 : sh_tau;
-    return state == 3 ? 1 : state == 4 ? 2 : 0;
+    return state == 3 ? 1 : state == 4 ? 2 : state == 1 || state == 2 ? 0 : -1;
 }
 
 // K1's window of vector v, after the fused pass: the CTAs' counts and sums
@@ -1314,8 +1320,7 @@ __global__ void __launch_bounds__(1024) k_project_small(const float* x, float* o
             for (unsigned e = threadIdx.x; e < n; e += blockDim.x) xs[e] *= kProjectDown;
             __syncthreads();
         }
-        (void)block_window(xs, n, 0.0, 0.0, 0.f, 0.f, radius * down, &tau);
-        tau /= down;
+        tau = block_window(xs, n, 0.0, 0.0, 0.f, 0.f, radius * down, &tau) == 0 ? tau / down : (double)NAN;
     }
     if (radius == 0.0) tau = (double)INFINITY;
     if (threadIdx.x == 0) {
@@ -1999,6 +2004,7 @@ int l1_project_standalone(const float* x, long long n, double radius, float* out
         const bool ok = cudaGetLastError() == cudaSuccess &&
                         cudaMemcpyAsync(&t, scr.p, sizeof(t), cudaMemcpyDeviceToHost, st) == cudaSuccess;
         if (cudaStreamSynchronize(st) != cudaSuccess || !ok) return -3;
+        if (std::isnan(t)) return -6;
         if (tau) *tau = t;
         return 0;
     }
