@@ -68,12 +68,16 @@ struct AdjArgs {
 
 // Float partial sums over a thread's voxels, moved into float pairs every 32
 // terms: float alone drifts over hundreds of terms, and FP64 issue is scarce on
-// this part.
+// this part.  A thread whose sums come near what a block's float pairs can hold
+// (kSpill: twice it from each of at most 2^9 threads is still a float) adds them to
+// the block's doubles `big` instead, so that the range is FP64's.
+constexpr float kSpill = 0x1p116f;
 template <int K>
 struct Partial {
     float f[K], hi[K], lo[K];
     int n;
-    __device__ __forceinline__ Partial() : n(0) {
+    double* big;                  // K sums of the block, in shared memory
+    __device__ __forceinline__ explicit Partial(double* b) : n(0), big(b) {
 #pragma unroll
         for (int k = 0; k < K; ++k) f[k] = hi[k] = lo[k] = 0.f;
     }
@@ -81,6 +85,16 @@ struct Partial {
         if (++n == 32) flush();
     }
     __device__ __forceinline__ void flush() {
+        float top = 0.f;
+#pragma unroll
+        for (int k = 0; k < K; ++k) top = fmaxf(top, fmaxf(fabsf(hi[k]), fabsf(f[k])));
+        if (top > kSpill) {
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                atomicAdd(big + k, ((double)hi[k] + (double)lo[k]) + (double)f[k]);
+                hi[k] = lo[k] = f[k] = 0.f;
+            }
+        }
 #pragma unroll
         for (int k = 0; k < K; ++k) { pair_add(hi[k], lo[k], f[k], 0.f); f[k] = 0.f; }
         n = 0;
@@ -123,8 +137,12 @@ struct NextRow {
 // voxel.
 __global__ void __launch_bounds__(NTA, 4) k_adj_sums(const AdjArgs a) {
     __shared__ float2 part[BY][kSlots];
+    __shared__ double big[NSUM];
     __shared__ bool last;
-    Partial<NSUM> p;
+    const int tid = threadIdx.y * BX + threadIdx.x;
+    if (tid < NSUM) big[tid] = 0.0;
+    __syncthreads();
+    Partial<NSUM> p(big);
     const float* const arr[12] = {a.x.u, a.x.s, a.x.t, a.x.y3, a.x.y4, a.x1.u, a.x1.s, a.x1.t,
                                   a.b1.s, a.b1.t, a.b1.y3, a.b1.y4};
     const NextRow nx(arr, a.d, a.v);
@@ -177,12 +195,11 @@ __global__ void __launch_bounds__(NTA, 4) k_adj_sums(const AdjArgs a) {
     }
     if (!(lane & 1)) part[threadIdx.y][lane >> 1] = make_float2(hi[0], lo[0]);
     __syncthreads();
-    const int tid = threadIdx.y * BX + threadIdx.x;
     if (tid < NSUM) {
         float h = part[0][tid].x, e = part[0][tid].y;
 #pragma unroll
         for (int k = 1; k < BY; ++k) pair_add(h, e, part[k][tid].x, part[k][tid].y);
-        atomicAdd(a.sc->sum + tid, (double)h + (double)e);
+        atomicAdd(a.sc->sum + tid, ((double)h + (double)e) + big[tid]);
         __threadfence();
     }
     __syncthreads();
@@ -331,8 +348,8 @@ __device__ __forceinline__ void L_at(const float* p, long long N, int n2, const 
 
 // The tile's voxels.
 template <int SET, bool IN>
-__device__ __forceinline__ void dual_tile(const AdjArgs& a, const DualSet& S, float* sm, int i0, int j0, int b0,
-                                          int b1) {
+__device__ __forceinline__ void dual_tile(const AdjArgs& a, const DualSet& S, float* sm, double* big, int i0, int j0,
+                                          int b0, int b1) {
     const Dims& d = a.d;
     const long long N = d.N;
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -341,7 +358,7 @@ __device__ __forceinline__ void dual_tile(const AdjArgs& a, const DualSet& S, fl
     const Nbr m(d, i, j);
     long long l = valid ? (long long)b0 * d.plane + (long long)i * d.n2 + j : 0;
     float* own = sm + (wid + 1) * DSW + lane + 1;
-    Partial<1> om;
+    Partial<1> om(big);
     float gn[3] = {0.f, 0.f, 0.f};                // SET 1: G_bar of the next band at (0,0), (1,0), (0,1)
     auto load_g = [&](long long lg, float g[3]) {
         const float* p = a.gbar + lg;
@@ -509,7 +526,7 @@ __device__ __forceinline__ void dual_ring(const AdjArgs& a, const DualSet& S, fl
 }
 
 template <int SET>
-__device__ __forceinline__ void dual_block(const AdjArgs& a, float* sm, int tiles_x, int run) {
+__device__ __forceinline__ void dual_block(const AdjArgs& a, float* sm, double* big, int tiles_x, int run) {
     const Dims& d = a.d;
     DualSet S;
     S.w = SET ? a.x.w2 : a.x.w1; S.y = SET ? a.x.y2 : a.x.y1;
@@ -522,8 +539,8 @@ __device__ __forceinline__ void dual_block(const AdjArgs& a, float* sm, int tile
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     auto inside = [&](int i, int j) { return i >= 1 && i <= d.n1 - 2 && j >= 1 && j <= d.n2 - 2; };
     if (wid < DTILE) {
-        if (__all_sync(0xffffffffu, inside(i0 + wid, j0 + lane))) dual_tile<SET, true>(a, S, sm, i0, j0, b0, b1);
-        else dual_tile<SET, false>(a, S, sm, i0, j0, b0, b1);
+        if (__all_sync(0xffffffffu, inside(i0 + wid, j0 + lane))) dual_tile<SET, true>(a, S, sm, big, i0, j0, b0, b1);
+        else dual_tile<SET, false>(a, S, sm, big, i0, j0, b0, b1);
     } else {
         const int q = wid - DTILE;
         // grid 0 at (-1, c), grids 1, 2 at (DTY, c) for a column c; grids 0, 2
@@ -558,7 +575,7 @@ __device__ __forceinline__ void dual_block(const AdjArgs& a, float* sm, int tile
             const float* red = sm + 12 * DPL;
             float h = red[0], e = red[1];
             for (int k = 1; k < DTILE; ++k) pair_add(h, e, red[2 * k], red[2 * k + 1]);
-            atomicAdd(a.pbar + 3, a.g_w1d * ((double)h + (double)e));
+            atomicAdd(a.pbar + 3, a.g_w1d * (((double)h + (double)e) + *big));
         }
     }
 }
@@ -566,11 +583,13 @@ __device__ __forceinline__ void dual_block(const AdjArgs& a, float* sm, int tile
 // blocks: (tile, run of bands x set), sets set0 .. set0 + nset - 1
 __global__ void __launch_bounds__(DNT, 2) k_adj_dual(const AdjArgs a, int tiles_x, int set0, int nset) {
     __shared__ float sm[12 * DPL + 2 * DTILE];
+    __shared__ double big;
+    if (threadIdx.x == 0) big = 0.0;
     for (int k = threadIdx.x; k < 12 * DPL; k += DNT) sm[k] = 0.f;
     __syncthreads();
     const int run = blockIdx.y / nset, set = set0 + (blockIdx.y - run * nset);
-    if (set == 0) dual_block<0>(a, sm, tiles_x, run);
-    else dual_block<1>(a, sm, tiles_x, run);
+    if (set == 0) dual_block<0>(a, sm, &big, tiles_x, run);
+    else dual_block<1>(a, sm, &big, tiles_x, run);
 }
 
 // Launch facts of one device: SM count and resident blocks of each kernel.

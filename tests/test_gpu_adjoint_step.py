@@ -44,3 +44,33 @@ def test_one_pass_at_tile_edges(shape, in_place):
     assert rel(vbar, vref) < 1e-5
     for k in GRAD_PARAMS:
         assert pbar[k] == pytest.approx(pref[k], rel=1e-5, abs=1e-9 * np.linalg.norm(vref)), k
+
+
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("shape", [(33, 65, 5), (157, 203, 21)])
+def test_one_pass_whose_sums_pass_the_largest_float(shape, in_place):
+    """y4 of 4e18: a square is an ordinary float32, a block's sum of them is not."""
+    n1, n2, n3 = shape
+    rs = synth.random_state(n1, n2, n3, seed=n2, scale=0.1)
+    rng = np.random.default_rng(6)
+    rs["y4"] = (4e18 * rng.standard_normal((n3, n1, n2))).astype(np.float32)
+    v = rng.uniform(0, 1, (n3, n1, n2)).astype(np.float32)
+    big = np.abs(rs["y4"]).sum(dtype=np.float64)
+    kw = dict(eps=0.02 * v.size ** 0.5, alpha=1e-4 * big, beta=1e-4 * big, omega=0.05)
+    bn = {k: rng.standard_normal(rs[k].shape).astype(np.float32) for k in STATE_KEYS}
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(x, dtype=np.float32)).cuda()  # noqa: E731
+    with GeoSSTVSolver(n1, n2, n3, make_params(graph_iters=0, **kw)) as sol:
+        sol.load(dev(v))
+        x = {k: dev(rs[k]) for k in STATE_KEYS}
+        sol.set_state(x)
+        sol.iterate(1)
+        bar, vbar, pbar = sol.vjp_step(x, sol.get_state(), {k: dev(bn[k]) for k in STATE_KEYS}, in_place=in_place)
+        got = {k: t.cpu().numpy().astype(np.float64) for k, t in bar.items()}
+        vbar = vbar.cpu().numpy().astype(np.float64)
+    ref, vref, pref = A.step_vjp(o.State(**{k: rs[k].astype(np.float64) for k in STATE_KEYS}), v.astype(np.float64),
+                                 o.Params(**kw), o.State(**{k: bn[k].astype(np.float64) for k in STATE_KEYS}))
+    for k in STATE_KEYS:
+        assert rel(got[k], getattr(ref, k)) < 1e-5, k
+    assert rel(vbar, vref) < 1e-5
+    for k in GRAD_PARAMS:
+        assert pbar[k] == pytest.approx(pref[k], rel=1e-5, abs=1e-9 * np.linalg.norm(vref)), k
