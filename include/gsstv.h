@@ -183,11 +183,13 @@ int gsstv_set_timing(gsstv_handle* h, int on);
  * this implementation, not part of Algorithm 1).  Picks the number of bands
  * each CTA of the fused stencil kernel runs through by measurement: times that kernel (CUDA events) over `passes`
  * passes from the standard start on the loaded observation for each of a few
- * candidate run lengths (the wave/prologue model's choice and the next best by
- * its estimate), keeps the fastest for this handle and resets the state.
- * *chunk_out (may be NULL) receives the bands per CTA chosen, or 0 when the
- * handle runs the cooperative kernel (16-bit storage), which has nothing to
- * tune.  Results do not depend on the choice beyond the summation order of
+ * candidate run lengths of at least 8 bands (all of them when there are fewer;
+ * the model's choice and the next best by its estimate), keeps the fastest of
+ * them for this handle and resets the state.  A cube of so few tiles that the
+ * model's own run is shorter than 8 bands is faster left untuned.
+ * *chunk_out (may be NULL) receives the bands per run chosen, or 0 when there is
+ * nothing to tune (16-bit storage, whose run follows from the order of its sums;
+ * the cooperative kernel).  Results do not depend on the choice beyond the summation order of
  * the l1 window statistics.  Synchronises the stream; the counters of
  * gsstv_get_stats are left as they were. */
 int gsstv_autotune(gsstv_handle* h, int passes, int* chunk_out);

@@ -675,7 +675,7 @@ int gsstv_autotune(gsstv_handle* h, int passes, int* chunk_out) {
     destroy_graphs(h);                                  // graphs hold the old launch shape
     TRY(rc);
     TRY(gsstv_reset_state(h));
-    if (chunk_out) *chunk_out = std::max(h->k1_chunk, std::min(8, h->g.n3));
+    if (chunk_out) *chunk_out = h->k1_chunk;
     return GSSTV_OK;
 }
 

@@ -1305,8 +1305,9 @@ int k1_tma_ctas(const Geom& g) {
     return std::max(device_sms(), tiles_of(g) * ((g.n3 + std::min(8, g.n3) - 1) / std::min(8, g.n3)));
 }
 
-// Run lengths worth timing: the model's choice first, then the next best of
-// at least 8 bands by its estimate, at most `cap` distinct lengths.
+// Run lengths worth timing: those of at least 8 bands (all of them when there are
+// fewer), the model's choice first, then the next best by its estimate, at most
+// `cap` distinct lengths.
 int k1_tma_chunk_candidates(const Geom& g, int* out, int cap) {
     const int tiles = tiles_of(g), sms = device_sms();
     std::vector<std::pair<double, int>> c;
@@ -1318,7 +1319,7 @@ int k1_tma_chunk_candidates(const Geom& g, int* out, int cap) {
     std::stable_sort(c.begin(), c.end(), [](const auto& x, const auto& y) { return x.first < y.first; });
     const int first = best_run(g.n3, tiles, sms);
     int n = 0;
-    if (cap > 0) out[n++] = first;
+    if (cap > 0 && first >= std::min(8, g.n3)) out[n++] = first;
     for (const auto& e : c)
         if (n < cap && e.second != first) out[n++] = e.second;
     return n;
