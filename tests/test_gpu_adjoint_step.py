@@ -47,7 +47,7 @@ def test_one_pass_at_tile_edges(shape, in_place):
 
 
 @pytest.mark.parametrize("in_place", [False, True])
-@pytest.mark.parametrize("shape", [(33, 65, 5), (157, 203, 21)])
+@pytest.mark.parametrize("shape", [(33, 65, 5)])
 def test_one_pass_whose_sums_pass_the_largest_float(shape, in_place):
     """y4 of 4e18: a square is an ordinary float32, a block's sum of them is not."""
     n1, n2, n3 = shape
