@@ -285,7 +285,8 @@ int gsstv_slabs_count(const gsstv_slabs* s, int* bands_out);
  * place; no other views may overlap).  Adds the adjoint of v to d_vbar (N
  * floats) and those of (eps, alpha, beta, omega) to h_pbar[0..3] (host).
  * All views: float32 device arrays in the layout of gsstv_state_view.  Uses
- * a workspace of about 10 N floats held by the handle from the first call.
+ * a workspace of about 2 N floats held by the handle from the first call, and of
+ * 8 N more from the first call in place.
  * Synchronises the stream to read the parameter adjoints back; with h_pbar
  * NULL it skips them and returns once the work is queued.
  *

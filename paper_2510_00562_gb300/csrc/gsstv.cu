@@ -37,6 +37,7 @@ struct gsstv_handle {
     float* v = nullptr;
     float* tmp = nullptr;         // dense float32 scratch for host copies (16-bit storage)
     void* adj_work = nullptr;     // scratch of gsstv_vjp_step (allocated on first use)
+    void* adj_spare = nullptr;    // and of its in-place form
     Scal* sc = nullptr;
     L1Work l1{};
     double* k2_part = nullptr;
@@ -758,10 +759,10 @@ void view_ptrs(const gsstv_state_view* v, float* out[9]) {
     out[5] = v->y1; out[6] = v->y2; out[7] = v->y3; out[8] = v->y4;
 }
 
-// single: 0 a pass of a run, 1 a single pass, 2 the same in place
+// single: 0 a pass of a run, 1 a single pass, 2 the same in place (with its spare set)
 int vjp_launch(gsstv_handle* h, const gsstv_state_view* x, const gsstv_state_view* x1,
                const gsstv_state_view* b1, const gsstv_state_view* bo, float* vbar, double* d_pbar,
-               void* work, int single = 0) {
+               void* work, int single = 0, void* spare = nullptr) {
     const gsstv_params& p = h->p;
     const double prm[16] = {p.gamma_u, p.gamma_w1, p.gamma_w2, p.gamma_s, p.gamma_t,
                             p.gamma_y1, p.gamma_y2, p.gamma_y3, p.gamma_y4,
@@ -770,8 +771,8 @@ int vjp_launch(gsstv_handle* h, const gsstv_state_view* x, const gsstv_state_vie
     view_ptrs(x, xa); view_ptrs(x1, x1a); view_ptrs(b1, b1a); view_ptrs(bo, boa);
     const Geom& g = h->g;
     if (single)
-        return map_launch(launch_adjoint_single(g.n1, g.n2, g.n3, xa, x1a, b1a, boa, single == 2, h->v, g.p2, vbar,
-                                                d_pbar, work, prm, h->st));
+        return map_launch(launch_adjoint_single(g.n1, g.n2, g.n3, xa, x1a, b1a, boa, single == 2 ? spare : nullptr,
+                                                h->v, g.p2, vbar, d_pbar, work, prm, h->st));
     return map_launch(launch_adjoint_step(g.n1, g.n2, g.n3, xa, x1a, b1a, boa, h->v, g.p2, vbar, d_pbar,
                                           work, prm, h->st));
 }
@@ -801,12 +802,13 @@ int gsstv_vjp_step(gsstv_handle* h, const gsstv_state_view* x, const gsstv_state
     if (h->p.storage != GSSTV_FP32) return GSSTV_ERR_ARG;
     const long long n = (long long)h->g.n1 * h->g.n2 * h->g.n3;
     const size_t wb = adjoint_step_bytes(n);
-    if (!h->adj_work) TRY(dalloc(h, &h->adj_work, wb + 4 * sizeof(double)));
-    double* d_pbar = (double*)((char*)h->adj_work + wb);
-    TRY(cuda_rc(cudaMemsetAsync(d_pbar, 0, 4 * sizeof(double), h->st)));
     const bool own = bar->w1 != bar_next->w1 && bar->w2 != bar_next->w2 && bar->y1 != bar_next->y1 &&
                      bar->y2 != bar_next->y2;
-    TRY(vjp_launch(h, x, x_next, bar_next, bar, d_vbar, d_pbar, h->adj_work, own ? 1 : 2));
+    if (!h->adj_work) TRY(dalloc(h, &h->adj_work, wb + 4 * sizeof(double)));
+    if (!own && !h->adj_spare) TRY(dalloc(h, &h->adj_spare, adjoint_spare_bytes(n)));
+    double* d_pbar = (double*)((char*)h->adj_work + wb);
+    TRY(cuda_rc(cudaMemsetAsync(d_pbar, 0, 4 * sizeof(double), h->st)));
+    TRY(vjp_launch(h, x, x_next, bar_next, bar, d_vbar, d_pbar, h->adj_work, own ? 1 : 2, h->adj_spare));
     if (!h_pbar) return GSSTV_OK;
     double pb[4];
     TRY(cuda_rc(cudaMemcpyAsync(pb, d_pbar, sizeof(pb), cudaMemcpyDeviceToHost, h->st)));

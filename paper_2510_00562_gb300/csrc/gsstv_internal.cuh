@@ -566,14 +566,15 @@ size_t adjoint_workspace_bytes(long long n);
 int launch_adjoint_step(int n1, int n2, int n3, const float* const x[9], const float* const x1[9],
                         const float* const b1[9], float* const bo[9], const float* v, int v_pitch,
                         float* vbar, double* pbar, void* work, const double prm[16], cudaStream_t st);
-// The same for a single pass (k_adjoint_step.cu).  in_place: w1, w2, y1, y2 of bo
-// may be b1's (else none of them is).  work: adjoint_step_bytes(N) bytes, its last
-// kAdjScalBytes (the scalars) zero before the first pass; every pass leaves them
-// ready for the next.
+// The same for a single pass (k_adjoint_step.cu).  spare: adjoint_spare_bytes(N)
+// bytes where w1, w2, y1, y2 of bo may be b1's, null where none of them is.  work:
+// adjoint_step_bytes(N) bytes, its last kAdjScalBytes (the scalars) zero before the
+// first pass; every pass leaves them ready for the next.
 constexpr size_t kAdjScalBytes = 256;
 size_t adjoint_step_bytes(long long n);
+size_t adjoint_spare_bytes(long long n);
 int launch_adjoint_single(int n1, int n2, int n3, const float* const x[9], const float* const x1[9],
-                          const float* const b1[9], float* const bo[9], bool in_place, const float* v, int v_pitch,
+                          const float* const b1[9], float* const bo[9], void* spare, const float* v, int v_pitch,
                           float* vbar, double* pbar, void* work, const double prm[16], cudaStream_t st);
 // y += a x on n floats
 int launch_axpy(float* y, const float* x, float a, long long n, cudaStream_t st);

@@ -658,11 +658,12 @@ const StepInfo& step_info() {
 }  // namespace
 
 size_t adjoint_step_bytes(long long n) {
-    return (size_t)adj_stride(n) * 10 * sizeof(float) + kAdjScalBytes;
+    return (size_t)adj_stride(n) * 2 * sizeof(float) + kAdjScalBytes;
 }
+size_t adjoint_spare_bytes(long long n) { return (size_t)adj_stride(n) * 8 * sizeof(float); }
 
 int launch_adjoint_single(int n1, int n2, int n3, const float* const x[9], const float* const x1[9],
-                        const float* const b1[9], float* const bo[9], bool in_place, const float* v, int v_pitch,
+                        const float* const b1[9], float* const bo[9], void* spare, const float* v, int v_pitch,
                         float* vbar, double* pbar, void* work, const double prm[16], cudaStream_t st) {
     const StepInfo& info = step_info();
     const int* res = info.res;
@@ -679,13 +680,12 @@ int launch_adjoint_single(int n1, int n2, int n3, const float* const x[9], const
     a.v = v;
     a.vbar = vbar;
     a.pbar = pbar;
-    // each region on a 256-byte boundary (the sums are doubles): G_bar, a_t_bar,
-    // the spare set (w: 6 regions, y: 2; their planes at the cube stride N)
+    // each region on a 256-byte boundary (the sums are doubles): G_bar, a_t_bar;
+    // in place, the spare set (w: 6 regions, y: 2; their planes at the cube stride N)
     float* f = (float*)work;
     const long long P = adj_stride(N);
     a.gbar = f; a.atb = f + P;
-    float *spare_w = f + 2 * P, *spare_y = f + 8 * P;
-    a.sc = (AdjScal*)(f + 10 * P);
+    a.sc = (AdjScal*)(f + 2 * P);
     a.g_u = (float)prm[0]; a.g_w1 = (float)prm[1]; a.g_w2 = (float)prm[2]; a.g_s = (float)prm[3];
     a.g_t = (float)prm[4]; a.g1 = (float)prm[5]; a.g2 = (float)prm[6]; a.g3 = (float)prm[7];
     a.g4 = (float)prm[8]; a.th1 = (float)prm[9]; a.th2 = (float)prm[10];
@@ -703,10 +703,11 @@ int launch_adjoint_single(int n1, int n2, int n3, const float* const x[9], const
         const dim3 grid((unsigned)tiles, (unsigned)(((n3 + a.len - 1) / a.len) * nset));
         k_adj_dual<<<grid, DNT, 0, st>>>(a, tx, set0, nset);
     };
-    if (!in_place) {
+    if (!spare) {
         dual(0, 2);
     } else {
         // in place: a set's inputs copied to the spare set first
+        float *spare_w = (float*)spare, *spare_y = spare_w + 6 * P;
         for (int s = 0; s < 2; ++s) {
             const float *&w = s ? a.b1.w2 : a.b1.w1, *&y = s ? a.b1.y2 : a.b1.y1;
             if (cudaMemcpyAsync(spare_w, w, 6 * N * sizeof(float), cudaMemcpyDeviceToDevice, st) != cudaSuccess ||

@@ -74,3 +74,27 @@ def test_one_pass_whose_sums_pass_the_largest_float(shape, in_place):
     assert rel(vbar, vref) < 1e-5
     for k in GRAD_PARAMS:
         assert pbar[k] == pytest.approx(pref[k], rel=1e-5, abs=1e-9 * np.linalg.norm(vref)), k
+
+
+def test_workspace_follows_the_form():
+    """A call that writes to buffers of its own takes 2 N floats; the spare set of
+    8 N is taken by the first call in place, and both forms agree after it."""
+    n1, n2, n3 = 48, 65, 4
+    n = n1 * n2 * n3
+    rs = synth.random_state(n1, n2, n3, seed=3, scale=0.1)
+    x = {k: torch.from_numpy(rs[k].astype(np.float32)).cuda() for k in STATE_KEYS}
+    with GeoSSTVSolver(n1, n2, n3, make_params(eps=1.0, alpha=10.0, beta=10.0, omega=0.05, graph_iters=0)) as sol:
+        sol.load(torch.zeros((n3, n1, n2), device="cuda"))
+        sol.set_state(x)
+        sol.iterate(1)
+        nxt = sol.get_state()
+        held, got = [sol.device_bytes()], []
+        for in_place in (False, True, False):
+            bar = {k: torch.full_like(v, 0.5) for k, v in x.items()}
+            got.append(sol.vjp_step(x, nxt, bar, in_place=in_place)[0])
+            held.append(sol.device_bytes())
+    grown = [b - a for a, b in zip(held, held[1:])]
+    assert 8 * n <= grown[0] <= 8 * n + 2048 and 32 * n <= grown[1] <= 32 * n + 4096 and grown[2] == 0
+    for k in STATE_KEYS:
+        for g in got[1:]:
+            assert rel(g[k].double().cpu().numpy(), got[0][k].double().cpu().numpy()) < 1e-6, k
