@@ -244,7 +244,7 @@ int enqueue_iteration(gsstv_handle* h, int par, bool timed, cudaStream_t st, boo
         };
         if (in_graph) {
             TRY(capture_if_search(st, h->cap2, [&](cudaGraphConditionalHandle c) {
-                return map_launch(launch_search_gate(&h->sc, 1, c, st));
+                return map_launch(launch_search_gate(h->sc, c, st));
             }, search));
         } else {
             TRY(search(st));

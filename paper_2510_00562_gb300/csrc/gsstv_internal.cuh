@@ -489,7 +489,7 @@ int launch_k2(int storage, const Geom& g, const IterBufs& b, const IterParams& p
 // Sets `cond` (a graph conditional handle) to whether any of the n cubes
 // whose scalars are sc[] needs a threshold search after K1's finish (for the
 // cooperative K1, whose last CTA finishes its windows itself).
-int launch_search_gate(Scal* const* sc, int n, cudaGraphConditionalHandle cond, cudaStream_t st);
+int launch_search_gate(Scal* sc, cudaGraphConditionalHandle cond, cudaStream_t st);
 // The finish of K1's windows (mode 2; parts: K1's CTAs, four partials each in
 // pn / ps), of the retry window (mode 0; parts: CTAs of the window pass(es),
 // their partial sums in pn / ps) or of the gathered radix bracket (mode 1),

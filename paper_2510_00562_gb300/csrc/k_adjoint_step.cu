@@ -321,11 +321,9 @@ __device__ __forceinline__ float shrink_adj(float xv, float xh, float pv, float 
 // itself with mv, mh (not on the last row / column).
 struct Nbr {
     bool mv, mh, up, dn, lf, rt;                  // last row/column; rows i-1, i+1, columns j-1, j+1 exist
-    bool vup;                                     // y_v at row i-1 (i >= 1)
     __device__ __forceinline__ Nbr(const Dims& d, int i, int j) {
         mv = i < d.n1 - 1; mh = j < d.n2 - 1;
         up = i >= 1; dn = i + 1 < d.n1; lf = j >= 1; rt = j + 1 < d.n2;
-        vup = up;
     }
 };
 // L y at (i, j) (p: the voxel's address in y's vertical plane, N to the

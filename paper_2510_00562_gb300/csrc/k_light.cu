@@ -1747,33 +1747,18 @@ int launch_window(int storage, const Geom& g, const IterBufs& b, const IterParam
     return -1;
 }
 
-// Whether any cube still needs a threshold search after K1's finish: sets the
-// condition of the graph node that holds the search launches (one thread, so
-// that no two calls race).
-struct GateArgs {
-    Scal* sc[kBatchMax];
-    int n;
-    cudaGraphConditionalHandle cond;
-};
-__global__ void k_search_gate(const __grid_constant__ GateArgs g) {
+// Whether a vector still needs a threshold search after the cooperative K1, which
+// finishes its window itself: sets the condition of the graph node that holds the
+// search launches.
+__global__ void k_search_gate(Scal* sc, cudaGraphConditionalHandle cond) {
     if (threadIdx.x != 0) return;
-    unsigned need = 0u;
-    for (int c = 0; c < g.n; ++c) {
-        const Scal* s = g.sc[c];
-        if (__ldcg(&s->done)) continue;
-        if (__ldcg(&s->ctl[0].need) != NEED_NONE || __ldcg(&s->ctl[1].need) != NEED_NONE) need = 1u;
-    }
-    if (need) g.sc[0]->gate_opens++;
-    cudaGraphSetConditional(g.cond, need);
+    const unsigned need = scal_needs_search(sc) ? 1u : 0u;
+    if (need) sc->gate_opens++;
+    cudaGraphSetConditional(cond, need);
 }
 
-int launch_search_gate(Scal* const* sc, int n, cudaGraphConditionalHandle cond, cudaStream_t st) {
-    if (n < 1 || n > kBatchMax) return -1;
-    GateArgs g{};
-    for (int c = 0; c < n; ++c) g.sc[c] = sc[c];
-    g.n = n;
-    g.cond = cond;
-    k_search_gate<<<1, 32, 0, st>>>(g);
+int launch_search_gate(Scal* sc, cudaGraphConditionalHandle cond, cudaStream_t st) {
+    k_search_gate<<<1, 32, 0, st>>>(sc, cond);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 

@@ -130,9 +130,6 @@ struct Lay {
     static constexpr int YPL = Y_B / ES, WRAW = W_B / ES;
     static constexpr int O_U = 4 * YPL, O_Q = O_U + U_B / ES, O_S = O_Q + U_B / ES, O_T = O_S + S_B / ES,
                          O_Y3 = O_T + S_B / ES;
-    // bytes each group's bulk copies deliver
-    static constexpr unsigned YG_TX = ES * (4u * YR * SW + 2u * UR * SW + 2u * TY * TX + (TY + 1u) * TX);
-    static constexpr unsigned WG_TX = ES * 12u * WR * SW;
     // dynamic plus the kernel's static shared memory within the 227 KB a CTA may use
     static_assert(SMEM + 512 <= 227 * 1024, "shared memory");
     static_assert(!F32 || WPL == WRAW, "w' in place");
@@ -879,6 +876,9 @@ __device__ __forceinline__ bool load_item(const Item& m, const Geom& g, Ring<Lay
 __device__ __forceinline__ void load_tma(const K1Maps& M, const K1Args<float>& a, const Sm<float>& S, int bid, int nblk,
                                          int items, int gx, int gy, unsigned& ny, unsigned& nw) {
     using L = Lay<float>;
+    // bytes each group's copies deliver
+    constexpr unsigned YG_TX = 4u * (4u * YR * SW + 2u * UR * SW + 2u * TY * TX + (TY + 1u) * TX);
+    constexpr unsigned WG_TX = 4u * 12u * WR * SW;
     Ring<L::NYS> y;
     Ring<L::NWS> w;
     const Geom& g = a.g;
@@ -890,7 +890,7 @@ __device__ __forceinline__ void load_tma(const K1Maps& M, const K1Args<float>& a
             [&](int band, int slot) {
                 unsigned char* s = reinterpret_cast<unsigned char*>(S.yg(slot));
                 uint64_t* bar = S.yfull + slot;
-                mbar_arrive_expect_tx(bar, L::YG_TX);
+                mbar_arrive_expect_tx(bar, YG_TX);
                 // (a cube of one row / column has no vertical / horizontal
                 // differences: start past its map's one row / aligned column)
                 const int iv = g.n1 > 1 ? m.i0 - 2 : 16, jh = g.n2 > 1 ? m.j0 - OX : 64;
@@ -908,7 +908,7 @@ __device__ __forceinline__ void load_tma(const K1Maps& M, const K1Args<float>& a
             [&](int band, int slot) {
                 unsigned char* s = reinterpret_cast<unsigned char*>(S.wg(slot));
                 uint64_t* bar = S.wfull + slot;
-                mbar_arrive_expect_tx(bar, L::WG_TX);
+                mbar_arrive_expect_tx(bar, WG_TX);
                 for (int k = 0; k < 6; ++k)
                     tma_load_3d(s + k * L::W_B, &M.w1, m.j0 - OX, m.i0 - 1, k * g.n3 + band, bar);
                 for (int k = 0; k < 6; ++k)
