@@ -201,8 +201,8 @@ int capture_if_search(cudaStream_t st, cudaStream_t side, D&& decide, F&& body) 
 }
 
 // One iteration from parity `par` (reads buffers par, writes par ^ 1) on `st`;
-// in_graph: `st` is being captured (the search launches then sit behind a
-// conditional node).
+// in_graph: `st` is being captured (the search launches of the cooperative K1 then
+// sit behind a conditional node).
 int enqueue_iteration(gsstv_handle* h, int par, bool timed, cudaStream_t st, bool in_graph = false) {
     const IterBufs b = bufs(h, par);
     const IterParams ip = iparams(h, par);
@@ -1039,8 +1039,6 @@ int batch_enqueue(gsstv_batch* b, const std::vector<int>& set, int par, cudaStre
         q.maps = b->dmaps + 2 * c + par;
     }
     TRY(map_launch(launch_k1_batch(cubes, nc, st)));
-    // K1's window finish, then the search launches behind a conditional node
-    // that it opens (the fused solve is always captured)
     TRY(map_launch(launch_search_batch(cubes, nc, st)));
     TRY(map_launch(launch_k2_batch(cubes, nc, st)));
     return GSSTV_OK;

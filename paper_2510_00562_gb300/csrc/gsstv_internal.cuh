@@ -486,20 +486,21 @@ int launch_window(int storage, const Geom& g, const IterBufs& b, const IterParam
                   const L1Work& w, int part_cap, const SlabPart& sp, cudaStream_t st);
 int launch_k2(int storage, const Geom& g, const IterBufs& b, const IterParams& p, Scal* sc,
               double* part, int part_cap, const SlabPart& sp, cudaStream_t st);
-// Sets `cond` (a graph conditional handle) to whether any of the n cubes
-// whose scalars are sc[] needs a threshold search after K1's finish (for the
-// cooperative K1, whose last CTA finishes its windows itself).
+// Sets `cond` (a graph conditional handle) to whether a threshold search is
+// needed after K1's finish (for the cooperative K1, whose last CTA finishes its
+// windows itself).
 int launch_search_gate(Scal* sc, cudaGraphConditionalHandle cond, cudaStream_t st);
-// The finish of K1's windows (mode 2; parts: K1's CTAs, four partials each in
-// pn / ps), of the retry window (mode 0; parts: CTAs of the window pass(es),
-// their partial sums in pn / ps) or of the gathered radix bracket (mode 1),
-// for every vector that needs it: one launch after the pass(es) it finishes.
-// gated (mode 2 in a graph): its last CTA also sets `cond` to whether a
-// threshold search is still needed.
 // K1's window finish and, where a vector needs it, the rest of the search, in
 // one launch.  parts: K1's CTAs; count: count the pass in gate_opens if it searched
 int launch_search(int storage, const Geom& g, const IterBufs& b, const IterParams& p, Scal* sc, const L1Work& w,
                   int part_cap, int parts, int count, cudaStream_t st);
+// The finish of K1's windows (mode 2; parts: K1's CTAs, four partials each in
+// pn / ps), of the retry window (mode 0; parts: CTAs of the window pass(es),
+// their partial sums in pn / ps) or of the gathered radix bracket (mode 1),
+// for every vector that needs it: one launch after the pass(es) it finishes
+// (band slabs, the cooperative K1, the allocation-free projection).  gated (mode 2
+// in a graph): its last CTA also sets `cond` to whether a threshold search is
+// still needed.
 int launch_search_finish(int mode, Scal* sc, const L1Work& w, int nvec, const unsigned long long* pn,
                          const double* ps, int parts, cudaStream_t st, int gated = 0,
                          cudaGraphConditionalHandle cond = 0);

@@ -264,8 +264,6 @@ __device__ __forceinline__ void k2_rows(const K2Args<float>& a, const int bid, c
     }
 }
 
-// The CTA `bid` of `nblk` that share one cube's K2 (a launch of its own, or
-// the cube's share of a batch launch).
 // The next windows of the threshold search, placed beside K2 by a CTA of its own
 // (one warp per vector): K1 needs them, K2 does not, and in the search launch
 // they stood 5 us in K2's way (code that runs once, in FP64).
@@ -277,7 +275,9 @@ __device__ __forceinline__ void k2_windows(Scal* sc) {
     l1_place_window(c, c.tau, c.rec_m, c.rec_w, c.rec_hit != 0, c.rec_hist != 0);
 }
 
-// (CTA -1, where the launch has one, places the next windows)
+// The CTA `bid` of `nblk` that share one cube's K2 (a launch of its own, or
+// the cube's share of a batch launch).  CTA -1, where the launch has one, places
+// the next windows.
 template <typename T, bool STRIPS = !std::is_same<T, float>::value>
 __device__ __forceinline__ void k2_body(const K2Args<T>& a, const int bid, const int nblk) {
     constexpr int NW = NT / 32;
