@@ -2,8 +2,15 @@
 //
 // For each band: the u step and u' of the next band; the w1, w2 group
 // soft-thresholds and w' on the tile plus a one-pixel ring; the y1, y2 ascent;
-// the window statistics of the l1 threshold search.  Tiles whose halo stays
-// off the image border take a specialised path with no boundary masks.
+// the window statistics of the l1 threshold search.
+//
+// Every tile runs the same code, with the masks of the image border.  Interior
+// tiles once had code of their own without masks: the two loops did not fit the
+// instruction cache that the two SMs of a pair share, and wherever a border tile
+// and an interior one ran on a pair both took 2.3 to 3.1 us a band step instead
+// of 2.0 (264x176x184 358 us a launch and 274 with one code, 176x104x94 111 and
+// 75, 256x256x128 263 and 237, bfloat16 512x512x224 2464 and 2364; sizes with few
+// such pairs 2 % slower to 3 % faster).
 //
 // One persistent CTA per SM works through (tile, band run) items, in the order
 // in which neighbouring tiles run at the same time over the same bands (their
@@ -355,9 +362,6 @@ __device__ __forceinline__ Item item_of(const K1Args<T>& a, int it, int gx, int 
     m.b1 = min(a.sp.o1, m.b0 + a.chunk);
     return m;
 }
-__device__ __forceinline__ bool item_edge(const Item& m, const Geom& g) {
-    return !(m.i0 >= 2 && m.i0 + TY + 3 <= g.n1 && m.j0 >= 2 && m.j0 + TX + 3 <= g.n2);
-}
 
 // Ring positions and phases of a warp that consumes bands (kept across items).
 template <typename T>
@@ -382,26 +386,22 @@ struct Cons {
 
 // D^T y2 of one band at row gi, column gj of the image, from global memory (y2
 // of the band at yv, yh): what D_s^T needs of the band before an item's first
-template <bool EDGE, typename T>
+template <typename T>
 __device__ __forceinline__ float dty_global(const T* yv, const T* yh, int gi, int gj, const Geom& g) {
     const long long k = (long long)gi * g.p2 + gj;
-    if constexpr (EDGE) {
-        if (gi >= g.n1 || gj >= g.n2) return 0.f;
-        float d = 0.f;
-        if (gi >= 1) d += ldT(yv + k - g.p2);
-        if (gi <= g.n1 - 2) d -= ldT(yv + k);
-        if (gj >= 1) d += ldT(yh + k - 1);
-        if (gj <= g.n2 - 2) d -= ldT(yh + k);
-        return d;
-    } else {
-        return ((ldT(yv + k - g.p2) - ldT(yv + k)) + ldT(yh + k - 1)) - ldT(yh + k);
-    }
+    if (gi >= g.n1 || gj >= g.n2) return 0.f;
+    float d = 0.f;
+    if (gi >= 1) d += ldT(yv + k - g.p2);
+    if (gi <= g.n1 - 2) d -= ldT(yv + k);
+    if (gj >= 1) d += ldT(yh + k - 1);
+    if (gj <= g.n2 - 2) d -= ldT(yh + k);
+    return d;
 }
 
 // u step (Eq. 21) and u' of one band at tile position (r, c) in [0, TY] x
 // [0, TX]: u' goes to upb, D^T y2 of the band replaces gprev (that of the
 // band before); returns u+.  gb: the band's place in the whole cube.
-template <bool EDGE, typename T>
+template <typename T>
 __device__ __forceinline__ float u_item(const K1Args<T>& a, const T* ys, float* upb, int gb, int r, int c, int gi,
                                         int gj, float cs, float& gprev) {
     using L = Lay<T>;
@@ -409,9 +409,7 @@ __device__ __forceinline__ float u_item(const K1Args<T>& a, const T* ys, float* 
     const Geom& g = a.g;
     const IterParams& P = a.p;
     const int kc = r * UC + c;
-    if constexpr (EDGE) {
-        if (gi >= g.n1 || gj >= g.n2) { upb[kc] = 0.f; gprev = 0.f; return 0.f; }
-    }
+    if (gi >= g.n1 || gj >= g.n2) { upb[kc] = 0.f; gprev = 0.f; return 0.f; }
     const int k = (r + 2) * SW + (c + OX);
     float d1, gcur;                                 // D^T y1 and D^T y2 of the band
     {
@@ -448,7 +446,6 @@ __device__ __forceinline__ YN load_yn(const T* yv, const T* yh) {
 
 // (L_v, L_h) at the three grids of one position: the dual entries themselves,
 // the four-point means and the centred means.
-template <bool EDGE>
 __device__ __forceinline__ void l_pairs(const YN& y, bool mv, bool mh, float2 (&Lg)[3]) {
     // (v, h) pairs: the centred means 0.5 (v00 + vm0), 0.5 (h00 + h0m), and
     // the four-point means 0.25 (v00 + vm0 + v01 + vm1), 0.25 (h00 + h0m + h10 + h1m)
@@ -456,15 +453,15 @@ __device__ __forceinline__ void l_pairs(const YN& y, bool mv, bool mh, float2 (&
     Lg[2] = mul2(sum, f2(0.5f, 0.5f));
     sum = add2(add2(sum, f2(y.v01, y.h10)), f2(y.vm1, y.h1m));
     const float2 four = mul2(sum, f2(0.25f, 0.25f));
-    Lg[0] = f2(!EDGE || mv ? y.v00 : 0.f, !EDGE || mv ? four.y : 0.f);
-    Lg[1] = f2(!EDGE || mh ? four.x : 0.f, !EDGE || mh ? y.h00 : 0.f);
+    Lg[0] = f2(mv ? y.v00 : 0.f, mv ? four.y : 0.f);
+    Lg[1] = f2(mh ? four.x : 0.f, mh ? y.h00 : 0.f);
 }
 
 // w step of one set (0 = w1, 1 = w2) from L y at each grid's position and the
 // six w values wk (k = 2 grid + component): w+ replaces wk, w' goes to the
 // set's planes 2 grid, 2 grid + 1 of wp at offset kw[grid] where L's output is
 // not structurally zero (on[grid]), zero elsewhere: L^T then reads w' unmasked.
-template <int SET, bool EDGE, typename T>
+template <int SET, typename T>
 __device__ __forceinline__ void w_step(const IterParams& P, const float2 (&Lg)[3], float (&wk)[6], float* wp,
                                        const int (&kw)[3], const bool (&on)[3]) {
     constexpr int WPL = Lay<T>::WPL;
@@ -489,15 +486,15 @@ __device__ __forceinline__ void w_step(const IterParams& P, const float2 (&Lg)[3
         wk[2 * gr] = nn.x;
         wk[2 * gr + 1] = nn.y;
         const float nv = 2.f * nn.x - wv, nh = 2.f * nn.y - wh;
-        wp[(6 * SET + 2 * gr) * WPL + kw[gr]] = !EDGE || on[gr] ? nv : 0.f;
-        wp[(6 * SET + 2 * gr + 1) * WPL + kw[gr]] = !EDGE || on[gr] ? nh : 0.f;
+        wp[(6 * SET + 2 * gr) * WPL + kw[gr]] = on[gr] ? nv : 0.f;
+        wp[(6 * SET + 2 * gr + 1) * WPL + kw[gr]] = on[gr] ? nh : 0.f;
     }
 }
 
 // ---------------------------------------------------------------------------
 // tile warps: one item
 // ---------------------------------------------------------------------------
-template <typename T, bool FIX, bool EDGE, bool HIST>
+template <typename T, bool FIX, bool HIST>
 __device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, const Item& m, Cons<T>& C, K1Stat& A,
                                           Ordered& O, const K1Win& W, float cs, int turn) {
     using L = Lay<T>;
@@ -509,10 +506,10 @@ __device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, co
     const unsigned plane = (unsigned)g.n1 * (unsigned)g.p2;
     const int r_t = tid / TX, c_t = tid % TX;
     const int gi = m.i0 + r_t, gj = m.j0 + c_t;
-    const bool valid = !EDGE || (gi < g.n1 && gj < g.n2);
+    const bool valid = gi < g.n1 && gj < g.n2;
     const unsigned o_t = valid ? (unsigned)gi * (unsigned)g.p2 + (unsigned)gj : 0u;
     const int ky = (r_t + 2) * SW + (c_t + OX), kw = (r_t + 1) * SW + (c_t + OX);
-    const bool mv = !EDGE || gi < g.n1 - 1, mh = !EDGE || gj < g.n2 - 1;
+    const bool mv = gi < g.n1 - 1, mh = gj < g.n2 - 1;
     const unsigned it32 = L::F32 ? 0u : (unsigned)a.sc->iter;      // seeds the 16-bit rounding streams
 
     // ---- dual ascent of y1, y2 at this thread's voxel of band tb ----
@@ -570,7 +567,7 @@ __device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, co
             // the same values), the (s, t) pair packed
             const float qv = ldT(ys + L::O_Q + r_t * SW + (c_t + OX));
             const float y3v = ldT(ys + L::O_Y3 + (r_t + 1) * TX + c_t);
-            const float y3u = (!EDGE || gi >= 1) ? ldT(ys + L::O_Y3 + r_t * TX + c_t) : 0.f;
+            const float y3u = gi >= 1 ? ldT(ys + L::O_Y3 + r_t * TX + c_t) : 0.f;
             const float y4 = __fmul_rn(cs, qv);
             const float dvt = __fsub_rn(y3u, gi <= g.n1 - 2 ? y3v : 0.f);
             const float2 mm = mul2(f2(P.gamma_s, P.gamma_t), f2(y4, __fadd_rn(dvt, y4)));
@@ -633,7 +630,7 @@ __device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, co
     float gprev = 0.f;
     if (m.b0 > 0) {
         const T* yv = a.y2 + (unsigned)(m.b0 - 1) * plane;
-        gprev = dty_global<EDGE>(yv, yv + cube, gi, gj, g);
+        gprev = dty_global(yv, yv + cube, gi, gj, g);
     }
     float yprev[4] = {0.f, 0.f, 0.f, 0.f};
     const int w_last = C.w.slot == 0 ? L::NWS - 1 : C.w.slot - 1;    // the previous item's last w
@@ -653,7 +650,7 @@ __device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, co
             const T* ys = S.yg(ys_slot);
             const T* wraw = S.wg(C.w.slot) + kw;
             float* wp = S.wp(C.w.slot, C.ps) + kw;
-            if (EDGE && !valid) {
+            if (!valid) {
 #pragma unroll
                 for (int k = 0; k < 12; ++k) wp[k * WPL] = 0.f;
             } else {
@@ -668,19 +665,17 @@ __device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, co
                 const YN ya = load_yn(ys + ky, ys + YPL + ky);
                 const YN yb = load_yn(ys + 2 * YPL + ky, ys + 3 * YPL + ky);
                 yprev[0] = ya.v00; yprev[1] = ya.h00; yprev[2] = yb.v00; yprev[3] = yb.h00;
-                if constexpr (EDGE) {
-                    // staged as zero where D is structurally zero (see
-                    // k1_tma_maps): the ascent leaves the stored values there
-                    if (!mv) { yprev[0] = ldT(a.y1 + ob); yprev[2] = ldT(a.y2 + ob); }
-                    if (!mh) { yprev[1] = ldT(a.y1 + (cube + ob)); yprev[3] = ldT(a.y2 + (cube + ob)); }
-                }
+                // staged as zero where D is structurally zero (see
+                // k1_tma_maps): the ascent leaves the stored values there
+                if (!mv) { yprev[0] = ldT(a.y1 + ob); yprev[2] = ldT(a.y2 + ob); }
+                if (!mh) { yprev[1] = ldT(a.y1 + (cube + ob)); yprev[3] = ldT(a.y2 + (cube + ob)); }
                 float2 La[3], Lb[3];
-                l_pairs<EDGE>(ya, mv, mh, La);
-                l_pairs<EDGE>(yb, mv, mh, Lb);
+                l_pairs(ya, mv, mh, La);
+                l_pairs(yb, mv, mh, Lb);
                 const int k3[3] = {0, 0, 0};
                 const bool on[3] = {mv, mh, true};
-                w_step<0, EDGE, T>(P, La, w1, wp, k3, on);
-                w_step<1, EDGE, T>(P, Lb, w2, wp, k3, on);
+                w_step<0, T>(P, La, w1, wp, k3, on);
+                w_step<1, T>(P, Lb, w2, wp, k3, on);
                 if constexpr (L::F32) {
 #pragma unroll
                     for (int k = 0; k < 6; ++k) {
@@ -698,7 +693,7 @@ __device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, co
             }
         }
         const T* yn = S.yg(C.y.slot);
-        const float un = u_item<EDGE>(a, yn, S.up(C.us), b + 1 + a.sp.band0, r_t, c_t, gi, gj, cs, gprev);
+        const float un = u_item(a, yn, S.up(C.us), b + 1 + a.sp.band0, r_t, c_t, gi, gj, cs, gprev);
         C.arrive(S);
         const bool more = b + 1 < m.b1;
         if (valid && more) store_u(ob + plane, un);
@@ -746,7 +741,7 @@ __device__ __forceinline__ bool tile_item(const K1Args<T>& a, const Sm<T>& S, co
 // ---------------------------------------------------------------------------
 // ring warps: one item
 // ---------------------------------------------------------------------------
-template <typename T, bool EDGE>
+template <typename T>
 __device__ __forceinline__ bool ring_item(const K1Args<T>& a, const Sm<T>& S, const Item& m, Cons<T>& C, float cs) {
     using L = Lay<T>;
     constexpr int YPL = L::YPL, WRAW = L::WRAW;
@@ -786,9 +781,9 @@ __device__ __forceinline__ bool ring_item(const K1Args<T>& a, const Sm<T>& S, co
         gj[k] = m.j0 + pc[k];
         ky[k] = (pr[k] + 2) * SW + (pc[k] + OX);
         kw[k] = (pr[k] + 1) * SW + (pc[k] + OX);
-        in[k] = !EDGE || (gi[k] >= 0 && gi[k] < g.n1 && gj[k] >= 0 && gj[k] < g.n2);
+        in[k] = gi[k] >= 0 && gi[k] < g.n1 && gj[k] >= 0 && gj[k] < g.n2;
     }
-    const bool mv = !EDGE || gi[0] < g.n1 - 1, mh = !EDGE || gj[1] < g.n2 - 1;
+    const bool mv = gi[0] < g.n1 - 1, mh = gj[1] < g.n2 - 1;
     in[0] = in[0] && mv;
     in[1] = in[1] && mh;
     // L y of one set at the three positions (as l_pairs; the planes read
@@ -806,7 +801,7 @@ __device__ __forceinline__ bool ring_item(const K1Args<T>& a, const Sm<T>& S, co
     float gprev = 0.f;
     if (has_u && m.b0 > 0) {
         const T* yv = a.y2 + (long long)(m.b0 - 1) * g.n1 * g.p2;
-        gprev = dty_global<EDGE>(yv, yv + g.cube, ui, uj, g);
+        gprev = dty_global(yv, yv + g.cube, ui, uj, g);
     }
     int ys_slot = 0;
 #pragma unroll 1
@@ -829,11 +824,11 @@ __device__ __forceinline__ bool ring_item(const K1Args<T>& a, const Sm<T>& S, co
             float2 La[3], Lb[3];
             ring_L(ys, ys + YPL, La);
             ring_L(ys + 2 * YPL, ys + 3 * YPL, Lb);
-            w_step<0, EDGE, T>(P, La, w1, wp, kw, in);
-            w_step<1, EDGE, T>(P, Lb, w2, wp, kw, in);
+            w_step<0, T>(P, La, w1, wp, kw, in);
+            w_step<1, T>(P, Lb, w2, wp, kw, in);
         }
         if (has_u && has_next)
-            u_item<EDGE>(a, S.yg(C.y.slot), S.up(C.us), b + 1 + a.sp.band0, ur, uc, ui, uj, cs, gprev);
+            u_item(a, S.yg(C.y.slot), S.up(C.us), b + 1 + a.sp.band0, ur, uc, ui, uj, cs, gprev);
         C.arrive(S);
         if (!C.wait(S)) return false;
         C.us = C.us == L::NUS - 1 ? 0 : C.us + 1;
@@ -1042,11 +1037,8 @@ __device__ __forceinline__ void k1_run(const K1Maps* maps, const K1Args<T>& a, c
         int turn = 0;
         for (int it = bid; it < items; it += nblk, ++turn) {
             const Item m = item_of(a, it, gx, gy);
-            const bool ok = item_edge(m, a.g)
-                                ? (hist ? tile_item<T, FIX, true, L::F32>(a, S, m, C, A, O, W, cs, turn)
-                                        : tile_item<T, FIX, true, false>(a, S, m, C, A, O, W, cs, turn))
-                                : (hist ? tile_item<T, FIX, false, L::F32>(a, S, m, C, A, O, W, cs, turn)
-                                        : tile_item<T, FIX, false, false>(a, S, m, C, A, O, W, cs, turn));
+            const bool ok = hist ? tile_item<T, FIX, L::F32>(a, S, m, C, A, O, W, cs, turn)
+                                 : tile_item<T, FIX, false>(a, S, m, C, A, O, W, cs, turn);
             if (!ok) break;
         }
     } else if (wid < kConsWarps) {
@@ -1057,8 +1049,7 @@ __device__ __forceinline__ void k1_run(const K1Maps* maps, const K1Args<T>& a, c
         int turn = 0;
         for (int it = bid; it < items; it += nblk, ++turn) {
             const Item m = item_of(a, it, gx, gy);
-            const bool ok = item_edge(m, a.g) ? ring_item<T, true>(a, S, m, C, cs) : ring_item<T, false>(a, S, m, C, cs);
-            if (!ok) break;
+            if (!ring_item<T>(a, S, m, C, cs)) break;
             if (mine)
                 flush_candidates(v, S.cbuf(v, turn & 1), S.cnt(v, turn & 1), a.sc, a.l1, v ? W.lo_t : W.lo_s,
                                  v ? W.hi_t : W.hi_s);
