@@ -1014,12 +1014,9 @@ int gsstv_batch_size(const gsstv_batch* b) { return b ? (int)b->h.size() : 0; }
 
 namespace {
 
-// One pass of the cubes in `set` from parity `par`: each stage one launch
-// (a cube that has stopped returns at once from each).
-int batch_enqueue(gsstv_batch* b, const std::vector<int>& set, int par, cudaStream_t st) {
-    const int nc = (int)set.size();
-    BatchCube cubes[kBatchMax];
-    for (int k = 0; k < nc; ++k) {
+// What the launches of a pass need of the cubes in `set` at parity `par` (k1: not set).
+void batch_cubes(gsstv_batch* b, const std::vector<int>& set, int par, BatchCube* cubes) {
+    for (int k = 0; k < (int)set.size(); ++k) {
         const int c = set[k];
         gsstv_handle* h = b->h[c];
         BatchCube& q = cubes[k];
@@ -1038,6 +1035,15 @@ int batch_enqueue(gsstv_batch* b, const std::vector<int>& set, int par, cudaStre
         q.k1_ctas = h->k1_ctas;
         q.maps = b->dmaps + 2 * c + par;
     }
+}
+
+// One pass of the cubes in `set` from parity `par`, K1 split as in plan: each stage
+// one launch (a cube that has stopped returns at once from each).
+int batch_enqueue(gsstv_batch* b, const std::vector<int>& set, int par, const BatchCube* plan, cudaStream_t st) {
+    const int nc = (int)set.size();
+    BatchCube cubes[kBatchMax];
+    batch_cubes(b, set, par, cubes);
+    for (int k = 0; k < nc; ++k) cubes[k].k1 = plan[k].k1;
     TRY(map_launch(launch_k1_batch(cubes, nc, st)));
     TRY(map_launch(launch_search_batch(cubes, nc, st)));
     TRY(map_launch(launch_k2_batch(cubes, nc, st)));
@@ -1051,10 +1057,13 @@ int batch_graph(gsstv_batch* b, const std::vector<int>& set, int G) {
     for (int c : set) chunks.push_back(b->h[c]->k1_chunk);   // (the autotuner may change them)
     if (b->gexec && b->graph_len == G && chunks == b->graph_chunks && set == b->graph_set) return GSSTV_OK;
     if (b->gexec) { cudaGraphExecDestroy(b->gexec); b->gexec = nullptr; }
+    BatchCube plan[kBatchMax];
+    batch_cubes(b, set, 0, plan);
+    k1_batch_plan(plan, (int)set.size());
     cudaGraph_t graph = nullptr;
     TRY(cuda_rc(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal)));
     int rc = GSSTV_OK;
-    for (int k = 0; k < G && rc == GSSTV_OK; ++k) rc = batch_enqueue(b, set, k & 1, b->cap);
+    for (int k = 0; k < G && rc == GSSTV_OK; ++k) rc = batch_enqueue(b, set, k & 1, plan, b->cap);
     const cudaError_t e = cudaStreamEndCapture(b->cap, &graph);
     if (rc != GSSTV_OK) { if (graph) cudaGraphDestroy(graph); return rc; }
     TRY(cuda_rc(e));

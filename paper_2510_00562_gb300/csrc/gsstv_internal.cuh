@@ -515,6 +515,10 @@ int k2_grid_ctas(int storage, const Geom& g);
 // every cube, each CTA finds its cube in a table of first CTAs, and the CTAs
 // of a cube that is done return at once.  Float32 storage.
 constexpr int kBatchMax = 64;
+// (K1Split: how K1 is split: bands per item, band runs, CTAs)
+struct K1Split {
+    int chunk, gz, ctas;
+};
 struct BatchCube {
     Geom g;
     IterBufs b;
@@ -525,12 +529,13 @@ struct BatchCube {
     int k2_cap;
     int k1_chunk;            // bands per K1 CTA (as the cube's handle runs it)
     int k1_ctas;             // capacity of the cube's per-CTA statistics
+    K1Split k1;              // K1's split in this batch (k1_batch_plan)
     const K1Maps* maps;      // the cube's tensor maps at this parity (device memory)
 };
+// Sets the split k1 of cubes[0..n) from their g, k1_chunk and k1_ctas.
+void k1_batch_plan(BatchCube* cubes, int n);
 // Each launches one stage for cubes[0..n) on st (n <= kBatchMax).
 int launch_k1_batch(const BatchCube* cubes, int n, cudaStream_t st);
-// how launch_k1_batch splits the cubes: bands per item, band runs and CTAs of each
-void k1_batch_plan(const BatchCube* cubes, int n, int* chunk, int* gz, int* ctas);
 int launch_search_batch(const BatchCube* cubes, int n, cudaStream_t st);
 int launch_k2_batch(const BatchCube* cubes, int n, cudaStream_t st);
 int batch_configure();

@@ -1767,8 +1767,6 @@ int launch_search_batch(const BatchCube* cubes, int n, cudaStream_t st) {
     static_assert(sizeof(SearchBatchTab) <= 32000, "kernel parameter space");
     SearchBatchTab t{};
     t.n = n;
-    int chunk[kBatchMax], gz[kBatchMax], ctas[kBatchMax];
-    k1_batch_plan(cubes, n, chunk, gz, ctas);            // K1's partials: one set per CTA of the cube
     double all = 0.0;
     for (int c = 0; c < n; ++c) all += (double)cubes[c].g.cube;
     const int helpers = std::max(0, device_sms() - 2 * n);
@@ -1784,7 +1782,7 @@ int launch_search_batch(const BatchCube* cubes, int n, cudaStream_t st) {
         e.ps = q.l1.k1_s;
         t.start[c] = total;
         const int share = (int)(helpers * ((double)q.g.cube / all));
-        e.h = search_shape(vox, window_grid_n(vox, q.k1_ctas), ctas[c], 1, 2 + share);
+        e.h = search_shape(vox, window_grid_n(vox, q.k1_ctas), q.k1.ctas, 1, 2 + share);
         total += share;
     }
     t.start[n] = total;

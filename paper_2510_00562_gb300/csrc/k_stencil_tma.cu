@@ -1379,48 +1379,71 @@ K1Args<T> k1_args(const Geom& g, const IterBufs& b, const IterParams& p, Scal* s
 }
 }  // namespace
 
-// The CTAs that each cube of a batch gets: persistent like a single cube's,
-// the SMs shared out so that the cube whose CTAs do the most band steps does
-// as few as possible (bisection on that count; every cube at least one CTA).
-void k1_batch_plan(const BatchCube* cubes, int n, int* chunk, int* gz, int* ctas) {
+// How the cubes of a batch share the SMs.  Within a number of CTAs, each cube gets
+// the fewest with which none of its CTAs does more than some number of band steps,
+// the same for all cubes (bisection on it).  With one CTA per SM that number is the
+// launch's time: best for a few cubes.  Many cubes leave most SMs with less than it
+// (a small cube's CTA ends early and nothing follows), so that several times as many
+// CTAs, which follow one another on the SMs, are weighed against it: their total
+// steps spread over the SMs, half a CTA for the last ones, a start for each.  (64
+// cubes of 0.05 to 59 million voxels: one CTA per SM 17.2 ms a launch, 16 times that
+// 10.6; the 8 cubes of 0.05 to 4.2 million: 0.27 and 0.36 ms.)
+constexpr double kCtaCost = 2.0;              // band steps that a CTA's start costs
+
+void k1_batch_plan(BatchCube* cubes, int n) {
     const int sms = device_sms();
-    // the fewest CTAs with which cube q stays within `steps` band steps
-    auto fewest = [&](const BatchCube& q, double steps, int* len_out) -> int {
-        const int nb = q.g.n3, tiles = tiles_of(q.g);
-        int best = 1 << 30, prev = 0;
-        for (int runs = 1; runs <= nb; ++runs) {
-            int len = (nb + runs - 1) / runs;
-            if (q.k1_chunk >= 1 && q.k1_chunk <= nb) len = q.k1_chunk;      // the cube's own (autotuned) run
-            if (len == prev) continue;
-            prev = len;
-            const long long per = (long long)(steps / (len + kItemCost));
-            if (len <= kMaxRun && per >= 1) {
-                const long long items = (long long)tiles * ((nb + len - 1) / len);
-                const long long c = (items + per - 1) / per;
-                if (c < best) { best = (int)c; *len_out = len; }
-            }
-            if (len == q.k1_chunk) break;
-        }
-        return best;
-    };
-    double lo = 0.0, hi = 1.0;
-    for (int c = 0; c < n; ++c) hi += (double)tiles_of(cubes[c].g) * (cubes[c].g.n3 + kItemCost) * 2.0;
-    const int budget = std::max(sms, n);
-    int len = 0;
-    for (int k = 0; k < 40 && hi - lo > 1e-3 * hi; ++k) {
-        const double mid = 0.5 * (lo + hi);
-        long long sum = 0;
-        for (int c = 0; c < n; ++c) sum += fewest(cubes[c], mid, &len);
-        if (sum <= budget) hi = mid; else lo = mid;
-    }
+    struct Run { int len; long long items; };
+    std::vector<std::vector<Run>> runs(n);
+    double all = 0.0;
     for (int c = 0; c < n; ++c) {
-        len = std::min(cubes[c].g.n3, kMaxRun);
-        const int want = std::min(std::max(1, fewest(cubes[c], hi, &len)), budget);
-        const Plan p = k1_plan(cubes[c].g, cubes[c].g.n3, len, want);
-        chunk[c] = p.chunk;
-        gz[c] = p.gz;
-        ctas[c] = p.ctas;
+        const BatchCube& q = cubes[c];
+        const int nb = q.g.n3, tiles = tiles_of(q.g);
+        const bool own = q.k1_chunk >= 1 && q.k1_chunk <= nb;      // the cube's own (autotuned) run
+        int prev = 0;
+        for (int k = 1; k <= nb; ++k) {
+            const int len = own ? q.k1_chunk : (nb + k - 1) / k;
+            if (len == prev) { if (own) break; continue; }
+            prev = len;
+            if (len <= kMaxRun) runs[c].push_back({len, (long long)tiles * ((nb + len - 1) / len)});
+        }
+        all += (double)tiles * (nb + kItemCost);
     }
+    // the fewest CTAs with which cube c stays within `steps` band steps, and its run
+    auto fewest = [&](int c, double steps, Run* best) -> long long {
+        long long ctas = 1ll << 40;
+        for (const Run& r : runs[c]) {
+            const long long per = (long long)(steps / (r.len + kItemCost));
+            if (per < 1) continue;
+            const long long k = (r.items + per - 1) / per;
+            if (k < ctas) { ctas = k; *best = r; }
+        }
+        return ctas;
+    };
+    std::vector<Plan> plan(n), best_plan(n);
+    double best = 1e300;
+    for (int wave = 1; wave <= 32; wave *= 2) {
+        const long long budget = (long long)wave * std::max(sms, n);
+        double lo = 0.0, hi = 1.0 + 2.0 * all;
+        Run r{1, 1};
+        for (int k = 0; k < 40 && hi - lo > 1e-3 * hi; ++k) {
+            const double mid = 0.5 * (lo + hi);
+            long long sum = 0;
+            for (int c = 0; c < n && sum <= budget; ++c) sum += fewest(c, mid, &r);
+            if (sum <= budget) hi = mid; else lo = mid;
+        }
+        double total = 0.0;
+        for (int c = 0; c < n; ++c) {
+            const BatchCube& q = cubes[c];
+            r = Run{std::min(q.g.n3, kMaxRun), 1};
+            // (the statistics of a cube's CTAs have k1_ctas places)
+            const int want = (int)std::max(1ll, std::min({fewest(c, hi, &r), budget, (long long)q.k1_ctas}));
+            plan[c] = k1_plan(q.g, q.g.n3, r.len, want);
+            total += (double)tiles_of(q.g) * plan[c].gz * (plan[c].chunk + kItemCost) + kCtaCost * plan[c].ctas;
+        }
+        const double t = wave == 1 ? hi + kCtaCost : total / sms + 0.5 * hi;
+        if (t < best) { best = t; best_plan.swap(plan); }
+    }
+    for (int c = 0; c < n; ++c) cubes[c].k1 = K1Split{best_plan[c].chunk, best_plan[c].gz, best_plan[c].ctas};
 }
 
 int launch_k1_batch(const BatchCube* cubes, int n, cudaStream_t st) {
@@ -1428,17 +1451,15 @@ int launch_k1_batch(const BatchCube* cubes, int n, cudaStream_t st) {
     static_assert(sizeof(K1BatchTab) <= 32000, "kernel parameter space");
     K1BatchTab t{};
     t.n = n;
-    int chunk[kBatchMax], gz[kBatchMax], ctas[kBatchMax];
-    k1_batch_plan(cubes, n, chunk, gz, ctas);
     int total = 0;
     for (int c = 0; c < n; ++c) {
         const BatchCube& q = cubes[c];
-        t.args[c] = k1_args<float>(q.g, q.b, q.p, q.sc, q.l1, chunk[c], whole_cube(q.g));
+        t.args[c] = k1_args<float>(q.g, q.b, q.p, q.sc, q.l1, q.k1.chunk, whole_cube(q.g));
         const int tx = (q.g.n2 + TX - 1) / TX, ty = (q.g.n1 + TY - 1) / TY;
-        t.gx[c] = tx; t.gy[c] = ty; t.gz[c] = gz[c];
+        t.gx[c] = tx; t.gy[c] = ty; t.gz[c] = q.k1.gz;
         t.maps[c] = q.maps;
         t.start[c] = total;
-        total += ctas[c];
+        total += q.k1.ctas;
     }
     t.start[n] = total;
     k1_tma_batch<<<total, Lay<float>::NT, Lay<float>::SMEM, st>>>(t);
