@@ -1624,9 +1624,14 @@ __global__ void __launch_bounds__(kFinishThreads) k_search_batch(const __grid_co
 }
 __global__ void __launch_bounds__(NT, 3) k2_batch(const __grid_constant__ K2BatchTab t) {
     const int c = batch_cube_of(t.start, t.n, blockIdx.x);
-    // by value: the table is indexed by a run-time cube, so each field is
-    // loaded once instead of at each use
-    const K2Args<float> a = t.c[c];
+    // the cube's arguments in shared memory: by value they did not fit the
+    // registers beside an item's eleven quads (28 bytes spilled)
+    __shared__ __align__(16) unsigned words[sizeof(K2Args<float>) / 4];
+    const K2Args<float>& a = *reinterpret_cast<const K2Args<float>*>(words);
+    static_assert(sizeof(K2Args<float>) % 4 == 0, "copied in words");
+    for (unsigned k = threadIdx.x; k < sizeof(words) / 4; k += NT)
+        words[k] = reinterpret_cast<const unsigned*>(&t.c[c])[k];
+    __syncthreads();
     if (__ldcg(&a.sc->done)) return;
     k2_body(a, (int)blockIdx.x - t.start[c] - 1, t.start[c + 1] - t.start[c] - 1);
 }
@@ -1802,9 +1807,14 @@ int launch_k2_batch(const BatchCube* cubes, int n, cudaStream_t st) {
     K2BatchTab t{};
     t.n = n;
     int total = 0;
-    // the CTAs that fit the GPU, shared out by size (each cube at least one)
+    // CTAs shared out by size (each cube at least one): up to eight times as many as
+    // fit the GPU, as long as a thread has about five quads.  With those that fit it
+    // once, rounded up per cube, a few ran a whole CTA's time after the rest (64 cubes
+    // of 0.05 to 59 million voxels: once 3.13, twice 2.81, four times 2.57, eight
+    // 2.47, sixteen 2.42 ms; 16 of 0.29 million: 47, 41, 47, 63, 71 us).
     double all = 0.0;
     for (int c = 0; c < n; ++c) all += (double)cubes[c].g.cube;
+    const double waves = std::min(8.0, std::max(1.0, all / (20.0 * NT * k2_resident())));
     for (int c = 0; c < n; ++c) {
         const BatchCube& q = cubes[c];
         K2Args<float>& a = t.c[c];
@@ -1817,7 +1827,7 @@ int launch_k2_batch(const BatchCube* cubes, int n, cudaStream_t st) {
         a.part = q.k2_part;
         a.sp = whole_cube(q.g);
         t.start[c] = total;
-        const int share = (int)std::ceil(k2_resident() * ((double)q.g.cube / all));
+        const int share = (int)std::ceil(waves * k2_resident() * ((double)q.g.cube / all));
         a.windows = 1;
         total += std::max(1, std::min({share, k2_grid_part(false, q.g, a.sp), q.k2_cap})) + 1;
     }
