@@ -131,11 +131,12 @@ int gsstv_set_params(gsstv_handle* h, const gsstv_params* p);
 /* on != 0: the passes of a float32 handle take the global sums behind the l1
  * thresholds and the l2-ball scale in one fixed order and rounding, in which
  * gsstv_unrolled_vjp always takes them; 0 (the default): in the order that
- * fills the GPU best, up to 15 % faster.  The iterates of the two agree to
- * float32 rounding, but a threshold that rounds to the neighbouring float moves
- * the FP64 adjoints of a run by 1e-8 to 1e-5: a forward run whose result seeds
- * gsstv_unrolled_vjp is best run with it on.  No effect on 16-bit storage, whose
- * sums always have one order, nor on a batch that runs its cubes in one launch. */
+ * fills the GPU best, up to 15 % faster (cubes of few tiles: up to twice).  The
+ * iterates of the two agree to float32 rounding, but a threshold that rounds to
+ * the neighbouring float moves the FP64 adjoints of a run by 1e-8 to 1e-5: a
+ * forward run whose result seeds gsstv_unrolled_vjp is best run with it on.  No
+ * effect on 16-bit storage, whose sums always have one order, nor on a batch that
+ * runs its cubes in one launch. */
 int gsstv_set_fixed_sums(gsstv_handle* h, int on);
 
 /* Releases every resource of the handle.  NULL is accepted. */

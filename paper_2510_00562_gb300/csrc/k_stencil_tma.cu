@@ -38,9 +38,9 @@
 // Each thread keeps the four y values of its own voxel that the ascent needs,
 // and D^T y2 of the previous band at its own u' position, in registers.
 //
-// What bounds it: instruction issue and the latency of 18 warps' dependency
-// chains (0.85 of the copy bandwidth at 512x512x224, 0.68 at 256x256x128, where
-// the split into whole items leaves 12 % of the band steps idle).
+// What bounds it: instruction issue (63 % of the slots) and the latency of 18
+// warps' dependency chains (0.88 of the copy bandwidth at 512x512x224, 0.77 at
+// 256x256x128, where the split into whole items leaves 12 % of the band steps idle).
 #include <algorithm>
 #include <vector>
 #include <cmath>
@@ -186,8 +186,8 @@ struct K1Stat {
 // in shared memory, one band late; finished pieces join a float pair.  (Sums
 // split otherwise, with a histogram and exact additions, moved one threshold in
 // 32 passes of a 256x256x200 float16 solve by an ulp and the result by up to a
-// float16 place; a pass took 0.91 ms either way, 1.47 ms in the cooperative
-// kernel's launches, and at 512x512x224 bfloat16 3.55 ms, 3.25 and 6.05 ms.)
+// float16 place, and a pass took the same time.  It takes 0.80 ms, 1.47 in the
+// cooperative kernel's launches; at 512x512x224 bfloat16 3.3 and 6.05 ms.)
 //
 // float32 storage with the sums in their fixed order (FIX, gsstv_set_fixed_sums):
 // a thread's Kahan sum over `unit` bands of its own voxel, in one launch shape for
