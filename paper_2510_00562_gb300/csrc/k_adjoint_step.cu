@@ -22,7 +22,7 @@
 //         output is never its input (see launch_adjoint_single).
 //
 // Against the five launches of k_adjoint.cu this moves 91 words a voxel instead
-// of 126 (512x256x64, 8.4 M voxels: SUMS 94, CUBE 199, DUAL 411 us, 4.3 TB/s in
+// of 126 (512x256x64, 8.4 M voxels: SUMS 93, CUBE 203, DUAL 393 us, 4.4 TB/s in
 // all, against 1085 us).  Without the next rows asked into L2 the three took 120,
 // 222 and 451 us.  Runs keep the five launches: their parameter adjoints are FP64
 // outputs summed over the passes, and sums split otherwise move them by 1e-7.
@@ -84,6 +84,11 @@ struct Partial {
     __device__ __forceinline__ void step() {
         if (++n == 32) flush();
     }
+    // the float sums into the pairs at once
+    __device__ __forceinline__ void fold() {
+#pragma unroll
+        for (int k = 0; k < K; ++k) { pair_add(hi[k], lo[k], f[k], 0.f); f[k] = 0.f; }
+    }
     __device__ __forceinline__ void flush() {
         float top = 0.f;
 #pragma unroll
@@ -95,8 +100,7 @@ struct Partial {
                 hi[k] = lo[k] = f[k] = 0.f;
             }
         }
-#pragma unroll
-        for (int k = 0; k < K; ++k) { pair_add(hi[k], lo[k], f[k], 0.f); f[k] = 0.f; }
+        fold();
         n = 0;
     }
 };
@@ -424,7 +428,10 @@ __device__ __forceinline__ void dual_tile(const AdjArgs& a, const DualSet& S, fl
                     buf[(2 * q + 1) * DPL] = ah;
                 }
             }
-            if (SET == 0) om.step();
+            if (SET == 0) {
+                om.fold();                        // (float sums of three terms, as where a thread has one voxel)
+                om.step();
+            }
         }
         __syncthreads();
         if (valid) {

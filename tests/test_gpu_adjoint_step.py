@@ -9,7 +9,7 @@ import torch
 from oracle import adjoint as A
 from oracle import ppds as o
 from paper_2510_00562_gb300 import synth
-from paper_2510_00562_gb300.solver import GRAD_PARAMS, STATE_KEYS, GeoSSTVSolver, make_params
+from paper_2510_00562_gb300.solver import GRAD_PARAMS, STATE_KEYS, STATE_LEAD, GeoSSTVSolver, make_params
 
 pytestmark = pytest.mark.gpu
 
@@ -98,3 +98,20 @@ def test_workspace_follows_the_form():
     for k in STATE_KEYS:
         for g in got[1:]:
             assert rel(g[k].double().cpu().numpy(), got[0][k].double().cpu().numpy()) < 1e-6, k
+
+
+def test_omega_sum_of_long_runs_does_not_drift():
+    """w = (2, 0), y = 0 and an adjoint of (1.3, 0) everywhere make every radial part
+    1.3 exactly, so the adjoint of omega is -g_w1 3 N 1.3 and what is left is the
+    rounding of the sum: one of three terms a band (2^-24 relative) and pairs."""
+    n1, n2, n3 = 192, 384, 32                       # blocks that march over all the bands
+    zero = {k: torch.zeros(STATE_LEAD[k] + (n3, n1, n2), device="cuda") for k in STATE_KEYS}
+    x = dict(zero, w1=zero["w1"].clone())
+    bar = dict(zero, w1=zero["w1"].clone())
+    x["w1"][:, 0], bar["w1"][:, 0] = 2.0, 1.3
+    p = make_params(eps=1.0, alpha=1.0, beta=1.0, omega=0.05, graph_iters=0)
+    with GeoSSTVSolver(n1, n2, n3, p) as sol:
+        sol.load(zero["u"])
+        _, _, pbar = sol.vjp_step(x, zero, bar)
+    want = -p.gamma_w1 * 3 * n1 * n2 * n3 * float(np.float32(1.3))
+    assert pbar["omega"] == pytest.approx(want, rel=2.0 ** -23)
