@@ -1210,14 +1210,19 @@ double run_cost(int nb, int tiles, int len, int ctas) {
     return (double)((items + ctas - 1) / ctas) * (len + kItemCost);
 }
 
+// The fewest runs of nb bands that are shorter than len (past nb where none is): the
+// next split to look at, so that a launch's plan takes some 2 sqrt(nb) steps.
+int next_split(int nb, int len) { return len > 1 ? (nb + len - 2) / (len - 1) : nb + 1; }
+
 // Bands per item for `ctas` persistent CTAs: the split of the bands (in multiples
 // of unit) whose slowest CTA does the fewest band steps.
 int best_run(int nb, int tiles, int ctas, int unit = 1) {
     int best_len = std::min(nb, kMaxRun);
     double best = 1e30;
     int prev = 0;
-    for (int runs = 1; runs <= nb; ++runs) {
+    for (int runs = 1, next; runs <= nb; runs = next) {
         int len = (nb + runs - 1) / runs;
+        next = next_split(nb, len);
         len = (len + unit - 1) / unit * unit;
         if (len == prev || (len > kMaxRun && unit == 1)) continue;
         prev = len;
@@ -1263,8 +1268,9 @@ int fixed_piece(int nb, int tiles) {
     const double sms = (double)device_sms();
     int len_best = nb;
     double best = 1e30;
-    for (int runs = 1; runs <= std::max(1, nb / 8); ++runs) {
+    for (int runs = 1, next; runs <= std::max(1, nb / 8); runs = next) {
         const int len = (nb + runs - 1) / runs;
+        next = next_split(nb, len);
         const double units = (double)tiles * ((nb + len - 1) / len);
         const double waves = std::ceil(units / sms);
         const double waste = (waves - units / sms) / waves + 1.5 / len;
@@ -1399,11 +1405,8 @@ void k1_batch_plan(BatchCube* cubes, int n) {
         const BatchCube& q = cubes[c];
         const int nb = q.g.n3, tiles = tiles_of(q.g);
         const bool own = q.k1_chunk >= 1 && q.k1_chunk <= nb;      // the cube's own (autotuned) run
-        int prev = 0;
-        for (int k = 1; k <= nb; ++k) {
-            const int len = own ? q.k1_chunk : (nb + k - 1) / k;
-            if (len == prev) { if (own) break; continue; }
-            prev = len;
+        for (int k = 1, len; k <= nb; k = own ? nb + 1 : next_split(nb, len)) {
+            len = own ? q.k1_chunk : (nb + k - 1) / k;
             if (len <= kMaxRun) runs[c].push_back({len, (long long)tiles * ((nb + len - 1) / len)});
         }
         all += (double)tiles * (nb + kItemCost);
